@@ -1,0 +1,627 @@
+// Resident leap-frog: a mesh that fits the chip's registers and shared memory is advanced by
+// many steps in one cooperative launch (eqs. 14-15 with eqs. 3-6, and the PML frame's cells).
+//
+// The plain step is two launches per step, each reading its tables again: on a mesh of a few
+// hundred thousand triangles a launch is latency, not bandwidth.  Here every CTA keeps a run of
+// consecutive stored triangles (and of frame cells) for the whole call: one thread holds a
+// triangle's B and its three edges' circulations, coefficients in registers or shared memory, and
+// only B crosses between CTAs.
+//
+// Edges as their triangles see them: with s_q the orientation sign of eq. 4, V_q = s_q U_q.  The
+// triangle is R of the edge exactly when s_q = +1, so eq. 3 reads
+//   V_q = fma(dt|e|/d, rn(b - b_neighbour), V_q)
+// on both sides, rounding as U += (dt|e|/d) rn(B_R - B_L) does (round-to-nearest is odd), and
+// eq. 4 is b = fma(-dt/S, rn(rn(V_0 + V_1) + V_2), b) as it stands.  The current (V and J change
+// sign together) and the source likewise.  Both triangles of an edge compute the same value.
+//
+// Exchange: no grid barrier.  A triangle with a neighbour in another CTA publishes its B as one
+// 64-bit word {value, tag} (FP64: two words), the tag counting steps; readers poll the word until
+// it carries the step they need.  Two words per triangle, alternating: a triangle writes step
+// s + 1 only after its neighbours' step s has arrived, hence after they have read its step s - 1,
+// which the word held.  Per step a CTA polls its remote neighbours once into shared memory, one
+// barrier, then every triangle reads its neighbours there.  All CTAs are resident (cooperative
+// launch) and every wait is bounded: one that runs out sets the error word and ends the launch.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "device.cuh"
+#include "frame.cuh"
+
+namespace ue {
+
+namespace {
+
+constexpr int kFar = 1 << 30;   // neighbour polled by its own thread (the CTA's list is full)
+
+template <typename T>
+struct FlowArgs {
+    const int4* tri;
+    const int2* rl;
+    const T* cU;
+    const double* cB64;
+    T* U;
+    T* B;
+    const T* pb;
+    T* J;
+    T pa, mdt;
+    const int2* hash;
+    unsigned bits;
+    const T* src_c;
+    const int32_t* src_grp;
+    const double* gtab;
+    int gstride;
+    int gbase;              // this launch's first entry in the g table
+    int has_src;
+    int n_t, n_ei, n_ei_pad;
+    int per;                // triangles per CTA
+    int hcap, scap;         // capacities of the CTA's lists: remote neighbours, source edges
+    unsigned long long* slots[2];
+    unsigned* ctl;          // {tag of the next launch, CTAs done, error word}
+    long long* step;
+    int n_steps;
+    int skip;               // tests only (-1 otherwise): this CTA returns at once
+    FrameDev f;
+    T* Uif;                 // circulations of the frame's interface edges
+    int fper;               // frame cells per CTA
+};
+
+// One published value: {32 bits, tag} words.  64-bit accesses are single-copy atomic.
+__device__ __forceinline__ void slot_put(unsigned long long* s, int i, unsigned tag, float v) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(s + i), "l"(w) : "memory");
+}
+__device__ __forceinline__ void slot_put(unsigned long long* s, int i, unsigned tag, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(s + 2 * (size_t)i), "l"(t | (b & 0xFFFFFFFFull)),
+                 "l"(t | (b >> 32))
+                 : "memory");
+}
+template <typename T>
+struct Word;
+template <>
+struct Word<float> {
+    unsigned long long w;
+    __device__ __forceinline__ void load(const unsigned long long* s, int i) {
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(s + i) : "memory");
+    }
+    __device__ __forceinline__ bool ready(unsigned tag) const { return (unsigned)(w >> 32) == tag; }
+    __device__ __forceinline__ float value() const { return __uint_as_float((unsigned)w); }
+};
+template <>
+struct Word<double> {
+    unsigned long long a, b;
+    __device__ __forceinline__ void load(const unsigned long long* s, int i) {
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(s + 2 * (size_t)i) : "memory");
+    }
+    __device__ __forceinline__ bool ready(unsigned tag) const {
+        return (unsigned)(a >> 32) == tag && (unsigned)(b >> 32) == tag;
+    }
+    __device__ __forceinline__ double value() const {
+        return __longlong_as_double((long long)((a & 0xFFFFFFFFull) | (b << 32)));
+    }
+};
+
+// Poll a word until it carries the tag; bounded (about a second of SM clock): false when the
+// wait runs out.
+template <typename T>
+__device__ __forceinline__ bool word_wait(Word<T>& w, const unsigned long long* s, int i, unsigned tag) {
+    if (w.ready(tag)) return true;
+    const long long t0 = clock64();
+    for (unsigned n = 1;; ++n) {
+        w.load(s, i);
+        if (w.ready(tag)) return true;
+        if ((n & 255u) == 0 && clock64() - t0 > (2LL << 30)) return false;
+    }
+}
+
+template <typename T>
+struct Vec4 {
+    T x, y, z, w;
+};
+template <>
+struct __align__(16) Vec4<float> {
+    float x, y, z, w;
+};
+
+template <typename T>
+struct SrcEntry {
+    T c;       // s_q dt |e| a
+    int g;     // offset of its group in the g table
+};
+
+// the source index of stored edge k (k_edge_half's table), or -1
+template <typename T>
+__device__ __forceinline__ int src_index(const FlowArgs<T>& a, int k) {
+    const unsigned size = 1u << a.bits;
+    unsigned h = ((unsigned)k * 2654435761u) >> (32 - a.bits);
+    int2 e = __ldg(a.hash + h);
+    for (unsigned p = 1; e.x != k && p < size; ++p) {
+        h = (h + 1) & (size - 1);
+        e = __ldg(a.hash + h);
+    }
+    return e.x == k ? e.y : -1;
+}
+
+__device__ __forceinline__ bool neg_bit(float c) { return __float_as_uint(c) >> 31; }
+__device__ __forceinline__ bool neg_bit(double c) { return (unsigned long long)__double_as_longlong(c) >> 63; }
+
+// Coefficients sit in registers while they fit beside the state, else in shared memory.
+template <typename T, int TS>
+constexpr bool kCoefRegs = sizeof(T) * TS <= 8;
+
+// Shared memory of a CTA of cap triangle slots.
+template <typename T, bool PLASMA>
+__host__ __device__ constexpr size_t flow_smem(bool coef_regs, int cap, int hcap, int scap) {
+    return (coef_regs ? 0 : sizeof(Vec4<T>) * (size_t)cap * (PLASMA ? 2 : 1)) + sizeof(SrcEntry<T>) * (size_t)scap +
+           2 * sizeof(T) * ((size_t)cap + hcap) + 4 * (size_t)hcap;
+}
+
+// NT: most threads of a CTA; a thread holds local triangles tid + i * blockDim.x, i < TS.
+// SOLO: one CTA holds the whole mesh, nothing is published.
+template <typename T, int NT, int TS, bool PLASMA, bool FRAME, bool SOLO>
+__global__ void __launch_bounds__(NT, 1) k_flow(const FlowArgs<T> a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ int s_hcnt, s_scnt;
+    const int tid = threadIdx.x, nth = blockDim.x, cap = TS * nth;
+    Vec4<T>* C = reinterpret_cast<Vec4<T>*>(smraw);                  // dt|e|/d of the three edges, dt/S
+    constexpr bool CR = kCoefRegs<T, TS>;
+    Vec4<T>* P = C + (CR ? 0 : cap);                                 // pb of the three edges
+    SrcEntry<T>* S = reinterpret_cast<SrcEntry<T>*>(P + (CR || !PLASMA ? 0 : cap));
+    const int bcap = cap + a.hcap;
+    T* Bb = reinterpret_cast<T*>(S + a.scap);                        // two buffers: own, then remote B
+    int* hlist = reinterpret_cast<int*>(Bb + 2 * bcap);
+    const int j0 = blockIdx.x * a.per;
+    const int nloc = max(0, min(a.per, a.n_t - j0));
+    if (tid == 0) s_hcnt = s_scnt = 0;
+    const unsigned tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
+    __syncthreads();
+    bool ok = true;
+    if (SOLO || (int)blockIdx.x != a.skip) {
+        T V[TS][3], J[TS][3], b[TS];
+        Vec4<T> Cr[CR ? TS : 1], Pr[CR && PLASMA ? TS : 1];
+        int nb[TS][3];
+        unsigned fl[TS];   // bits 0-2 source edges, 3 publishes, 4-6 no current on the edge, 8-: first list entry
+        auto remote = [&](int o) {
+            const int pos = atomicAdd(&s_hcnt, 1);
+            if (pos >= a.hcap) return o | kFar;
+            hlist[pos] = o;
+            return cap + pos;
+        };
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = tid + i * nth;
+            fl[i] = 0;
+            b[i] = T(0);
+            if (l >= nloc) continue;
+            const int j = j0 + l;
+            const int4 t = __ldg(a.tri + j);
+            const int code[3] = {t.x, t.y, t.z};
+            T c[3], pb[3];
+            int src[3] = {-1, -1, -1};
+            unsigned f = 0;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int k = code[q] >> 1;
+                const bool neg = code[q] & 1;
+                c[q] = pb[q] = T(0);
+                V[i][q] = T(0);
+                if constexpr (PLASMA) J[i][q] = T(0);
+                nb[i][q] = -1;
+                if (k < a.n_ei) {
+                    const int2 r = __ldg(a.rl + k);
+                    const int o = neg ? r.x : r.y;
+                    const T cu = __ldg(a.cU + k), u = a.U[k];
+                    c[q] = fabs(cu);
+                    V[i][q] = neg ? -u : u;
+                    if constexpr (PLASMA) {
+                        const T jj = a.J[k];
+                        J[i][q] = neg ? -jj : jj;
+                        pb[q] = __ldg(a.pb + k);
+                    }
+                    if (SOLO || (o >= j0 && o < j0 + nloc)) nb[i][q] = o - j0;
+                    else {
+                        nb[i][q] = remote(o);
+                        f |= 8u;
+                    }
+                    if (a.has_src && neg_bit(cu)) src[q] = src_index(a, k);
+                } else if (FRAME && k >= a.n_ei_pad) {
+                    const int e = k - a.n_ei_pad;
+                    const T u = a.Uif[e];
+                    c[q] = ((const T*)a.f.icU)[e];
+                    V[i][q] = neg ? -u : u;
+                    nb[i][q] = remote(a.n_t + a.f.icell[e]);
+                    f |= 8u | (16u << q);
+                }
+            }
+            T cb;
+            if constexpr (sizeof(T) == 4) cb = __int_as_float(t.w);
+            else cb = __ldg(a.cB64 + j);
+            const Vec4<T> cv{c[0], c[1], c[2], cb}, pv{pb[0], pb[1], pb[2], T(0)};
+            if constexpr (CR) Cr[i] = cv;
+            else C[l] = cv;
+            if constexpr (CR && PLASMA) Pr[i] = pv;
+            else if constexpr (PLASMA) P[l] = pv;
+            const int ns = (src[0] >= 0) + (src[1] >= 0) + (src[2] >= 0);
+            if (ns > 0) {
+                int e = atomicAdd(&s_scnt, ns);
+                if (e + ns > a.scap) {
+                    f |= 7u | (0xFFFFu << 8);   // the list is full: looked up again at every step
+                } else {
+                    f |= (unsigned)e << 8;
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (src[q] < 0) continue;
+                        const T sc = __ldg(a.src_c + src[q]);
+                        S[e++] = SrcEntry<T>{(code[q] & 1) ? -sc : sc, (int)__ldg(a.src_grp + src[q]) * a.gstride};
+                        f |= 1u << q;
+                    }
+                }
+            }
+            fl[i] = f;
+            b[i] = a.B[j];
+            Bb[l] = b[i];
+        }
+        // a frame cell: sides X in bottom, top, left, right order, each with the cell's own
+        // counter-clockwise sign, so that every one advances by (own B - neighbour's B)
+        unsigned ifm = 0;   // sides that are interface edges: no decay, one fused multiply-add
+        T X[4], ca[4], cd[4], Bx = T(0), By = T(0), ax = T(0), bx = T(0), ay = T(0), by = T(0);
+        int cn[4];
+        const int cell = FRAME ? (int)blockIdx.x * a.fper + tid : 0;
+        const bool has_cell = FRAME && tid < a.fper && cell < (int)a.f.n_fc;
+        int I = 0, Jc = 0;
+        if constexpr (FRAME) {
+            if (has_cell) {
+                const FrameDev& f = a.f;
+                const Tab<T> tb = tabs<T>(f);
+                frame_ij(f, cell, I, Jc);
+                const bool in_x = I >= f.W && I < f.W + f.nx, in_y = Jc >= f.W && Jc < f.W + f.ny;
+                const int di[4] = {0, 0, -1, 1}, dj[4] = {-1, 1, 0, 0};
+                // interface edge on that side, or -1
+                const int kif[4] = {in_x && Jc == f.W + f.ny ? f.nx + (I - f.W) : -1, in_x && Jc == f.W - 1 ? I - f.W : -1,
+                                    in_y && I == f.W + f.nx ? 2 * f.nx + f.ny + (Jc - f.W) : -1,
+                                    in_y && I == f.W - 1 ? 2 * f.nx + (Jc - f.W) : -1};
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    X[d] = ca[d] = cd[d] = T(0);
+                    cn[d] = -1;
+                    if (frame_is_cell(f, I + di[d], Jc + dj[d])) {
+                        if (d < 2) {
+                            const int at = Jc + d;
+                            const T u = ((const T*)f.H)[(int64_t)at * f.NX + I];
+                            X[d] = d == 0 ? u : -u;
+                            ca[d] = tb.aH[at];
+                            cd[d] = tb.bH[at];
+                        } else {
+                            const int at = I + (d - 2);
+                            const T u = ((const T*)f.V)[(int64_t)Jc * (f.NX + 1) + at];
+                            X[d] = d == 2 ? -u : u;
+                            ca[d] = tb.aV[at];
+                            cd[d] = tb.bV[at];
+                        }
+                        cn[d] = remote(a.n_t + (int)frame_cell(f, I + di[d], Jc + dj[d]));
+                    } else if (kif[d] >= 0) {
+                        const int code = f.itri[kif[d]];
+                        const T u = a.Uif[kif[d]];
+                        X[d] = code >= 0 ? -u : u;
+                        ifm |= 1u << d;
+                        cd[d] = ((const T*)f.icU)[kif[d]];
+                        cn[d] = remote(code >= 0 ? code : ~code);
+                    }
+                }
+                Bx = ((const T*)f.Bx)[cell];
+                By = ((const T*)f.By)[cell];
+                ax = tb.axc[I];
+                bx = tb.bxc[I];
+                ay = tb.ayc[Jc];
+                by = tb.byc[Jc];
+            }
+        }
+        if constexpr (!SOLO) {
+            // published only after this thread's reads of U, J and the frame are done: their
+            // owners write them back after later steps
+            __threadfence();
+#pragma unroll
+            for (int i = 0; i < TS; ++i)
+                if (fl[i] & 8u) slot_put(a.slots[0], j0 + tid + i * nth, tag0, b[i]);
+            if (has_cell) slot_put(a.slots[0], a.n_t + cell, tag0, rn_add(Bx, By));
+        }
+        __syncthreads();
+        const int hn = SOLO ? 0 : min(s_hcnt, a.hcap);
+        auto near = [&](const T* Bp, int p, unsigned tag, int n) -> T {
+            if (SOLO || !(n & kFar)) return Bp[n];
+            Word<T> w;
+            w.load((p ? a.slots[1] : a.slots[0]), n & ~kFar);
+            if (!word_wait(w, (p ? a.slots[1] : a.slots[0]), n & ~kFar, tag)) ok = false;
+            return w.value();
+        };
+#pragma unroll 1
+        for (int s = 1; s <= a.n_steps; ++s) {
+            const int p = (s - 1) & 1;
+            const unsigned tag = tag0 + (unsigned)(s - 1);
+            T* Bp = Bb + (p ? bcap : 0);
+            T* Bn = Bb + (p ? 0 : bcap);
+            if constexpr (SOLO) {
+                if (s > 1) __syncthreads();
+            } else {
+                // the remote neighbours' B of the last step, a few polls in flight per thread
+                constexpr int kPoll = 4;
+                for (int e0 = tid; e0 < hn; e0 += kPoll * nth) {
+                    Word<T> w[kPoll];
+#pragma unroll
+                    for (int u = 0; u < kPoll; ++u)
+                        if (e0 + u * nth < hn) w[u].load((p ? a.slots[1] : a.slots[0]), hlist[e0 + u * nth]);
+#pragma unroll
+                    for (int u = 0; u < kPoll; ++u) {
+                        const int e = e0 + u * nth;
+                        if (e < hn) {
+                            if (!word_wait(w[u], (p ? a.slots[1] : a.slots[0]), hlist[e], tag)) ok = false;
+                            Bp[cap + e] = w[u].value();
+                        }
+                    }
+                }
+                ok = __syncthreads_and(ok ? 1 : 0) != 0;
+                if (!ok) break;
+            }
+#pragma unroll
+            for (int i = 0; i < TS; ++i) {
+                const int l = tid + i * nth;
+                if (l >= nloc) break;
+                Vec4<T> c, pv;
+                if constexpr (CR) c = Cr[i];
+                else c = C[l];
+                if constexpr (CR && PLASMA) pv = Pr[i];
+                else if constexpr (PLASMA) pv = P[l];
+                const T cq[3] = {c.x, c.y, c.z};
+                const T pq[3] = {PLASMA ? pv.x : T(0), PLASMA ? pv.y : T(0), PLASMA ? pv.z : T(0)};
+                T nv[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) nv[q] = nb[i][q] >= 0 ? near(Bp, p, tag, nb[i][q]) : b[i];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const T uo = V[i][q];
+                    T un = rn_fma(cq[q], rn_sub(b[i], nv[q]), uo);
+                    if constexpr (PLASMA) {
+                        if (!FRAME || !(fl[i] & (16u << q))) {
+                            const T jn = rn_fma(a.pa, J[i][q], rn_mul(pq[q], uo));
+                            un = rn_fma(a.mdt, jn, un);
+                            J[i][q] = nb[i][q] >= 0 ? jn : T(0);
+                        }
+                    }
+                    V[i][q] = nb[i][q] >= 0 ? un : T(0);   // a conductor's edge stays 0
+                }
+                if (fl[i] & 7u) {
+                    int e = (int)(fl[i] >> 8);
+                    if (e != 0xFFFF) {
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) {
+                            if (!((fl[i] >> q) & 1u)) continue;
+                            const SrcEntry<T> se = S[e++];
+                            V[i][q] = rn_fma(se.c, (T)__ldg(a.gtab + se.g + a.gbase + s - 1), V[i][q]);
+                        }
+                    } else {
+                        const int4 t = __ldg(a.tri + j0 + l);
+                        const int code[3] = {t.x, t.y, t.z};
+#pragma unroll
+                        for (int q = 0; q < 3; ++q) {
+                            const int k = code[q] >> 1;
+                            if (k >= a.n_ei || !neg_bit(__ldg(a.cU + k))) continue;
+                            const int x = src_index(a, k);
+                            if (x < 0) continue;
+                            const T sc = __ldg(a.src_c + x);
+                            const T g = (T)__ldg(a.gtab + (size_t)__ldg(a.src_grp + x) * a.gstride + a.gbase + s - 1);
+                            V[i][q] = rn_fma((code[q] & 1) ? -sc : sc, g, V[i][q]);
+                        }
+                    }
+                }
+                b[i] = rn_fma(-c.w, rn_add(rn_add(V[i][0], V[i][1]), V[i][2]), b[i]);
+                Bn[l] = b[i];
+                if constexpr (!SOLO) {
+                    if ((fl[i] & 8u) && s < a.n_steps) slot_put((p ? a.slots[0] : a.slots[1]), j0 + l, tag + 1u, b[i]);
+                }
+            }
+            if constexpr (FRAME) {
+                if (has_cell) {
+                    const T F = rn_add(Bx, By);
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) {
+                        if (cn[d] < 0) continue;
+                        const T df = rn_sub(F, near(Bp, p, tag, cn[d]));
+                        X[d] = (ifm >> d) & 1u ? rn_fma(cd[d], df, X[d]) : rn_fma(ca[d], X[d], rn_mul(cd[d], df));
+                    }
+                    Bx = rn_sub(rn_mul(ax, Bx), rn_mul(bx, rn_add(X[3], X[2])));
+                    By = rn_sub(rn_mul(ay, By), rn_mul(by, rn_add(X[0], X[1])));
+                    if (s < a.n_steps) slot_put((p ? a.slots[0] : a.slots[1]), a.n_t + cell, tag + 1u, rn_add(Bx, By));
+                }
+            }
+        }
+        if (!SOLO) ok = __syncthreads_and(ok ? 1 : 0) != 0;
+        if (ok) {
+            if (!SOLO) __threadfence();
+            // each edge by its R triangle, each interface edge by its triangle, each frame side
+            // by the cell above or to its right
+#pragma unroll
+            for (int i = 0; i < TS; ++i) {
+                const int l = tid + i * nth;
+                if (l >= nloc) break;
+                const int4 t = __ldg(a.tri + j0 + l);
+                const int code[3] = {t.x, t.y, t.z};
+                a.B[j0 + l] = b[i];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int k = code[q] >> 1;
+                    const bool neg = code[q] & 1;
+                    if (k < a.n_ei) {
+                        if (neg) continue;
+                        a.U[k] = V[i][q];
+                        if constexpr (PLASMA) a.J[k] = J[i][q];
+                    } else if (FRAME && k >= a.n_ei_pad) {
+                        a.Uif[k - a.n_ei_pad] = neg ? -V[i][q] : V[i][q];
+                    }
+                }
+            }
+            if constexpr (FRAME) {
+                if (has_cell) {
+                    ((T*)a.f.Bx)[cell] = Bx;
+                    ((T*)a.f.By)[cell] = By;
+                    if (frame_is_cell(a.f, I, Jc - 1)) ((T*)a.f.H)[(int64_t)Jc * a.f.NX + I] = X[0];
+                    if (frame_is_cell(a.f, I - 1, Jc)) ((T*)a.f.V)[(int64_t)Jc * (a.f.NX + 1) + I] = -X[2];
+                }
+            }
+        }
+    }
+    if (tid == 0) {
+        if (!ok) atomicOr(a.ctl + 2, 1u);
+        if (blockIdx.x == 0) *a.step += a.n_steps;
+        if constexpr (!SOLO) {
+            // the last CTA moves the tags on: every CTA has read this launch's by then
+            __threadfence();
+            if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
+                a.ctl[1] = 0u;
+                a.ctl[0] = tag0 + (unsigned)a.n_steps + 1u;
+                __threadfence();
+            }
+        }
+    }
+}
+
+__global__ void k_flow_init(unsigned* ctl) {
+    if (threadIdx.x == 0) {
+        ctl[0] = 1u;   // words start with tag 0
+        ctl[1] = ctl[2] = 0u;
+    }
+}
+
+struct FlowShape {
+    int nt, ts;        // most threads, slots per thread
+};
+constexpr FlowShape kShapes[3] = {{1024, 1}, {1024, 2}, {512, 8}};
+
+template <typename T, bool PLASMA, bool FRAME, bool SOLO, int SH>
+cudaError_t launch_shape(const FlowArgs<T>& a, int grid, int threads, cudaStream_t s) {
+    auto kern = k_flow<T, kShapes[SH].nt, kShapes[SH].ts, PLASMA, FRAME, SOLO>;
+    const size_t smem = flow_smem<T, PLASMA>(kCoefRegs<T, kShapes[SH].ts>, kShapes[SH].ts * threads, a.hcap, a.scap);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = SOLO ? 0 : 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <typename T, bool PLASMA, bool FRAME>
+cudaError_t launch_flow_pf(const FlowArgs<T>& a, const FlowDev& fl, cudaStream_t s) {
+    if (fl.grid == 1) {
+        if constexpr (FRAME) return cudaErrorInvalidValue;
+        else {
+            if (fl.shape == 0) return launch_shape<T, PLASMA, false, true, 0>(a, 1, fl.threads, s);
+            return launch_shape<T, PLASMA, false, true, 1>(a, 1, fl.threads, s);
+        }
+    }
+    if (fl.shape == 0) return launch_shape<T, PLASMA, FRAME, false, 0>(a, fl.grid, fl.threads, s);
+    if (fl.shape == 1) return launch_shape<T, PLASMA, FRAME, false, 1>(a, fl.grid, fl.threads, s);
+    if constexpr (sizeof(T) == 4) return launch_shape<T, PLASMA, FRAME, false, 2>(a, fl.grid, fl.threads, s);
+    return cudaErrorInvalidValue;
+}
+
+template <typename T>
+cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
+    FlowArgs<T> a;
+    a.tri = m.tri;
+    a.rl = m.rl;
+    a.cU = (const T*)m.cU;
+    a.cB64 = (const double*)m.cB;
+    a.U = (T*)m.U;
+    a.B = (T*)m.B;
+    a.pb = (const T*)m.pb;
+    a.J = (T*)m.J;
+    a.pa = (T)m.pa;
+    a.mdt = (T)(-m.dt);
+    a.hash = m.src_hash;
+    a.bits = (unsigned)m.src_bits;
+    a.src_c = (const T*)m.src_c;
+    a.src_grp = m.src_grp;
+    a.gtab = m.gtab;
+    a.gstride = m.gtab_size;
+    a.gbase = gbase;
+    a.has_src = m.n_src > 0;
+    a.n_t = (int)m.n_t;
+    a.n_ei = (int)m.n_ei;
+    a.n_ei_pad = (int)m.n_ei_pad;
+    a.per = fl.per;
+    a.hcap = fl.hcap;
+    a.scap = fl.scap;
+    a.slots[0] = fl.slots;
+    a.slots[1] = fl.slots + fl.slot_words;
+    a.ctl = fl.ctl;
+    a.step = m.step;
+    a.n_steps = n_steps;
+    a.skip = fl.skip;
+    if (m.frame) a.f = *m.frame;
+    a.Uif = (T*)Uif;
+    a.fper = fl.fper;
+    if (m.frame) return m.plasma ? launch_flow_pf<T, true, true>(a, fl, s) : launch_flow_pf<T, false, true>(a, fl, s);
+    return m.plasma ? launch_flow_pf<T, true, false>(a, fl, s) : launch_flow_pf<T, false, false>(a, fl, s);
+}
+
+constexpr size_t kFlowSmem = 226 * 1024;
+
+}  // namespace
+
+bool flow_plan(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
+    fl = FlowDev();
+    if (n_t < 1 || sms < 1 || n_t + n_fc >= kFar / 2) return false;
+    const int esz = f64 ? 8 : 4;
+    if (n_fc == 0 && n_t <= 2048) {
+        fl.grid = 1;
+        fl.shape = n_t <= 1024 ? 0 : 1;
+        fl.per = (int)n_t;
+    } else {
+        const int64_t per = (n_t + sms - 1) / sms, fper = (n_fc + sms - 1) / sms;
+        fl.shape = -1;
+        for (int i = 0; i < (f64 ? 2 : 3) && fl.shape < 0; ++i)
+            if (per <= (int64_t)kShapes[i].nt * kShapes[i].ts && fper <= kShapes[i].nt) fl.shape = i;
+        if (fl.shape < 0) return false;
+        fl.per = (int)((per + 31) / 32 * 32);
+        fl.per = std::min(fl.per, kShapes[fl.shape].nt * kShapes[fl.shape].ts);
+        fl.grid = std::max((int)((n_t + fl.per - 1) / fl.per), 2);
+        fl.fper = (int)((n_fc + fl.grid - 1) / fl.grid);
+        if (fl.fper > kShapes[fl.shape].nt) return false;
+    }
+    const int ts = kShapes[fl.shape].ts;
+    int threads = std::max((fl.per + ts - 1) / ts, fl.fper);
+    fl.threads = std::min((threads + 31) / 32 * 32, kShapes[fl.shape].nt);
+    const int cap = ts * fl.threads;
+    // what shared memory the coefficients (with a current's, which may come later) and the own
+    // B values leave goes to the lists: source edges, then remote neighbours
+    const bool cr = (f64 ? 8 : 4) * ts <= 8;   // kCoefRegs
+    const size_t fixed = f64 ? flow_smem<double, true>(cr, cap, 0, 0) : flow_smem<float, true>(cr, cap, 0, 0);
+    if (fixed + 8192 > kFlowSmem) return false;
+    const size_t left = kFlowSmem - fixed;
+    fl.scap = (int)std::min<size_t>(std::min(3 * cap, 0x8000), left / 3 / (f64 ? 16 : 8)) & ~1;
+    if (fl.grid > 1)
+        fl.hcap = (int)std::min<size_t>((size_t)3 * cap + 4 * (size_t)fl.fper,
+                                        (left - (size_t)fl.scap * (f64 ? 16 : 8)) / (2 * esz + 4)) & ~3;
+    fl.slot_words = fl.grid > 1 ? (n_t + n_fc) * (f64 ? 2 : 1) : 0;
+    return true;
+}
+
+cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s) {
+    k_flow_init<<<1, 32, 0, s>>>(fl.ctl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
+    if (n_steps < 1) return cudaErrorInvalidValue;
+    return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, Uif, n_steps, gbase, s)
+                                       : launch_flow_t<float>(fl, m, Uif, n_steps, gbase, s);
+}
+
+}  // namespace ue

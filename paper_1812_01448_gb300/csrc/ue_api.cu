@@ -1073,6 +1073,8 @@ int fields_f32(ue_mesh* m, float* E, float* B, float* j, bool write, cudaStream_
         if (!write) std::memset(j, 0, 4 * (size_t)h.n_edges);   // no current in this medium
         j = nullptr;
     }
+    const int mrc = ensure_caller_maps(m, s);   // a batch has none until its first transfer
+    if (mrc != UE_OK) return mrc;
     const void *dE = nullptr, *dB = nullptr, *dj = nullptr;
     const bool direct = direct_transfer(m, E, B, j, 4, dE, dB, dj);
     if (!direct) {

@@ -121,7 +121,8 @@ typedef struct ue_options {
     int32_t test_skip_cta; /* tests only (-1 otherwise): UE_VARIANT_PERSISTENT: this CTA     */
                            /* never arrives at the grid barrier; UE_VARIANT_BLOCKED: this CTA */
                            /* of the pipelined forms waits for record bytes that never come.  */
-                           /* Either way the bounded wait runs out: UE_ERR_TIMEOUT            */
+                           /* UE_VARIANT_PLAIN: this CTA of the resident launch returns at    */
+                           /* once.  Each way the bounded wait runs out: UE_ERR_TIMEOUT       */
 } ue_options;
 
 typedef struct ue_stats_t {
@@ -139,6 +140,7 @@ typedef struct ue_stats_t {
     int64_t direct_fields;       /* field arrays that ue_write_fields / ue_read_fields moved  */
                                  /* in place in pinned host memory (no staging copy)          */
     int32_t tb_kernel_used;      /* UE_VARIANT_BLOCKED: the kernel its launches run (UE_TBK_*) */
+                                 /* (long calls on small meshes run resident: ue_step_n)      */
     int32_t reserved2;
 } ue_stats_t;
 
@@ -223,7 +225,11 @@ int ue_exchange_tris(ue_mesh* m, const int32_t* ids, int64_t n, void* buf, int32
 int ue_write_fields_f32(ue_mesh* m, const float* E, const float* B, const float* j, void* stream);
 int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
 
-/* Advance n_steps leap-frog steps, asynchronously on `stream`.  Errors of the launches are
+/* Advance n_steps leap-frog steps, asynchronously on `stream`.  A call of a graph chunk of steps
+ * or more on a mesh small enough for the chip's registers and shared memory (about 600k triangles
+ * in FP32, 300k in FP64; plain and blocked variants, graph_chunk >= 0) runs resident: one
+ * cooperative launch for up to 1024 steps, with the same results bit for bit.  Its waits are
+ * bounded; one that runs out is reported by ue_check (UE_ERR_TIMEOUT).  Errors of the launches are
  * reported here; device-side conditions surface at the next synchronous call. */
 int ue_step_n(ue_mesh* m, int64_t n_steps, void* stream);
 

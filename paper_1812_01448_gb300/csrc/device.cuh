@@ -232,6 +232,24 @@ int persistent_grid(int device);
 cudaError_t launch_persistent(const DevMesh& m, int n_steps, unsigned* sync, int* err,
                               long long budget, int skip_cta, int grid, cudaStream_t s);
 
+// Resident step (kernels_flow.cu): the launch shape for a mesh that fits the chip, its exchange
+// words and its control words {tag of the next launch, CTAs done, error}.
+constexpr int kFlowSteps = 1024;  // most steps of one resident launch (and its g table)
+struct FlowDev {
+    int grid = 0;                 // CTAs; 0: the mesh does not fit, 1: one CTA holds it all
+    int threads = 0, shape = 0, per = 0, fper = 0, hcap = 0, scap = 0;
+    unsigned long long* slots = nullptr;   // 2 * slot_words, zeroed
+    int64_t slot_words = 0;
+    unsigned* ctl = nullptr;
+    int skip = -1;                // tests only: this CTA returns at once
+};
+// n_fc: cells of a PML frame stepped with the mesh.  False when the mesh does not fit.
+bool flow_plan(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl);
+cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s);
+// n_steps steps of m in place in one launch; the source uses g-table entries gbase ..
+// gbase + n_steps - 1.  Uif: the circulations of a frame's interface edges.
+cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s);
+
 // Launchers (kernels_step.cu).
 // g(t) table for the next `count` steps (no-op without a source).
 cudaError_t launch_gtab(const DevMesh& m, int count, cudaStream_t s);

@@ -25,6 +25,7 @@ namespace {
 
 thread_local std::string g_err;
 
+
 int fail(int code, const std::string& msg) {
     g_err = msg;
     return code;
@@ -117,6 +118,7 @@ struct ue_mesh {
     int tb_threads = 512;
     int tb_kernel = UE_TB_SPLIT;
     int tb_test_cta = -1;
+    int flow_skip = -1;
     int cur = 0;                     // buffer holding the current fields
 
     // dt selection
@@ -135,6 +137,10 @@ struct ue_mesh {
     long long p_budget = 0;
     int p_skip = -1;
     int p_grid = 0;
+
+    // resident step (kernels_flow.cu); grid 0: the mesh does not fit, or a test or an option
+    // asks for the launches
+    ue::FlowDev flow;
 
     // PML frame
     FrameHost fr;
@@ -935,8 +941,22 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
          alloc_into(m, dm.U, dm.n_ei_pad + (n_if + 3) / 4 * 4, esz, s) &&
          alloc_into(m, dm.B, dm.n_t_pad, esz, s) && alloc_into(m, dm.step, 1, 8, s);
     if (ok && m->precision == UE_PREC_FP64) ok = alloc_into(m, dm.cB, dm.n_t_pad, 8, s);
+    m->flow = ue::FlowDev();
+    if (m->variant != UE_VARIANT_PERSISTENT && m->graph_chunk > 0 && m->tb_test_cta < 0) {
+        int dev = 0, sms = 0, coop = 0;
+        UE_CUDA(cudaGetDevice(&dev));
+        UE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        const int64_t W = m->fr.W, NX = m->fr.nx + 2 * W;
+        const int64_t n_fc = 2 * W * NX + 2 * W * m->fr.ny;
+        if (coop && ue::flow_plan(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) {
+            m->flow.skip = m->flow_skip;
+            ok = ok && alloc_into(m, m->flow.ctl, 4, 4, s) &&
+                 (m->flow.slot_words == 0 || alloc_into(m, m->flow.slots, 2 * m->flow.slot_words, 8, s));
+        }
+    }
     {
-        int g = 64;
+        int g = m->flow.grid > 0 ? ue::kFlowSteps : 64;
         if (m->graph_chunk > g) g = m->graph_chunk;
         if (m->variant == UE_VARIANT_BLOCKED && tb_chunk_launches(m) * m->block_depth > g)
             g = tb_chunk_launches(m) * m->block_depth;
@@ -948,9 +968,14 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         dev_free_all(m, s);
         m->d_tri_nb = nullptr;
         m->d_kof = m->d_inv = nullptr;
+        m->flow = ue::FlowDev();
         return fail(UE_ERR_ALLOC, "device allocation failed");
     }
     {
+        if (m->flow.grid > 0) {
+            UE_CUDA(ue::launch_flow_init(m->flow, s));
+            if (m->flow.slot_words > 0) UE_CUDA(cudaMemsetAsync(m->flow.slots, 0, 16 * m->flow.slot_words, s));
+        }
         const double w0[4] = {0.0, 0.0, m->watchdog_growth, 0.0};
         UE_CUDA(cudaMemcpyAsync(m->wd, w0, sizeof(w0), cudaMemcpyHostToDevice, s));
         UE_CUDA(cudaStreamSynchronize(s));
@@ -1028,7 +1053,7 @@ bool direct_transfer(const ue_mesh* m, const void* E, const void* B, const void*
 
 // The watchdog words (energy, reference, growth limit, flag) and the error words reset in one
 // launch: values travel as kernel arguments, so no host buffer outlives the call.
-__global__ void k_rearm(double* wd, double growth, int* p_err, unsigned* tb_err) {
+__global__ void k_rearm(double* wd, double growth, int* p_err, unsigned* tb_err, unsigned* flow_err) {
     if (threadIdx.x != 0) return;
     wd[0] = 0.0;
     wd[1] = 0.0;
@@ -1036,6 +1061,7 @@ __global__ void k_rearm(double* wd, double growth, int* p_err, unsigned* tb_err)
     wd[3] = 0.0;
     if (p_err) *p_err = 0;
     if (tb_err) *tb_err = 0u;
+    if (flow_err) *flow_err = 0u;
 }
 
 __global__ void k_put_step(long long* step, long long v) {
@@ -1046,7 +1072,7 @@ __global__ void k_put_step(long long* step, long long v) {
 int rearm(ue_mesh* m, cudaStream_t s) {
     m->since_check = 0;
     unsigned* tb_err = (m->variant == UE_VARIANT_BLOCKED && m->tb.done) ? m->tb.done + 1 : nullptr;
-    k_rearm<<<1, 32, 0, s>>>(m->wd, m->watchdog_growth, m->p_err, tb_err);
+    k_rearm<<<1, 32, 0, s>>>(m->wd, m->watchdog_growth, m->p_err, tb_err, m->flow.ctl ? m->flow.ctl + 2 : nullptr);
     UE_CUDA(cudaGetLastError());
     return UE_OK;
 }
@@ -1058,6 +1084,39 @@ int flush_step(ue_mesh* m, cudaStream_t s) {
     k_put_step<<<1, 32, 0, s>>>(m->dm.step, (long long)m->step_pending);
     UE_CUDA(cudaGetLastError());
     m->step_pending = -1;
+    return UE_OK;
+}
+
+// n steps by the resident kernel, in place in the current field buffer.  `unit`: the steps between
+// watchdog checks of the launches this replaces.  *used is false, and nothing stepped, when the
+// device cannot hold the launch's CTAs at once (the caller then makes its launches).
+int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) {
+    DevMesh& dm = m->dm;
+    const int64_t most = m->watchdog_every > 0 ? unit : dm.n_src > 0 ? (int64_t)dm.gtab_size : ue::kFlowSteps;
+    void* Uif = nullptr;
+    if (m->has_reg) Uif = (float*)m->reg.dm.U + m->reg.f.u_off;
+    else if (m->fr.W > 0) Uif = (char*)dm.U + (m->precision == UE_PREC_FP64 ? 8 : 4) * dm.n_ei_pad;
+    DevMesh v = dm;
+    v.frame = m->fr.W > 0 ? &m->fd : nullptr;
+    int64_t launched = 0;
+    *used = true;
+    for (int64_t left = n; left > 0;) {
+        const int batch = (int)std::min(left, most);
+        UE_CUDA(ue::launch_gtab(dm, batch, s));
+        const cudaError_t e = ue::launch_flow(m->flow, v, Uif, batch, 0, s);
+        if (e == cudaErrorCooperativeLaunchTooLarge && left == n) {
+            cudaGetLastError();
+            m->flow.grid = 0;
+            *used = false;
+            return UE_OK;
+        }
+        UE_CUDA(e);
+        launched += 1 + (dm.n_src > 0 ? 1 : 0);
+        left -= batch;
+        UE_CUDA(watchdog_tick(m, batch, s, &launched));
+    }
+    m->steps_done += n;
+    m->launches += launched;
     return UE_OK;
 }
 
@@ -1291,6 +1350,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     m->built = false;
     m->dm = DevMesh();
     m->tb = ue::TBDev();
+    m->flow = ue::FlowDev();
     m->fd = ue::FrameDev();
     m->has_reg = false;
     m->reg = ue::RegionDev();
@@ -1302,6 +1362,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     if (o.tb_kernel != UE_TB_SPLIT && o.tb_kernel != UE_TB_FUSED) return fail(UE_ERR_ARG, "tb_kernel must be UE_TB_SPLIT or UE_TB_FUSED");
     m->tb_kernel = o.tb_kernel;
     m->tb_test_cta = m->variant == UE_VARIANT_BLOCKED ? o.test_skip_cta : -1;
+    m->flow_skip = m->variant == UE_VARIANT_PLAIN ? o.test_skip_cta : -1;
     m->precision = o.precision;
     m->graph_chunk = o.graph_chunk == 0 ? 32 : o.graph_chunk;
     if (o.watchdog_every < 0 || !(o.watchdog_growth > 1.0))
@@ -1824,6 +1885,15 @@ int ue_step_n(ue_mesh* m, int64_t n, void* stream) {
         m->launches += launched;
         return UE_OK;
     }
+    if (m->flow.grid > 0) {
+        const int64_t unit = m->variant == UE_VARIANT_BLOCKED ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
+        // calls of a graph chunk or more, which would replay graphs; shorter ones launch step by step
+        if (n >= unit) {
+            bool used = false;
+            const int rc = flow_steps(m, n, unit, s, &used);
+            if (rc != UE_OK || used) return rc;
+        }
+    }
     if (m->variant == UE_VARIANT_BLOCKED) {
         const int64_t k = m->block_depth;
         const int64_t chunk = (int64_t)tb_chunk_launches(m) * k;
@@ -1901,6 +1971,7 @@ int ue_step_prepare(ue_mesh* m, void* stream) {
         }
         return UE_OK;
     }
+    if (m->flow.grid > 0) return UE_OK;   // the calls long enough for a graph run resident
     const int rc = ensure_graph(m);
     if (rc != UE_OK) return rc;
     UE_CUDA(cudaGraphUpload(m->gexec, s));
@@ -1981,6 +2052,14 @@ int ue_check(ue_mesh* m, double* W, int32_t* flag) {
         if (e) {
             if (flag) *flag = 3;
             return fail(UE_ERR_TIMEOUT, "a copy wait of the pipelined blocked kernel ran out of time");
+        }
+    }
+    if (m->flow.ctl) {
+        unsigned e = 0;
+        UE_CUDA(cudaMemcpy(&e, m->flow.ctl + 2, 4, cudaMemcpyDeviceToHost));
+        if (e) {
+            if (flag) *flag = 3;
+            return fail(UE_ERR_TIMEOUT, "a wait of the resident step kernel ran out of time");
         }
     }
     if (wd[3] != 0.0)

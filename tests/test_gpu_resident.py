@@ -1,0 +1,156 @@
+"""The resident step (one cooperative launch for many steps) against the plain launches, bit for
+bit: every medium, precision and order it takes, at the edges of its launch shapes."""
+import math
+
+import numpy as np
+import pytest
+
+import meshgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ue():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1812_01448_gb300 import build
+    build.build()
+    import paper_1812_01448_gb300 as ue
+    return ue
+
+
+def _lattice(n_t, seed, shuffle=False):
+    """About n_t triangles: a strip of equilateral rows cut to exactly n_t, jittered, the caller's
+    triangle order shuffled on request."""
+    rows = max(1, int(math.sqrt(n_t / 2)))
+    cols = -(-n_t // (2 * rows))
+    r, c = np.meshgrid(np.arange(rows + 1), np.arange(cols + 1), indexing="ij")
+    xy = np.stack([(c + 0.5 * r).ravel(), (math.sqrt(3) / 2 * r).ravel()], axis=1).astype(np.float64)
+    w = cols + 1
+    p = (np.arange(rows)[:, None] * w + np.arange(cols)[None, :]).ravel()
+    tris = np.stack([np.stack([p, p + 1, p + w], 1), np.stack([p + 1, p + w + 1, p + w], 1)], 1).reshape(-1, 3)[:n_t]
+    rng = np.random.default_rng(seed)
+    xy = (xy + rng.uniform(-0.08, 0.08, xy.shape)) / max(rows, cols)
+    if shuffle:
+        tris = tris[rng.permutation(len(tris))]
+    used = np.zeros(len(xy), bool)
+    used[tris.ravel()] = True
+    return xy[used], (np.cumsum(used) - 1)[tris].astype(np.int32), 1.0 / max(rows, cols)
+
+
+def _run(ue, xy, tris, h, steps, chunk, load=None, plasma=False, source=True, frame=0, calls=1, **opt):
+    m = ue.Mesh(xy, tris, **(load or {}))
+    if frame:
+        m.frame_attach(frame)
+    m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=chunk, **opt)
+    w0 = 2.0 / h
+    if source:
+        ids, amp = meshgen.source_line_amplitudes(xy, tris, float(xy[:, 0].mean()), h)
+        if ids.size:
+            m.set_source(ids, amp, w0, 0.0, 0.3)
+    if plasma:
+        m.set_plasma((0.3 / h) ** 2 * (1 + xy[:, 0]), 0.5)
+    rng = np.random.default_rng(3)
+    B, E, j = rng.standard_normal(m.n_tris), rng.standard_normal(m.n_edges), rng.standard_normal(m.n_edges)
+    m.write_fields(E, B, j if plasma else None)
+    m.set_step(7)
+    for _ in range(calls):
+        m.step_n(steps)
+    assert m.check()[0]
+    out = list(m.read_fields(j=plasma))[:3 if plasma else 2]
+    if frame:
+        out += list(m.frame_fields())
+    out += [m.get_step(), m.energy(), m.stats()["kernel_launches"]]
+    m.close()
+    return out
+
+
+def _same(a, b):
+    for x, y in zip(a[:-1], b[:-1]):
+        assert np.array_equal(x, y)
+    assert a[-1] < b[-1]      # the resident calls launch fewer kernels
+
+
+@pytest.mark.parametrize("n_t", [1, 2, 33, 1024, 1025, 2048, 2049, 2081, 4865])
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("plasma", [False, True])
+def test_resident_is_bit_identical_to_plain(ue, n_t, fp64, plasma):
+    xy, tris, h = _lattice(n_t, n_t)
+    kw = dict(plasma=plasma, calls=2, precision=ue.UE_PREC_FP64 if fp64 else ue.UE_PREC_FP32)
+    _same(_run(ue, xy, tris, h, 45, 32, **kw), _run(ue, xy, tris, h, 45, -1, **kw))
+
+
+@pytest.mark.parametrize("n_t", [155_648, 155_649, 311_297, 622_592])
+@pytest.mark.parametrize("plasma", [False, True])
+def test_resident_at_the_edges_of_its_shapes(ue, n_t, plasma):
+    """152 CTAs of 1,024, 2,048 and 4,096 triangles."""
+    xy, tris, h = _lattice(n_t, 5)
+    kw = dict(plasma=plasma)
+    _same(_run(ue, xy, tris, h, 33, 32, **kw), _run(ue, xy, tris, h, 33, -1, **kw))
+
+
+def test_resident_fp64_with_two_slots(ue):
+    xy, tris, h = _lattice(200_001, 5)
+    kw = dict(plasma=True, precision=ue.UE_PREC_FP64)
+    _same(_run(ue, xy, tris, h, 33, 32, **kw), _run(ue, xy, tris, h, 33, -1, **kw))
+
+
+@pytest.mark.parametrize("n_t", [7_000, 400_000])
+def test_resident_with_scattered_neighbours(ue, n_t):
+    """The caller's order kept and random: nearly every neighbour is in another CTA, more than a
+    CTA lists, so threads poll their own."""
+    xy, tris, h = _lattice(n_t, 5, shuffle=True)
+    kw = dict(plasma=True, load=dict(reorder=ue.UE_REORDER_NONE))
+    _same(_run(ue, xy, tris, h, 40, 32, **kw), _run(ue, xy, tris, h, 40, -1, **kw))
+
+
+@pytest.mark.parametrize("tiled", [False, True])
+@pytest.mark.parametrize("plasma", [False, True])
+@pytest.mark.parametrize("frame,order", [(1, 3), (16, 3), (5, 1)])
+def test_resident_with_a_frame(ue, tiled, plasma, frame, order):
+    ms = meshgen.graded_square(0.05, 0.05, holes=[meshgen.polygon_triangle((0.5, 0.5), 0.3)], seed=4)
+    kw = dict(plasma=plasma, frame=frame)
+    plain = _run(ue, ms.xy, ms.tris, 0.05, 70, -1, load=dict(reorder=ue.UE_REORDER_GREEDY_RINGS, tile_tris=200) if tiled else None, **kw)
+    if tiled:
+        kw.update(load=dict(reorder=ue.UE_REORDER_GREEDY_RINGS, tile_tris=200), variant=ue.UE_VARIANT_BLOCKED, block_depth=4)
+    _same(_run(ue, ms.xy, ms.tris, 0.05, 70, 32, **kw), plain)
+
+
+def test_resident_batch_and_watchdog(ue):
+    """A batch of meshes with their own sources, and the watchdog's checks at the same steps."""
+    out = []
+    for chunk in (32, -1):
+        meshes = []
+        for n_t in (300, 4097, 2500):
+            xy, tris, h = _lattice(n_t, n_t)
+            m = ue.Mesh(xy, tris)
+            m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=chunk, watchdog_every=32)
+            ids, amp = meshgen.source_line_amplitudes(xy, tris, float(xy[:, 0].mean()), h)
+            m.set_source(ids, amp, 1.0 / h, 0.0, 0.3)
+            meshes.append(m)
+        b = ue.batch_create(meshes)
+        b.write_fields(B=np.cos(np.arange(b.n_tris)))
+        b.step_n(64)
+        ok, W, flag = b.check()
+        E, B, _ = b.read_fields()
+        assert ok and flag == 0
+        out.append((E, B, W))
+        b.close()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+
+
+def test_resident_wait_that_runs_out_is_reported(ue):
+    """One CTA that never publishes (test hook): the others' waits end after about a second,
+    UE_ERR_TIMEOUT is reported, and the rebuilt mesh steps normally."""
+    xy, tris, h = _lattice(5000, 2)
+    m = ue.Mesh(xy, tris)
+    m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=32, test_skip_cta=1)
+    m.write_fields(B=np.ones(m.n_tris))
+    m.step_n(32)
+    ok, _, flag = m.check()
+    m.close()
+    assert not ok and flag == 3
+    _same(_run(ue, xy, tris, h, 40, 32), _run(ue, xy, tris, h, 40, -1))

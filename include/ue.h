@@ -392,7 +392,7 @@ int ue_mesh_flip(const double* xy, int64_t n_nodes, const int32_t* tris, int64_t
  * n_modes in [1, 24], iters >= 1, seed: start vectors (SplitMix64 of the caller triangle id and
  * column).  omega: n_modes doubles, descending.  B: NULL or n_modes * n_tris doubles, mode i
  * at B + i*n_tris in caller triangle order, normalised to sum_j S_j B_j^2 = 1 (sign
- * arbitrary).  Synchronous; the work space, about (2 n_tris + n_interior_edges) * 2 n_modes
+ * arbitrary).  Synchronous; the work space, about 3 n_tris * 2 n_modes
  * doubles, comes from the mesh's allocator and is returned.
  * Errors: UE_ERR_ARG (also on a mesh with a PML frame); UE_ERR_ALLOC; UE_ERR_DUAL if the block
  * loses rank; UE_ERR_CUDA. */

@@ -6,8 +6,9 @@
 // the same way while keeping the ones already found from growing back.  Here the m columns of
 // a block are advanced together: V <- K V, then the block is made S-orthonormal again
 // (Cholesky QR: G = W^T S W = R^T R, V = W R^{-1}).  Column i is thereby kept clear of the
-// directions of columns 0..i-1 at every step, which is the deflation applied to all columns at
-// once.  A final Rayleigh-Ritz step on the block (eigenvectors of V^T S K V) gives the modes.
+// directions of columns 0..i-1, which is the deflation applied to all columns at once.  Cholesky
+// QR only changes the basis of the columns' span, so K V may be taken several times before it: as
+// many as keep the block well conditioned (modes_run).  A final Rayleigh-Ritz step on the block (eigenvectors of V^T S K V) gives the modes.
 // Everything is FP64.  Blocks of vectors are row-major [n_t][m]: a triangle's m values are
 // contiguous, so each gather reads one contiguous row.
 #include <cuda_runtime.h>
@@ -35,13 +36,32 @@ __device__ __forceinline__ uint64_t md_splitmix64(uint64_t x) {
 
 unsigned md_blocks(int64_t n) { return (unsigned)((n + kMdThreads - 1) / kMdThreads); }
 
-// c_k = |e_k| / d_k and 1/S_j (FP64 divisions once, not per product)
-__global__ void k_md_prep(const double* __restrict__ elen, const double* __restrict__ d,
-                          const double* __restrict__ S, double* __restrict__ c,
-                          double* __restrict__ invS, int64_t n_ei, int64_t n_t) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_ei) c[i] = elen[i] / d[i];
-    if (i < n_t) invS[i] = 1.0 / S[i];
+// Records of K's rows, made once per call: the triangles across the three edges (the triangle
+// itself on the boundary, with weight 0) and the weights c_q / S_j, c = |e| / d.
+__global__ void k_md_prep(const int4* __restrict__ tri, const int2* __restrict__ rl,
+                          const double* __restrict__ elen, const double* __restrict__ d,
+                          const double* __restrict__ S, int4* __restrict__ nb, double2* __restrict__ w,
+                          int64_t n_ei, int64_t n_t) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n_t) return;
+    const int4 t = tri[j];
+    const int code[3] = {t.x, t.y, t.z};
+    int o[3];
+    double x[3];
+    const double inv = 1.0 / S[j];
+    for (int q = 0; q < 3; ++q) {
+        const int64_t k = code[q] >> 1;
+        o[q] = (int)j;
+        x[q] = 0.0;
+        if (k < n_ei) {
+            const int2 r = rl[k];
+            o[q] = (code[q] & 1) ? r.x : r.y;
+            x[q] = elen[k] / d[k] * inv;
+        }
+    }
+    nb[j] = make_int4(o[0], o[1], o[2], 0);
+    w[2 * j] = make_double2(x[0], x[1]);
+    w[2 * j + 1] = make_double2(x[2], x[0] + x[1] + x[2]);
 }
 
 // V[j][col] uniform in [-1, 1), keyed by the caller id of triangle j and the column
@@ -55,37 +75,50 @@ __global__ void k_md_init(double* __restrict__ V, const int64_t* __restrict__ pe
     V[i] = (double)(z >> 11) * 0x1.0p-53 * 2.0 - 1.0;
 }
 
-// g[k][col] = c_k (V[R][col] - V[L][col]); row n_ei of g is the zero row of boundary edges
-__global__ void k_md_edge(const int2* __restrict__ rl, const double* __restrict__ c,
-                          const double* __restrict__ V, double* __restrict__ g, int64_t n_ei, int m) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_ei * m) return;
-    const int64_t k = i / m;
-    const int col = (int)(i - k * m);
-    const int2 e = rl[k];
-    g[i] = c[k] * (V[(int64_t)e.x * m + col] - V[(int64_t)e.y * m + col]);
-}
-
-// W[j][col] = (1/S_j) sum_q s(j,q) g[k_q][col]  (K V)
-__global__ void k_md_tri(const int4* __restrict__ tri, const double* __restrict__ invS,
-                         const double* __restrict__ g, double* __restrict__ W, int64_t n_t, int m) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_t * m) return;
-    const int64_t j = i / m;
-    const int col = (int)(i - j * m);
-    const int4 q = tri[j];
-    double a = g[(int64_t)(q.x >> 1) * m + col], b = g[(int64_t)(q.y >> 1) * m + col],
-           e = g[(int64_t)(q.z >> 1) * m + col];
-    if (q.x & 1) a = -a;
-    if (q.y & 1) b = -b;
-    if (q.z & 1) e = -e;
-    W[i] = (a + b + e) * invS[j];
+// W = K V in one pass: each triangle reads its own row and its three neighbours' (a signed sum of
+// edge differences c (V_R - V_L) is a sum of c (V_j - V_neighbour): both signs turn together).
+// Written as two passes over edges and triangles, each product moved the block's edge values,
+// 1.5 rows per triangle, out and in again: 11 + 18 us against 10 us here on 90k triangles and 16
+// columns (L2-resident; FP64 issue is the bound).  threadIdx.x: pair of columns, y: row.
+// CHEB: one step of the Chebyshev recurrence with it, Y1 = a (K Y - c Y) + b Y0 (Y0 may be NULL),
+// the product in difference form, which keeps the small values of smooth fields; without it
+// K_jj V_j - sum w V (four operations per value; FP64 is scarce), for the top of the spectrum.
+template <bool CHEB>
+__global__ void __launch_bounds__(kMdThreads) k_md_K(const int4* __restrict__ nb, const double2* __restrict__ w,
+                                                     const double2* __restrict__ Y, const double2* __restrict__ Y0,
+                                                     double2* __restrict__ out, double a, double c, double b,
+                                                     int64_t n_t, int m2) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+    if (j >= n_t) return;
+    const int col = threadIdx.x;
+    const int4 o = __ldg(nb + j);
+    const double2 w01 = __ldg(w + 2 * j), w2k = __ldg(w + 2 * j + 1);
+    const double2 v = __ldg(Y + j * m2 + col);
+    const double2 p = __ldg(Y + (int64_t)o.x * m2 + col), q = __ldg(Y + (int64_t)o.y * m2 + col),
+                  r = __ldg(Y + (int64_t)o.z * m2 + col);
+    double2 y;
+    if constexpr (CHEB) {
+        y.x = fma(w2k.x, v.x - r.x, fma(w01.y, v.x - q.x, w01.x * (v.x - p.x)));
+        y.y = fma(w2k.x, v.y - r.y, fma(w01.y, v.y - q.y, w01.x * (v.y - p.y)));
+        y.x = a * (y.x - c * v.x);
+        y.y = a * (y.y - c * v.y);
+        if (Y0) {
+            const double2 u = __ldg(Y0 + j * m2 + col);
+            y.x = fma(b, u.x, y.x);
+            y.y = fma(b, u.y, y.y);
+        }
+    } else {
+        y.x = fma(-w2k.x, r.x, fma(-w01.y, q.x, fma(-w01.x, p.x, w2k.y * v.x)));
+        y.y = fma(-w2k.x, r.y, fma(-w01.y, q.y, fma(-w01.x, p.y, w2k.y * v.y)));
+    }
+    out[j * m2 + col] = y;
 }
 
 // Block partials of the upper triangle of G[a][b] = sum_j S_j X[j][a] Y[j][b] (a <= b; G is
 // symmetric for X = Y, and for Y = K X up to rounding): rows in tiles of kMdRows staged in
 // shared memory, each thread owning the pairs tid, tid + 256, ... (m <= 32: at most 3 pairs of
-// the 528).  Pair p enumerates (a, b) row by row.
+// the 528).  Pair p enumerates (a, b) row by row.  Narrow blocks (at most 128 pairs) split each
+// tile's rows among 256 / pairs groups of threads, summed at the end in group order.
 constexpr int kMdRows = 32, kMdMaxM = 32;
 __global__ void __launch_bounds__(kMdThreads) k_md_gram(const double* __restrict__ S,
                                                         const double* __restrict__ X,
@@ -93,10 +126,12 @@ __global__ void __launch_bounds__(kMdThreads) k_md_gram(const double* __restrict
                                                         int m, double* __restrict__ part) {
     __shared__ double xs[kMdRows][kMdMaxM + 1], ys[kMdRows][kMdMaxM + 1];
     const int tid = threadIdx.x, npair = m * (m + 1) / 2;
+    const int groups = npair <= kMdThreads / 2 ? kMdThreads / npair : 1;
+    const int grp = groups > 1 ? tid / npair : 0, first = groups > 1 ? tid - grp * npair : tid;
     int pa[3], pb[3];
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
-        int p = tid + u * kMdThreads, a = 0;
+        int p = first + u * kMdThreads, a = 0;
         while (a < m && p >= m - a) {
             p -= m - a;
             ++a;
@@ -120,15 +155,35 @@ __global__ void __launch_bounds__(kMdThreads) k_md_gram(const double* __restrict
             ys[r][col] = y;
         }
         __syncthreads();
+        if (groups > 1) {
+            if (grp < groups) {
+                double s = acc[0];
+                for (int r = grp; r < kMdRows; r += groups) s = fma(xs[r][pa[0]], ys[r][pb[0]], s);
+                acc[0] = s;
+            }
+        } else {
 #pragma unroll
-        for (int u = 0; u < 3; ++u) {
-            if (tid + u * kMdThreads < npair) {
-                const int a = pa[u], b = pb[u];
-                double s = acc[u];
-                for (int r = 0; r < kMdRows; ++r) s = fma(xs[r][a], ys[r][b], s);
-                acc[u] = s;
+            for (int u = 0; u < 3; ++u) {
+                if (tid + u * kMdThreads < npair) {
+                    const int a = pa[u], b = pb[u];
+                    double s = acc[u];
+                    for (int r = 0; r < kMdRows; ++r) s = fma(xs[r][a], ys[r][b], s);
+                    acc[u] = s;
+                }
             }
         }
+    }
+    if (groups > 1) {
+        __syncthreads();
+        double* red = &xs[0][0];   // kMdRows * (kMdMaxM + 1) >= kMdThreads values
+        red[tid] = acc[0];
+        __syncthreads();
+        if (tid < npair) {
+            double s = 0.0;
+            for (int g = 0; g < groups; ++g) s += red[tid + g * npair];
+            part[(int64_t)blockIdx.x * npair + tid] = s;
+        }
+        return;
     }
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
@@ -137,13 +192,16 @@ __global__ void __launch_bounds__(kMdThreads) k_md_gram(const double* __restrict
     }
 }
 
-// G[p] = sum over blocks of part[b][p], in block order (deterministic)
+// G[p] = sum over blocks of part[b][p], one warp per pair, in an order that does not change (one
+// thread per pair summed 608 partials in a row: 50 us against 5)
 __global__ void k_md_sum(const double* __restrict__ part, int nb, int npair, double* __restrict__ G) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (p >= npair) return;
     double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[(int64_t)b * npair + p];
-    G[p] = s;
+#pragma unroll 4
+    for (int b = lane; b < nb; b += 32) s += part[(int64_t)b * npair + p];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) G[p] = s;
 }
 
 // V[j][col] = sum_a W[j][a] T[a][col] (T is m x m, row-major; upper: T[a][col] = 0 for
@@ -162,17 +220,23 @@ __global__ void __launch_bounds__(kMdThreads) k_md_apply(const double* __restric
     __syncthreads();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_t) return;
-    const double* w = W + j * m;
+    const double2* w = reinterpret_cast<const double2*>(W + j * m);   // m is even
     double x[MW];
 #pragma unroll
-    for (int a = 0; a < MW; ++a) x[a] = a < m ? w[a] : 0.0;
-    double* v = V + j * m;
+    for (int a = 0; a < MW; a += 2) {
+        const double2 v = a < m ? __ldg(w + a / 2) : make_double2(0.0, 0.0);
+        x[a] = v.x;
+        x[a + 1] = v.y;
+    }
+    double2* v = reinterpret_cast<double2*>(V + j * m);
 #pragma unroll
-    for (int col = 0; col < MW; ++col) {
-        double s = 0.0;
+    for (int col = 0; col < MW; col += 2) {
+        double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-        for (int a = 0; a < (UPPER ? col + 1 : MW); ++a) s = fma(x[a], ts[a * MW + col], s);
-        if (col < m) v[col] = s;
+        for (int a = 0; a < (UPPER ? col + 1 : MW); ++a) s0 = fma(x[a], ts[a * MW + col], s0);
+#pragma unroll
+        for (int a = 0; a < (UPPER ? col + 2 : MW); ++a) s1 = fma(x[a], ts[a * MW + col + 1], s1);
+        if (col < m) v[col / 2] = make_double2(s0, s1);
     }
 }
 
@@ -195,23 +259,14 @@ __global__ void k_md_scatter(const double* __restrict__ V, const int64_t* __rest
     out[(int64_t)col * n_t + perm[j]] = V[j * m + col];
 }
 
-// One step of the Chebyshev recurrence on blocks: Y1 = a (W - c Y) + b Y0, with W = K Y.
-__global__ void k_md_cheb(const double* __restrict__ W, const double* __restrict__ Y,
-                          const double* __restrict__ Y0, double* __restrict__ Y1, double a, double c,
-                          double b, int64_t n) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double y = a * (W[i] - c * Y[i]);
-    Y1[i] = Y0 ? fma(b, Y0[i], y) : y;
-}
-
 // Gershgorin bound of S^(1/2) K S^(-1/2) (the S-symmetric form of K, same eigenvalues): row j
-// has K_jj = sum_q c_q / S_j and off-diagonal c_q / sqrt(S_j S_k) for the triangle k across
-// interior edge q; the largest row sum bounds lambda_max from above.  Positive doubles order
+// has K_jj = sum_q c_q / S_j and off-diagonal c_q / sqrt(S_j S_k), c = |e| / d, for the triangle k
+// across interior edge q; the largest row sum bounds lambda_max from above.  Positive doubles order
 // like their bit patterns, so the maximum is an integer atomic.
 __global__ void k_md_gersh(const int4* __restrict__ tri, const int2* __restrict__ rl,
-                           const double* __restrict__ c, const double* __restrict__ S,
-                           int64_t n_t, int64_t n_ei, unsigned long long* __restrict__ out) {
+                           const double* __restrict__ elen, const double* __restrict__ d,
+                           const double* __restrict__ S, int64_t n_t, int64_t n_ei,
+                           unsigned long long* __restrict__ out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_t) return;
     const int4 q = tri[j];
@@ -223,7 +278,8 @@ __global__ void k_md_gersh(const int4* __restrict__ tri, const int2* __restrict_
         if (e >= n_ei) continue;
         const int2 t = rl[e];
         const int64_t o = t.x == j ? t.y : t.x;
-        row += c[e] / sj + c[e] / sqrt(sj * S[o]);
+        const double c = elen[e] / d[e];
+        row += c / sj + c / sqrt(sj * S[o]);
     }
     atomicMax(out, (unsigned long long)__double_as_longlong(row));
 }
@@ -313,11 +369,94 @@ void jacobi_eigen(std::vector<double> A, int m, std::vector<double>& lam, std::v
 
 }  // namespace
 
+namespace {
+
+// What both iterations share: K's records, the small dense matrices and the block operations.
+struct Block {
+    int64_t n_t;
+    int m, npair, nup, nb;
+    const double* S;
+    int4* onb;
+    double2* w;
+    double *part, *G, *T;
+    cudaStream_t s;
+    std::vector<double> Gu, Gh, R, Th;
+    bool lost = false;
+
+    // the work space after `bufs` blocks of n_t * m values
+    Block(int64_t n_t_, int m_, const double* S_, double* work, int bufs, cudaStream_t s_)
+        : n_t(n_t_), m(m_), npair(m_ * m_), nup(m_ * (m_ + 1) / 2),
+          nb((int)std::min<int64_t>(152 * 4, (n_t_ + kMdRows - 1) / kMdRows)), S(S_), s(s_), Gu(nup), Gh(npair) {
+        double* p = work + (int64_t)bufs * n_t * m;
+        onb = reinterpret_cast<int4*>(p);
+        w = reinterpret_cast<double2*>(p + 2 * n_t);
+        part = p + 6 * n_t;
+        G = part + (int64_t)nb * nup;
+        T = G + npair;
+    }
+    static size_t doubles(int64_t n_t, int m, int bufs) {
+        const int64_t nb = std::min<int64_t>(152 * 4, (n_t + kMdRows - 1) / kMdRows);
+        return (size_t)(bufs * n_t * m + 6 * n_t + nb * (int64_t)m * (m + 1) / 2 + 2 * m * m + 8);
+    }
+    void prep(const int4* tri, const int2* rl, const double* elen, const double* d, int64_t n_ei) {
+        k_md_prep<<<md_blocks(n_t), kMdThreads, 0, s>>>(tri, rl, elen, d, S, onb, w, n_ei, n_t);
+    }
+    template <bool CHEB>
+    void K(const double* Y, const double* Y0, double* out, double a, double c, double b) {
+        const int m2 = m / 2, rows = kMdThreads / m2;
+        k_md_K<CHEB><<<(unsigned)((n_t + rows - 1) / rows), dim3(m2, rows), 0, s>>>(
+            onb, w, (const double2*)Y, (const double2*)Y0, (double2*)out, a, c, b, n_t, m2);
+    }
+    void product(const double* X, double* Y) { K<false>(X, nullptr, Y, 0.0, 0.0, 0.0); }
+    cudaError_t gram(const double* X, const double* Y) {   // Gh = X^T S Y
+        k_md_gram<<<nb, kMdThreads, 0, s>>>(S, X, Y, n_t, m, part);
+        k_md_sum<<<(nup + 7) / 8, 256, 0, s>>>(part, nb, nup, G);
+        cudaError_t e = cudaMemcpyAsync(Gu.data(), G, sizeof(double) * nup, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+        for (int a = 0, p = 0; a < m; ++a)
+            for (int b = a; b < m; ++b, ++p) Gh[(size_t)a * m + b] = Gh[(size_t)b * m + a] = Gu[p];
+        return cudaSuccess;
+    }
+    template <bool UPPER>
+    cudaError_t rotate(const double* X, const std::vector<double>& M, double* Y) {   // Y = X M
+        const cudaError_t e = cudaMemcpyAsync(T, M.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return e;
+        md_apply<UPPER>(X, T, Y, n_t, m, s);
+        return cudaGetLastError();
+    }
+    // Y = X R^{-1}, X^T S X = R^T R; sets lost (and leaves Y) when X has lost rank
+    cudaError_t orthonormalize(const double* X, double* Y) {
+        const cudaError_t e = gram(X, X);
+        if (e != cudaSuccess) return e;
+        lost = !cholesky_upper(Gh, m, R);
+        if (lost) return cudaSuccess;
+        upper_inverse(R, m, Th);
+        return rotate<true>(X, Th, Y);
+    }
+};
+
+}  // namespace
+
 int modes_block_size(int n_modes) { return std::min(kMdMaxM, 2 * n_modes); }
 
-size_t modes_work_doubles(int64_t n_t, int64_t n_ei, int m) {
-    const int64_t nb = std::min<int64_t>(152 * 4, (n_t + kMdRows - 1) / kMdRows);
-    return (size_t)(2 * n_t * m + (n_ei + 1) * m + n_ei + n_t + nb * (int64_t)m * (m + 1) / 2 + 2 * m * m + 8);
+size_t modes_work_doubles(int64_t n_t, int m) { return Block::doubles(n_t, m, 3); }
+
+// How many products K V to take before the next Cholesky QR.  It only has to come before the
+// columns' norms and angles drift so far apart that forming W^T S W loses digits; the diagonal of
+// R, over the `p` products that led to it, tells the drift per product.  Products until it
+// reaches 100 (an error of the basis, not of its span, of 1e-12, gone at the next QR), at most 8,
+// and none that could overflow the Gram matrix.  One QR per product took 150 of the 180 us of an
+// iteration on 90k triangles with 16 columns; with up to 8 products it is 25 us per iteration.
+static int products_until_qr(const std::vector<double>& R, int m, int p) {
+    double lo = R[0], hi = R[0];
+    for (int i = 1; i < m; ++i) {
+        lo = std::min(lo, R[(size_t)i * m + i]);
+        hi = std::max(hi, R[(size_t)i * m + i]);
+    }
+    const double drift = std::log10(hi / lo) / p, size = std::fabs(std::log10(hi)) / p;
+    const double most = std::min(drift > 0 ? 2.0 / drift : 8.0, size > 0 ? 140.0 / size : 8.0);
+    return (int)std::max(1.0, std::min(8.0, most));
 }
 
 cudaError_t modes_run(const int2* rl, const int4* tri, const double* elen, const double* d,
@@ -325,75 +464,56 @@ cudaError_t modes_run(const int2* rl, const int4* tri, const double* elen, const
                       int iters, uint32_t seed, double* work, double* omega, double* B_dev,
                       bool* lost_rank, cudaStream_t s) {
     const int m = modes_block_size(n_modes);
-    const int npair = m * m, nup = m * (m + 1) / 2;
-    const int nb = (int)std::min<int64_t>(152 * 4, (n_t + kMdRows - 1) / kMdRows);
-    double* V = work;
-    double* W = V + n_t * m;
-    double* g = W + n_t * m;
-    double* c = g + (n_ei + 1) * m;
-    double* invS = c + n_ei;
-    double* part = invS + n_t;
-    double* G = part + (int64_t)nb * nup;
-    double* T = G + npair;
+    Block k(n_t, m, S, work, 3, s);
+    double *V = work, *W = V + n_t * m, *W2 = W + n_t * m;
     *lost_rank = false;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(g + n_ei * m, 0, sizeof(double) * m, s)) != cudaSuccess) return e;
-    k_md_prep<<<md_blocks(std::max(n_ei, n_t)), kMdThreads, 0, s>>>(elen, d, S, c, invS, n_ei, n_t);
+    k.prep(tri, rl, elen, d, n_ei);
     k_md_init<<<md_blocks(n_t * m), kMdThreads, 0, s>>>(V, perm, seed, n_t, m);
-    std::vector<double> Gu(nup), Gh(npair), R, Th;
-    auto apply_K = [&](const double* X, double* Y) {
-        if (n_ei > 0) k_md_edge<<<md_blocks(n_ei * m), kMdThreads, 0, s>>>(rl, c, X, g, n_ei, m);
-        k_md_tri<<<md_blocks(n_t * m), kMdThreads, 0, s>>>(tri, invS, g, Y, n_t, m);
-    };
-    auto gram = [&](const double* X, const double* Y) -> cudaError_t {
-        k_md_gram<<<nb, kMdThreads, 0, s>>>(S, X, Y, n_t, m, part);
-        k_md_sum<<<(nup + 255) / 256, 256, 0, s>>>(part, nb, nup, G);
-        cudaError_t e2 = cudaMemcpyAsync(Gu.data(), G, sizeof(double) * nup, cudaMemcpyDeviceToHost, s);
-        if (e2 != cudaSuccess) return e2;
-        if ((e2 = cudaStreamSynchronize(s)) != cudaSuccess) return e2;
-        for (int a = 0, p = 0; a < m; ++a)
-            for (int b = a; b < m; ++b, ++p) Gh[(size_t)a * m + b] = Gh[(size_t)b * m + a] = Gu[p];
-        return cudaSuccess;
-    };
-    auto orthonormalize = [&](const double* X, double* Y) -> cudaError_t {   // Y = X R^{-1}
-        cudaError_t e2 = gram(X, X);
-        if (e2 != cudaSuccess) return e2;
-        if (!cholesky_upper(Gh, m, R)) {
-            *lost_rank = true;
-            return cudaSuccess;
-        }
-        upper_inverse(R, m, Th);
-        if ((e2 = cudaMemcpyAsync(T, Th.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-            return e2;
-        md_apply<true>(X, T, Y, n_t, m, s);
-        return cudaGetLastError();
-    };
-    // start: the random block made S-orthonormal (into W, then copied back by the first step)
-    if ((e = orthonormalize(V, W)) != cudaSuccess || *lost_rank) return e;
+    // start: the random block made S-orthonormal
+    if ((e = k.orthonormalize(V, W)) != cudaSuccess || (*lost_rank = k.lost)) return e;
     std::swap(V, W);
-    for (int it = 0; it < iters; ++it) {
-        apply_K(V, W);                                   // W = K V
-        if ((e = orthonormalize(W, V)) != cudaSuccess || *lost_rank) return e;   // V = W R^{-1}
+    int p = 1;
+    for (int it = 0; it < iters;) {
+        p = std::min(p, iters - it);
+        const double* X = V;   // V stays: a block that lost rank over p products is taken again one by one
+        for (int i = 0; i < p; ++i) {
+            double* Y = X == W ? W2 : W;
+            k.product(X, Y);
+            X = Y;
+        }
+        double* Y = X == W ? W2 : W;
+        if ((e = k.orthonormalize(X, Y)) != cudaSuccess) return e;
+        if (k.lost) {
+            if (p == 1) {
+                *lost_rank = true;
+                return cudaSuccess;
+            }
+            p = 1;
+            continue;
+        }
+        it += p;
+        std::swap(V, Y == W ? W : W2);
+        p = products_until_qr(k.R, m, p);
     }
+    // once more, now near identity: columns S-orthonormal to rounding for Rayleigh-Ritz
+    if ((e = k.orthonormalize(V, W)) != cudaSuccess || (*lost_rank = k.lost)) return e;
+    std::swap(V, W);
     // Rayleigh-Ritz: H = V^T S K V, its eigenvectors rotate V into the modes
-    apply_K(V, W);
-    if ((e = gram(V, W)) != cudaSuccess) return e;
+    k.product(V, W);
+    if ((e = k.gram(V, W)) != cudaSuccess) return e;
     std::vector<double> lam, Q;
-    jacobi_eigen(Gh, m, lam, Q);
+    jacobi_eigen(k.Gh, m, lam, Q);
     for (int i = 0; i < n_modes; ++i) omega[i] = std::sqrt(std::max(lam[i], 0.0));
     if (B_dev) {
-        if ((e = cudaMemcpyAsync(T, Q.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-            return e;
-        md_apply<false>(V, T, W, n_t, m, s);
+        if ((e = k.rotate<false>(V, Q, W)) != cudaSuccess) return e;
         k_md_scatter<<<md_blocks(n_t * n_modes), kMdThreads, 0, s>>>(W, perm, B_dev, n_t, m, n_modes);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return cudaStreamSynchronize(s);
 }
 
-size_t modes_low_work_doubles(int64_t n_t, int64_t n_ei, int m) {
-    return modes_work_doubles(n_t, n_ei, m) + 2 * (size_t)n_t * m + 8;
-}
+size_t modes_low_work_doubles(int64_t n_t, int m) { return Block::doubles(n_t, m, 4) + 8; }
 
 // The lowest n_modes eigenpairs of K by Chebyshev-filtered subspace iteration: each outer
 // iteration applies to the block the degree-`degree` Chebyshev polynomial that stays within
@@ -406,81 +526,44 @@ cudaError_t modes_low_run(const int2* rl, const int4* tri, const double* elen, c
                           int iters, int degree, uint32_t seed, double* work, double* omega,
                           double* B_dev, bool* lost_rank, cudaStream_t s) {
     const int m = modes_block_size(n_modes);
-    const int npair = m * m, nup = m * (m + 1) / 2;
-    const int nb = (int)std::min<int64_t>(152 * 4, (n_t + kMdRows - 1) / kMdRows);
-    double* V = work;
-    double* W = V + n_t * m;
-    double* g = W + n_t * m;
-    double* c = g + (n_ei + 1) * m;
-    double* invS = c + n_ei;
-    double* part = invS + n_t;
-    double* G = part + (int64_t)nb * nup;
-    double* T = G + npair;
-    double* Y0 = work + modes_work_doubles(n_t, n_ei, m);
-    double* Y1 = Y0 + n_t * m;
-    unsigned long long* gmax = reinterpret_cast<unsigned long long*>(Y1 + n_t * m);
+    Block k(n_t, m, S, work, 4, s);
+    double* buf[4];
+    for (int i = 0; i < 4; ++i) buf[i] = work + (int64_t)i * n_t * m;
+    unsigned long long* gmax = reinterpret_cast<unsigned long long*>(work + Block::doubles(n_t, m, 4));
     *lost_rank = false;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(g + n_ei * m, 0, sizeof(double) * m, s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(gmax, 0, 8, s)) != cudaSuccess) return e;
-    k_md_prep<<<md_blocks(std::max(n_ei, n_t)), kMdThreads, 0, s>>>(elen, d, S, c, invS, n_ei, n_t);
-    k_md_gersh<<<md_blocks(n_t), kMdThreads, 0, s>>>(tri, rl, c, S, n_t, n_ei, gmax);
-    k_md_init<<<md_blocks(n_t * m), kMdThreads, 0, s>>>(V, perm, seed, n_t, m);
+    k.prep(tri, rl, elen, d, n_ei);
+    k_md_gersh<<<md_blocks(n_t), kMdThreads, 0, s>>>(tri, rl, elen, d, S, n_t, n_ei, gmax);
+    k_md_init<<<md_blocks(n_t * m), kMdThreads, 0, s>>>(buf[0], perm, seed, n_t, m);
     unsigned long long hb = 0;
     if ((e = cudaMemcpyAsync(&hb, gmax, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     double hi;
     std::memcpy(&hi, &hb, 8);
     hi *= 1.0 + 1e-12;
-    std::vector<double> Gu(nup), Gh(npair), R, Th, lam, Q;
-    auto apply_K = [&](const double* X, double* Y) {
-        if (n_ei > 0) k_md_edge<<<md_blocks(n_ei * m), kMdThreads, 0, s>>>(rl, c, X, g, n_ei, m);
-        k_md_tri<<<md_blocks(n_t * m), kMdThreads, 0, s>>>(tri, invS, g, Y, n_t, m);
+    std::vector<double> lam, Q;
+    // The block is buf[v]; the recurrence and the basis changes move it among the four buffers.
+    int v = 0;
+    auto orthonormal = [&]() -> cudaError_t {
+        const cudaError_t e2 = k.orthonormalize(buf[v], buf[(v + 1) & 3]);
+        v = (v + 1) & 3;
+        return e2;
     };
-    auto gram = [&](const double* X, const double* Y) -> cudaError_t {
-        k_md_gram<<<nb, kMdThreads, 0, s>>>(S, X, Y, n_t, m, part);
-        k_md_sum<<<(nup + 255) / 256, 256, 0, s>>>(part, nb, nup, G);
-        cudaError_t e2 = cudaMemcpyAsync(Gu.data(), G, sizeof(double) * nup, cudaMemcpyDeviceToHost, s);
-        if (e2 != cudaSuccess) return e2;
-        if ((e2 = cudaStreamSynchronize(s)) != cudaSuccess) return e2;
-        for (int a = 0, p = 0; a < m; ++a)
-            for (int b = a; b < m; ++b, ++p) Gh[(size_t)a * m + b] = Gh[(size_t)b * m + a] = Gu[p];
-        return cudaSuccess;
-    };
-    auto orthonormalize = [&](const double* X, double* Y) -> cudaError_t {   // Y = X R^{-1}
-        cudaError_t e2 = gram(X, X);
-        if (e2 != cudaSuccess) return e2;
-        if (!cholesky_upper(Gh, m, R)) {
-            *lost_rank = true;
-            return cudaSuccess;
-        }
-        upper_inverse(R, m, Th);
-        if ((e2 = cudaMemcpyAsync(T, Th.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-            return e2;
-        md_apply<true>(X, T, Y, n_t, m, s);
-        return cudaGetLastError();
-    };
-    // The block always lives in V (the work space's first n_t * m values), W is scratch; the
-    // filter's recurrence rotates among V, Y0 and Y1.
-    const int64_t n = n_t * m;
-    auto copy_to_V = [&](const double* X) -> cudaError_t {
-        return X == V ? cudaSuccess : cudaMemcpyAsync(V, X, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
-    };
-    // V -> its Ritz vectors (V^T S K V diagonal), lam ascending
+    // the block -> its Ritz vectors (V^T S K V diagonal), lam ascending
     auto rayleigh_ritz = [&]() -> cudaError_t {
-        apply_K(V, W);
-        cudaError_t e2 = gram(V, W);
+        double* W = buf[(v + 1) & 3];
+        k.K<true>(buf[v], nullptr, W, 1.0, 0.0, 0.0);   // K V, in difference form
+        cudaError_t e2 = k.gram(buf[v], W);
         if (e2 != cudaSuccess) return e2;
-        jacobi_eigen(Gh, m, lam, Q);
+        jacobi_eigen(k.Gh, m, lam, Q);
         std::reverse(lam.begin(), lam.end());
         for (int r = 0; r < m; ++r) std::reverse(Q.begin() + (size_t)r * m, Q.begin() + (size_t)(r + 1) * m);
-        if ((e2 = cudaMemcpyAsync(T, Q.data(), sizeof(double) * npair, cudaMemcpyHostToDevice, s)) != cudaSuccess)
-            return e2;
-        md_apply<false>(V, T, W, n_t, m, s);
-        return copy_to_V(W);
+        e2 = k.rotate<false>(buf[v], Q, W);
+        v = (v + 1) & 3;
+        return e2;
     };
-    if ((e = orthonormalize(V, W)) != cudaSuccess || *lost_rank) return e;
-    if ((e = copy_to_V(W)) != cudaSuccess) return e;
+    if ((e = orthonormal()) != cudaSuccess || (*lost_rank = k.lost)) return e;
     if ((e = rayleigh_ritz()) != cudaSuccess) return e;
     std::vector<double> prev(n_modes, -1.0);
     for (int it = 0; it < iters; ++it) {
@@ -491,23 +574,19 @@ cudaError_t modes_low_run(const int2* rl, const int4* tri, const double* elen, c
         // scaled three-term recurrence: T_k((x - cc)/ee) / T_k((0 - cc)/ee) (Zhou and Saad)
         const double sig1 = ee / (0.0 - cc);
         double sig = sig1;
-        apply_K(V, W);
-        k_md_cheb<<<md_blocks(n), kMdThreads, 0, s>>>(W, V, nullptr, Y1, sig1 / ee, cc, 0.0, n);
-        double* Yp = V;    // T_{k-1}
-        double* Yc = Y1;   // T_k
-        double* Yn = Y0;
-        for (int k = 2; k <= degree; ++k) {
+        int yp = v, yc = (v + 1) & 3, yn = (v + 2) & 3;   // T_{k-1}, T_k, T_{k+1}
+        k.K<true>(buf[yp], nullptr, buf[yc], sig1 / ee, cc, 0.0);
+        for (int q = 2; q <= degree; ++q) {
             const double sn = 1.0 / (2.0 / sig1 - sig);
-            apply_K(Yc, W);
-            k_md_cheb<<<md_blocks(n), kMdThreads, 0, s>>>(W, Yc, Yp, Yn, 2.0 * sn / ee, cc, -sig * sn, n);
+            k.K<true>(buf[yc], buf[yp], buf[yn], 2.0 * sn / ee, cc, -sig * sn);
             sig = sn;
-            double* t = Yp;
-            Yp = Yc;
-            Yc = Yn;
-            Yn = t;
+            const int t = yp;
+            yp = yc;
+            yc = yn;
+            yn = t;
         }
-        if ((e = orthonormalize(Yc, W)) != cudaSuccess || *lost_rank) return e;
-        if ((e = copy_to_V(W)) != cudaSuccess) return e;
+        v = yc;
+        if ((e = orthonormal()) != cudaSuccess || (*lost_rank = k.lost)) return e;
         if ((e = rayleigh_ritz()) != cudaSuccess) return e;
         bool done = true;
         for (int i = 0; i < n_modes; ++i) {
@@ -517,7 +596,7 @@ cudaError_t modes_low_run(const int2* rl, const int4* tri, const double* elen, c
         if (done && it > 0) break;
     }
     for (int i = 0; i < n_modes; ++i) omega[i] = std::sqrt(std::max(lam[i], 0.0));
-    if (B_dev) k_md_scatter<<<md_blocks(n_t * n_modes), kMdThreads, 0, s>>>(V, perm, B_dev, n_t, m, n_modes);
+    if (B_dev) k_md_scatter<<<md_blocks(n_t * n_modes), kMdThreads, 0, s>>>(buf[v], perm, B_dev, n_t, m, n_modes);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return cudaStreamSynchronize(s);
 }

@@ -2526,7 +2526,7 @@ int ue_modes_low(ue_mesh* m, int32_t n_modes, int32_t iters, int32_t degree, uin
     if (nt < bw) return fail(UE_ERR_ARG, "ue_modes_low: the mesh has fewer triangles than the block of vectors");
     double* work = nullptr;
     double* Bd = nullptr;
-    if (!alloc_into(m, work, ue::modes_low_work_doubles(nt, nei, bw), 8, s) ||
+    if (!alloc_into(m, work, ue::modes_low_work_doubles(nt, bw), 8, s) ||
         (B && !alloc_into(m, Bd, (size_t)n_modes * nt, 8, s)))
         return fail(UE_ERR_ALLOC, "ue_modes_low work space");
     bool lost = false;
@@ -2558,7 +2558,7 @@ int ue_modes(ue_mesh* m, int32_t n_modes, int32_t iters, uint32_t seed, double* 
         return fail(UE_ERR_ARG, "ue_modes: the mesh has fewer triangles than the block of vectors");
     double* work = nullptr;
     double* Bd = nullptr;
-    if (!alloc_into(m, work, ue::modes_work_doubles(nt, nei, ue::modes_block_size(n_modes)), 8, s) ||
+    if (!alloc_into(m, work, ue::modes_work_doubles(nt, ue::modes_block_size(n_modes)), 8, s) ||
         (B && !alloc_into(m, Bd, (size_t)n_modes * nt, 8, s)))
         return fail(UE_ERR_ALLOC, "ue_modes work space");
     bool lost = false;

@@ -276,6 +276,11 @@ cudaError_t power_iteration(const int2* rl, const int4* tri, const double* elen,
                             int iters, uint32_t seed, double* work, double* rho, cudaStream_t s,
                             const FrameDev* frame = nullptr);
 size_t power_iteration_work_doubles(int64_t n_t, int64_t n_ei, const FrameDev* frame = nullptr);
+// The same without a frame (kernels_power.cu); work holds power_work_doubles doubles.
+size_t power_work_doubles(int64_t n_t);
+cudaError_t power_iteration_mesh(const int2* rl, const int4* tri, const double* elen, const double* d,
+                                 const double* S, const int64_t* perm, int64_t n_t, int64_t n_ei, int iters,
+                                 uint32_t seed, double* work, double* rho, cudaStream_t s);
 cudaError_t launch_fields_in(const DevMesh& m, const double* E_caller, const double* B_caller,
                              const double* J_caller, const int64_t* edge_caller,
                              const int64_t* perm_tri, const double* elen, cudaStream_t s);

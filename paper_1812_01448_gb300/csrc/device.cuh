@@ -264,6 +264,15 @@ cudaError_t launch_geom_tri(const double* xy, const int32_t* tri_nodes, double* 
                             int64_t n_t, cudaStream_t s);
 cudaError_t launch_geom_edge(const double* xy, const int32_t* edge_nodes, const int32_t* edge_opp,
                              double* elen, double* d, int64_t n_ei, cudaStream_t s);
+// Edge tables (R, L), (low, high) nodes and opposite nodes from the triangles' nodes and codes.
+cudaError_t launch_edge_tables(const int32_t* tri_nodes, const int32_t* tri_code, int2* rl, int32_t* edge_nodes,
+                               int32_t* edge_opp, int64_t n_t, int64_t n_ei, cudaStream_t s);
+// k_of[n_e] = stored interior edge of each caller edge or -1; inv[n_t] = stored triangle of each
+// caller triangle.
+cudaError_t launch_caller_maps(const int64_t* edge_caller, const int64_t* perm_tri, int32_t* k_of, int32_t* inv,
+                               int64_t n_ei, int64_t n_t, int64_t n_e, cudaStream_t s);
+// *first (device) = the smallest stored edge whose dual length is not > 1e-12 |e|, or all ones.
+cudaError_t launch_dual_check(const double* d, const double* elen, int64_t n_ei, unsigned long long* first, cudaStream_t s);
 // cU = dt|e|/d on [0, n_ei), triangle records on [0, n_t) and their padding (codes on the zero
 // slot, coefficient 0).  Edge padding must be zeroed by the caller.
 cudaError_t launch_coeff(const DevMesh& m, const double* elen, const double* d, const double* S,

@@ -40,6 +40,43 @@ __device__ __forceinline__ double cot_at(double ax, double ay, double bx, double
     return (ux * vx + uy * vy) / fabs(ux * vy - uy * vx);
 }
 
+// Edge tables from the triangles' (two uploads instead of five): each triangle writes itself, its
+// node opposite the edge and, as the edge's R, the edge's nodes.  Edge q joins vertices q and q + 1.
+__global__ void k_edge_tables(const int32_t* __restrict__ tn, const int32_t* __restrict__ code,
+                              int32_t* __restrict__ rl, int32_t* __restrict__ en, int32_t* __restrict__ eo,
+                              int64_t n_t, int64_t n_ei) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n_t) return;
+    const int32_t v[3] = {tn[3 * j], tn[3 * j + 1], tn[3 * j + 2]};
+    for (int q = 0; q < 3; ++q) {
+        const int32_t c = code[3 * j + q];
+        const int64_t k = c >> 1;
+        if (k >= n_ei) continue;
+        const int neg = c & 1;
+        rl[2 * k + neg] = (int32_t)j;
+        eo[2 * k + neg] = v[q == 0 ? 2 : q - 1];
+        if (!neg) {
+            en[2 * k] = v[q];
+            en[2 * k + 1] = v[q == 2 ? 0 : q + 1];
+        }
+    }
+}
+
+// Caller -> stored maps: k_of filled with -1 before.
+__global__ void k_caller_maps(const int64_t* __restrict__ ec, const int64_t* __restrict__ perm,
+                              int32_t* __restrict__ k_of, int32_t* __restrict__ inv, int64_t n_ei, int64_t n_t) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_ei) k_of[ec[i]] = (int32_t)i;
+    if (i < n_t) inv[perm[i]] = (int32_t)i;
+}
+
+// *first = smallest stored edge without d > 1e-12 |e| (NaN included); all ones before.
+__global__ void k_dual_check(const double* __restrict__ d, const double* __restrict__ elen, int64_t n_ei,
+                             unsigned long long* __restrict__ first) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n_ei && !(d[k] > 1e-12 * elen[k])) atomicMin(first, (unsigned long long)k);
+}
+
 // |e_i| and the dual length |O_R O_L| of eq. 3 in the cotangent form
 // d_i = |e_i|/2 (cot alpha_R + cot alpha_L), alpha = angle opposite e_i (stable for
 // near-degenerate triangles, where subtracting two circumcentres would cancel).
@@ -545,6 +582,27 @@ __global__ void k_recip(const double* __restrict__ elen, double* __restrict__ re
 
 cudaError_t launch_recip(const double* elen, double* relen, int64_t n_ei, cudaStream_t s) {
     k_recip<<<blocks_for(n_ei + 1), kThreads, 0, s>>>(elen, relen, n_ei);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_edge_tables(const int32_t* tri_nodes, const int32_t* tri_code, int2* rl, int32_t* edge_nodes,
+                               int32_t* edge_opp, int64_t n_t, int64_t n_ei, cudaStream_t s) {
+    k_edge_tables<<<blocks_for(n_t), kThreads, 0, s>>>(tri_nodes, tri_code, (int32_t*)rl, edge_nodes, edge_opp, n_t, n_ei);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_caller_maps(const int64_t* edge_caller, const int64_t* perm_tri, int32_t* k_of, int32_t* inv,
+                               int64_t n_ei, int64_t n_t, int64_t n_e, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(k_of, 0xFF, 4 * n_e, s);
+    if (e != cudaSuccess) return e;
+    k_caller_maps<<<blocks_for(n_ei > n_t ? n_ei : n_t), kThreads, 0, s>>>(edge_caller, perm_tri, k_of, inv, n_ei, n_t);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dual_check(const double* d, const double* elen, int64_t n_ei, unsigned long long* first, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(first, 0xFF, 8, s);
+    if (e != cudaSuccess || n_ei == 0) return e;
+    k_dual_check<<<blocks_for(n_ei), kThreads, 0, s>>>(d, elen, n_ei, first);
     return cudaGetLastError();
 }
 

@@ -562,20 +562,16 @@ int build_host_mesh(const double* xy, int64_t n_nodes, const int32_t* tris, int6
     hm.edge_caller.resize(n_ei);
     hm.k_of_edge.assign(ne, -1);
     hm.edge_tri.resize(2 * n_ei);
-    hm.edge_nodes.resize(2 * n_ei);
     for (int64_t k = 0; k < n_ei; ++k) {
         const int64_t e = ie[k].second;
         hm.edge_caller[k] = e;
         hm.k_of_edge[e] = k;
         hm.edge_tri[2 * k] = (int32_t)new_of[c.R[e]];
         hm.edge_tri[2 * k + 1] = (int32_t)new_of[c.L[e]];
-        hm.edge_nodes[2 * k] = (int32_t)c.edges[2 * e];
-        hm.edge_nodes[2 * k + 1] = (int32_t)c.edges[2 * e + 1];
     }
     // per stored triangle: vertices rotated to start at the smallest caller node id
     hm.tri_nodes.resize(3 * n_tris);
     hm.tri_code.resize(3 * n_tris);
-    hm.edge_opp.assign(2 * n_ei, -1);
     for (int64_t j = 0; j < n_tris; ++j) {
         const int64_t cj = hm.perm_tri[j];
         const int64_t* v = &c.tri[3 * cj];
@@ -592,7 +588,6 @@ int build_host_mesh(const double* xy, int64_t n_nodes, const int32_t* tris, int6
             } else {
                 const int neg = c.tri_neg[3 * cj + src];
                 hm.tri_code[3 * j + q] = (int32_t)(2 * k + neg);
-                hm.edge_opp[2 * k + neg] = (int32_t)v[(src + 2) % 3];
             }
         }
     }

@@ -20,8 +20,6 @@ struct HostMesh {
     std::vector<int32_t> edge_tri;      // 2*n_ei: (R, L) stored triangle ids
     std::vector<int32_t> tri_code;      // 3*n_tris: 2*k + neg (k = n_ei for a boundary edge)
     std::vector<int32_t> tri_nodes;     // 3*n_tris: caller node ids, rotated, CCW
-    std::vector<int32_t> edge_nodes;    // 2*n_ei: (low, high) caller node ids
-    std::vector<int32_t> edge_opp;      // 2*n_ei: node opposite the edge in R, in L
     std::vector<int64_t> tile_tri_off;  // KD order: n_tiles+1 stored-triangle offsets
 };
 

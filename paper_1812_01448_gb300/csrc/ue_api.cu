@@ -62,6 +62,13 @@ struct ue_mesh {
     ue_free_fn free_fn = nullptr;
     void* alloc_ctx = nullptr;
     std::vector<void*> allocs;
+    // without callbacks: small blocks are cut from a few large ones (Arena below)
+    struct Piece {
+        char* p;
+        size_t bytes;
+    };
+    std::vector<Piece> chunks, spare, pieces;   // from cudaMalloc; free parts of them; parts in use
+    size_t reserve = 0;                         // least size of the next chunk
 
     bool built = false;
     int precision = UE_PREC_FP32;
@@ -158,6 +165,83 @@ struct ue_mesh {
 
 namespace {
 
+// Device memory without allocator callbacks.  A cudaMalloc and its cudaFree cost about 60 us and a
+// setup makes some 27 of them: blocks up to kDirect are cut, first fit, from chunks (the first as
+// large as a setup's arrays), larger ones come from cudaMalloc as before.  A released block is reused
+// only after the device has gone idle, as cudaFree waits too, so work on another stream that
+// still reads it is safe.  A rebuild starts from one chunk of the size that the last build took.
+constexpr size_t kDirect = (size_t)64 << 20, kChunk = (size_t)2 << 20, kAlign = 256;
+
+void* arena_alloc(ue_mesh* m, size_t bytes) {
+    bytes = (bytes + kAlign - 1) / kAlign * kAlign;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (size_t i = 0; i < m->spare.size(); ++i) {
+            ue_mesh::Piece& f = m->spare[i];
+            if (f.bytes < bytes) continue;
+            char* p = f.p;
+            f.p += bytes;
+            f.bytes -= bytes;
+            if (f.bytes == 0) m->spare.erase(m->spare.begin() + i);
+            m->pieces.push_back({p, bytes});
+            return p;
+        }
+        if (pass == 1) break;
+        size_t held = 0;
+        for (const ue_mesh::Piece& c : m->chunks) held += c.bytes;
+        const size_t want = std::max(bytes, std::max(kChunk, std::min(std::max(held / 4, m->reserve), 4 * kDirect)));
+        m->reserve = 0;
+        void* c = nullptr;
+        size_t got = want;
+        if (cudaMalloc(&c, want) != cudaSuccess) {   // little memory left: no more than asked for
+            cudaGetLastError();
+            got = bytes;
+            if (want == bytes || cudaMalloc(&c, bytes) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+        }
+        m->chunks.push_back({(char*)c, got});
+        m->spare.push_back({(char*)c, got});
+    }
+    return nullptr;
+}
+
+bool arena_release(ue_mesh* m, void* p) {
+    for (size_t i = 0; i < m->pieces.size(); ++i)
+        if (m->pieces[i].p == p) {
+            cudaDeviceSynchronize();
+            m->spare.push_back(m->pieces[i]);
+            m->pieces[i] = m->pieces.back();
+            m->pieces.pop_back();
+            return true;
+        }
+    return false;
+}
+
+// All blocks of the arena free again.  keep: as one chunk for the next build.
+void arena_reset(ue_mesh* m, bool keep) {
+    m->pieces.clear();
+    m->spare.clear();
+    size_t held = 0;
+    for (const ue_mesh::Piece& c : m->chunks) held += c.bytes;
+    if (keep && m->chunks.size() == 1) {
+        cudaDeviceSynchronize();
+        m->spare = m->chunks;
+        return;
+    }
+    for (const ue_mesh::Piece& c : m->chunks) cudaFree(c.p);
+    m->chunks.clear();
+    void* c = nullptr;
+    if (keep && held > 0) {
+        if (cudaMalloc(&c, held) == cudaSuccess) {
+            m->chunks.push_back({(char*)c, held});
+            m->spare = m->chunks;
+        } else {
+            cudaGetLastError();
+        }
+    }
+}
+
 void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s) {
     if (bytes == 0) bytes = 16;
     void* p = nullptr;
@@ -167,6 +251,8 @@ void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s) {
             if (m->free_fn) m->free_fn(p, (void*)s, m->alloc_ctx);
             p = nullptr;
         }
+    } else if (bytes <= kDirect) {
+        return arena_alloc(m, bytes);
     } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         p = nullptr;
@@ -175,12 +261,13 @@ void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s) {
     return p;
 }
 
-void dev_free_all(ue_mesh* m, cudaStream_t s) {
+void dev_free_all(ue_mesh* m, cudaStream_t s, bool keep_arena = false) {
     for (void* p : m->allocs) {
         if (m->free_fn) m->free_fn(p, (void*)s, m->alloc_ctx);
         else cudaFree(p);
     }
     m->allocs.clear();
+    arena_reset(m, keep_arena);
 }
 
 template <typename P>
@@ -191,7 +278,7 @@ bool alloc_into(ue_mesh* m, P*& out, size_t count, size_t elem, cudaStream_t s) 
 
 // Release one allocation made by dev_alloc (no-op for NULL).
 void dev_release(ue_mesh* m, void* p, cudaStream_t s) {
-    if (!p) return;
+    if (!p || arena_release(m, p)) return;
     for (size_t i = 0; i < m->allocs.size(); ++i)
         if (m->allocs[i] == p) {
             if (m->free_fn) m->free_fn(p, (void*)s, m->alloc_ctx);
@@ -917,6 +1004,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
     const HostMesh& h = m->hm;
     const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;
     const int64_t nt = h.n_tris, nei = h.n_ei, nn = h.n_nodes, ne = h.n_edges;
+    m->reserve = (size_t)(16 * nn + nt * (104 + 3 * (int64_t)esz) + nei * (56 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
     bool ok = alloc_into(m, m->d_xy, 2 * nn, 8, s) && alloc_into(m, m->d_tri_nodes, 3 * nt, 4, s) &&
               alloc_into(m, m->d_edge_nodes, 2 * nei + 2, 4, s) &&
               alloc_into(m, m->d_edge_opp, 2 * nei + 2, 4, s) &&
@@ -1337,7 +1425,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     // a rebuild starts from scratch
     drop_graph(m);
     UE_CUDA(cudaStreamSynchronize(s));
-    dev_free_all(m, s);
+    dev_free_all(m, s, true);
     m->d_tri_nb = nullptr;
     m->d_kof = m->d_inv = nullptr;
     m->d_xbad = nullptr;

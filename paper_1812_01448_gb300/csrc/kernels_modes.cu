@@ -445,18 +445,20 @@ size_t modes_work_doubles(int64_t n_t, int m) { return Block::doubles(n_t, m, 3)
 // How many products K V to take before the next Cholesky QR.  It only has to come before the
 // columns' norms and angles drift so far apart that forming W^T S W loses digits; the diagonal of
 // R, over the `p` products that led to it, tells the drift per product.  Products until it
-// reaches 100 (an error of the basis, not of its span, of 1e-12, gone at the next QR), at most 8,
+// reaches 100 (an error of the basis, not of its span, of 1e-12, gone at the next QR), at most 16,
 // and none that could overflow the Gram matrix.  One QR per product took 150 of the 180 us of an
-// iteration on 90k triangles with 16 columns; with up to 8 products it is 25 us per iteration.
+// iteration on 90k triangles with 16 columns; with up to 8 products an iteration takes 31 us, with up to
+// 16 25 us (12 of them the product).
 static int products_until_qr(const std::vector<double>& R, int m, int p) {
+    constexpr double kMost = 16.0;
     double lo = R[0], hi = R[0];
     for (int i = 1; i < m; ++i) {
         lo = std::min(lo, R[(size_t)i * m + i]);
         hi = std::max(hi, R[(size_t)i * m + i]);
     }
     const double drift = std::log10(hi / lo) / p, size = std::fabs(std::log10(hi)) / p;
-    const double most = std::min(drift > 0 ? 2.0 / drift : 8.0, size > 0 ? 140.0 / size : 8.0);
-    return (int)std::max(1.0, std::min(8.0, most));
+    const double most = std::min(drift > 0 ? 2.0 / drift : kMost, size > 0 ? 140.0 / size : kMost);
+    return (int)std::max(1.0, std::min(kMost, most));
 }
 
 cudaError_t modes_run(const int2* rl, const int4* tri, const double* elen, const double* d,

@@ -18,6 +18,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstddef>
 
@@ -253,29 +254,112 @@ __device__ __forceinline__ void mlp16(const PackedNet& N, uint32_t a0, uint32_t 
     s1 = x1;
 }
 
-// Forward on BF16 tensor cores (mma.sync m16n8k16, FP32 accumulation): one warp per 16 rows.
-__global__ void __launch_bounds__(128) k_mlp_fwd_bf16(const float* __restrict__ P,
-                                                      const float* __restrict__ X, int64_t n,
-                                                      float* __restrict__ z) {
-    __shared__ __align__(16) PackedNet net;
-    pack_net(net, P, threadIdx.x, blockDim.x);
-    __syncthreads();
-    const float b3 = net.b3[0];
+// Forward on BF16 tensor cores (mma.sync m16n8k16, FP32 accumulation): one warp per 16 rows.  The
+// whole network sits in a warp's registers as B fragments (16 for layer 1, 64 for layer 2), so a
+// tile is its loads, its products and its ReLUs; the next tile's inputs are loaded a tile ahead.
+// Bound by the warp-level tensor pipe: 40 products per 16 rows, about 15 cycles each on every SM
+// quarter, which is why the gain over fragments read from shared memory at every tile (460
+// instructions per tile, scalar input loads) is small.  5.07M rows: 192 -> 177 us at 384 threads per
+// SM (197 at 256, 195 at 512, where registers spill); 100k rows: 17 -> 13 us at 256 (15 at 384).
+template <int NT>
+__global__ void __launch_bounds__(NT, 1) k_mlp_fwd_bf16(const float* __restrict__ P,
+                                                        const float* __restrict__ X, int64_t n,
+                                                        float* __restrict__ z) {
+    __shared__ __align__(16) float bias[3 * kH];   // b1, b2, w3
+    for (int i = threadIdx.x; i < kH; i += NT) {
+        bias[i] = P[kOffB1 + i];
+        bias[kH + i] = P[kOffB2 + i];
+        bias[2 * kH + i] = P[kOffW3 + i];
+    }
+    const float b3 = __ldg(P + kOffB3);
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); tile * 16 < n;
-         tile += warps) {
+    // B fragments: column n = 8 nt + g, rows 2t, 2t + 1 and 2t + 8, 2t + 9 of each k-tile
+    uint32_t w1[8][2], w2[4][8][2];
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        const float* r1 = P + kOffW1 + (8 * nt + g) * kD;
+        const float* r2 = P + kOffW2 + (8 * nt + g) * kH;
+        w1[nt][0] = pack_bf16(__ldg(r1 + 2 * t), __ldg(r1 + 2 * t + 1));
+        w1[nt][1] = t < 2 ? pack_bf16(__ldg(r1 + 2 * t + 8), __ldg(r1 + 2 * t + 9)) : 0u;
+#pragma unroll
+        for (int kt = 0; kt < 4; ++kt) {
+            w2[kt][nt][0] = pack_bf16(__ldg(r2 + 16 * kt + 2 * t), __ldg(r2 + 16 * kt + 2 * t + 1));
+            w2[kt][nt][1] = pack_bf16(__ldg(r2 + 16 * kt + 2 * t + 8), __ldg(r2 + 16 * kt + 2 * t + 9));
+        }
+    }
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * (NT / 32);
+    const bool pair = ((uintptr_t)X & 7u) == 0;   // rows are 48 bytes: pairs of floats together
+    auto load2 = [&](int64_t r, int c) {
+        float2 v = make_float2(0.f, 0.f);
+        if (r < n) {
+            const float* x = X + r * kD + c;
+            if (pair) v = __ldg(reinterpret_cast<const float2*>(x));
+            else v = make_float2(__ldg(x), __ldg(x + 1));
+        }
+        return v;
+    };
+    auto load = [&](int64_t tile, float2 (&x)[4]) {
         const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
-        auto xv = [&](int64_t r, int c) { return (r < n && c < kD) ? __ldg(X + r * kD + c) : 0.f; };
-        const uint32_t a0 = pack_bf16(xv(r0, 2 * t), xv(r0, 2 * t + 1));
-        const uint32_t a1 = pack_bf16(xv(r1, 2 * t), xv(r1, 2 * t + 1));
-        const uint32_t a2 = pack_bf16(xv(r0, 2 * t + 8), xv(r0, 2 * t + 9));
-        const uint32_t a3 = pack_bf16(xv(r1, 2 * t + 8), xv(r1, 2 * t + 9));
-        float s0, s1;
-        mlp16(net, a0, a1, a2, a3, s0, s1);
+        x[0] = load2(r0, 2 * t);
+        x[1] = load2(r1, 2 * t);
+        x[2] = t < 2 ? load2(r0, 2 * t + 8) : make_float2(0.f, 0.f);
+        x[3] = t < 2 ? load2(r1, 2 * t + 8) : make_float2(0.f, 0.f);
+    };
+    int64_t tile = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5);
+    float2 x[4];
+    if (tile * 16 < n) load(tile, x);
+    for (; tile * 16 < n; tile += stride) {
+        const uint32_t a0 = pack_bf16(x[0].x, x[0].y), a1 = pack_bf16(x[1].x, x[1].y);
+        const uint32_t a2 = pack_bf16(x[2].x, x[2].y), a3 = pack_bf16(x[3].x, x[3].y);
+        if ((tile + stride) * 16 < n) load(tile + stride, x);
+        // relu, then BF16: the C fragments of layer 1 (n-tiles 2kt, 2kt + 1) are the A fragments
+        // of layer 2's k-tile kt
+        uint32_t c[4][4];
+#pragma unroll
+        for (int kt = 0; kt < 4; ++kt) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int nt = 2 * kt + h;
+                const float2 bb = *reinterpret_cast<const float2*>(bias + nt * 8 + 2 * t);
+                float h1[4] = {bb.x, bb.y, bb.x, bb.y};
+                mma_bf16(h1, a0, a1, a2, a3, w1[nt][0], w1[nt][1]);
+                c[kt][2 * h] = pack_bf16(fmaxf(h1[0], 0.f), fmaxf(h1[1], 0.f));
+                c[kt][2 * h + 1] = pack_bf16(fmaxf(h1[2], 0.f), fmaxf(h1[3], 0.f));
+            }
+        }
+        float x0 = 0.f, x1 = 0.f;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {   // four n-tiles at a time: 16 accumulators, not 32
+            float h2[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 bb = *reinterpret_cast<const float2*>(bias + kH + (4 * half + i) * 8 + 2 * t);
+                h2[i][0] = bb.x;
+                h2[i][1] = bb.y;
+                h2[i][2] = bb.x;
+                h2[i][3] = bb.y;
+            }
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    mma_bf16(h2[i], c[kt][0], c[kt][1], c[kt][2], c[kt][3], w2[kt][4 * half + i][0], w2[kt][4 * half + i][1]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 w = *reinterpret_cast<const float2*>(bias + 2 * kH + (4 * half + i) * 8 + 2 * t);
+                x0 += w.x * fmaxf(h2[i][0], 0.f) + w.y * fmaxf(h2[i][1], 0.f);
+                x1 += w.x * fmaxf(h2[i][2], 0.f) + w.y * fmaxf(h2[i][3], 0.f);
+            }
+        }
+        x0 += __shfl_xor_sync(0xffffffffu, x0, 1);
+        x0 += __shfl_xor_sync(0xffffffffu, x0, 2);
+        x1 += __shfl_xor_sync(0xffffffffu, x1, 1);
+        x1 += __shfl_xor_sync(0xffffffffu, x1, 2);
         if (t == 0) {
-            if (r0 < n) z[r0] = s0 + b3;
-            if (r1 < n) z[r1] = s1 + b3;
+            const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
+            if (r0 < n) z[r0] = x0 + b3;
+            if (r1 < n) z[r1] = x1 + b3;
         }
     }
 }
@@ -657,53 +741,102 @@ __global__ void k_mlp_fwd_f32(const float* __restrict__ P, const float* __restri
 }
 
 // ---------------------------------------------------------------------------------------
-// backward for selected rows: per-row gradient rows (deterministic), reduced in fixed order.
+// backward for selected rows, summed over the rows in an order that does not change.
 // bf16 = 1 repeats the forward's BF16 rounding of x, W1, W2 and h1.
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float rb(float x, int bf16) {
     return bf16 ? __bfloat162float(__float2bfloat16_rn(x)) : x;
 }
 
-__global__ void __launch_bounds__(64) k_mlp_bwd_rows(const float* __restrict__ P,
-                                                     const float* __restrict__ X,
-                                                     const int64_t* __restrict__ rows,
-                                                     const float* __restrict__ dz, int bf16,
-                                                     float* __restrict__ G) {
-    const int64_t m = blockIdx.x;
-    const int o = threadIdx.x;   // hidden unit
-    __shared__ float x[kD], h1[kH], d2[kH];
-    const int64_t r = rows[m];
-    if (o < kD) x[o] = rb(X[r * kD + o], bf16);
-    __syncthreads();
-    float a1 = P[kOffB1 + o];
-    for (int i = 0; i < kD; ++i) a1 += rb(P[kOffW1 + o * kD + i], bf16) * x[i];
-    h1[o] = rb(fmaxf(a1, 0.f), bf16);
-    __syncthreads();
-    float a2 = P[kOffB2 + o];
-    for (int i = 0; i < kH; ++i) a2 += rb(P[kOffW2 + o * kH + i], bf16) * h1[i];
-    const float g = dz[m];
-    float* Gm = G + m * (int64_t)kNParams;
-    const float h2 = fmaxf(a2, 0.f);
-    Gm[kOffW3 + o] = g * h2;
-    if (o == 0) Gm[kOffB3] = g;
-    const float dd2 = a2 > 0.f ? g * P[kOffW3 + o] : 0.f;
-    d2[o] = dd2;
-    Gm[kOffB2 + o] = dd2;
-    for (int i = 0; i < kH; ++i) Gm[kOffW2 + o * kH + i] = dd2 * h1[i];
-    __syncthreads();
-    float d1 = 0.f;
-    for (int i = 0; i < kH; ++i) d1 += d2[i] * rb(P[kOffW2 + i * kH + o], bf16);
-    d1 = a1 > 0.f ? d1 : 0.f;
-    Gm[kOffB1 + o] = d1;
-    for (int i = 0; i < kD; ++i) Gm[kOffW1 + o * kD + i] = d1 * x[i];
+// A block keeps the network in shared memory and its share of the gradient in registers (16 + 3
+// weights per thread and its unit's biases) over its rows, four rows at a time: 64 threads, one per
+// hidden unit, take a row forward and back, then all 256 add the four outer products.  One sum per
+// block is written; with one gradient row per mesh row (20 KB) the sum over them read it all
+// again, one thread per parameter in a row: 19 + 16 us on 400 rows, milliseconds on 20,000, against
+// 16 + 4 us here on 400 rows (bound by the latency of a row's chain of sums).
+constexpr int kBwdRows = 4, kBwdThreads = kH * kBwdRows, kW2P = kH + 1;   // padded row: no bank conflicts
+__global__ void __launch_bounds__(kBwdThreads) k_mlp_bwd(const float* __restrict__ P, const float* __restrict__ X,
+                                                         const int64_t* __restrict__ rows, const float* __restrict__ dz,
+                                                         int64_t m, int bf16, float* __restrict__ part) {
+    __shared__ float w1[kH * (kD + 1)], w2[kH * kW2P], b1[kH], b2[kH], w3[kH];
+    __shared__ float x[kBwdRows][kD], h1[kBwdRows][kH], h2[kBwdRows][kH], d1[kBwdRows][kH], d2[kBwdRows][kH], dzr[kBwdRows];
+    const int tid = threadIdx.x, o = tid & (kH - 1), p = tid / kH;   // hidden unit, row of the group
+    for (int i = tid; i < kH * kD; i += kBwdThreads) w1[(i / kD) * (kD + 1) + i % kD] = rb(P[kOffW1 + i], bf16);
+    for (int i = tid; i < kH * kH; i += kBwdThreads) w2[(i / kH) * kW2P + i % kH] = rb(P[kOffW2 + i], bf16);
+    if (tid < kH) {
+        b1[tid] = P[kOffB1 + tid];
+        b2[tid] = P[kOffB2 + tid];
+        w3[tid] = P[kOffW3 + tid];
+    }
+    float gw2[kH / kBwdRows] = {}, gw1[kD / kBwdRows] = {}, gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f;
+    for (int64_t i0 = (int64_t)blockIdx.x * kBwdRows; i0 < m; i0 += (int64_t)gridDim.x * kBwdRows) {
+        const int64_t i = i0 + p;
+        const int64_t r = i < m ? rows[i] : -1;   // -1: an empty segment's row adds nothing
+        __syncthreads();
+        if (o < kD) x[p][o] = r >= 0 ? rb(X[r * kD + o], bf16) : 0.f;
+        if (o == 0) dzr[p] = r >= 0 ? dz[i] : 0.f;
+        __syncthreads();
+        float a1 = b1[o];
+        for (int k = 0; k < kD; ++k) a1 += w1[o * (kD + 1) + k] * x[p][k];
+        h1[p][o] = rb(fmaxf(a1, 0.f), bf16);
+        __syncthreads();
+        float a2 = b2[o];
+#pragma unroll 16
+        for (int k = 0; k < kH; ++k) a2 += w2[o * kW2P + k] * h1[p][k];
+        const float g = dzr[p];
+        h2[p][o] = g * fmaxf(a2, 0.f);
+        d2[p][o] = a2 > 0.f ? g * w3[o] : 0.f;
+        __syncthreads();
+        float s = 0.f;
+#pragma unroll 16
+        for (int k = 0; k < kH; ++k) s += d2[p][k] * w2[k * kW2P + o];
+        d1[p][o] = a1 > 0.f ? s : 0.f;
+        __syncthreads();
+        for (int q = 0; q < kBwdRows; ++q) {
+            const float e2 = d2[q][o], e1 = d1[q][o];
+#pragma unroll
+            for (int k = 0; k < kH / kBwdRows; ++k) gw2[k] += e2 * h1[q][p * (kH / kBwdRows) + k];
+#pragma unroll
+            for (int k = 0; k < kD / kBwdRows; ++k) gw1[k] += e1 * x[q][p * (kD / kBwdRows) + k];
+            if (p == 0) {
+                gb1 += e1;
+                gb2 += e2;
+                gw3 += h2[q][o];
+                if (o == 0) gb3 += dzr[q];
+            }
+        }
+    }
+    float* G = part + (int64_t)blockIdx.x * kNParams;
+#pragma unroll
+    for (int k = 0; k < kH / kBwdRows; ++k) G[kOffW2 + o * kH + p * (kH / kBwdRows) + k] = gw2[k];
+#pragma unroll
+    for (int k = 0; k < kD / kBwdRows; ++k) G[kOffW1 + o * kD + p * (kD / kBwdRows) + k] = gw1[k];
+    if (p == 0) {
+        G[kOffB1 + o] = gb1;
+        G[kOffB2 + o] = gb2;
+        G[kOffW3 + o] = gw3;
+        if (o == 0) G[kOffB3] = gb3;
+    }
 }
 
-__global__ void k_colsum(const float* __restrict__ G, int64_t m, float* __restrict__ g) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kNParams) return;
+// grad[p] = sum of the blocks' shares: 64 parameters and 16 slices of the blocks per block
+constexpr int kSumParams = 64, kSumSlices = 16;
+__global__ void __launch_bounds__(kSumParams * kSumSlices) k_colsum(const float* __restrict__ G, int nb,
+                                                                    float* __restrict__ g) {
+    __shared__ float red[kSumSlices][kSumParams];
+    const int c = threadIdx.x & (kSumParams - 1), q = threadIdx.x / kSumParams;
+    const int p = blockIdx.x * kSumParams + c;
     float s = 0.f;
-    for (int64_t i = 0; i < m; ++i) s += G[i * kNParams + p];
-    g[p] = s;
+    if (p < kNParams) {
+#pragma unroll 4
+        for (int i = q; i < nb; i += kSumSlices) s += G[(int64_t)i * kNParams + p];
+    }
+    red[q][c] = s;
+    __syncthreads();
+    if (q == 0 && p < kNParams) {
+        for (int i = 1; i < kSumSlices; ++i) s += red[i][c];
+        g[p] = s;
+    }
 }
 
 // Adam (Kingma & Ba 2015) with bias correction.
@@ -719,40 +852,58 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-// Per segment (mesh): best = max_j (z_j + base_j) and its row (first on ties).
-__global__ void k_seg_argmax(const float* __restrict__ z, const float* __restrict__ base,
-                             const int64_t* __restrict__ off, int n_seg, float* __restrict__ best,
-                             int64_t* __restrict__ arg) {
+// Per segment (mesh): best = max_j (z_j + base_j) and its row (first on ties).  Eight rows per thread
+// in flight: one at a time in blocks of 256, the longest of 400 segments (50k rows) took 66 us
+// of latency; 15 us so.
+constexpr int kArgThreads = 512, kArgRows = 8;
+__global__ void __launch_bounds__(kArgThreads) k_seg_argmax(const float* __restrict__ z, const float* __restrict__ base,
+                                                            const int64_t* __restrict__ off, int n_seg,
+                                                            float* __restrict__ best, int64_t* __restrict__ arg) {
     const int s = blockIdx.x;
     if (s >= n_seg) return;
-    __shared__ float bv[256];
-    __shared__ int64_t bi[256];
+    __shared__ float bv[kArgThreads / 32];
+    __shared__ int64_t bi[kArgThreads / 32];
     float v = -INFINITY;
     int64_t a = -1;
-    for (int64_t j = off[s] + threadIdx.x; j < off[s + 1]; j += blockDim.x) {
-        const float x = z[j] + base[j];
-        if (x > v) {
-            v = x;
-            a = j;
+    const int64_t end = off[s + 1];
+    for (int64_t j0 = off[s] + threadIdx.x; j0 < end; j0 += kArgThreads * kArgRows) {
+        float x[kArgRows], b[kArgRows];
+#pragma unroll
+        for (int u = 0; u < kArgRows; ++u) {
+            const int64_t j = j0 + u * kArgThreads;
+            x[u] = j < end ? __ldg(z + j) : 0.f;
+            b[u] = j < end ? __ldg(base + j) : -INFINITY;
         }
-    }
-    bv[threadIdx.x] = v;
-    bi[threadIdx.x] = a;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            const float w = bv[threadIdx.x + o];
-            const int64_t wi = bi[threadIdx.x + o];
-            if (w > bv[threadIdx.x] || (w == bv[threadIdx.x] && wi >= 0 && (bi[threadIdx.x] < 0 || wi < bi[threadIdx.x]))) {
-                bv[threadIdx.x] = w;
-                bi[threadIdx.x] = wi;
+#pragma unroll
+        for (int u = 0; u < kArgRows; ++u) {
+            const float t = x[u] + b[u];
+            if (t > v) {
+                v = t;
+                a = j0 + u * kArgThreads;
             }
         }
-        __syncthreads();
     }
+    auto take = [&](float w, int64_t wi) {
+        if (w > v || (w == v && wi >= 0 && (a < 0 || wi < a))) {
+            v = w;
+            a = wi;
+        }
+    };
+    for (int o = 16; o > 0; o >>= 1) {
+        const float w = __shfl_xor_sync(0xffffffffu, v, o);
+        const int64_t wi = __shfl_xor_sync(0xffffffffu, (long long)a, o);
+        take(w, wi);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) {
+        bv[warp] = v;
+        bi[warp] = a;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        best[s] = bv[0];
-        arg[s] = bi[0];
+        for (int w = 1; w < kArgThreads / 32; ++w) take(bv[w], bi[w]);
+        best[s] = v;
+        arg[s] = a;
     }
 }
 
@@ -783,10 +934,12 @@ cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf
                                cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     if (bf16) {
+        // one block per SM (a warp's registers hold the network); few tiles per warp: 8 warps, whose
+        // start is shorter, else 12
         const int64_t tiles = (n + 15) / 16;
-        int blocks = (int)((tiles + 3) / 4);
-        if (blocks > 152 * 16) blocks = 152 * 16;
-        k_mlp_fwd_bf16<<<blocks, 128, 0, s>>>(P, X, n, z);
+        auto grid = [&](int nt) { return (unsigned)std::min<int64_t>((tiles + nt / 32 - 1) / (nt / 32), 152); };
+        if (tiles < 152 * 8 * 32) k_mlp_fwd_bf16<256><<<grid(256), 256, 0, s>>>(P, X, n, z);
+        else k_mlp_fwd_bf16<384><<<grid(384), 384, 0, s>>>(P, X, n, z);
     } else {
         k_mlp_fwd_f32<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(P, X, n, z);
     }
@@ -796,8 +949,11 @@ cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf
 cudaError_t launch_mlp_backward(const float* P, const float* X, const int64_t* rows, const float* dz,
                                 int64_t m, int bf16, float* work, float* grad, cudaStream_t s) {
     if (m <= 0) return cudaMemsetAsync(grad, 0, sizeof(float) * kNParams, s);
-    k_mlp_bwd_rows<<<(unsigned)m, 64, 0, s>>>(P, X, rows, dz, bf16, work);
-    k_colsum<<<(kNParams + 255) / 256, 256, 0, s>>>(work, m, grad);
+    // at most two blocks per SM; no more shares than the m gradient rows `work` holds
+    const int64_t groups = (m + kBwdRows - 1) / kBwdRows;
+    const int blocks = (int)(groups < 304 ? groups : 304);
+    k_mlp_bwd<<<blocks, kBwdThreads, 0, s>>>(P, X, rows, dz, m, bf16, work);
+    k_colsum<<<(kNParams + kSumParams - 1) / kSumParams, kSumParams * kSumSlices, 0, s>>>(work, blocks, grad);
     return cudaGetLastError();
 }
 
@@ -811,7 +967,7 @@ cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, flo
 cudaError_t launch_seg_argmax(const float* z, const float* base, const int64_t* off, int n_seg,
                               float* best, int64_t* arg, cudaStream_t s) {
     if (n_seg <= 0) return cudaSuccess;
-    k_seg_argmax<<<n_seg, 256, 0, s>>>(z, base, off, n_seg, best, arg);
+    k_seg_argmax<<<n_seg, kArgThreads, 0, s>>>(z, base, off, n_seg, best, arg);
     return cudaGetLastError();
 }
 

@@ -226,8 +226,9 @@ int ue_write_fields_f32(ue_mesh* m, const float* E, const float* B, const float*
 int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
 
 /* Advance n_steps leap-frog steps, asynchronously on `stream`.  A call of a graph chunk of steps
- * or more on a mesh small enough for the chip's registers and shared memory (about 600k triangles
- * in FP32, 300k in FP64; plain and blocked variants, graph_chunk >= 0) runs resident: one
+ * or more on a mesh small enough for the chip's registers and shared memory (about 1.2M
+ * triangles in FP32, 600k with a current or a frame, 300k in FP64, provided neighbouring triangles
+ * are mostly stored close together; plain and blocked variants, graph_chunk >= 0) runs resident: one
  * cooperative launch for up to 1024 steps, with the same results bit for bit.  Its waits are
  * bounded; one that runs out is reported by ue_check (UE_ERR_TIMEOUT).  Errors of the launches are
  * reported here; device-side conditions surface at the next synchronous call. */

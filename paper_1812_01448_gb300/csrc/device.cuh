@@ -232,20 +232,32 @@ int persistent_grid(int device);
 cudaError_t launch_persistent(const DevMesh& m, int n_steps, unsigned* sync, int* err,
                               long long budget, int skip_cta, int grid, cudaStream_t s);
 
-// Resident step (kernels_flow.cu): the launch shape for a mesh that fits the chip, its exchange
-// words and its control words {tag of the next launch, CTAs done, error}.
+// Resident step (kernels_flow.cu): the launch shape for a mesh that fits the chip, its plan, its
+// exchange words and its control words {tag of the next launch, CTAs done, error, plan overflow}.
 constexpr int kFlowSteps = 1024;  // most steps of one resident launch (and its g table)
 struct FlowDev {
     int grid = 0;                 // CTAs; 0: the mesh does not fit, 1: one CTA holds it all
-    int threads = 0, shape = 0, per = 0, fper = 0, hcap = 0, scap = 0;
+    int shape = 0, per = 0, fper = 0, cap = 0, halo = 0;
     unsigned long long* slots = nullptr;   // 2 * slot_words, zeroed
     int64_t slot_words = 0;
-    unsigned* ctl = nullptr;
+    unsigned* ctl = nullptr;      // 4 words
+    int* place = nullptr;         // [n_t] CTA * cap + slot of each triangle
+    int4* rec = nullptr;          // [grid * cap] slot records
+    void* sent = nullptr;         // sent_bytes: source entries
+    size_t sent_bytes = 0;
+    int* hlist = nullptr;         // [grid * halo] remote neighbours
+    int2* cnt = nullptr;          // [grid]
+    int4* crec = nullptr;         // [frame cells]
     int skip = -1;                // tests only: this CTA returns at once
 };
 // n_fc: cells of a PML frame stepped with the mesh.  False when the mesh does not fit.
-bool flow_plan(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl);
+bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl);
+// Whether m, as it stands, steps by it (the largest shape takes vacuum media only).
+bool flow_takes(const FlowDev& fl, const DevMesh& m);
 cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s);
+// The plan from the mesh's tables and source (again when the source changes); sets ctl[3] when a
+// CTA has more remote neighbours than it can list.
+cudaError_t launch_flow_plan(const FlowDev& fl, const DevMesh& m, cudaStream_t s);
 // n_steps steps of m in place in one launch; the source uses g-table entries gbase ..
 // gbase + n_steps - 1.  Uif: the circulations of a frame's interface edges.
 cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s);

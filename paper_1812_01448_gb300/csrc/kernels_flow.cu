@@ -22,12 +22,20 @@
 // barrier, then every triangle reads its neighbours there.  All CTAs are resident (cooperative
 // launch) and every wait is bounded: one that runs out sets the error word and ends the launch.
 //
-// What bounds it: a step is at least one exchange through L2 (store, poll, barrier: 1.2 us here)
-// up to about 1,000 triangles per SM, then the SM's issue slots.  Measured per step on GB300 with
-// a line source, against graph replays of the two plain kernels: 90k triangles 1.23 us (6.2 us),
-// 305k 1.89; one CTA alone 0.35 us on 1,040 triangles (2.9 us).  Against k_tbp (8 steps per launch,
-// ring-ordered tiles) on 480k to 500k triangles 2.4 us (5.0 us), with a plasma current 4.4
-// (k_tb 4.7), with a 16-cell PML frame 4.3 (10.0, the frame's tiles stepping by plain launches).
+// A plan made once (k_flow_plan, after the source is set) orders each CTA's triangles into slots:
+// those that publish first, so that their values travel while the rest is computed, then those
+// with a source or a conductor's edge, so that few warps take that branch, then the others in
+// stored order; and it turns each triangle's neighbours into shared-memory addresses.
+//
+// What bounds it: one exchange through L2 (store, poll, barrier: about 0.9 us) up to some 1,000
+// triangles per SM, then the SM's issue slots (about 25 instructions per triangle; everything a slot
+// needs is at a compile-time offset from one register).  Measured per step on GB300, with a line
+// source, against graph replays of the two plain kernels: 90k triangles 0.97 us (6.2), 305k 1.20,
+// 1.2M 3.06 (9.3); one CTA alone 0.41 us on 1,040 triangles, 0.30 without a source (2.9).  Against
+// k_tbp (8 steps per launch, ring-ordered tiles) on 500k triangles 1.38 us (5.0), with a plasma
+// current 1.70 (k_tb 4.7), with a 16-cell PML frame 1.75 (10.0: the frame's tiles step by plain
+// launches).  With slots in stored order, neighbours found at each launch and unpacked addresses
+// hoisted into (then spilled) registers the same steps took 1.23, 1.89, -, 0.52, 2.44, 4.4 and 4.3.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,47 +48,25 @@ namespace ue {
 
 namespace {
 
-// Per triangle slot, two words: byte offsets of the three neighbours' B in the CTA's buffer (16
-// bits each), then flags.
-constexpr unsigned kSrc = 1u << 16;        // 3 bits: the edge has a source
-constexpr unsigned kPublish = 1u << 19;    // a neighbour is in another CTA
-constexpr unsigned kIface = 1u << 20;      // 3 bits: the edge borders a frame cell
-constexpr unsigned kWall = 1u << 23;       // 3 bits: a conductor's edge (its offset is the triangle's own)
-constexpr unsigned kFar = 1u << 26;        // 3 bits: neighbour polled by this thread (the CTA's list is full)
-constexpr int kCellFar = 1 << 30;          // the same for a frame cell's neighbour
-constexpr int kNoEntry = 0xFFFF;
-
-template <typename T>
-struct FlowArgs {
-    const int4* tri;
-    const int2* rl;
-    const T* cU;
-    const double* cB64;
-    T* U;
-    T* B;
-    const T* pb;
-    T* J;
-    T pa, mdt;
-    const int2* hash;
-    unsigned bits;
-    const T* src_c;
-    const int32_t* src_grp;
-    const double* gtab;
-    int gstride;
-    int gbase;              // this launch's first entry in the g table
-    int has_src, n_grp;
-    int n_t, n_ei, n_ei_pad;
-    int per;                // triangles per CTA
-    int hcap, scap;         // capacities of the CTA's lists: remote neighbours, source edges
-    unsigned long long* slots[2];
-    unsigned* ctl;          // {tag of the next launch, CTAs done, error word}
-    long long* step;
-    int n_steps;
-    int skip;               // tests only (-1 otherwise): this CTA returns at once
-    FrameDev f;
-    T* Uif;                 // circulations of the frame's interface edges
-    int fper;               // frame cells per CTA
+// Launch shapes, the first that fits: threads of a CTA, triangle slots per thread, and remote
+// neighbours a CTA lists (FP32, FP64).  Up to two slots (one in FP64) the coefficients sit in
+// registers too, else in shared memory.  The last shape is for vacuum media without a frame: 6 words
+// of state per slot leave room for 16 of them, a current's 9 do not.
+struct FlowShape {
+    int nt, ts, halo32, halo64;
 };
+constexpr FlowShape kShapes[4] = {{1024, 1, 3072, 3072}, {1024, 2, 6144, 3072}, {512, 8, 3456, 0}, {512, 16, 2560, 0}};
+constexpr int kVacuumShape = 3;
+template <typename T, int SH>
+constexpr int kHalo = sizeof(T) == 4 ? kShapes[SH].halo32 : kShapes[SH].halo64;
+template <typename T, int SH>
+constexpr int kBuffer = kShapes[SH].nt * kShapes[SH].ts + kHalo<T, SH>;   // B values per buffer
+
+// Slot record {triangle, n01, n2f, 0}: byte offsets of the three neighbours' B in a buffer, 16 bits
+// each (own slots, then the CTA's remote neighbours), and flags above the third.
+constexpr unsigned kSrc = 1u << 16;     // 3 bits: the edge has a source
+constexpr unsigned kWall = 1u << 19;    // 3 bits: a conductor's edge (the offset is the slot's own)
+constexpr unsigned kIface = 1u << 22;   // 3 bits: the edge borders a frame cell
 
 template <typename T>
 struct Vec4 {
@@ -91,17 +77,80 @@ struct __align__(16) Vec4<float> {
     float x, y, z, w;
 };
 
-// A triangle with source edges: s_q dt |e| a of each edge (0 without a source), and its group's
-// offset in the g table.
+// A source triangle's s_q dt |e| a of its edges (0 without a source) and its group's offset in the g
+// table; indexed like the slot records.
 template <typename T>
 struct SrcEntry {
     T c[3];
     int g;
 };
+template <>
+struct __align__(16) SrcEntry<float> {
+    float c[3];
+    int g;
+};
+template <>
+struct __align__(16) SrcEntry<double> {
+    double c[3];
+    int g;
+};
+
+template <typename T>
+struct FlowArgs {
+    const int4* tri;
+    const T* cU;
+    const double* cB64;
+    T* U;
+    T* B;
+    const T* pb;
+    T* J;
+    T pa, mdt;
+    const int4* rec;        // cap per CTA
+    const SrcEntry<T>* sent;
+    const int* hlist;       // halo per CTA: places (CTA * cap + slot, then the frame cells)
+    const int2* cnt;        // per CTA: publishing triangles, remote neighbours
+    const int4* crec;       // fper per CTA: offsets of a frame cell's neighbours, -1 none
+    const double* gtab;
+    int gbase;              // this launch's first entry in the g table
+    int one_grp;            // one source group: its g is staged in shared memory
+    int n_t, n_ei, n_ei_pad;
+    int per;                // triangles per CTA
+    unsigned long long* slots[2];
+    unsigned* ctl;          // {tag of the next launch, CTAs done, error word, plan overflow}
+    long long* step;
+    int n_steps;
+    int skip;               // tests only (-1 otherwise): this CTA returns at once
+    FrameDev f;
+    T* Uif;                 // circulations of the frame's interface edges
+    int fper;               // frame cells per CTA
+};
+
+__device__ __forceinline__ bool neg_bit(float c) { return __float_as_uint(c) >> 31; }
+__device__ __forceinline__ bool neg_bit(double c) { return (unsigned long long)__double_as_longlong(c) >> 63; }
+
+struct PlanArgs {
+    const int4* tri;
+    const int2* rl;
+    const void* cU;
+    const int2* hash;
+    unsigned bits;
+    const void* src_c;
+    const int32_t* src_grp;
+    int gstride, has_src;
+    int n_t, n_ei, n_ei_pad, per, cap, halo;
+    int* place;             // [n_t]
+    int4* rec;
+    void* sent;
+    int* hlist;
+    int2* cnt;
+    int4* crec;
+    unsigned* ctl;
+    FrameDev f;
+    int fper;
+};
 
 // the source index of stored edge k (k_edge_half's table), or -1
-template <typename T>
-__device__ __forceinline__ int src_index(const FlowArgs<T>& a, int k) {
+__device__ __forceinline__ int src_index(const PlanArgs& a, int k) {
     const unsigned size = 1u << a.bits;
     unsigned h = ((unsigned)k * 2654435761u) >> (32 - a.bits);
     int2 e = __ldg(a.hash + h);
@@ -112,174 +161,363 @@ __device__ __forceinline__ int src_index(const FlowArgs<T>& a, int k) {
     return e.x == k ? e.y : -1;
 }
 
-// Rare paths of a step, out of line so that they cost the common one no registers: the source
-// term of edge k looked up again (the CTA's source list is full), and a neighbour's B polled by
-// the thread that needs it (the CTA's list of remote neighbours is full).
+// The plan, one block per CTA of the resident launch.  First each triangle's place (CTA * cap +
+// slot) and how many publish; then the records, and the CTA's remote neighbours as places.  A CTA
+// with more of these than its list holds sets ctl[3]: the mesh then keeps its launches.
 template <typename T>
-__device__ __noinline__ T source_again(const FlowArgs<T>* a, int code, int at, T v) {
-    const int x = src_index(*a, code >> 1);
-    if (x < 0) return v;
-    const T sc = __ldg(a->src_c + x);
-    const T g = (T)__ldg(a->gtab + (size_t)__ldg(a->src_grp + x) * a->gstride + at);
-    return rn_fma((code & 1) ? -sc : sc, g, v);
-}
-template <typename T>
-__device__ __noinline__ T poll_one(const unsigned long long* slots, int o, unsigned tag, bool* ok) {
-    Word<T> w;
-    w.load(slots, o);
-    if (!word_wait(w, slots, o, tag)) *ok = false;
-    return w.value();
+__global__ void __launch_bounds__(1024) k_flow_order(const __grid_constant__ PlanArgs a) {
+    __shared__ int wsum[3][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int j0 = blockIdx.x * a.per, nloc = max(0, min(a.per, a.n_t - j0));
+    const T* cU = (const T*)a.cU;
+    // class 0: a neighbour in another CTA (or a frame cell), 1: a source or a conductor, 2: others
+    auto classify = [&](int l) {
+        const int4 t = __ldg(a.tri + j0 + l);
+        const int code[3] = {t.x, t.y, t.z};
+        int cls = 2;
+        for (int q = 0; q < 3; ++q) {
+            const int k = code[q] >> 1;
+            if (k < a.n_ei) {
+                const int2 r = __ldg(a.rl + k);
+                const int o = (code[q] & 1) ? r.x : r.y;
+                if (o < j0 || o >= j0 + nloc) return 0;
+                if (a.has_src && neg_bit(__ldg(cU + k))) cls = 1;
+            } else if (k >= a.n_ei_pad && a.fper > 0) {
+                return 0;
+            } else {
+                cls = 1;
+            }
+        }
+        return cls;
+    };
+    int cls[8];   // of local triangles tid + 1024 i (cap <= 8192)
+    int total[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (1024 * i >= a.per) break;
+        const int l = tid + 1024 * i;
+        cls[i] = l < nloc ? classify(l) : -1;
+        for (int k = 0; k < 3; ++k) total[k] += __syncthreads_count(cls[i] == k);
+    }
+    int base[3] = {0, total[0], total[0] + total[1]};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {   // stable: rank in class, in stored order
+        if (1024 * i >= a.per) break;
+        const int l = tid + 1024 * i;
+        unsigned m[3];
+        for (int k = 0; k < 3; ++k) {
+            m[k] = __ballot_sync(0xffffffffu, cls[i] == k);
+            if (lane == 0) wsum[k][warp] = __popc(m[k]);
+        }
+        __syncthreads();
+        for (int k = 0; k < 3; ++k) {
+            int before = 0, all = 0;
+            for (int w = 0; w < 32; ++w) {
+                before += w < warp ? wsum[k][w] : 0;
+                all += wsum[k][w];
+            }
+            if (cls[i] == k)
+                a.place[j0 + l] = (int)blockIdx.x * a.cap + base[k] + before + __popc(m[k] & ((1u << lane) - 1u));
+            base[k] += all;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) a.cnt[blockIdx.x].x = total[0];
 }
 
-__device__ __forceinline__ bool neg_bit(float c) { return __float_as_uint(c) >> 31; }
-__device__ __forceinline__ bool neg_bit(double c) { return (unsigned long long)__double_as_longlong(c) >> 63; }
+template <typename T>
+__global__ void __launch_bounds__(1024) k_flow_plan(const __grid_constant__ PlanArgs a) {
+    __shared__ int s_halo;
+    const int tid = threadIdx.x;
+    const int j0 = blockIdx.x * a.per, nloc = max(0, min(a.per, a.n_t - j0)), p0 = (int)blockIdx.x * a.cap;
+    const int cell0 = (int)gridDim.x * a.cap;   // place of frame cell 0
+    const T* cU = (const T*)a.cU;
+    if (tid == 0) s_halo = 0;
+    __syncthreads();
+    int* hl = a.hlist + (size_t)blockIdx.x * a.halo;
+    auto remote = [&](int place) -> unsigned {   // its offset; the first of the list when that is full
+        const int h = atomicAdd(&s_halo, 1);
+        if (h >= a.halo) return (unsigned)a.cap * (unsigned)sizeof(T);
+        hl[h] = place;
+        return (unsigned)(a.cap + h) * (unsigned)sizeof(T);
+    };
+    for (int l = tid; l < nloc; l += 1024) {
+        const int slot = a.place[j0 + l] - p0;
+        const int4 t = __ldg(a.tri + j0 + l);
+        const int code[3] = {t.x, t.y, t.z};
+        unsigned off[3], f = 0;
+        SrcEntry<T> se{{T(0), T(0), T(0)}, 0};
+        for (int q = 0; q < 3; ++q) {
+            const int k = code[q] >> 1;
+            off[q] = (unsigned)slot * (unsigned)sizeof(T);
+            if (k < a.n_ei) {
+                const int2 r = __ldg(a.rl + k);
+                const int o = (code[q] & 1) ? r.x : r.y, place = a.place[o];
+                if (o >= j0 && o < j0 + nloc) off[q] = (unsigned)(place - p0) * (unsigned)sizeof(T);
+                else off[q] = remote(place);
+                const int x = a.has_src && neg_bit(__ldg(cU + k)) ? src_index(a, k) : -1;
+                if (x >= 0) {
+                    const T sc = __ldg((const T*)a.src_c + x);
+                    se.c[q] = (code[q] & 1) ? -sc : sc;
+                    se.g = (int)__ldg(a.src_grp + x) * a.gstride;
+                    f |= kSrc << q;
+                }
+            } else if (k >= a.n_ei_pad && a.fper > 0) {
+                off[q] = remote(cell0 + a.f.icell[k - a.n_ei_pad]);
+                f |= kIface << q;
+            } else {
+                f |= kWall << q;
+            }
+        }
+        a.rec[p0 + slot] = make_int4(j0 + l, (int)(off[0] | (off[1] << 16)), (int)(off[2] | f), 0);
+        if (f & (7u * kSrc)) ((SrcEntry<T>*)a.sent)[p0 + slot] = se;
+    }
+    for (int t = tid; t < a.fper; t += 1024) {
+        const int cell = (int)blockIdx.x * a.fper + t;
+        if (cell >= (int)a.f.n_fc) break;
+        const FrameDev& f = a.f;
+        int I, J;
+        frame_ij(f, cell, I, J);
+        const bool in_x = I >= f.W && I < f.W + f.nx, in_y = J >= f.W && J < f.W + f.ny;
+        const int di[4] = {0, 0, -1, 1}, dj[4] = {-1, 1, 0, 0};   // bottom, top, left, right
+        const int kif[4] = {in_x && J == f.W + f.ny ? f.nx + (I - f.W) : -1, in_x && J == f.W - 1 ? I - f.W : -1,
+                            in_y && I == f.W + f.nx ? 2 * f.nx + f.ny + (J - f.W) : -1,
+                            in_y && I == f.W - 1 ? 2 * f.nx + (J - f.W) : -1};
+        int cn[4];
+        for (int d = 0; d < 4; ++d) {
+            cn[d] = -1;
+            if (frame_is_cell(f, I + di[d], J + dj[d])) {
+                cn[d] = (int)remote(cell0 + (int)frame_cell(f, I + di[d], J + dj[d]));
+            } else if (kif[d] >= 0) {
+                const int code = f.itri[kif[d]];
+                cn[d] = (int)remote(a.place[code >= 0 ? code : ~code]);
+            }
+        }
+        a.crec[cell] = make_int4(cn[0], cn[1], cn[2], cn[3]);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        a.cnt[blockIdx.x].y = min(s_halo, a.halo);
+        if (s_halo > a.halo) atomicOr(a.ctl + 3, 1u);
+    }
+}
 
-// Coefficients sit in registers while they fit beside the state, else in shared memory.
 template <typename T, int TS>
 constexpr bool kCoefRegs = sizeof(T) * TS <= 8;
 
-// Shared memory of a CTA of cap triangle slots and `cells` frame cells.
-template <typename T, bool PLASMA>
-__host__ __device__ constexpr size_t flow_smem(bool coef_regs, int cap, int hcap, int scap, int cells) {
-    return (coef_regs ? 0 : sizeof(Vec4<T>) * (size_t)cap * (PLASMA ? 2 : 1)) + sizeof(SrcEntry<T>) * (size_t)scap +
-           2 * sizeof(T) * ((size_t)cap + hcap) + sizeof(T) * (size_t)kFlowSteps + 4 * (size_t)hcap + 2 * (size_t)cap +
-           3 * sizeof(Vec4<T>) * (size_t)cells;
+// Shared memory of a CTA: two buffers of B, the coefficients (with a current's), g, the remote
+// neighbours, the frame cells' coefficients.
+template <typename T, bool PLASMA, int SH>
+constexpr size_t flow_smem(int cells) {
+    const size_t cap = (size_t)kShapes[SH].nt * kShapes[SH].ts;
+    return 2 * sizeof(T) * (size_t)kBuffer<T, SH> +
+           (kCoefRegs<T, kShapes[SH].ts> ? 0 : sizeof(T) * cap * (PLASMA ? 7 : 4)) + sizeof(T) * (size_t)kFlowSteps +
+           4 * (size_t)kHalo<T, SH> + 3 * sizeof(Vec4<T>) * (size_t)cells;
 }
 
-// NT: threads of a CTA (at most, for TS = 1); a thread holds local triangles tid + i * NT, i < TS.
-// SOLO: one CTA holds the whole mesh, nothing is published.
-template <typename T, int NT, int TS, bool PLASMA, bool FRAME, bool SOLO>
-__global__ void __launch_bounds__(NT, 1) k_flow(const __grid_constant__ FlowArgs<T> a) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ int s_hcnt, s_scnt;
-    const int tid = threadIdx.x, nth = TS > 1 ? NT : (int)blockDim.x, cap = TS * nth;
-    Vec4<T>* C = reinterpret_cast<Vec4<T>*>(smraw);                  // dt|e|/d of the three edges, dt/S
-    constexpr bool CR = kCoefRegs<T, TS>;
-    Vec4<T>* P = C + (CR ? 0 : cap);                                 // pb of the three edges
-    Vec4<T>* Fc = P + (CR || !PLASMA ? 0 : cap);                     // a frame cell's a, b of its sides and itself
-    SrcEntry<T>* S = reinterpret_cast<SrcEntry<T>*>(Fc + (FRAME ? 3 * a.fper : 0));
-    const int bcap = cap + a.hcap;
-    T* Bb = reinterpret_cast<T*>(S + a.scap);                        // two buffers: own, then remote B
-    T* gs = Bb + 2 * bcap;                                           // g of the launch's steps (one group)
-    int* hlist = reinterpret_cast<int*>(gs + kFlowSteps);            // the remote neighbours
-    unsigned short* spos = reinterpret_cast<unsigned short*>(hlist + a.hcap);   // source entry of a triangle
-    const int j0 = blockIdx.x * a.per;
-    const int nloc = max(0, min(a.per, a.n_t - j0));
-    if (tid == 0) s_hcnt = s_scnt = 0;
-    const unsigned tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
-    __syncthreads();
-    bool ok = true;
-    if (SOLO || (int)blockIdx.x != a.skip) {
-        T V[TS][3], J[TS][3], b[TS];
-        Vec4<T> Cr[CR ? TS : 1], Pr[CR && PLASMA ? TS : 1];
-        unsigned n01[TS], n2f[TS];
-        // the list entry of a neighbour in another CTA, or -1 when the list is full
-        auto remote = [&](int o) {
-            const int pos = atomicAdd(&s_hcnt, 1);
-            if (pos >= a.hcap) return -1;
-            hlist[pos] = o;
-            return cap + pos;
-        };
+// Shared accesses at an address plus a compile-time offset.  A step's loads read the buffer that
+// its stores do not touch, so they may move among the stores.
+template <int OFF>
+__device__ __forceinline__ float lds_at(uint32_t addr, float) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(addr), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ double lds_at(uint32_t addr, double) {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1+%2];" : "=d"(v) : "r"(addr), "n"(OFF));
+    return v;
+}
+// The same at the address in the low (HI = false) or high half of a word; one volatile statement, as
+// the unpacked addresses of all slots, hoisted out of the step loop, would not fit the registers.
+template <int OFF, bool HI>
+__device__ __forceinline__ float lds_half(unsigned w, float) {
+    float v;
+    if constexpr (HI) asm volatile("{.reg .b32 t; shr.u32 t, %1, 16; ld.shared.f32 %0, [t+%2];}" : "=f"(v) : "r"(w), "n"(OFF));
+    else asm volatile("{.reg .b32 t; and.b32 t, %1, 65535; ld.shared.f32 %0, [t+%2];}" : "=f"(v) : "r"(w), "n"(OFF));
+    return v;
+}
+template <int OFF, bool HI>
+__device__ __forceinline__ double lds_half(unsigned w, double) {
+    double v;
+    if constexpr (HI) asm volatile("{.reg .b32 t; shr.u32 t, %1, 16; ld.shared.f64 %0, [t+%2];}" : "=d"(v) : "r"(w), "n"(OFF));
+    else asm volatile("{.reg .b32 t; and.b32 t, %1, 65535; ld.shared.f64 %0, [t+%2];}" : "=d"(v) : "r"(w), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ Vec4<float> lds4_at(uint32_t addr, float) {
+    Vec4<float> v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4+%5];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ Vec4<double> lds4_at(uint32_t addr, double) {
+    Vec4<double> v;
+    asm volatile("ld.shared.v2.f64 {%0,%1}, [%2+%3];" : "=d"(v.x), "=d"(v.y) : "r"(addr), "n"(OFF));
+    asm volatile("ld.shared.v2.f64 {%0,%1}, [%2+%3];" : "=d"(v.z), "=d"(v.w) : "r"(addr), "n"(OFF + 16));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ void sts_at(uint32_t addr, float v) {
+    asm volatile("st.shared.f32 [%0+%1], %2;" ::"r"(addr), "n"(OFF), "f"(v));
+}
+template <int OFF>
+__device__ __forceinline__ void sts_at(uint32_t addr, double v) {
+    asm volatile("st.shared.f64 [%0+%1], %2;" ::"r"(addr), "n"(OFF), "d"(v));
+}
+
+// slot_put at a pointer plus a compile-time number of values, and a source entry likewise: one
+// pointer per thread serves all its slots.
+template <int N>
+__device__ __forceinline__ void slot_put_at(unsigned long long* s, unsigned tag, float v) {
+    const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.u64 [%0+%1], %2;" ::"l"(s), "n"(8 * N), "l"(w) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void slot_put_at(unsigned long long* s, unsigned tag, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0+%1], {%2, %3};" ::"l"(s), "n"(16 * N), "l"(t | (b & 0xFFFFFFFFull)),
+                 "l"(t | (b >> 32))
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ SrcEntry<float> entry_at(const SrcEntry<float>* e) {
+    SrcEntry<float> v;
+    asm volatile("ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4+%5];"
+                 : "=f"(v.c[0]), "=f"(v.c[1]), "=f"(v.c[2]), "=r"(v.g)
+                 : "l"(e), "n"((int)sizeof(v) * N));
+    return v;
+}
+template <int N>
+__device__ __forceinline__ SrcEntry<double> entry_at(const SrcEntry<double>* e) {
+    SrcEntry<double> v;
+    asm volatile("ld.global.nc.v2.f64 {%0,%1}, [%2+%3];" : "=d"(v.c[0]), "=d"(v.c[1]) : "l"(e), "n"((int)sizeof(v) * N));
+    asm volatile("ld.global.nc.f64 %0, [%1+%2];" : "=d"(v.c[2]) : "l"(e), "n"((int)sizeof(v) * N + 16));
+    asm volatile("ld.global.nc.b32 %0, [%1+%2];" : "=r"(v.g) : "l"(e), "n"((int)sizeof(v) * N + 24));
+    return v;
+}
+
+// A thread holds slots tid + i * NT, i < TS.  SOLO: one CTA holds the whole mesh, nothing is
+// published.
+template <typename T, int SH, bool PLASMA, bool FRAME, bool SOLO>
+struct Flow {
+    static constexpr int NT = kShapes[SH].nt, TS = kShapes[SH].ts, CAP = NT * TS;
+    static constexpr int STRIDE = kBuffer<T, SH> * (int)sizeof(T);   // bytes between the two buffers
+    static constexpr bool CR = kCoefRegs<T, TS>;
+    static_assert(STRIDE + 2048 < 65536, "16-bit shared addresses");
+
+    T V[TS][3], J[PLASMA ? TS : 1][3], b[TS];
+    Vec4<T> Cr[CR ? TS : 1];
+    T Pr[CR && PLASMA ? TS : 1][3];
+    unsigned n01[TS], n2f[TS];
+    // frame cell: sides X in bottom, top, left, right order, each with the cell's own
+    // counter-clockwise sign, so that every one advances by (own B - neighbour's B)
+    T X[FRAME ? 4 : 1], Bx, By;
+    int cn[FRAME ? 4 : 1];
+    unsigned ifm;           // sides that are interface edges: no decay, one fused multiply-add
+    bool has_cell, ok;
+    int nloc, npub, hn;
+    uint32_t bufs, own;     // shared addresses: the buffers, this thread's first slot
+    Vec4<T>* C;
+    T* P;
+    Vec4<T>* Fc;
+    T* gs;
+    int* hl;
+    unsigned tag0;
+    unsigned long long* put[2];   // this thread's first slot's exchange words
+    const SrcEntry<T>* sent;      // its first source entry
+
+    __device__ __forceinline__ void setup(const FlowArgs<T>& a, unsigned char* sm) {
+        const int tid = threadIdx.x;
+        bufs = smem_addr(sm);
+        own = bufs + (uint32_t)tid * (uint32_t)sizeof(T);
+        C = reinterpret_cast<Vec4<T>*>(sm + 2 * STRIDE);
+        P = reinterpret_cast<T*>(C + (CR ? 0 : CAP));
+        Fc = reinterpret_cast<Vec4<T>*>(P + (CR || !PLASMA ? 0 : 3 * CAP));
+        gs = reinterpret_cast<T*>(Fc + (FRAME ? 3 * a.fper : 0));
+        hl = reinterpret_cast<int*>(gs + kFlowSteps);
+        const int j0 = blockIdx.x * a.per;
+        nloc = max(0, min(a.per, a.n_t - j0));
+        const int2 cn2 = __ldg(a.cnt + blockIdx.x);
+        npub = SOLO ? 0 : cn2.x;
+        hn = SOLO ? 0 : cn2.y;
+        tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
+        ok = true;
+        const size_t first = (size_t)blockIdx.x * CAP + tid;
+        for (int p = 0; p < 2; ++p) put[p] = a.slots[p] + first * (sizeof(T) / 4);
+        sent = a.sent + first;
+        const int4* rec = a.rec + (size_t)blockIdx.x * CAP;
 #pragma unroll
         for (int i = 0; i < TS; ++i) {
-            const int l = tid + i * nth;
+            const int l = tid + i * NT;
             n01[i] = n2f[i] = 0;
             b[i] = T(0);
             if (l >= nloc) continue;
-            const int j = j0 + l;
-            const int4 t = __ldg(a.tri + j);
+            const int4 r = __ldg(rec + l);
+            n01[i] = (unsigned)r.y + (bufs | (bufs << 16));
+            n2f[i] = (unsigned)r.z + bufs;
+            const int4 t = __ldg(a.tri + r.x);
             const int code[3] = {t.x, t.y, t.z};
             T c[3], pb[3];
-            int src[3] = {-1, -1, -1};
-            unsigned f = 0, off[3];
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 const int k = code[q] >> 1;
                 const bool neg = code[q] & 1;
-                c[q] = pb[q] = T(0);
-                V[i][q] = T(0);
+                c[q] = pb[q] = V[i][q] = T(0);
                 if constexpr (PLASMA) J[i][q] = T(0);
-                int n = -1;
                 if (k < a.n_ei) {
-                    const int2 r = __ldg(a.rl + k);
-                    const int o = neg ? r.x : r.y;
-                    const T cu = __ldg(a.cU + k), u = a.U[k];
-                    c[q] = fabs(cu);
+                    const T u = a.U[k];
+                    c[q] = fabs(__ldg(a.cU + k));
                     V[i][q] = neg ? -u : u;
                     if constexpr (PLASMA) {
                         const T jj = a.J[k];
                         J[i][q] = neg ? -jj : jj;
                         pb[q] = __ldg(a.pb + k);
                     }
-                    if (SOLO || (o >= j0 && o < j0 + nloc)) n = o - j0;
-                    else {
-                        n = remote(o);
-                        f |= kPublish | (n < 0 ? kFar << q : 0u);
-                    }
-                    if (a.has_src && neg_bit(cu)) src[q] = src_index(a, k);
                 } else if (FRAME && k >= a.n_ei_pad) {
-                    const int e = k - a.n_ei_pad;
-                    const T u = a.Uif[e];
-                    c[q] = ((const T*)a.f.icU)[e];
+                    const T u = a.Uif[k - a.n_ei_pad];
+                    c[q] = ((const T*)a.f.icU)[k - a.n_ei_pad];
                     V[i][q] = neg ? -u : u;
-                    n = remote(a.n_t + a.f.icell[e]);
-                    f |= kPublish | (kIface << q) | (n < 0 ? kFar << q : 0u);
-                } else {
-                    f |= kWall << q;
                 }
-                off[q] = (unsigned)(n < 0 ? l : n) * (unsigned)sizeof(T);
             }
             T cb;
             if constexpr (sizeof(T) == 4) cb = __int_as_float(t.w);
-            else cb = __ldg(a.cB64 + j);
-            const Vec4<T> cv{c[0], c[1], c[2], cb}, pv{pb[0], pb[1], pb[2], T(0)};
+            else cb = __ldg(a.cB64 + r.x);
+            const Vec4<T> cv{c[0], c[1], c[2], cb};
             if constexpr (CR) Cr[i] = cv;
             else C[l] = cv;
-            if constexpr (CR && PLASMA) Pr[i] = pv;
-            else if constexpr (PLASMA) P[l] = pv;
-            if (src[0] >= 0 || src[1] >= 0 || src[2] >= 0) {
-                const int e = atomicAdd(&s_scnt, 1);
-                spos[l] = (unsigned short)(e < a.scap ? e : kNoEntry);   // the list is full: looked up at every step
-                SrcEntry<T> se{{T(0), T(0), T(0)}, 0};
+            if constexpr (PLASMA) {
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    if (src[q] < 0) continue;
-                    const T sc = __ldg(a.src_c + src[q]);
-                    se.c[q] = (code[q] & 1) ? -sc : sc;
-                    se.g = (int)__ldg(a.src_grp + src[q]) * a.gstride;
-                    f |= kSrc << q;
+                    if constexpr (CR) Pr[i][q] = pb[q];
+                    else P[q * CAP + l] = pb[q];
                 }
-                if (e < a.scap) S[e] = se;
             }
-            n01[i] = off[0] | (off[1] << 16);
-            n2f[i] = off[2] | f;
-            b[i] = a.B[j];
-            Bb[l] = b[i];
+            b[i] = a.B[r.x];
+            reinterpret_cast<T*>(sm)[l] = b[i];
         }
-        // a frame cell: sides X in bottom, top, left, right order, each with the cell's own
-        // counter-clockwise sign, so that every one advances by (own B - neighbour's B)
-        unsigned ifm = 0;   // sides that are interface edges: no decay, one fused multiply-add
-        T X[4], Bx = T(0), By = T(0);
-        int cn[4];
-        const int cell = FRAME ? (int)blockIdx.x * a.fper + tid : 0;
-        const bool has_cell = FRAME && tid < a.fper && cell < (int)a.f.n_fc;
+        has_cell = false;
         if constexpr (FRAME) {
+            const int cell = (int)blockIdx.x * a.fper + tid;
+            has_cell = tid < a.fper && cell < (int)a.f.n_fc;
+            ifm = 0;
+            Bx = By = T(0);
             if (has_cell) {
                 const FrameDev& f = a.f;
                 const Tab<T> tb = tabs<T>(f);
                 T ca[4], cd[4];
                 int I, Jc;
                 frame_ij(f, cell, I, Jc);
-                const bool in_x = I >= f.W && I < f.W + f.nx, in_y = Jc >= f.W && Jc < f.W + f.ny;
+                const int4 cr = __ldg(a.crec + cell);
+                const int off[4] = {cr.x, cr.y, cr.z, cr.w};
                 const int di[4] = {0, 0, -1, 1}, dj[4] = {-1, 1, 0, 0};
-                // interface edge on that side, or -1
-                const int kif[4] = {in_x && Jc == f.W + f.ny ? f.nx + (I - f.W) : -1, in_x && Jc == f.W - 1 ? I - f.W : -1,
-                                    in_y && I == f.W + f.nx ? 2 * f.nx + f.ny + (Jc - f.W) : -1,
-                                    in_y && I == f.W - 1 ? 2 * f.nx + (Jc - f.W) : -1};
+                const int kif[4] = {f.nx + (I - f.W), I - f.W, 2 * f.nx + f.ny + (Jc - f.W), 2 * f.nx + (Jc - f.W)};
 #pragma unroll
                 for (int d = 0; d < 4; ++d) {
                     X[d] = ca[d] = cd[d] = T(0);
-                    cn[d] = -1;
+                    cn[d] = off[d] < 0 ? -1 : (int)bufs + off[d];
+                    if (off[d] < 0) continue;
                     if (frame_is_cell(f, I + di[d], Jc + dj[d])) {
                         if (d < 2) {
                             const int at = Jc + d;
@@ -294,16 +532,11 @@ __global__ void __launch_bounds__(NT, 1) k_flow(const __grid_constant__ FlowArgs
                             ca[d] = tb.aV[at];
                             cd[d] = tb.bV[at];
                         }
-                        const int o = a.n_t + (int)frame_cell(f, I + di[d], Jc + dj[d]), n = remote(o);
-                        cn[d] = n < 0 ? o | kCellFar : n;
-                    } else if (kif[d] >= 0) {
-                        const int code = f.itri[kif[d]];
+                    } else {   // interface edge kif[d]
                         const T u = a.Uif[kif[d]];
-                        X[d] = code >= 0 ? -u : u;
+                        X[d] = f.itri[kif[d]] >= 0 ? -u : u;
                         ifm |= 1u << d;
                         cd[d] = ((const T*)f.icU)[kif[d]];
-                        const int o = code >= 0 ? code : ~code, n = remote(o);
-                        cn[d] = n < 0 ? o | kCellFar : n;
                     }
                 }
                 Bx = ((const T*)f.Bx)[cell];
@@ -314,183 +547,184 @@ __global__ void __launch_bounds__(NT, 1) k_flow(const __grid_constant__ FlowArgs
             }
         }
         if constexpr (!SOLO) {
+            for (int e = tid; e < hn; e += NT) hl[e] = __ldg(a.hlist + (size_t)blockIdx.x * kHalo<T, SH> + e);
             // published only after this thread's reads of U, J and the frame are done: their
             // owners write them back after later steps
             __threadfence();
 #pragma unroll
             for (int i = 0; i < TS; ++i)
-                if (n2f[i] & kPublish) slot_put(a.slots[0], j0 + tid + i * nth, tag0, b[i]);
-            if (has_cell) slot_put(a.slots[0], a.n_t + cell, tag0, rn_add(Bx, By));
+                if (tid + i * NT < npub) slot_put(a.slots[0], (int)blockIdx.x * CAP + tid + i * NT, tag0, b[i]);
+            if (FRAME && has_cell) slot_put(a.slots[0], ((int)gridDim.x * CAP) + (int)blockIdx.x * a.fper + tid, tag0, rn_add(Bx, By));
         }
-        const bool one_g = a.has_src && a.n_grp == 1;
-        if (one_g)
-            for (int e = tid; e < a.n_steps; e += nth) gs[e] = (T)__ldg(a.gtab + a.gbase + e);
+        if (a.one_grp)
+            for (int e = tid; e < a.n_steps; e += NT) gs[e] = (T)__ldg(a.gtab + a.gbase + e);
         __syncthreads();
-        const int hn = SOLO ? 0 : min(s_hcnt, a.hcap);
-        auto poll = [&](int p, unsigned tag, int o) -> T {
-            bool fine = true;
-            const T v = poll_one<T>(p ? a.slots[1] : a.slots[0], o, tag, &fine);
-            if (!fine) ok = false;
-            return v;
-        };
-#pragma unroll 1
-        for (int s = 1; s <= a.n_steps; ++s) {
-            const int p = (s - 1) & 1;
-            const unsigned tag = tag0 + (unsigned)(s - 1);
-            T* Bp = Bb + (p ? bcap : 0);
-            T* Bn = Bb + (p ? 0 : bcap);
-            const uint32_t ba = smem_addr(Bp);
-            if constexpr (SOLO) {
-                if (s > 1) __syncthreads();
-            } else {
-                // the remote neighbours' B of the last step, a few polls in flight per thread
-                constexpr int kPoll = 4;
-                for (int e0 = tid; e0 < hn; e0 += kPoll * nth) {
-                    Word<T> w[kPoll];
+    }
+
+    // Step s + 1 from the B of step s in buffer PB = s & 1.
+    template <int PB>
+    __device__ __forceinline__ bool step(const FlowArgs<T>& a, int s) {
+        constexpr int RD = PB * STRIDE;
+        const int tid = threadIdx.x;
+        const unsigned tag = tag0 + (unsigned)s;
+        if constexpr (SOLO) {
+            if (s > 0) __syncthreads();
+        } else {
+            // the remote neighbours' B, a few polls in flight per thread
+            constexpr int kPoll = 4;
+            const unsigned long long* sl = a.slots[PB];
+            for (int e0 = tid; e0 < hn; e0 += kPoll * NT) {
+                Word<T> w[kPoll];
 #pragma unroll
-                    for (int u = 0; u < kPoll; ++u)
-                        if (e0 + u * nth < hn) w[u].load(p ? a.slots[1] : a.slots[0], hlist[e0 + u * nth]);
+                for (int u = 0; u < kPoll; ++u)
+                    if (e0 + u * NT < hn) w[u].load(sl, hl[e0 + u * NT]);
 #pragma unroll
-                    for (int u = 0; u < kPoll; ++u) {
-                        const int e = e0 + u * nth;
-                        if (e < hn) {
-                            if (!word_wait(w[u], p ? a.slots[1] : a.slots[0], hlist[e], tag)) ok = false;
-                            Bp[cap + e] = w[u].value();
-                        }
+                for (int u = 0; u < kPoll; ++u) {
+                    const int e = e0 + u * NT;
+                    if (e < hn) {
+                        if (!word_wait(w[u], sl, hl[e], tag)) ok = false;
+                        sts_at<RD>(bufs + (uint32_t)(CAP + e) * (uint32_t)sizeof(T), w[u].value());
                     }
                 }
-                ok = __syncthreads_and(ok ? 1 : 0) != 0;
-                if (!ok) break;
             }
-            const T g1 = one_g ? gs[s - 1] : T(0);
+            ok = __syncthreads_and(ok ? 1 : 0) != 0;
+            if (!ok) return false;
+        }
+        if constexpr (FRAME) {
+            if (has_cell) {
+                const T F = rn_add(Bx, By);
+                const Vec4<T> va = Fc[3 * tid], vd = Fc[3 * tid + 1], vc = Fc[3 * tid + 2];
+                const T ca[4] = {va.x, va.y, va.z, va.w}, cd[4] = {vd.x, vd.y, vd.z, vd.w};
 #pragma unroll
-            for (int i = 0; i < TS; ++i) {
-                const int l = tid + i * nth;
-                if (l >= nloc) break;
-                Vec4<T> c, pv;
-                if constexpr (CR) c = Cr[i];
-                else c = C[l];
-                if constexpr (CR && PLASMA) pv = Pr[i];
-                else if constexpr (PLASMA) pv = P[l];
-                T nv[3] = {lds_val<T>(ba + (n01[i] & 0xFFFFu)), lds_val<T>(ba + (n01[i] >> 16)),
-                           lds_val<T>(ba + (n2f[i] & 0xFFFFu))};
-                const T cq[3] = {c.x, c.y, c.z};
-                const T pq[3] = {PLASMA ? pv.x : T(0), PLASMA ? pv.y : T(0), PLASMA ? pv.z : T(0)};
-                if (!SOLO && (n2f[i] & (7u * kFar))) {
-                    const int4 t = __ldg(a.tri + j0 + l);
-                    const int code[3] = {t.x, t.y, t.z};
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        if (!(n2f[i] & (kFar << q))) continue;
-                        const int k = code[q] >> 1;
-                        int o;
-                        if (k < a.n_ei) {
-                            const int2 r = __ldg(a.rl + k);
-                            o = (code[q] & 1) ? r.x : r.y;
-                        } else {
-                            o = a.n_t + a.f.icell[k - a.n_ei_pad];
-                        }
-                        nv[q] = poll(p, tag, o);
-                    }
+                for (int d = 0; d < 4; ++d) {
+                    if (cn[d] < 0) continue;
+                    const T df = rn_sub(F, lds_at<RD>((uint32_t)cn[d], T(0)));
+                    X[d] = (ifm >> d) & 1u ? rn_fma(cd[d], df, X[d]) : rn_fma(ca[d], X[d], rn_mul(cd[d], df));
                 }
+                Bx = rn_sub(rn_mul(vc.x, Bx), rn_mul(vc.y, rn_add(X[3], X[2])));
+                By = rn_sub(rn_mul(vc.z, By), rn_mul(vc.w, rn_add(X[0], X[1])));
+                slot_put(a.slots[PB ^ 1], (int)gridDim.x * CAP + (int)blockIdx.x * a.fper + tid, tag + 1u, rn_add(Bx, By));
+            }
+        }
+        slots_from<PB, 0>(a, s, tag);
+        return true;
+    }
+
+    template <int PB, int I>
+    __device__ __forceinline__ void slots_from(const FlowArgs<T>& a, int s, unsigned tag) {
+        if constexpr (I < TS) {
+            constexpr int RD = PB * STRIDE, WR = (PB ^ 1) * STRIDE;
+            // pb of the slot's edges, after the buffers and the coefficients
+            constexpr int PS = CAP * (int)sizeof(T), PO = 2 * STRIDE + CAP * (int)sizeof(Vec4<T>) + I * NT * (int)sizeof(T);
+            const int l = threadIdx.x + I * NT;
+            if (l < nloc) {
+                Vec4<T> c;
+                if constexpr (CR) c = Cr[I];
+                else c = lds4_at<2 * STRIDE + I * NT * (int)sizeof(Vec4<T>)>(bufs + threadIdx.x * (uint32_t)sizeof(Vec4<T>), T(0));
+                const T cq[3] = {c.x, c.y, c.z};
+                const T nv[3] = {lds_half<RD, false>(n01[I], T(0)), lds_half<RD, true>(n01[I], T(0)),
+                                 lds_half<RD, false>(n2f[I], T(0))};
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const T uo = V[i][q];
-                    T un = rn_fma(cq[q], rn_sub(b[i], nv[q]), uo);
+                    const T uo = V[I][q];
+                    T un = rn_fma(cq[q], rn_sub(b[I], nv[q]), uo);
                     if constexpr (PLASMA) {
+                        T pq;
+                        if constexpr (CR) pq = Pr[I][q];
+                        else pq = q == 0 ? lds_at<PO>(own, T(0)) : q == 1 ? lds_at<PO + PS>(own, T(0)) : lds_at<PO + 2 * PS>(own, T(0));
                         // an interface edge carries no current
-                        const T x = FRAME && (n2f[i] & (kIface << q)) ? T(0) : rn_mul(pq[q], uo);
-                        const T jn = rn_fma(a.pa, J[i][q], x);
+                        const T x = FRAME && (n2f[I] & (kIface << q)) ? T(0) : rn_mul(pq, uo);
+                        const T jn = rn_fma(a.pa, J[I][q], x);
                         un = rn_fma(a.mdt, jn, un);
-                        J[i][q] = jn;
+                        J[I][q] = jn;
                     }
-                    V[i][q] = un;
+                    V[I][q] = un;
                 }
-                if (n2f[i] & (7u * kWall)) {   // a conductor's edge stays 0, whatever the fields
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        if (!(n2f[i] & (kWall << q))) continue;
-                        V[i][q] = T(0);
-                        if constexpr (PLASMA) J[i][q] = T(0);
-                    }
-                }
-                if (n2f[i] & (7u * kSrc)) {
-                    const int e = spos[l];
-                    if (e != kNoEntry) {
-                        const SrcEntry<T> se = S[e];
-                        const T g = one_g ? g1 : (T)__ldg(a.gtab + se.g + a.gbase + s - 1);
-#pragma unroll
-                        for (int q = 0; q < 3; ++q)
-                            if (n2f[i] & (kSrc << q)) V[i][q] = rn_fma(se.c[q], g, V[i][q]);
-                    } else {
-                        const int4 t = __ldg(a.tri + j0 + l);
-                        const int code[3] = {t.x, t.y, t.z};
-#pragma unroll
-                        for (int q = 0; q < 3; ++q)
-                            if (n2f[i] & (kSrc << q)) V[i][q] = source_again<T>(&a, code[q], a.gbase + s - 1, V[i][q]);
-                    }
-                }
-                b[i] = rn_fma(-c.w, rn_add(rn_add(V[i][0], V[i][1]), V[i][2]), b[i]);
-                Bn[l] = b[i];
-                if constexpr (!SOLO) {
-                    if ((n2f[i] & kPublish) && s < a.n_steps) slot_put(p ? a.slots[0] : a.slots[1], j0 + l, tag + 1u, b[i]);
-                }
+                if (n2f[I] & (7u * (kSrc | kWall))) special<I>(a, s);
+                b[I] = rn_fma(-c.w, rn_add(rn_add(V[I][0], V[I][1]), V[I][2]), b[I]);
+                sts_at<WR + I * NT * (int)sizeof(T)>(own, b[I]);
+                if (!SOLO && l < npub) slot_put_at<I * NT>(put[PB ^ 1], tag + 1u, b[I]);
             }
-            if constexpr (FRAME) {
-                if (has_cell) {
-                    const T F = rn_add(Bx, By);
-                    const Vec4<T> va = Fc[3 * tid], vd = Fc[3 * tid + 1], vc = Fc[3 * tid + 2];
-                    const T ca[4] = {va.x, va.y, va.z, va.w}, cd[4] = {vd.x, vd.y, vd.z, vd.w};
+            slots_from<PB, I + 1>(a, s, tag);
+        }
+    }
+
+    // Source terms, and conductors' edges, which stay 0 whatever the fields.
+    template <int I>
+    __device__ __forceinline__ void special(const FlowArgs<T>& a, int s) {
+        if (n2f[I] & (7u * kSrc)) {
+            const SrcEntry<T> se = entry_at<I * NT>(sent);
+            const T g = a.one_grp ? gs[s] : (T)__ldg(a.gtab + se.g + a.gbase + s);
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) {
-                        if (cn[d] < 0) continue;
-                        const T df = rn_sub(F, cn[d] >= kCellFar ? poll(p, tag, cn[d] & ~kCellFar) : Bp[cn[d]]);
-                        X[d] = (ifm >> d) & 1u ? rn_fma(cd[d], df, X[d]) : rn_fma(ca[d], X[d], rn_mul(cd[d], df));
-                    }
-                    Bx = rn_sub(rn_mul(vc.x, Bx), rn_mul(vc.y, rn_add(X[3], X[2])));
-                    By = rn_sub(rn_mul(vc.z, By), rn_mul(vc.w, rn_add(X[0], X[1])));
-                    if (s < a.n_steps) slot_put(p ? a.slots[0] : a.slots[1], a.n_t + cell, tag + 1u, rn_add(Bx, By));
+            for (int q = 0; q < 3; ++q)
+                if (n2f[I] & (kSrc << q)) V[I][q] = rn_fma(se.c[q], g, V[I][q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            if (!(n2f[I] & (kWall << q))) continue;
+            V[I][q] = T(0);
+            if constexpr (PLASMA) J[I][q] = T(0);
+        }
+    }
+
+    // Each edge by its R triangle, each interface edge by its triangle, each frame side by the
+    // cell above or to its right.
+    __device__ __forceinline__ void write_back(const FlowArgs<T>& a) {
+        const int tid = threadIdx.x;
+        if (!SOLO) __threadfence();
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = tid + i * NT;
+            if (l >= nloc) break;
+            const int j = __ldg(&a.rec[(size_t)blockIdx.x * CAP + l].x);
+            const int4 t = __ldg(a.tri + j);
+            const int code[3] = {t.x, t.y, t.z};
+            a.B[j] = b[i];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int k = code[q] >> 1;
+                const bool neg = code[q] & 1;
+                if (k < a.n_ei) {
+                    if (neg) continue;
+                    a.U[k] = V[i][q];
+                    if constexpr (PLASMA) a.J[k] = J[i][q];
+                } else if (FRAME && k >= a.n_ei_pad) {
+                    a.Uif[k - a.n_ei_pad] = neg ? -V[i][q] : V[i][q];
                 }
             }
         }
-        if (!SOLO) ok = __syncthreads_and(ok ? 1 : 0) != 0;
-        if (ok) {
-            if (!SOLO) __threadfence();
-            // each edge by its R triangle, each interface edge by its triangle, each frame side
-            // by the cell above or to its right
-#pragma unroll
-            for (int i = 0; i < TS; ++i) {
-                const int l = tid + i * nth;
-                if (l >= nloc) break;
-                const int4 t = __ldg(a.tri + j0 + l);
-                const int code[3] = {t.x, t.y, t.z};
-                a.B[j0 + l] = b[i];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const int k = code[q] >> 1;
-                    const bool neg = code[q] & 1;
-                    if (k < a.n_ei) {
-                        if (neg) continue;
-                        a.U[k] = V[i][q];
-                        if constexpr (PLASMA) a.J[k] = J[i][q];
-                    } else if (FRAME && k >= a.n_ei_pad) {
-                        a.Uif[k - a.n_ei_pad] = neg ? -V[i][q] : V[i][q];
-                    }
-                }
-            }
-            if constexpr (FRAME) {
-                if (has_cell) {
-                    int I, Jc;
-                    frame_ij(a.f, cell, I, Jc);
-                    ((T*)a.f.Bx)[cell] = Bx;
-                    ((T*)a.f.By)[cell] = By;
-                    if (frame_is_cell(a.f, I, Jc - 1)) ((T*)a.f.H)[(int64_t)Jc * a.f.NX + I] = X[0];
-                    if (frame_is_cell(a.f, I - 1, Jc)) ((T*)a.f.V)[(int64_t)Jc * (a.f.NX + 1) + I] = -X[2];
-                }
+        if constexpr (FRAME) {
+            if (has_cell) {
+                const int cell = (int)blockIdx.x * a.fper + tid;
+                int I, Jc;
+                frame_ij(a.f, cell, I, Jc);
+                ((T*)a.f.Bx)[cell] = Bx;
+                ((T*)a.f.By)[cell] = By;
+                if (frame_is_cell(a.f, I, Jc - 1)) ((T*)a.f.H)[(int64_t)Jc * a.f.NX + I] = X[0];
+                if (frame_is_cell(a.f, I - 1, Jc)) ((T*)a.f.V)[(int64_t)Jc * (a.f.NX + 1) + I] = -X[2];
             }
         }
     }
-    if (tid == 0) {
+};
+
+template <typename T, int SH, bool PLASMA, bool FRAME, bool SOLO>
+__global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constant__ FlowArgs<T> a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const unsigned tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
+    bool ok = true;
+    if (SOLO || (int)blockIdx.x != a.skip) {
+        Flow<T, SH, PLASMA, FRAME, SOLO> f;
+        f.setup(a, smraw);
+#pragma unroll 1
+        for (int s = 0; s < a.n_steps; s += 2) {
+            if (!f.template step<0>(a, s)) break;
+            if (s + 1 == a.n_steps) break;
+            if (!f.template step<1>(a, s + 1)) break;
+        }
+        ok = SOLO || __syncthreads_and(f.ok ? 1 : 0) != 0;
+        if (ok) f.write_back(a);
+    }
+    if (threadIdx.x == 0) {
         if (!ok) atomicOr(a.ctl + 2, 1u);
         if (blockIdx.x == 0) *a.step += a.n_steps;
         if constexpr (!SOLO) {
@@ -508,28 +742,19 @@ __global__ void __launch_bounds__(NT, 1) k_flow(const __grid_constant__ FlowArgs
 __global__ void k_flow_init(unsigned* ctl) {
     if (threadIdx.x == 0) {
         ctl[0] = 1u;   // words start with tag 0
-        ctl[1] = ctl[2] = 0u;
+        ctl[1] = ctl[2] = ctl[3] = 0u;
     }
 }
 
-// Launch shapes, the first that fits.  One slot per thread keeps everything in registers (64 at
-// 1,024 threads); eight at 512 threads (128 registers) keep the state in registers and read the
-// coefficients from shared memory: 2.4 us per step on 500k triangles, the same as four slots at
-// 1,024 threads, and 2.0 against 2.4 without a source.
-struct FlowShape {
-    int nt, ts;        // most threads, slots per thread
-};
-constexpr FlowShape kShapes[3] = {{1024, 1}, {1024, 2}, {512, 8}};
-
 template <typename T, bool PLASMA, bool FRAME, bool SOLO, int SH>
-cudaError_t launch_shape(const FlowArgs<T>& a, int grid, int threads, cudaStream_t s) {
-    auto kern = k_flow<T, kShapes[SH].nt, kShapes[SH].ts, PLASMA, FRAME, SOLO>;
-    const size_t smem = flow_smem<T, PLASMA>(kCoefRegs<T, kShapes[SH].ts>, kShapes[SH].ts * threads, a.hcap, a.scap, FRAME ? a.fper : 0);
+cudaError_t launch_shape(const FlowArgs<T>& a, int grid, cudaStream_t s) {
+    auto kern = k_flow<T, SH, PLASMA, FRAME, SOLO>;
+    const size_t smem = flow_smem<T, PLASMA, SH>(FRAME ? a.fper : 0);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
+    cfg.blockDim = dim3((unsigned)kShapes[SH].nt);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -545,13 +770,16 @@ cudaError_t launch_flow_pf(const FlowArgs<T>& a, const FlowDev& fl, cudaStream_t
     if (fl.grid == 1) {
         if constexpr (FRAME) return cudaErrorInvalidValue;
         else {
-            if (fl.shape == 0) return launch_shape<T, PLASMA, false, true, 0>(a, 1, fl.threads, s);
-            return launch_shape<T, PLASMA, false, true, 1>(a, 1, fl.threads, s);
+            if (fl.shape == 0) return launch_shape<T, PLASMA, false, true, 0>(a, 1, s);
+            return launch_shape<T, PLASMA, false, true, 1>(a, 1, s);
         }
     }
-    if (fl.shape == 0) return launch_shape<T, PLASMA, FRAME, false, 0>(a, fl.grid, fl.threads, s);
-    if (fl.shape == 1) return launch_shape<T, PLASMA, FRAME, false, 1>(a, fl.grid, fl.threads, s);
-    if constexpr (sizeof(T) == 4) return launch_shape<T, PLASMA, FRAME, false, 2>(a, fl.grid, fl.threads, s);
+    if (fl.shape == 0) return launch_shape<T, PLASMA, FRAME, false, 0>(a, fl.grid, s);
+    if (fl.shape == 1) return launch_shape<T, PLASMA, FRAME, false, 1>(a, fl.grid, s);
+    if constexpr (sizeof(T) == 4) {
+        if (fl.shape == 2) return launch_shape<T, PLASMA, FRAME, false, 2>(a, fl.grid, s);
+        if constexpr (!PLASMA && !FRAME) return launch_shape<T, false, false, false, kVacuumShape>(a, fl.grid, s);
+    }
     return cudaErrorInvalidValue;
 }
 
@@ -559,7 +787,6 @@ template <typename T>
 cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
     FlowArgs<T> a;
     a.tri = m.tri;
-    a.rl = m.rl;
     a.cU = (const T*)m.cU;
     a.cB64 = (const double*)m.cB;
     a.U = (T*)m.U;
@@ -568,21 +795,18 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
     a.J = (T*)m.J;
     a.pa = (T)m.pa;
     a.mdt = (T)(-m.dt);
-    a.hash = m.src_hash;
-    a.bits = (unsigned)m.src_bits;
-    a.src_c = (const T*)m.src_c;
-    a.src_grp = m.src_grp;
+    a.rec = fl.rec;
+    a.sent = (const SrcEntry<T>*)fl.sent;
+    a.hlist = fl.hlist;
+    a.cnt = fl.cnt;
+    a.crec = fl.crec;
     a.gtab = m.gtab;
-    a.gstride = m.gtab_size;
     a.gbase = gbase;
-    a.has_src = m.n_src > 0;
-    a.n_grp = m.n_grp;
+    a.one_grp = m.n_src > 0 && m.n_grp == 1;
     a.n_t = (int)m.n_t;
     a.n_ei = (int)m.n_ei;
     a.n_ei_pad = (int)m.n_ei_pad;
     a.per = fl.per;
-    a.hcap = fl.hcap;
-    a.scap = fl.scap;
     a.slots[0] = fl.slots;
     a.slots[1] = fl.slots + fl.slot_words;
     a.ctl = fl.ctl;
@@ -596,16 +820,22 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
     return m.plasma ? launch_flow_pf<T, true, false>(a, fl, s) : launch_flow_pf<T, false, false>(a, fl, s);
 }
 
-constexpr size_t kFlowSmem = 226 * 1024;
+// Most shared memory of a CTA, a current's coefficients counted in (it may be set later).
+size_t smem_of(bool f64, int sh, int cells) {
+    if (f64) return sh == 0 ? flow_smem<double, true, 0>(cells) : flow_smem<double, true, 1>(cells);
+    return sh == 0   ? flow_smem<float, true, 0>(cells)
+           : sh == 1 ? flow_smem<float, true, 1>(cells)
+           : sh == 2 ? flow_smem<float, true, 2>(cells)
+                     : flow_smem<float, false, kVacuumShape>(cells);
+}
 
 }  // namespace
 
-bool flow_plan(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
+bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
     fl = FlowDev();
-    if (n_t < 1 || sms < 1 || n_t + n_fc >= kCellFar / 2) return false;
-    const int esz = f64 ? 8 : 4;
-    // one CTA holds up to 2,048 triangles: without an exchange its step takes 0.35-0.5 us, less
-    // than the 1.2 us of one
+    if (n_t < 1 || sms < 1 || n_t + n_fc >= INT32_MAX / 2) return false;
+    // one CTA holds up to 2,048 triangles: without an exchange its step takes 0.3 to 0.6 us, less
+    // than the 0.9 us of one
     if (n_fc == 0 && n_t <= 2048) {
         fl.grid = 1;
         fl.shape = n_t <= 1024 ? 0 : 1;
@@ -613,41 +843,68 @@ bool flow_plan(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
     } else {
         const int64_t per = (n_t + sms - 1) / sms, fper = (n_fc + sms - 1) / sms;
         fl.shape = -1;
-        for (int i = 0; i < (f64 ? 2 : 3) && fl.shape < 0; ++i)
+        for (int i = 0; i < (f64 ? 2 : n_fc > 0 ? kVacuumShape : 4) && fl.shape < 0; ++i)
             if (per <= (int64_t)kShapes[i].nt * kShapes[i].ts && fper <= kShapes[i].nt) fl.shape = i;
         if (fl.shape < 0) return false;
-        fl.per = (int)((per + 31) / 32 * 32);
-        fl.per = std::min(fl.per, kShapes[fl.shape].nt * kShapes[fl.shape].ts);
+        fl.per = std::min((int)((per + 31) / 32 * 32), kShapes[fl.shape].nt * kShapes[fl.shape].ts);
         fl.grid = std::max((int)((n_t + fl.per - 1) / fl.per), 2);
         if (n_fc > 0) fl.grid = std::max<int>(fl.grid, (int)std::min<int64_t>(sms, (n_fc + 63) / 64));
         fl.fper = (int)((n_fc + fl.grid - 1) / fl.grid);
         if (fl.fper > kShapes[fl.shape].nt) return false;
     }
-    const int ts = kShapes[fl.shape].ts;
-    fl.threads = ts > 1 ? kShapes[fl.shape].nt : std::min((std::max(fl.per, fl.fper) + 31) / 32 * 32, kShapes[fl.shape].nt);
-    const int cap = ts * fl.threads;
-    // what shared memory the coefficients (with a current's, which may come later) and the own
-    // B values leave goes to the lists: source edges, then remote neighbours
-    const bool cr = (f64 ? 8 : 4) * ts <= 8;   // kCoefRegs
-    const size_t fixed = f64 ? flow_smem<double, true>(cr, cap, 0, 0, fl.fper) : flow_smem<float, true>(cr, cap, 0, 0, fl.fper);
-    if (fixed + 8192 > kFlowSmem) return false;
-    const size_t left = kFlowSmem - fixed;
-    fl.scap = (int)std::min<size_t>(std::min(cap, 0x8000), left / 3 / (f64 ? 32 : 16)) & ~1;
-    if (fl.grid > 1)
-        fl.hcap = (int)std::min(std::min<size_t>((size_t)3 * cap + 4 * (size_t)fl.fper,
-                                                 (left - (size_t)fl.scap * (f64 ? 32 : 16)) / (2 * esz + 4)),
-                                (size_t)(65536 / esz - cap)) & ~3;   // 16-bit byte offsets
-    fl.slot_words = fl.grid > 1 ? (n_t + n_fc) * (f64 ? 2 : 1) : 0;
+    if (smem_of(f64, fl.shape, fl.fper) > (size_t)226 * 1024) return false;
+    fl.cap = kShapes[fl.shape].nt * kShapes[fl.shape].ts;
+    fl.halo = f64 ? kShapes[fl.shape].halo64 : kShapes[fl.shape].halo32;
+    fl.slot_words = fl.grid > 1 ? ((int64_t)fl.grid * fl.cap + n_fc) * (f64 ? 2 : 1) : 0;
+    fl.sent_bytes = (size_t)fl.grid * fl.cap * (f64 ? sizeof(SrcEntry<double>) : sizeof(SrcEntry<float>));
     return true;
 }
+
+bool flow_takes(const FlowDev& fl, const DevMesh& m) { return fl.grid > 0 && (fl.shape != kVacuumShape || !m.plasma); }
 
 cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s) {
     k_flow_init<<<1, 32, 0, s>>>(fl.ctl);
     return cudaGetLastError();
 }
 
+cudaError_t launch_flow_plan(const FlowDev& fl, const DevMesh& m, cudaStream_t s) {
+    PlanArgs a;
+    a.tri = m.tri;
+    a.rl = m.rl;
+    a.cU = m.cU;
+    a.hash = m.src_hash;
+    a.bits = (unsigned)m.src_bits;
+    a.src_c = m.src_c;
+    a.src_grp = m.src_grp;
+    a.gstride = m.gtab_size;
+    a.has_src = m.n_src > 0;
+    a.n_t = (int)m.n_t;
+    a.n_ei = (int)m.n_ei;
+    a.n_ei_pad = (int)m.n_ei_pad;
+    a.per = fl.per;
+    a.cap = fl.cap;
+    a.halo = fl.halo;
+    a.rec = fl.rec;
+    a.sent = fl.sent;
+    a.hlist = fl.hlist;
+    a.cnt = fl.cnt;
+    a.crec = fl.crec;
+    a.ctl = fl.ctl;
+    if (m.frame) a.f = *m.frame;
+    a.fper = fl.fper;
+    a.place = fl.place;
+    if (m.precision == UE_PREC_FP64) {
+        k_flow_order<double><<<fl.grid, 1024, 0, s>>>(a);
+        k_flow_plan<double><<<fl.grid, 1024, 0, s>>>(a);
+    } else {
+        k_flow_order<float><<<fl.grid, 1024, 0, s>>>(a);
+        k_flow_plan<float><<<fl.grid, 1024, 0, s>>>(a);
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
-    if (n_steps < 1) return cudaErrorInvalidValue;
+    if (n_steps < 1 || n_steps > kFlowSteps) return cudaErrorInvalidValue;
     return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, Uif, n_steps, gbase, s)
                                        : launch_flow_t<float>(fl, m, Uif, n_steps, gbase, s);
 }

@@ -613,6 +613,15 @@ int region_sources(ue_mesh* m, cudaStream_t s) {
 int bake_source(ue_mesh* m, cudaStream_t s) {
     int rc = bake_source_mesh(m, s);
     if (rc != UE_OK) return rc;
+    if (m->flow.grid > 0) {
+        DevMesh v = m->dm;
+        v.frame = m->fr.W > 0 ? &m->fd : nullptr;
+        unsigned over = 0;
+        UE_CUDA(ue::launch_flow_plan(m->flow, v, s));
+        UE_CUDA(cudaMemcpyAsync(&over, m->flow.ctl + 3, 4, cudaMemcpyDeviceToHost, s));
+        UE_CUDA(cudaStreamSynchronize(s));
+        if (over) m->flow.grid = 0;   // neighbours too scattered: this mesh keeps its launches
+    }
     if (m->variant == UE_VARIANT_BLOCKED && m->tb.erec) {
         // the tile records carry the source flags of the coefficients (the pipelined kernel
         // takes a source edge's value back after the source is added)
@@ -1037,10 +1046,16 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         const int64_t W = m->fr.W, NX = m->fr.nx + 2 * W;
         const int64_t n_fc = 2 * W * NX + 2 * W * m->fr.ny;
-        if (coop && ue::flow_plan(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) {
-            m->flow.skip = m->flow_skip;
-            ok = ok && alloc_into(m, m->flow.ctl, 4, 4, s) &&
-                 (m->flow.slot_words == 0 || alloc_into(m, m->flow.slots, 2 * m->flow.slot_words, 8, s));
+        if (coop && ue::flow_shape(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) {
+            ue::FlowDev& fl = m->flow;
+            fl.skip = m->flow_skip;
+            const size_t slots = (size_t)fl.grid * fl.cap;
+            ok = ok && alloc_into(m, fl.ctl, 4, 4, s) && alloc_into(m, fl.place, nt, 4, s) &&
+                 alloc_into(m, fl.rec, slots, 16, s) &&
+                 alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
+                 (fl.grid == 1 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
+                 (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
+                 (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));
         }
     }
     {
@@ -1964,7 +1979,7 @@ int ue_step_n(ue_mesh* m, int64_t n, void* stream) {
         m->launches += launched;
         return UE_OK;
     }
-    if (m->flow.grid > 0) {
+    if (ue::flow_takes(m->flow, m->dm)) {
         const int64_t unit = m->variant == UE_VARIANT_BLOCKED ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
         // calls of a graph chunk or more, which would replay graphs; shorter ones launch step by step
         if (n >= unit) {
@@ -2050,7 +2065,7 @@ int ue_step_prepare(ue_mesh* m, void* stream) {
         }
         return UE_OK;
     }
-    if (m->flow.grid > 0) return UE_OK;   // the calls long enough for a graph run resident
+    if (ue::flow_takes(m->flow, m->dm)) return UE_OK;   // the calls long enough for a graph run resident
     const int rc = ensure_graph(m);
     if (rc != UE_OK) return rc;
     UE_CUDA(cudaGraphUpload(m->gexec, s));

@@ -82,13 +82,18 @@ def test_resident_is_bit_identical_to_plain(ue, n_t, fp64, plasma):
     _same(_run(ue, xy, tris, h, 45, 32, **kw), _run(ue, xy, tris, h, 45, -1, **kw))
 
 
-@pytest.mark.parametrize("n_t", [155_648, 155_649, 311_297, 622_592])
+@pytest.mark.parametrize("n_t", [155_648, 155_649, 311_297, 622_592, 622_593, 1_245_184, 1_245_185])
 @pytest.mark.parametrize("plasma", [False, True])
 def test_resident_at_the_edges_of_its_shapes(ue, n_t, plasma):
-    """152 CTAs of 1,024, 2,048 and 4,096 triangles."""
+    """152 CTAs of 1,024, 2,048, 4,096 and, without a current, 8,192 triangles (which of the
+    largest run resident depends on how many neighbours of a CTA lie in others)."""
     xy, tris, h = _lattice(n_t, 5)
     kw = dict(plasma=plasma)
-    _same(_run(ue, xy, tris, h, 33, 32, **kw), _run(ue, xy, tris, h, 33, -1, **kw))
+    a, b = _run(ue, xy, tris, h, 33, 32, **kw), _run(ue, xy, tris, h, 33, -1, **kw)
+    for x, y in zip(a[:-1], b[:-1]):
+        assert np.array_equal(x, y)
+    assert a[-1] < b[-1] if n_t <= (622_592 if plasma else 622_593) else True
+    assert a[-1] >= b[-1] if n_t > (622_592 if plasma else 1_245_184) else True
 
 
 def test_resident_fp64_with_two_slots(ue):
@@ -99,11 +104,14 @@ def test_resident_fp64_with_two_slots(ue):
 
 @pytest.mark.parametrize("n_t", [7_000, 400_000])
 def test_resident_with_scattered_neighbours(ue, n_t):
-    """The caller's order kept and random: nearly every neighbour is in another CTA, more than a
-    CTA lists, so threads poll their own."""
+    """The caller's order kept and random: nearly every neighbour is in another CTA; the larger
+    mesh has more than a CTA lists and keeps its launches."""
     xy, tris, h = _lattice(n_t, 5, shuffle=True)
     kw = dict(plasma=True, load=dict(reorder=ue.UE_REORDER_NONE))
-    _same(_run(ue, xy, tris, h, 40, 32, **kw), _run(ue, xy, tris, h, 40, -1, **kw))
+    a, b = _run(ue, xy, tris, h, 40, 32, **kw), _run(ue, xy, tris, h, 40, -1, **kw)
+    for x, y in zip(a[:-1], b[:-1]):
+        assert np.array_equal(x, y)
+    assert (a[-1] < b[-1]) == (n_t < 10_000)
 
 
 @pytest.mark.parametrize("tiled", [False, True])

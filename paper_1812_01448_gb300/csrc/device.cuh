@@ -85,6 +85,17 @@ __device__ __forceinline__ double rn_sub(double a, double b) { return __dsub_rn(
 __device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
 
+// wd = {W at the previous check, W now, growth factor, flag}: flag 1 = non-finite energy,
+// 2 = energy grew by more than the factor since the previous check.  A set flag stays set.
+__device__ __forceinline__ void watchdog_update(double* wd, double W) {
+    wd[1] = W;
+    if (wd[3] == 0.0) {
+        if (!isfinite(W)) wd[3] = 1.0;
+        else if (wd[2] > 0.0 && wd[0] > 0.0 && W > wd[2] * wd[0]) wd[3] = 2.0;
+    }
+    wd[0] = W;
+}
+
 // g(t) of the soft source at t = (n + 1/2) dt, in FP64: sin(w0 t) exp(-((t - t0)/tau)^2).
 // One out-of-line definition with explicit rounding, shared by every variant of the step.
 static __device__ __noinline__ double source_g(long long n, double dt, double w0, double t0,
@@ -248,6 +259,8 @@ struct FlowDev {
     int* hlist = nullptr;         // [grid * halo] remote neighbours
     int2* cnt = nullptr;          // [grid]
     int4* crec = nullptr;         // [frame cells]
+    double* epart = nullptr;      // [kFlowChecks * grid] energy sums of a launch's checks, then
+                                  // kFlowChecks counters (zero between launches)
     int skip = -1;                // tests only: this CTA returns at once
 };
 // n_fc: cells of a PML frame stepped with the mesh.  False when the mesh does not fit.
@@ -258,9 +271,17 @@ cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s);
 // The plan from the mesh's tables and source (again when the source changes); sets ctl[3] when a
 // CTA has more remote neighbours than it can list.
 cudaError_t launch_flow_plan(const FlowDev& fl, const DevMesh& m, cudaStream_t s);
-// n_steps steps of m in place in one launch; the source uses g-table entries gbase ..
-// gbase + n_steps - 1.  Uif: the circulations of a frame's interface edges.
-cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s);
+// n_steps steps of m in place in one launch; the source uses g-table entries 0 .. n_steps - 1.  Uif:
+// the circulations of a frame's interface edges.  The energy watchdog's checks inside the launch:
+// after `first` steps (0: none) and every `period` more, and after the last step when `end` is
+// set; at most kFlowChecks.
+constexpr int kFlowChecks = 64;
+struct FlowChecks {
+    int first = 0, period = 0, end = 0;
+    const double *we = nullptr, *S = nullptr;
+    double* wd = nullptr;
+};
+cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, const FlowChecks& chk, cudaStream_t s);
 
 // Launchers (kernels_step.cu).
 // g(t) table for the next `count` steps (no-op without a source).
@@ -319,7 +340,7 @@ cudaError_t launch_fields_in_caller(const DevMesh& m, const void* E_caller, cons
 cudaError_t launch_fields_out_caller(const DevMesh& m, void* E_caller, void* B_caller, void* J_caller, bool f32,
                                      const int32_t* k_of, const int32_t* inv, const double* relen, int64_t n_e,
                                      cudaStream_t s);
-cudaError_t launch_recip(const double* elen, double* relen, int64_t n_ei, cudaStream_t s);
+cudaError_t launch_recip(const double* elen, const double* d, double* relen, double* we, int64_t n_ei, cudaStream_t s);
 // Halo exchange of a partitioned mesh: B at caller triangle ids[0..n) to buf (scatter = 0) or
 // from buf (scatter = 1), in the field type; inv[n_t] = stored triangle of each caller one.
 // Ids outside [0, n_t) are skipped and counted in *bad (device).
@@ -387,8 +408,8 @@ int mesh_flip(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, con
 
 // Energy watchdog: W of eq. 8 into wd[1], compared with the previous check (see kernels_geom.cu).
 size_t energy_parts(int64_t n_ei, int64_t n_t);
-cudaError_t launch_energy(const DevMesh& m, const double* elen, const double* d, const double* S,
-                          double* part, double* wd, cudaStream_t s);
+// we: d/|e| per interior edge (launch_recip).
+cudaError_t launch_energy(const DevMesh& m, const double* we, const double* S, double* part, double* wd, cudaStream_t s);
 // Batch assembly: dst[i] = |src[i]| (coefficients without source flags), and triangle
 // records re-pointed at the batch's edge numbering.
 cudaError_t launch_copy_abs(void* dst, const void* src, int64_t n, bool f64, cudaStream_t s);

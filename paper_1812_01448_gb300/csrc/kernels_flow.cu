@@ -111,7 +111,6 @@ struct FlowArgs {
     const int2* cnt;        // per CTA: publishing triangles, remote neighbours
     const int4* crec;       // fper per CTA: offsets of a frame cell's neighbours, -1 none
     const double* gtab;
-    int gbase;              // this launch's first entry in the g table
     int one_grp;            // one source group: its g is staged in shared memory
     int n_t, n_ei, n_ei_pad;
     int per;                // triangles per CTA
@@ -123,6 +122,9 @@ struct FlowArgs {
     FrameDev f;
     T* Uif;                 // circulations of the frame's interface edges
     int fper;               // frame cells per CTA
+    FlowChecks chk;
+    double* epart;
+    unsigned* ecount;       // kFlowChecks counters
 };
 
 __device__ __forceinline__ bool neg_bit(float c) { return __float_as_uint(c) >> 31; }
@@ -557,7 +559,7 @@ struct Flow {
             if (FRAME && has_cell) slot_put(a.slots[0], ((int)gridDim.x * CAP) + (int)blockIdx.x * a.fper + tid, tag0, rn_add(Bx, By));
         }
         if (a.one_grp)
-            for (int e = tid; e < a.n_steps; e += NT) gs[e] = (T)__ldg(a.gtab + a.gbase + e);
+            for (int e = tid; e < a.n_steps; e += NT) gs[e] = (T)__ldg(a.gtab + e);
         __syncthreads();
     }
 
@@ -654,7 +656,7 @@ struct Flow {
     __device__ __forceinline__ void special(const FlowArgs<T>& a, int s) {
         if (n2f[I] & (7u * kSrc)) {
             const SrcEntry<T> se = entry_at<I * NT>(sent);
-            const T g = a.one_grp ? gs[s] : (T)__ldg(a.gtab + se.g + a.gbase + s);
+            const T g = a.one_grp ? gs[s] : (T)__ldg(a.gtab + se.g + s);
 #pragma unroll
             for (int q = 0; q < 3; ++q)
                 if (n2f[I] & (kSrc << q)) V[I][q] = rn_fma(se.c[q], g, V[I][q]);
@@ -665,6 +667,54 @@ struct Flow {
             V[I][q] = T(0);
             if constexpr (PLASMA) J[I][q] = T(0);
         }
+    }
+
+    // The energy of eq. 8 after a step (check c of the launch), without leaving the launch: each
+    // triangle adds its own term and those of the edges it is R of, and the last CTA to arrive sums
+    // the CTAs' shares in order and updates the watchdog.  Checks are handled in turn: the last
+    // arrival at one has arrived, and finished, at those before.  It is bound by the latency of its
+    // loads (three deep); ending the launch at every check instead and summing in two kernels cost
+    // 19 us more per check at 92k triangles (256 steps, a check every 32: 606 us, now 454 us).
+    __device__ __forceinline__ void energy(const FlowArgs<T>& a, int c) {
+        __shared__ double red[NT / 32];
+        __shared__ bool last;
+        const int tid = threadIdx.x;
+        double x = 0.0;
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = tid + i * NT;
+            if (l >= nloc) break;
+            const int j = __ldg(&a.rec[(size_t)blockIdx.x * CAP + l].x);
+            const int4 t = __ldg(a.tri + j);
+            const int code[3] = {t.x, t.y, t.z};
+            x += __ldg(a.chk.S + j) * (double)b[i] * (double)b[i];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int k = code[q] >> 1;
+                if (k < a.n_ei && !(code[q] & 1)) x += __ldg(a.chk.we + k) * (double)V[i][q] * (double)V[i][q];
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((tid & 31) == 0) red[tid >> 5] = x;
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < NT / 32; ++w) x += red[w];
+            a.epart[(size_t)c * gridDim.x + blockIdx.x] = x;
+            __threadfence();
+            last = SOLO || atomicAdd(a.ecount + c, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (last && tid < 32) {
+            __threadfence();
+            double w = 0.0;
+            for (int i = tid; i < (int)gridDim.x; i += 32) w += __ldcg(a.epart + (size_t)c * gridDim.x + i);
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (tid == 0) {
+                watchdog_update(a.chk.wd, w);
+                __threadfence();
+            }
+        }
+        __syncthreads();
     }
 
     // Each edge by its R triangle, each interface edge by its triangle, each frame side by the
@@ -715,11 +765,22 @@ __global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constan
     if (SOLO || (int)blockIdx.x != a.skip) {
         Flow<T, SH, PLASMA, FRAME, SOLO> f;
         f.setup(a, smraw);
+        int c = 0, next = a.chk.first > 0 ? a.chk.first : a.n_steps + 1;
+        bool go = true;
 #pragma unroll 1
-        for (int s = 0; s < a.n_steps; s += 2) {
-            if (!f.template step<0>(a, s)) break;
-            if (s + 1 == a.n_steps) break;
-            if (!f.template step<1>(a, s + 1)) break;
+        for (int s = 0; s < a.n_steps && go;) {
+            const int end = min(next, a.n_steps);
+#pragma unroll 1
+            for (;;) {
+                if (!(s & 1)) {
+                    if (!(go = f.template step<0>(a, s)) || ++s == end) break;
+                }
+                if (!(go = f.template step<1>(a, s)) || ++s == end) break;
+            }
+            if (go && (s == next || (s == a.n_steps && a.chk.end))) {
+                f.energy(a, c++);
+                next += a.chk.period;
+            }
         }
         ok = SOLO || __syncthreads_and(f.ok ? 1 : 0) != 0;
         if (ok) f.write_back(a);
@@ -731,6 +792,8 @@ __global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constan
             // the last CTA moves the tags on: every CTA has read this launch's by then
             __threadfence();
             if (atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
+                if (a.chk.first > 0 || a.chk.end)
+                    for (int i = 0; i < kFlowChecks; ++i) a.ecount[i] = 0u;
                 a.ctl[1] = 0u;
                 a.ctl[0] = tag0 + (unsigned)a.n_steps + 1u;
                 __threadfence();
@@ -784,7 +847,7 @@ cudaError_t launch_flow_pf(const FlowArgs<T>& a, const FlowDev& fl, cudaStream_t
 }
 
 template <typename T>
-cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
+cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, const FlowChecks& chk, cudaStream_t s) {
     FlowArgs<T> a;
     a.tri = m.tri;
     a.cU = (const T*)m.cU;
@@ -801,7 +864,6 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
     a.cnt = fl.cnt;
     a.crec = fl.crec;
     a.gtab = m.gtab;
-    a.gbase = gbase;
     a.one_grp = m.n_src > 0 && m.n_grp == 1;
     a.n_t = (int)m.n_t;
     a.n_ei = (int)m.n_ei;
@@ -816,6 +878,9 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
     if (m.frame) a.f = *m.frame;
     a.Uif = (T*)Uif;
     a.fper = fl.fper;
+    a.chk = chk;
+    a.epart = fl.epart;
+    a.ecount = fl.epart ? reinterpret_cast<unsigned*>(fl.epart + (size_t)kFlowChecks * fl.grid) : nullptr;
     if (m.frame) return m.plasma ? launch_flow_pf<T, true, true>(a, fl, s) : launch_flow_pf<T, false, true>(a, fl, s);
     return m.plasma ? launch_flow_pf<T, true, false>(a, fl, s) : launch_flow_pf<T, false, false>(a, fl, s);
 }
@@ -903,10 +968,11 @@ cudaError_t launch_flow_plan(const FlowDev& fl, const DevMesh& m, cudaStream_t s
     return cudaGetLastError();
 }
 
-cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, int gbase, cudaStream_t s) {
+cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, const FlowChecks& chk, cudaStream_t s) {
     if (n_steps < 1 || n_steps > kFlowSteps) return cudaErrorInvalidValue;
-    return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, Uif, n_steps, gbase, s)
-                                       : launch_flow_t<float>(fl, m, Uif, n_steps, gbase, s);
+    if ((chk.first > 0 || chk.end) && (!fl.epart || !chk.we || !chk.S || !chk.wd)) return cudaErrorInvalidValue;
+    return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, Uif, n_steps, chk, s)
+                                       : launch_flow_t<float>(fl, m, Uif, n_steps, chk, s);
 }
 
 }  // namespace ue

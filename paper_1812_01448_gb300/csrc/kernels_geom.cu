@@ -572,16 +572,22 @@ cudaError_t launch_geom_tri(const double* xy, const int32_t* tri_nodes, double* 
     return cudaGetLastError();
 }
 
-// 1/|e| of every interior edge (the zero slot n_ei gets 0): the readout multiplies by it, since
-// an FP64 division per element costs more than the transfer on GB300's FP64 pipes.
-__global__ void k_recip(const double* __restrict__ elen, double* __restrict__ relen, int64_t n_ei) {
+// 1/|e| of every interior edge (the zero slot n_ei gets 0) and the energy's weight d/|e|: the readout
+// and the energy multiply by them, since an FP64 division per element costs more than the transfer
+// or the sum on GB300's FP64 pipes.
+__global__ void k_recip(const double* __restrict__ elen, const double* __restrict__ d, double* __restrict__ relen,
+                        double* __restrict__ we, int64_t n_ei) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n_ei) relen[k] = 1.0 / elen[k];
-    else if (k == n_ei) relen[k] = 0.0;
+    if (k < n_ei) {
+        relen[k] = 1.0 / elen[k];
+        we[k] = d[k] / elen[k];
+    } else if (k == n_ei) {
+        relen[k] = 0.0;
+    }
 }
 
-cudaError_t launch_recip(const double* elen, double* relen, int64_t n_ei, cudaStream_t s) {
-    k_recip<<<blocks_for(n_ei + 1), kThreads, 0, s>>>(elen, relen, n_ei);
+cudaError_t launch_recip(const double* elen, const double* d, double* relen, double* we, int64_t n_ei, cudaStream_t s) {
+    k_recip<<<blocks_for(n_ei + 1), kThreads, 0, s>>>(elen, d, relen, we, n_ei);
     return cudaGetLastError();
 }
 
@@ -654,38 +660,40 @@ namespace {
 
 // Energy of eq. 8 with the eq. 7 weights, in circulation variables:
 //   W = sum_i (d_i / |e_i|) U_i^2 + sum_j S_j B_j^2   (U = |e| E).
-// Blocks [0, nbe) cover edges, [nbe, nbe + nbt) triangles; fixed-order partial sums.
+// Blocks [0, nbe) cover edges, [nbe, nbe + nbt) triangles, kEnergyPer consecutive runs of elements
+// per thread; fixed-order partial sums.
+constexpr int kEnergyPer = 4;
 template <typename T>
 __global__ void k_energy_parts(const T* __restrict__ U, const T* __restrict__ B,
-                               const double* __restrict__ elen, const double* __restrict__ d,
-                               const double* __restrict__ S, int64_t n_ei, int64_t n_t, int nbe,
-                               double* __restrict__ part) {
-    __shared__ double a[kThreads];
+                               const double* __restrict__ we, const double* __restrict__ S, int64_t n_ei,
+                               int64_t n_t, int nbe, double* __restrict__ part) {
+    __shared__ double a[kThreads / 32];
+    const bool edges = (int)blockIdx.x < nbe;
+    const T* F = edges ? U : B;
+    const double* w = edges ? we : S;
+    const int64_t n = edges ? n_ei : n_t;
+    const int64_t i0 = (int64_t)(edges ? blockIdx.x : blockIdx.x - nbe) * kThreads * kEnergyPer + threadIdx.x;
+    double f[kEnergyPer], c[kEnergyPer];
+#pragma unroll
+    for (int u = 0; u < kEnergyPer; ++u) {
+        const int64_t i = i0 + u * kThreads;
+        f[u] = i < n ? (double)F[i] : 0.0;
+        c[u] = i < n ? w[i] : 0.0;
+    }
     double x = 0.0;
-    if ((int)blockIdx.x < nbe) {
-        const int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-        if (k < n_ei) {
-            const double u = (double)U[k];
-            x = d[k] / elen[k] * u * u;
-        }
-    } else {
-        const int64_t j = (int64_t)(blockIdx.x - nbe) * kThreads + threadIdx.x;
-        if (j < n_t) {
-            const double b = (double)B[j];
-            x = S[j] * b * b;
-        }
-    }
-    a[threadIdx.x] = x;
+#pragma unroll
+    for (int u = 0; u < kEnergyPer; ++u)
+        if (i0 + u * kThreads < n) x += c[u] * f[u] * f[u];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) a[threadIdx.x >> 5] = x;
     __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) a[threadIdx.x] += a[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kThreads / 32; ++i) x += a[i];
+        part[blockIdx.x] = x;
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = a[0];
 }
 
-// wd = {W at the previous check, W now, growth factor, flag}: flag 1 = non-finite energy,
-// 2 = energy grew by more than the factor since the previous check.  A set flag stays set.
+// The watchdog words (watchdog_update) from the partials.
 __global__ void k_energy_check(const double* __restrict__ part, int nb, double* __restrict__ wd) {
     __shared__ double a[kThreads];
     double x = 0.0;
@@ -696,33 +704,27 @@ __global__ void k_energy_check(const double* __restrict__ part, int nb, double* 
         if (threadIdx.x < o) a[threadIdx.x] += a[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        const double W = a[0];
-        wd[1] = W;
-        if (wd[3] == 0.0) {
-            if (!isfinite(W)) wd[3] = 1.0;
-            else if (wd[2] > 0.0 && wd[0] > 0.0 && W > wd[2] * wd[0]) wd[3] = 2.0;
-        }
-        wd[0] = W;
-    }
+    if (threadIdx.x == 0) watchdog_update(wd, a[0]);
 }
 
 }  // namespace
 
 size_t energy_parts(int64_t n_ei, int64_t n_t) {
-    return (size_t)((n_ei + kThreads - 1) / kThreads + (n_t + kThreads - 1) / kThreads);
+    const int64_t per = kThreads * kEnergyPer;
+    return (size_t)((n_ei + per - 1) / per + (n_t + per - 1) / per);
 }
 
-cudaError_t launch_energy(const DevMesh& m, const double* elen, const double* d, const double* S,
-                          double* part, double* wd, cudaStream_t s) {
-    const int nbe = (int)((m.n_ei + kThreads - 1) / kThreads);
-    const int nbt = (int)((m.n_t + kThreads - 1) / kThreads);
+cudaError_t launch_energy(const DevMesh& m, const double* we, const double* S, double* part, double* wd,
+                          cudaStream_t s) {
+    const int64_t per = kThreads * kEnergyPer;
+    const int nbe = (int)((m.n_ei + per - 1) / per);
+    const int nbt = (int)((m.n_t + per - 1) / per);
     if (m.precision == UE_PREC_FP64)
-        k_energy_parts<double><<<nbe + nbt, kThreads, 0, s>>>((const double*)m.U, (const double*)m.B,
-                                                              elen, d, S, m.n_ei, m.n_t, nbe, part);
+        k_energy_parts<double><<<nbe + nbt, kThreads, 0, s>>>((const double*)m.U, (const double*)m.B, we, S, m.n_ei,
+                                                              m.n_t, nbe, part);
     else
-        k_energy_parts<float><<<nbe + nbt, kThreads, 0, s>>>((const float*)m.U, (const float*)m.B,
-                                                             elen, d, S, m.n_ei, m.n_t, nbe, part);
+        k_energy_parts<float><<<nbe + nbt, kThreads, 0, s>>>((const float*)m.U, (const float*)m.B, we, S, m.n_ei,
+                                                             m.n_t, nbe, part);
     k_energy_check<<<1, kThreads, 0, s>>>(part, nbe + nbt, wd);
     return cudaGetLastError();
 }

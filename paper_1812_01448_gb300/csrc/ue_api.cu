@@ -92,6 +92,7 @@ struct ue_mesh {
     int64_t* d_ecaller = nullptr;
     double *d_O = nullptr, *d_S = nullptr, *d_elen = nullptr, *d_d = nullptr;
     double* d_relen = nullptr;   // 1/|e| (the readout of E)
+    double* d_we = nullptr;      // d/|e| (the energy)
     // transfer buffers in caller numbering
     double *d_Ec = nullptr, *d_Bc = nullptr, *d_Jc = nullptr;
     // caller -> stored maps of the direct transfers (made on first use)
@@ -503,7 +504,7 @@ cudaError_t watchdog_tick(ue_mesh* m, int64_t steps, cudaStream_t s, int64_t* la
     if (m->since_check < m->watchdog_every) return cudaSuccess;
     m->since_check = 0;
     *launched += 2;
-    return ue::launch_energy(m->dm, m->d_elen, m->d_d, m->d_S, m->wd_part, m->wd, s);
+    return ue::launch_energy(m->dm, m->d_we, m->d_S, m->wd_part, m->wd, s);
 }
 
 // kernels launched for `steps` plain steps issued in batches of `batch` (one g-table kernel
@@ -1013,7 +1014,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
     const HostMesh& h = m->hm;
     const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;
     const int64_t nt = h.n_tris, nei = h.n_ei, nn = h.n_nodes, ne = h.n_edges;
-    m->reserve = (size_t)(16 * nn + nt * (104 + 3 * (int64_t)esz) + nei * (56 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
+    m->reserve = (size_t)(16 * nn + nt * (150 + 3 * (int64_t)esz) + nei * (64 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
     bool ok = alloc_into(m, m->d_xy, 2 * nn, 8, s) && alloc_into(m, m->d_tri_nodes, 3 * nt, 4, s) &&
               alloc_into(m, m->d_edge_nodes, 2 * nei + 2, 4, s) &&
               alloc_into(m, m->d_edge_opp, 2 * nei + 2, 4, s) &&
@@ -1022,7 +1023,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
               alloc_into(m, m->d_perm, nt, 8, s) && alloc_into(m, m->d_ecaller, nei + 1, 8, s) &&
               alloc_into(m, m->d_O, 2 * nt, 8, s) && alloc_into(m, m->d_S, nt, 8, s) &&
               alloc_into(m, m->d_elen, nei + 1, 8, s) && alloc_into(m, m->d_d, nei + 1, 8, s) &&
-              alloc_into(m, m->d_relen, nei + 1, 8, s) &&
+              alloc_into(m, m->d_relen, nei + 1, 8, s) && alloc_into(m, m->d_we, nei + 1, 8, s) &&
               alloc_into(m, m->d_Ec, ne, 8, s) && alloc_into(m, m->d_Bc, nt, 8, s) &&
               alloc_into(m, m->d_Jc, ne, 8, s);
     DevMesh& dm = m->dm;
@@ -1055,6 +1056,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
                  alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
                  (fl.grid == 1 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
                  (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
+                 (m->watchdog_every <= 0 || alloc_into(m, fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8, s)) &&
                  (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));
         }
     }
@@ -1078,6 +1080,8 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         if (m->flow.grid > 0) {
             UE_CUDA(ue::launch_flow_init(m->flow, s));
             if (m->flow.slot_words > 0) UE_CUDA(cudaMemsetAsync(m->flow.slots, 0, 16 * m->flow.slot_words, s));
+            if (m->flow.epart)   // its counters
+                UE_CUDA(cudaMemsetAsync(m->flow.epart + (size_t)ue::kFlowChecks * m->flow.grid, 0, 8 * ue::kFlowChecks, s));
         }
         const double w0[4] = {0.0, 0.0, m->watchdog_growth, 0.0};
         UE_CUDA(cudaMemcpyAsync(m->wd, w0, sizeof(w0), cudaMemcpyHostToDevice, s));
@@ -1189,7 +1193,16 @@ int flush_step(ue_mesh* m, cudaStream_t s) {
 // device cannot hold the launch's CTAs at once (the caller then makes its launches).
 int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) {
     DevMesh& dm = m->dm;
-    const int64_t most = m->watchdog_every > 0 ? unit : dm.n_src > 0 ? (int64_t)dm.gtab_size : ue::kFlowSteps;
+    const int64_t every = m->watchdog_every;
+    // whole units per launch when the watchdog is on: its checks fall on their ends, the first where
+    // the steps since the last check reach `every`, then every `period`
+    const int64_t period = every > 0 ? (every + unit - 1) / unit * unit : 0;
+    int64_t most = ue::kFlowSteps;
+    if (every > 0) most = unit > most ? unit : std::max(unit, std::min(most / unit * unit, ue::kFlowChecks / 2 * period));
+    if (most > ue::kFlowSteps) {   // a unit beyond one launch (a very long graph chunk)
+        *used = false;
+        return UE_OK;
+    }
     void* Uif = nullptr;
     if (m->has_reg) Uif = (float*)m->reg.dm.U + m->reg.f.u_off;
     else if (m->fr.W > 0) Uif = (char*)dm.U + (m->precision == UE_PREC_FP64 ? 8 : 4) * dm.n_ei_pad;
@@ -1199,8 +1212,28 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
     *used = true;
     for (int64_t left = n; left > 0;) {
         const int batch = (int)std::min(left, most);
+        ue::FlowChecks chk;
+        int64_t since = m->since_check;
+        if (every > 0) {
+            chk.we = m->d_we;
+            chk.S = m->d_S;
+            chk.wd = m->wd;
+            chk.period = (int)period;
+            for (int64_t t = unit; t <= batch; t += unit)
+                if (since + unit >= every) {
+                    if (chk.first == 0) chk.first = (int)t;
+                    since = 0;
+                } else {
+                    since += unit;
+                }
+            const int64_t rest = batch % unit;   // the call's last steps: checked at their end
+            if (rest > 0 && (since += rest) >= every) {
+                since = 0;
+                chk.end = 1;
+            }
+        }
         UE_CUDA(ue::launch_gtab(dm, batch, s));
-        const cudaError_t e = ue::launch_flow(m->flow, v, Uif, batch, 0, s);
+        const cudaError_t e = ue::launch_flow(m->flow, v, Uif, batch, chk, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && left == n) {
             cudaGetLastError();
             m->flow.grid = 0;
@@ -1210,7 +1243,7 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
         UE_CUDA(e);
         launched += 1 + (dm.n_src > 0 ? 1 : 0);
         left -= batch;
-        UE_CUDA(watchdog_tick(m, batch, s, &launched));
+        m->since_check = since;
     }
     m->steps_done += n;
     m->launches += launched;
@@ -1474,7 +1507,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     const int64_t nt = h.n_tris, nei = h.n_ei;
     UE_CUDA(ue::launch_geom_tri(m->d_xy, m->d_tri_nodes, m->d_O, m->d_S, nt, s));
     UE_CUDA(ue::launch_geom_edge(m->d_xy, m->d_edge_nodes, m->d_edge_opp, m->d_elen, m->d_d, nei, s));
-    UE_CUDA(ue::launch_recip(m->d_elen, m->d_relen, nei, s));
+    UE_CUDA(ue::launch_recip(m->d_elen, m->d_d, m->d_relen, m->d_we, nei, s));
     // dual lengths must be positive (eq. 3 divides by |O_R O_L|); looked at on the device, eight
     // bytes come back (the two arrays and a host loop took 0.5 ms on 234k triangles)
     {
@@ -1703,7 +1736,7 @@ int ue_batch_create(ue_mesh* const* meshes, int32_t n, void* stream, ue_mesh** o
             UE_BATCH_CUDA(cudaMemcpyAsync((char*)dm.U + esz * ko, m->dm.U, esz * nei, cudaMemcpyDeviceToDevice, s));
         }
     }
-    UE_BATCH_CUDA(ue::launch_recip(B->d_elen, B->d_relen, NEI, s));   // the readout's 1/|e|
+    UE_BATCH_CUDA(ue::launch_recip(B->d_elen, B->d_d, B->d_relen, B->d_we, NEI, s));   // the readout's 1/|e|, the energy's d/|e|
     {
         // padding records of the batch point at its zero slot with coefficient 0
         std::vector<int4> pad(dm.n_t_pad - H.n_tris);
@@ -2118,7 +2151,7 @@ int ue_read_fields(ue_mesh* m, double* E, double* B, double* j, void* stream) {
 int ue_energy(ue_mesh* m, double* W, void* stream) {
     if (!m || !m->built || !W) return fail(UE_ERR_ARG, "geometry not built or NULL output");
     cudaStream_t s = (cudaStream_t)stream;
-    UE_CUDA(ue::launch_energy(m->dm, m->d_elen, m->d_d, m->d_S, m->wd_part, m->wd, s));
+    UE_CUDA(ue::launch_energy(m->dm, m->d_we, m->d_S, m->wd_part, m->wd, s));
     double wd[4];
     UE_CUDA(cudaMemcpyAsync(wd, m->wd, sizeof(wd), cudaMemcpyDeviceToHost, s));
     UE_CUDA(cudaStreamSynchronize(s));

@@ -128,7 +128,7 @@ def test_resident_with_a_frame(ue, tiled, plasma, frame, order):
 
 def test_resident_batch_and_watchdog(ue):
     """A batch of meshes with their own sources, and the watchdog's checks at the same steps."""
-    out = []
+    out, energy = [], []
     for chunk in (32, -1):
         meshes = []
         for n_t in (300, 4097, 2500):
@@ -144,10 +144,55 @@ def test_resident_batch_and_watchdog(ue):
         ok, W, flag = b.check()
         E, B, _ = b.read_fields()
         assert ok and flag == 0
-        out.append((E, B, W))
+        out.append((E, B))
+        energy.append(W)
         b.close()
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+    assert abs(energy[0] / energy[1] - 1) < 1e-13      # the same terms, summed in another order
+
+
+@pytest.mark.parametrize("every", [1, 32, 40, 100])
+@pytest.mark.parametrize("n_t", [500, 5000])
+def test_resident_watchdog_checks_at_the_same_steps(ue, every, n_t):
+    """The energy at the last check over calls that end inside and between the checks' steps, and a
+    run above the stability bound flagged."""
+    xy, tris, h = _lattice(n_t, 3)
+    calls, unit = (70, 32, 110, 45, 2000), 32
+    # the launches' checks: at the ends of the graph chunks and of the call, once `every` is reached
+    ends, since, at, last = [], 0, 0, 0
+    for n in calls:
+        for part in [unit] * (n // unit) + ([n % unit] if n % unit else []):
+            at, since = at + part, since + part
+            if since >= every:
+                since, last = 0, at
+        ends.append((at, last))
+    m = ue.Mesh(xy, tris)
+    m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=unit, watchdog_every=every)
+    m.write_fields(B=np.cos(np.arange(m.n_tris)))
+    r = ue.Mesh(xy, tris)
+    r.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=-1)
+    r.write_fields(B=np.cos(np.arange(r.n_tris)))
+    stepped, ref = 0, 0.0
+    for n, (_, last) in zip(calls, ends):
+        m.step_n(n)
+        if last > stepped:
+            r.step_n(last - stepped)
+            stepped, ref = last, r.energy()
+        ok, W, flag = m.check()
+        assert ok and flag == 0
+        # the same positive terms summed in another order, fewer than n_t + n_ei additions deep
+        assert abs(W - ref) <= 4 * n_t * 2.3e-16 * ref
+    m.close()
+    r.close()
+    # a step above the stability bound is flagged inside the launch
+    m = ue.Mesh(xy, tris)
+    m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.8 * h, graph_chunk=unit, watchdog_every=every, watchdog_growth=10.0)
+    m.write_fields(B=np.cos(np.arange(m.n_tris)))
+    m.step_n(960)
+    ok, _, flag = m.check()
+    m.close()
+    assert not ok and flag in (1, 2)
 
 
 def test_resident_wait_that_runs_out_is_reported(ue):

@@ -13,15 +13,18 @@
 // most 3 d L + 4 d^2 <= 0.54 h L (L its longest edge), less than the h L it has, so no triangle
 // turns over.
 // GPU, FP64, positions double-buffered: per step one thread per triangle evaluates its three
-// height springs and its cap once, then one thread per node gathers its edge springs and its
-// triangles' shares (node -> edge and node -> triangle lists).
-// Host: the lists, and the flips (a flip changes the lists).
+// height springs, its cap and the edge springs it owns once each, then one thread per node gathers
+// its edges' and its triangles' shares.  The lists are made on the device after every round of
+// flips, which also marks the edges that may not be Delaunay; the flips themselves, whose order
+// decides the result's rows, are made on the host from those marks.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <string>
+#include <type_traits>
 #include <unordered_set>
 #include <utility>
 #include <vector>
@@ -33,102 +36,361 @@ namespace ue {
 namespace {
 
 constexpr int kRxThreads = 256;
+// The two step kernels use small blocks: 40k triangles are 636 blocks for 152 SMs, where 159 of 256
+// threads gave seven SMs twice the work of the others.
+constexpr int kRxStepThreads = 64;
 
-// adjacency of one triangulation, as uploaded
-struct RxLists {
-    std::vector<int32_t> e_off, e_nb;     // node -> (neighbour node) of each incident edge
-    std::vector<double> e_L0;             // rest length of that edge
-    std::vector<int32_t> t_off, t_tri;    // node -> incident triangle
-    std::vector<int32_t> t_loc;           // local index of the node in it (0..2)
-    std::vector<double> H0;               // rest height per triangle
-    std::vector<double> cap;              // displacement cap per node
-    std::vector<uint8_t> fixed;           // boundary node
+// Device arrays of one relaxation.  A corner or an edge is a code s = 3 i + q of triangle i: the
+// corner q, the edge from it to the next corner.
+struct RxDev {
+    double *x0, *x1;      // positions, before and after a step
+    double* h;            // size per node
+    double* H0;           // rest height per triangle
+    double* cap;          // displacement cap per node
+    double* tri_out;      // per triangle: {F_0, F_1, F_2 (x, y each), cap, 0}
+    double* edge_out;     // per owned edge s: its pull on its first node
+    int32_t *t, *nb;      // corners; the triangle across edge s, -1 none
+    int32_t *off, *cnt;   // node v: its corners at code[off[v] .. off[v] + cnt[v]), ascending
+    int32_t* code;
+    int32_t* e_cnt;       // node v: its edges at e_ref[2 off[v] ..], by the other node's number
+    uint32_t* e_ref;      // 2 s + (1: v is the edge's second node) of the slot s that owns the edge
+    uint8_t *own, *fixed; // slot s owns its edge; boundary nodes and anchors
+    uint8_t* anchor;
+    uint8_t* marks;       // per slot, for the flips: kSeed, kSeed | kLook
+    int32_t* ctl;         // {list cursor, a node has too many triangles, an edge is not shared by two}
+    size_t cleared;       // bytes from cnt on that a rebuild starts at zero
 };
+
+// Corners per node that one thread sorts (about 6 in a triangulation of any quality); a mesh with a
+// node of more is listed on the host.
+constexpr int kRxValence = 32;
+constexpr uint8_t kSeed = 1, kLook = 2;
+
+// 1/|w| and |w| of w^2 = n2: one Heron step on n2 rsqrt(n2) gives the root to about half an ulp, so
+// springs and caps keep the precision of a square root and a division at the cost of one rsqrt.
+__device__ __forceinline__ double root(double n2, double* r) {
+    *r = rsqrt(n2);
+    const double y = n2 * *r;
+    return fma(fma(-y, y, n2), 0.5 * *r, y);
+}
 
 // Per triangle, once per step: the three height springs' pulls on its vertices and the cap
 // 0.15 * (2 area / longest edge).  Spring q (apex q over the edge (q+1, q+2)) with
 // g_q = ((|w| - H0) / |w|) w, w = x_q - (x_{q+1} + x_{q+2}) / 2, pulls the apex by -g_q and each
-// end of its edge by g_q / 2, so vertex j takes -g_j + (g_{j+1} + g_{j+2}) / 2.
-// out: 8 doubles per triangle {F_0, F_1, F_2 (x, y each), cap, 0}.
-__global__ void k_rx_tri(const double* __restrict__ x, const int32_t* __restrict__ tris,
-                         const double* __restrict__ H0, double* __restrict__ out, int64_t n_tris) {
+// end of its edge by g_q / 2, so vertex j takes -g_j + (g_{j+1} + g_{j+2}) / 2.  The springs along
+// the edges that it owns: the pull on the second node is the negative.
+// Bound by the FP64 pipe (two lanes per SM and clock): every edge and height is evaluated once,
+// with one rsqrt for its root and its division.  40k triangles: 17 us, the FP64 pipe busy for 78% of
+// the active cycles (23 us with an edge length per triangle and a root and a division per spring).
+__global__ void __launch_bounds__(kRxStepThreads) k_rx_tri(const __grid_constant__ RxDev a, const double* __restrict__ x,
+                                                           int64_t n_tris) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t n[3];
+    double h[3], h0 = 0.0;
+    uint8_t own[3];
+    if (t < n_tris) {
+        for (int q = 0; q < 3; ++q) {
+            n[q] = a.t[3 * t + q];
+            h[q] = a.h[n[q]];
+            own[q] = a.own[3 * t + q];
+        }
+        h0 = a.H0[t];
+    }
+    grid_dependency_wait();
+    grid_dependents_launch();
     if (t >= n_tris) return;
     double px[3], py[3];
     for (int q = 0; q < 3; ++q) {
-        const int32_t n = tris[3 * t + q];
-        px[q] = x[2 * n];
-        py[q] = x[2 * n + 1];
+        const double2 p = __ldcg(reinterpret_cast<const double2*>(x) + n[q]);
+        px[q] = p.x;
+        py[q] = p.y;
     }
     const double a2 = fabs((px[1] - px[0]) * (py[2] - py[0]) - (py[1] - py[0]) * (px[2] - px[0]));
-    double lm = 0.0;
+    double l2[3];
+    double2* eo = reinterpret_cast<double2*>(a.edge_out) + 3 * t;
     for (int q = 0; q < 3; ++q) {
         const int p = q == 2 ? 0 : q + 1;
         const double ex = px[p] - px[q], ey = py[p] - py[q];
-        lm = fmax(lm, sqrt(ex * ex + ey * ey));
+        l2[q] = ex * ex + ey * ey;
+        if (own[q]) {
+            double r;
+            const double s = (root(l2[q], &r) - 0.5 * (h[q] + h[p])) * r;
+            eo[q] = make_double2(s * ex, s * ey);
+        }
     }
-    const double h0 = H0[t];
     double gx[3], gy[3];
     for (int q = 0; q < 3; ++q) {
         const int p = q == 2 ? 0 : q + 1, r = q == 0 ? 2 : q - 1;
         const double wx = px[q] - 0.5 * (px[p] + px[r]), wy = py[q] - 0.5 * (py[p] + py[r]);
-        const double hm = sqrt(wx * wx + wy * wy);
-        const double sc = (hm - h0) / hm;
+        double rm;
+        const double hm = root(wx * wx + wy * wy, &rm);
+        const double sc = (hm - h0) * rm;
         gx[q] = sc * wx;
         gy[q] = sc * wy;
     }
-    double* o = out + 8 * t;
+    double f[6];
     for (int j = 0; j < 3; ++j) {
         const int p = j == 2 ? 0 : j + 1, r = j == 0 ? 2 : j - 1;
-        o[2 * j] = 0.5 * (gx[p] + gx[r]) - gx[j];
-        o[2 * j + 1] = 0.5 * (gy[p] + gy[r]) - gy[j];
+        f[2 * j] = 0.5 * (gx[p] + gx[r]) - gx[j];
+        f[2 * j + 1] = 0.5 * (gy[p] + gy[r]) - gy[j];
     }
-    o[6] = 0.15 * (a2 / lm);
-    o[7] = 0.0;
+    double rl;
+    const double lm = root(fmax(fmax(l2[0], l2[1]), l2[2]), &rl);
+    double ht = a2 * rl;
+    ht = fma(fma(-lm, ht, a2), rl, ht);
+    double2* o = reinterpret_cast<double2*>(a.tri_out) + 4 * t;
+    o[0] = make_double2(f[0], f[1]);
+    o[1] = make_double2(f[2], f[3]);
+    o[2] = make_double2(f[4], f[5]);
+    o[3] = make_double2(0.15 * ht, 0.0);
 }
 
 // Per node: its edge springs, its shares of its triangles' height springs, the smallest cap;
-// then the capped Euler step (fixed nodes copy through).
-__global__ void k_rx_node(const double* __restrict__ x, double* __restrict__ xn,
-                          const int32_t* __restrict__ e_off, const int32_t* __restrict__ e_nb,
-                          const double* __restrict__ e_L0, const int32_t* __restrict__ t_off,
-                          const int32_t* __restrict__ t_tri, const int32_t* __restrict__ t_loc,
-                          const double* __restrict__ tri_out, const double* __restrict__ cap,
-                          const uint8_t* __restrict__ fixed, double tau, int64_t n_nodes) {
+// then the capped Euler step (fixed nodes copy through).  Bound by the latency of its gathers: the
+// first kRxHeld entries of both lists are read before the triangles' kernel has finished, and what
+// they name is then loaded at once.  20k nodes: 12 us (30 us with every edge's spring evaluated here,
+// at both of its ends).
+constexpr int kRxHeld = 8;
+__global__ void __launch_bounds__(kRxStepThreads) k_rx_node(const __grid_constant__ RxDev a, const double* __restrict__ x,
+                                                            double* __restrict__ xn, double tau, int64_t n_nodes) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t ne = 0, nt = 0;
+    double c = 0.0;
+    bool fixed = true;
+    const uint32_t* er = nullptr;
+    const int32_t* cd = nullptr;
+    if (v < n_nodes) {
+        const int32_t off = a.off[v];
+        ne = a.e_cnt[v];
+        nt = a.cnt[v];
+        c = a.cap[v];
+        fixed = a.fixed[v];
+        er = a.e_ref + 2 * (int64_t)off;
+        cd = a.code + off;
+    }
+    uint32_t r[kRxHeld];
+    int32_t s[kRxHeld];
+#pragma unroll
+    for (int i = 0; i < kRxHeld; ++i) {
+        r[i] = i < ne ? er[i] : 0u;
+        s[i] = i < nt ? cd[i] : 0;
+    }
+    grid_dependency_wait();
+    grid_dependents_launch();
     if (v >= n_nodes) return;
-    const double vx = x[2 * v], vy = x[2 * v + 1];
-    if (fixed[v]) {
-        xn[2 * v] = vx;
-        xn[2 * v + 1] = vy;
+    const double2 p = __ldcg(reinterpret_cast<const double2*>(x) + v);
+    if (fixed) {
+        reinterpret_cast<double2*>(xn)[v] = p;
         return;
     }
-    double fx = 0.0, fy = 0.0;
-    for (int32_t i = e_off[v]; i < e_off[v + 1]; ++i) {   // edge springs
-        const int32_t b = e_nb[i];
-        const double dx = x[2 * b] - vx, dy = x[2 * b + 1] - vy;
-        const double L = sqrt(dx * dx + dy * dy);
-        const double s = (L - e_L0[i]) / L;
-        fx += s * dx;
-        fy += s * dy;
+    auto edge = [&](uint32_t ref) { return __ldcg(reinterpret_cast<const double2*>(a.edge_out) + (ref >> 1)); };
+    auto share = [&](int32_t code, double* cap) {
+        const int32_t t = code / 3;
+        const double2* o = reinterpret_cast<const double2*>(a.tri_out) + 4 * (int64_t)t;
+        *cap = __ldcg(reinterpret_cast<const double*>(o + 3));
+        return __ldcg(o + (code - 3 * t));
+    };
+    double2 ev[kRxHeld], tv[kRxHeld];
+    double cv[kRxHeld];
+#pragma unroll
+    for (int i = 0; i < kRxHeld; ++i) {
+        if (i < ne) ev[i] = edge(r[i]);
+        if (i < nt) tv[i] = share(s[i], &cv[i]);
     }
-    double c = cap[v];
-    for (int32_t i = t_off[v]; i < t_off[v + 1]; ++i) {   // its triangles' height springs
-        const double* o = tri_out + 8 * (int64_t)t_tri[i];
-        const int l = t_loc[i];
-        fx += o[2 * l];
-        fy += o[2 * l + 1];
-        c = fmin(c, o[6]);
+    double fx = 0.0, fy = 0.0;
+    auto pull = [&](uint32_t ref, double2 e) {   // edge springs
+        fx += ref & 1 ? -e.x : e.x;
+        fy += ref & 1 ? -e.y : e.y;
+    };
+    auto height = [&](double2 f, double cap) {   // its triangles' height springs
+        fx += f.x;
+        fy += f.y;
+        c = fmin(c, cap);
+    };
+#pragma unroll
+    for (int i = 0; i < kRxHeld; ++i)
+        if (i < ne) pull(r[i], ev[i]);
+    for (int32_t i = kRxHeld; i < ne; ++i) pull(er[i], edge(er[i]));
+#pragma unroll
+    for (int i = 0; i < kRxHeld; ++i)
+        if (i < nt) height(tv[i], cv[i]);
+    for (int32_t i = kRxHeld; i < nt; ++i) {
+        double cap;
+        const double2 f = share(cd[i], &cap);
+        height(f, cap);
     }
     double dx = tau * fx, dy = tau * fy;
-    const double n = sqrt(dx * dx + dy * dy);
-    if (n > c) {
-        const double k = c / n;
-        dx *= k;
-        dy *= k;
+    const double n2 = dx * dx + dy * dy;
+    if (!(n2 < c * c * (1.0 - 1e-15))) {   // else the root is below c too
+        const double n = sqrt(n2);
+        if (n > c) {
+            const double k = c / n;
+            dx *= k;
+            dy *= k;
+        }
     }
-    xn[2 * v] = vx + dx;
-    xn[2 * v + 1] = vy + dy;
+    reinterpret_cast<double2*>(xn)[v] = make_double2(p.x + dx, p.y + dy);
+}
+
+// --- the lists: corners counted, offsets handed out block by block (any order serves), corners
+// filled in and sorted per node.  Five launches, 55 us together for 40k triangles; on the host the lists,
+// their upload and the flips' matching of edges took 6 ms per round of flips.
+
+__global__ void k_rx_count(const __grid_constant__ RxDev a, int64_t n_tris) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_tris) return;
+    double s = 0.0;
+    for (int q = 0; q < 3; ++q) {
+        const int32_t n = a.t[3 * t + q], m = a.t[3 * t + (q == 2 ? 0 : q + 1)];
+        atomicAdd(a.cnt + n, 1);
+        s += 0.5 * (a.h[n] + a.h[m]);
+    }
+    a.H0[t] = sqrt(3.0) / 2.0 * s / 3.0;
+}
+
+__global__ void __launch_bounds__(kRxThreads) k_rx_offsets(const __grid_constant__ RxDev a, int64_t n_nodes) {
+    __shared__ int32_t w[kRxThreads / 32];
+    __shared__ int32_t base;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int32_t n = v < n_nodes ? a.cnt[v] : 0;
+    if (n > kRxValence) a.ctl[1] = 1;
+    int32_t inc = n;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+    }
+    if (lane == 31) w[threadIdx.x >> 5] = inc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int32_t sum = 0;
+        for (int i = 0; i < kRxThreads / 32; ++i) {
+            const int32_t u = w[i];
+            w[i] = sum;
+            sum += u;
+        }
+        base = atomicAdd(a.ctl, sum);
+    }
+    __syncthreads();
+    if (v < n_nodes) a.off[v] = base + w[threadIdx.x >> 5] + inc - n;
+}
+
+__global__ void k_rx_fill(const __grid_constant__ RxDev a, int64_t n_slots) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n_slots) return;
+    const int32_t n = a.t[s];
+    a.code[a.off[n] + atomicAdd(a.e_cnt + n, 1)] = (int32_t)s;   // e_cnt: a cursor until k_rx_lists
+}
+
+// Node v's corners in ascending order, its edges by the other node's number (each owned by the lowest
+// slot that names it, as at its other end), its cap; an edge named once is on the boundary, its
+// ends fixed.
+__global__ void __launch_bounds__(kRxStepThreads) k_rx_lists(const __grid_constant__ RxDev a, int64_t n_nodes) {
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n_nodes) return;
+    const int32_t n = a.cnt[v];
+    if (n > kRxValence) return;
+    int32_t* cd = a.code + a.off[v];
+    unsigned long long key[2 * kRxValence];
+    key[0] = 0;
+    int m = 0;
+    auto put = [&](int32_t b, int32_t s, uint32_t second) {
+        const unsigned long long k = (unsigned long long)b << 32 | ((unsigned)s << 1 | second);
+        int i = m++;
+        for (; i > 0 && key[i - 1] > k; --i) key[i] = key[i - 1];
+        key[i] = k;
+    };
+    for (int32_t k = 0; k < n; ++k) {
+        const int32_t s = cd[k];
+        int32_t i = k;
+        for (; i > 0 && cd[i - 1] > s; --i) cd[i] = cd[i - 1];
+        cd[i] = s;
+        const int32_t t = s / 3, q = s - 3 * t, p = q == 2 ? 0 : q + 1, r = q == 0 ? 2 : q - 1;
+        put(a.t[3 * (int64_t)t + p], s, 0);
+        put(a.t[3 * (int64_t)t + r], 3 * t + r, 1);
+    }
+    uint32_t* er = a.e_ref + 2 * (int64_t)a.off[v];
+    int32_t ne = 0;
+    double cap = INFINITY;
+    for (int k = 0; k < m;) {
+        int r = k + 1;
+        while (r < m && key[r] >> 32 == key[k] >> 32) ++r;
+        const int32_t b = (int32_t)(key[k] >> 32);
+        const uint32_t ref = (uint32_t)key[k];
+        if (r - k == 1) a.fixed[v] = a.fixed[b] = 1;
+        a.own[ref >> 1] = 1;
+        er[ne++] = ref;
+        cap = fmin(cap, 0.1 * (0.5 * (a.h[v] + a.h[b])));
+        k = r;
+    }
+    a.e_cnt[v] = ne;
+    a.cap[v] = cap;
+    if (a.anchor[v]) a.fixed[v] = 1;
+}
+
+// The triangle across each edge, from the corners of its second node.  Edges of more than two
+// triangles, or of two on one side, are reported: the host's order of matching then decides.
+__global__ void k_rx_nb(const __grid_constant__ RxDev a, int64_t n_slots) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n_slots || a.ctl[1] != 0) return;
+    const int64_t i = s / 3;
+    const int q = (int)(s - 3 * i);
+    const int32_t n0 = a.t[s], n1 = a.t[3 * i + (q == 2 ? 0 : q + 1)];
+    int32_t nb = -1;
+    int twins = 0, same = 0;
+    for (int32_t k = a.off[n1], e = k + a.cnt[n1]; k < e; ++k) {
+        const int32_t c = a.code[k], j = c / 3, r = c - 3 * j;
+        if (j == (int32_t)i) continue;
+        if (a.t[3 * (int64_t)j + (r == 2 ? 0 : r + 1)] == n0) {
+            nb = j;
+            ++twins;
+        }
+        if (a.t[3 * (int64_t)j + (r == 0 ? 2 : r - 1)] == n0) ++same;
+    }
+    if (twins > 1 || same > 0) a.ctl[2] = 1;
+    a.nb[s] = nb;
+}
+
+// Marks for the flips: every edge once (the slot of its lower triangle), and whether the in-circle
+// test of in_circle() below could hold at these positions: the threshold is lowered by a
+// thousandth, far above the test's rounding (about 1e-14 of s^2), and what is not a number, or so
+// small that products underflow, is marked.
+__global__ void k_rx_marks(const __grid_constant__ RxDev m, const double* __restrict__ x, int64_t n_slots) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n_slots) return;
+    const int64_t i = s / 3, j = m.nb[s];
+    uint8_t mark = 0;
+    if (j > i) {
+        const int q = (int)(s - 3 * i);
+        const int32_t a = m.t[s], b = m.t[3 * i + (q == 2 ? 0 : q + 1)], c = m.t[3 * i + (q == 0 ? 2 : q - 1)];
+        int32_t d = m.t[3 * j];
+        for (int r = 1; r < 3; ++r)
+            if (d == a || d == b) d = m.t[3 * j + r];
+        const double2* p = reinterpret_cast<const double2*>(x);
+        const double2 pa = p[a], pb = p[b], pc = p[c], pd = p[d];
+        const double ax = pa.x - pd.x, ay = pa.y - pd.y, bx = pb.x - pd.x, by = pb.y - pd.y, cx = pc.x - pd.x,
+                     cy = pc.y - pd.y;
+        const double a2 = ax * ax + ay * ay, b2 = bx * bx + by * by, c2 = cx * cx + cy * cy;
+        const double det = a2 * (bx * cy - by * cx) - b2 * (ax * cy - ay * cx) + c2 * (ax * by - ay * bx);
+        const double l = fmax(a2, fmax(b2, c2));
+        mark = kSeed;
+        if (!(det <= 0.999e-10 * l * l) || !(l * l > 1e-280) || !(l * l < 1e280)) mark |= kLook;
+    }
+    m.marks[s] = mark;
+}
+
+template <typename K, typename... A>
+cudaError_t launch_after(K kern, unsigned grid, int threads, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 double orient2d(const std::vector<double>& x, int a, int b, int c) {
@@ -147,150 +409,164 @@ bool in_circle(const std::vector<double>& x, int a, int b, int c, int d) {
     return det > 1e-10 * s * s;
 }
 
-// Lawson flips until every interior edge is locally Delaunay; returns the number of flips.
-// nb[3 i + q] is the triangle across edge q = (t[q], t[q+1]) of triangle i (-1 on the boundary).
-// The stack holds (triangle, a, b) for a directed CCW edge a->b; an entry whose triangle no longer
-// holds that edge is stale and skipped: every flip pushes its four outer edges with their current
-// triangles, so no live edge is lost.
-// node -> incident triangles (CSR by counting), in triangle order
-void node_tris(int64_t nn, const std::vector<int32_t>& t, std::vector<int32_t>& off,
-               std::vector<int32_t>& tri, std::vector<int32_t>* loc) {
-    const int64_t nt = (int64_t)t.size() / 3;
-    off.assign(nn + 1, 0);
-    for (int32_t n : t) ++off[n + 1];
-    for (int64_t v = 0; v < nn; ++v) off[v + 1] += off[v];
-    tri.assign(off[nn], 0);
-    if (loc) loc->assign(off[nn], 0);
-    std::vector<int32_t> p(off.begin(), off.end() - 1);
-    for (int64_t i = 0; i < nt; ++i)
-        for (int q = 0; q < 3; ++q) {
-            const int32_t n = t[3 * i + q];
-            if (loc) (*loc)[p[n]] = q;
-            tri[p[n]++] = (int32_t)i;
-        }
-}
-
 uint64_t edge_key(int32_t a, int32_t b) {
     return ((uint64_t)(uint32_t)std::min(a, b) << 32) | (uint32_t)std::max(a, b);
 }
 
-// keep: edges (edge_key) that are never flipped (the input geometry's).
-int64_t lawson(const std::vector<double>& x, std::vector<int32_t>& t, const std::unordered_set<uint64_t>& keep) {
+// node -> corners 3 i + q (CSR by counting), ascending
+void node_corners(int64_t nn, const std::vector<int32_t>& t, std::vector<int32_t>& off, std::vector<int32_t>& code) {
+    off.assign(nn + 1, 0);
+    for (int32_t n : t) ++off[n + 1];
+    for (int64_t v = 0; v < nn; ++v) off[v + 1] += off[v];
+    code.assign(off[nn], 0);
+    std::vector<int32_t> p(off.begin(), off.end() - 1);
+    for (size_t s = 0; s < t.size(); ++s) code[p[t[s]]++] = (int32_t)s;
+}
+
+// nb[3 i + q]: the triangle across edge q = (t[q], t[q+1]) of triangle i (-1 on the boundary); marks
+// of all edges.
+void host_neighbours(int64_t nn, const std::vector<int32_t>& t, std::vector<int32_t>& nb, std::vector<uint8_t>& marks) {
     const int64_t nt = (int64_t)t.size() / 3;
-    const int64_t nn = (int64_t)x.size() / 2;
-    std::vector<int64_t> nb(3 * nt, -1);
-    {   // the twin of a -> b in triangle i is b -> a in one of b's other triangles
-        std::vector<int32_t> off, tri;
-        node_tris(nn, t, off, tri, nullptr);
-        for (int64_t i = 0; i < nt; ++i)
-            for (int q = 0; q < 3; ++q) {
-                if (nb[3 * i + q] >= 0) continue;   // found from the other side
-                const int32_t a = t[3 * i + q], b = t[3 * i + (q + 1) % 3];
-                for (int32_t k = off[b]; k < off[b + 1] && nb[3 * i + q] < 0; ++k) {
-                    const int32_t j = tri[k];
-                    if (j == i) continue;
-                    for (int r = 0; r < 3; ++r)
-                        if (t[3 * j + r] == b && t[3 * j + (r + 1) % 3] == a) {
-                            nb[3 * i + q] = j;
-                            nb[3 * j + r] = i;
-                            break;
-                        }
-                }
+    nb.assign(3 * nt, -1);
+    // the twin of a -> b in triangle i is b -> a in one of b's other triangles
+    std::vector<int32_t> off, code;
+    node_corners(nn, t, off, code);
+    for (int64_t i = 0; i < nt; ++i)
+        for (int q = 0; q < 3; ++q) {
+            if (nb[3 * i + q] >= 0) continue;   // found from the other side
+            const int32_t a = t[3 * i + q], b = t[3 * i + (q + 1) % 3];
+            for (int32_t k = off[b]; k < off[b + 1] && nb[3 * i + q] < 0; ++k) {
+                const int32_t j = code[k] / 3;
+                if (j == i) continue;
+                for (int r = 0; r < 3; ++r)
+                    if (t[3 * j + r] == b && t[3 * j + (r + 1) % 3] == a) {
+                        nb[3 * i + q] = j;
+                        nb[3 * j + r] = (int32_t)i;
+                        break;
+                    }
             }
-    }
-    struct Item { int64_t tri; int32_t a, b; };
+        }
+    marks.assign(3 * nt, 0);
+    for (int64_t s = 0; s < 3 * nt; ++s)
+        if (nb[s] > s / 3) marks[s] = kSeed | kLook;
+}
+
+// Lawson flips until every interior edge is locally Delaunay; returns the number of flips.
+// nb: as host_neighbours; it follows the flips.
+// Edges are taken in the order of their slots, those that flips bring up before the next: a
+// stack holds (triangle, a, b) for a directed CCW edge a->b; an entry whose triangle no longer
+// holds that edge is stale and skipped: every flip pushes its four outer edges with their current
+// triangles, so no live edge is lost.  An edge marked kSeed alone is Delaunay and passed by unless a
+// flip has changed one of its two triangles since.
+// keep: edges (edge_key) that are never flipped (the input geometry's).
+int64_t lawson(const std::vector<double>& x, std::vector<int32_t>& t, std::vector<int32_t>& nb,
+               std::vector<uint8_t>& marks, const std::unordered_set<uint64_t>& keep) {
+    const int64_t n_slots = (int64_t)t.size();
+    const std::vector<int32_t> t0 = t;   // the seeds' edges
+    struct Item { int32_t tri, a, b; };
     std::vector<Item> stack;
-    stack.reserve(3 * nt);
-    for (int64_t s = 3 * nt - 1; s >= 0; --s)
-        if (nb[s] > s / 3) stack.push_back({s / 3, t[s], t[3 * (s / 3) + (s % 3 + 1) % 3]});
     auto slot_of = [&](int64_t i, int32_t a, int32_t b) -> int {
         for (int q = 0; q < 3; ++q)
             if (t[3 * i + q] == a && t[3 * i + (q + 1) % 3] == b) return q;
         return -1;
     };
+    auto look = [&](int64_t i) {
+        if (i >= 0)
+            for (int q = 0; q < 3; ++q) marks[3 * i + q] |= kLook;
+    };
     int64_t flips = 0;
-    while (!stack.empty()) {
-        const Item it = stack.back();
-        stack.pop_back();
-        const int64_t i = it.tri;
-        const int qi = slot_of(i, it.a, it.b);
-        if (qi < 0) continue;                       // stale: the edge left this triangle
-        const int64_t j = nb[3 * i + qi];
-        if (j < 0) continue;
-        const int32_t a = it.a, b = it.b, c = t[3 * i + (qi + 2) % 3];
-        if (!keep.empty() && keep.count(edge_key(a, b))) continue;
-        const int qj = slot_of(j, b, a);
-        const int32_t d = t[3 * j + (qj + 2) % 3];
-        if (!in_circle(x, a, b, c, d)) continue;
-        if (orient2d(x, a, d, c) <= 0 || orient2d(x, d, b, c) <= 0) continue;   // not convex
-        const int64_t X_bc = nb[3 * i + (qi + 1) % 3], X_ca = nb[3 * i + (qi + 2) % 3];
-        const int64_t X_ad = nb[3 * j + (qj + 1) % 3], X_db = nb[3 * j + (qj + 2) % 3];
-        // new i = (a, d, c), new j = (d, b, c)
-        t[3 * i] = a; t[3 * i + 1] = d; t[3 * i + 2] = c;
-        t[3 * j] = d; t[3 * j + 1] = b; t[3 * j + 2] = c;
-        nb[3 * i] = X_ad; nb[3 * i + 1] = j; nb[3 * i + 2] = X_ca;
-        nb[3 * j] = X_db; nb[3 * j + 1] = X_bc; nb[3 * j + 2] = i;
-        auto repoint = [&](int64_t X, int64_t from, int64_t to) {
-            if (X < 0) return;
-            for (int q = 0; q < 3; ++q)
-                if (nb[3 * X + q] == from) { nb[3 * X + q] = to; return; }
-        };
-        repoint(X_ad, j, i);
-        repoint(X_bc, i, j);
-        ++flips;
-        stack.push_back({i, a, d});
-        stack.push_back({j, d, b});
-        stack.push_back({j, b, c});
-        stack.push_back({i, c, a});
+    for (int64_t seed = 0; seed < n_slots; ++seed) {
+        uint64_t eight;
+        if (seed + 8 <= n_slots && (std::memcpy(&eight, &marks[seed], 8), (eight & (0x0101010101010101ull * kLook)) == 0)) {
+            seed += 7;
+            continue;
+        }
+        if (marks[seed] != (kSeed | kLook)) continue;
+        const int32_t si = (int32_t)(seed / 3);
+        stack.push_back({si, t0[seed], t0[3 * (int64_t)si + (seed % 3 + 1) % 3]});
+        while (!stack.empty()) {
+            const Item it = stack.back();
+            stack.pop_back();
+            const int64_t i = it.tri;
+            const int qi = slot_of(i, it.a, it.b);
+            if (qi < 0) continue;                       // stale: the edge left this triangle
+            const int64_t j = nb[3 * i + qi];
+            if (j < 0) continue;
+            const int32_t a = it.a, b = it.b, c = t[3 * i + (qi + 2) % 3];
+            if (!keep.empty() && keep.count(edge_key(a, b))) continue;
+            const int qj = slot_of(j, b, a);
+            const int32_t d = t[3 * j + (qj + 2) % 3];
+            if (!in_circle(x, a, b, c, d)) continue;
+            if (orient2d(x, a, d, c) <= 0 || orient2d(x, d, b, c) <= 0) continue;   // not convex
+            const int32_t X_bc = nb[3 * i + (qi + 1) % 3], X_ca = nb[3 * i + (qi + 2) % 3];
+            const int32_t X_ad = nb[3 * j + (qj + 1) % 3], X_db = nb[3 * j + (qj + 2) % 3];
+            // new i = (a, d, c), new j = (d, b, c)
+            t[3 * i] = a; t[3 * i + 1] = d; t[3 * i + 2] = c;
+            t[3 * j] = d; t[3 * j + 1] = b; t[3 * j + 2] = c;
+            nb[3 * i] = X_ad; nb[3 * i + 1] = (int32_t)j; nb[3 * i + 2] = X_ca;
+            nb[3 * j] = X_db; nb[3 * j + 1] = X_bc; nb[3 * j + 2] = (int32_t)i;
+            auto repoint = [&](int64_t X, int64_t from, int64_t to) {
+                if (X < 0) return;
+                for (int q = 0; q < 3; ++q)
+                    if (nb[3 * X + q] == from) { nb[3 * X + q] = (int32_t)to; return; }
+            };
+            repoint(X_ad, j, i);
+            repoint(X_bc, i, j);
+            for (int64_t X : {i, j, (int64_t)X_ad, (int64_t)X_db, (int64_t)X_bc, (int64_t)X_ca}) look(X);
+            ++flips;
+            stack.push_back({(int32_t)i, a, d});
+            stack.push_back({(int32_t)j, d, b});
+            stack.push_back({(int32_t)j, b, c});
+            stack.push_back({(int32_t)i, c, a});
+        }
     }
     return flips;
 }
 
-void build_lists(int64_t nn, const std::vector<int32_t>& t, const std::vector<double>& h, RxLists& L) {
-    const int64_t nt = (int64_t)t.size() / 3;
-    // node -> triangles (with the node's local index), in triangle order
-    node_tris(nn, t, L.t_off, L.t_tri, &L.t_loc);
-    L.H0.assign(nt, 0.0);
-    for (int64_t i = 0; i < nt; ++i) {
-        double s = 0.0;
-        for (int q = 0; q < 3; ++q) s += 0.5 * (h[t[3 * i + q]] + h[t[3 * i + (q + 1) % 3]]);
-        L.H0[i] = std::sqrt(3.0) / 2.0 * s / 3.0;
-    }
-    // node -> edges in increasing neighbour order (each triangle names each of its vertices'
-    // two neighbours; an edge named once is on the boundary, its ends fixed)
-    L.fixed.assign(nn, 0);
-    L.e_off.assign(nn + 1, 0);
-    L.e_nb.clear();
-    L.e_L0.clear();
+// The lists of k_rx_offsets, k_rx_fill and k_rx_lists on the host, for meshes with a node of more
+// than kRxValence triangles: sorted in n log n.
+struct RxLists {
+    std::vector<int32_t> off, cnt, code, e_cnt;
+    std::vector<uint32_t> e_ref;
+    std::vector<uint8_t> own, fixed;
+    std::vector<double> cap;
+};
+
+void build_lists(int64_t nn, const std::vector<int32_t>& t, const std::vector<double>& h, const std::vector<uint8_t>& anchor,
+                 RxLists& L) {
+    node_corners(nn, t, L.off, L.code);
+    L.cnt.resize(nn);
+    L.e_cnt.assign(nn, 0);
+    L.e_ref.assign(2 * L.code.size(), 0);
+    L.own.assign(t.size(), 0);
+    L.fixed = anchor;
     L.cap.assign(nn, INFINITY);
-    std::vector<int32_t> nbr;
+    std::vector<uint64_t> key;
     for (int64_t v = 0; v < nn; ++v) {
-        nbr.clear();
-        for (int32_t k = L.t_off[v]; k < L.t_off[v + 1]; ++k) {
-            const int32_t i = L.t_tri[k], q = L.t_loc[k];
-            nbr.push_back(t[3 * i + (q + 1) % 3]);
-            nbr.push_back(t[3 * i + (q + 2) % 3]);
+        key.clear();
+        L.cnt[v] = L.off[v + 1] - L.off[v];
+        for (int32_t k = L.off[v]; k < L.off[v + 1]; ++k) {
+            const int32_t s = L.code[k], q = s % 3, p = s - q + (q + 1) % 3, r = s - q + (q + 2) % 3;
+            key.push_back((uint64_t)t[p] << 32 | (uint32_t)s << 1);
+            key.push_back((uint64_t)t[r] << 32 | (uint32_t)r << 1 | 1);
         }
-        std::sort(nbr.begin(), nbr.end());
-        for (size_t k = 0; k < nbr.size();) {
+        std::sort(key.begin(), key.end());
+        uint32_t* er = L.e_ref.data() + 2 * (size_t)L.off[v];
+        for (size_t k = 0; k < key.size();) {
             size_t r = k + 1;
-            while (r < nbr.size() && nbr[r] == nbr[k]) ++r;
-            const int32_t b = nbr[k];
+            while (r < key.size() && key[r] >> 32 == key[k] >> 32) ++r;
+            const int32_t b = (int32_t)(key[k] >> 32);
             if (r - k == 1) L.fixed[v] = L.fixed[b] = 1;
-            const double l0 = 0.5 * (h[v] + h[b]);
-            L.e_nb.push_back(b);
-            L.e_L0.push_back(l0);
-            L.cap[v] = std::min(L.cap[v], 0.1 * l0);
+            L.own[(uint32_t)key[k] >> 1] = 1;
+            er[L.e_cnt[v]++] = (uint32_t)key[k];
+            L.cap[v] = std::min(L.cap[v], 0.1 * (0.5 * (h[v] + h[b])));
             k = r;
         }
-        L.e_off[v + 1] = (int32_t)L.e_nb.size();
     }
 }
 
 }  // namespace
 
-// See include/ue.h (ue_mesh_relax).  Device buffers are owned here (cudaMalloc/cudaFree):
-// the call is a one-off preprocessing step outside any mesh.
 namespace {
 
 // Orients the triangles CCW in t (a copy of tris); accumulates the area.
@@ -343,7 +619,10 @@ int mesh_flip(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, con
     int rc = orient_input(x, nn, t, &area, err);
     if (rc == UE_OK) rc = keep_set(segs, n_segs, nn, keep, err);
     if (rc != UE_OK) return rc;
-    const int64_t k = lawson(x, t, keep);
+    std::vector<int32_t> nb;
+    std::vector<uint8_t> marks;
+    host_neighbours(nn, t, nb, marks);
+    const int64_t k = lawson(x, t, nb, marks, keep);
     std::copy(t.begin(), t.end(), tris_out);
     if (n_flips) *n_flips = k;
     return UE_OK;
@@ -379,81 +658,118 @@ int mesh_relax(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, co
     } else {
         std::fill(h.begin(), h.end(), std::sqrt(4.0 * area / (std::sqrt(3.0) * (double)nt)));
     }
-    RxLists L;
-    // the boundary nodes are fixed by build_lists; the caller's anchors join them
-    auto lists = [&]() {
-        build_lists(nn, t, h, L);
-        for (int64_t k = 0; k < n_anchors; ++k) L.fixed[anchors[k]] = 1;
+    std::vector<uint8_t> anchor(nn, 0);
+    for (int64_t k = 0; k < n_anchors; ++k) anchor[anchors[k]] = 1;
+
+    // one device block for the call, a one-off preprocessing step outside any mesh
+    RxDev a = {};
+    size_t bytes = 0;
+    char* block = nullptr;
+    auto lay = [&]() {   // twice: the size, then the pointers
+        bytes = 0;
+        auto cut = [&](auto*& p, size_t n) {
+            p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(block + bytes);
+            bytes += (n * sizeof(*p) + 255) / 256 * 256;
+        };
+        cut(a.x0, 2 * nn);
+        cut(a.x1, 2 * nn);
+        cut(a.h, nn);
+        cut(a.H0, nt);
+        cut(a.cap, nn);
+        cut(a.tri_out, 8 * nt);
+        cut(a.edge_out, 6 * nt);
+        cut(a.t, 3 * nt);
+        cut(a.nb, 3 * nt);
+        cut(a.off, nn);
+        cut(a.code, 3 * nt);
+        cut(a.e_ref, 6 * nt);
+        cut(a.anchor, nn);
+        cut(a.marks, 3 * nt);
+        const size_t z = bytes;
+        cut(a.cnt, nn);
+        cut(a.e_cnt, nn);
+        cut(a.own, 3 * nt);
+        cut(a.fixed, nn);
+        cut(a.ctl, 4);
+        a.cleared = bytes - z;
     };
-    lists();
-    // device buffers, sized for the lists (their sizes do not change under flips)
-    double *dx0 = nullptr, *dx1 = nullptr, *dL0 = nullptr, *dH0 = nullptr, *dcap = nullptr,
-           *dtri = nullptr;
-    int32_t *dt = nullptr, *deo = nullptr, *den = nullptr, *dto = nullptr, *dtt = nullptr, *dtl = nullptr;
-    uint8_t* dfix = nullptr;
-    const size_t ne2 = L.e_nb.size(), nt3 = L.t_tri.size();
-    cudaError_t e = cudaSuccess;
+    lay();
+    cudaError_t e = cudaMalloc(&block, bytes);
+    lay();
     auto ck = [&](cudaError_t r) {
         if (e == cudaSuccess && r != cudaSuccess) e = r;
     };
-    ck(cudaMalloc(&dx0, 16 * nn));
-    ck(cudaMalloc(&dx1, 16 * nn));
-    ck(cudaMalloc(&dt, 12 * nt));
-    ck(cudaMalloc(&deo, 4 * (nn + 1)));
-    ck(cudaMalloc(&den, 4 * ne2));
-    ck(cudaMalloc(&dL0, 8 * ne2));
-    ck(cudaMalloc(&dto, 4 * (nn + 1)));
-    ck(cudaMalloc(&dtt, 4 * nt3));
-    ck(cudaMalloc(&dtl, 4 * nt3));
-    ck(cudaMalloc(&dH0, 8 * nt));
-    ck(cudaMalloc(&dcap, 8 * nn));
-    ck(cudaMalloc(&dfix, nn));
-    ck(cudaMalloc(&dtri, 64 * nt));
-    auto upload_lists = [&]() {
-        ck(cudaMemcpyAsync(dt, t.data(), 12 * nt, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(deo, L.e_off.data(), 4 * (nn + 1), cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(den, L.e_nb.data(), 4 * ne2, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dL0, L.e_L0.data(), 8 * ne2, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dto, L.t_off.data(), 4 * (nn + 1), cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dtt, L.t_tri.data(), 4 * nt3, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dtl, L.t_loc.data(), 4 * nt3, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dH0, L.H0.data(), 8 * nt, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dcap, L.cap.data(), 8 * nn, cudaMemcpyHostToDevice, s));
-        ck(cudaMemcpyAsync(dfix, L.fixed.data(), nn, cudaMemcpyHostToDevice, s));
-        ck(cudaStreamSynchronize(s));   // the host lists may change after this
+    const int64_t n_slots = 3 * nt;
+    auto blocks = [](int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); };
+    int32_t ctl[4] = {};
+    // after a change of t: the lists of every node and, where flips follow, the neighbours
+    auto relist = [&]() {
+        ck(cudaMemcpyAsync(a.t, t.data(), 4 * n_slots, cudaMemcpyHostToDevice, s));
+        ck(cudaMemsetAsync(a.cnt, 0, a.cleared, s));
+        if (e != cudaSuccess) return;
+        k_rx_count<<<blocks(nt, kRxThreads), kRxThreads, 0, s>>>(a, nt);
+        k_rx_offsets<<<blocks(nn, kRxThreads), kRxThreads, 0, s>>>(a, nn);
+        k_rx_fill<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, n_slots);
+        k_rx_lists<<<blocks(nn, kRxStepThreads), kRxStepThreads, 0, s>>>(a, nn);
+        if (flip_every > 0) k_rx_nb<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, n_slots);
+        ck(cudaGetLastError());
+        ck(cudaMemcpyAsync(ctl, a.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
+        ck(cudaStreamSynchronize(s));   // t may change after this
+        if (e != cudaSuccess || ctl[1] == 0) return;
+        RxLists L;
+        build_lists(nn, t, h, anchor, L);
+        ck(cudaMemcpyAsync(a.off, L.off.data(), 4 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.cnt, L.cnt.data(), 4 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.code, L.code.data(), 4 * n_slots, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.e_cnt, L.e_cnt.data(), 4 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.e_ref, L.e_ref.data(), 8 * n_slots, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.own, L.own.data(), n_slots, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.fixed, L.fixed.data(), nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.cap, L.cap.data(), 8 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaStreamSynchronize(s));
     };
     if (e == cudaSuccess) {
-        ck(cudaMemcpyAsync(dx0, x.data(), 16 * nn, cudaMemcpyHostToDevice, s));
-        upload_lists();
+        ck(cudaMemcpyAsync(a.x0, x.data(), 16 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.h, h.data(), 8 * nn, cudaMemcpyHostToDevice, s));
+        ck(cudaMemcpyAsync(a.anchor, anchor.data(), nn, cudaMemcpyHostToDevice, s));
+        relist();
     }
     int64_t flips = 0;
-    const unsigned grid = (unsigned)((nn + kRxThreads - 1) / kRxThreads);
-    const unsigned grid_t = (unsigned)((nt + kRxThreads - 1) / kRxThreads);
+    std::vector<int32_t> nb;
+    std::vector<uint8_t> marks;
+    bool nb_fresh = false;   // nb follows t
     for (int32_t it = 0; it < iters && e == cudaSuccess; ++it) {
-        k_rx_tri<<<grid_t, kRxThreads, 0, s>>>(dx0, dt, dH0, dtri, nt);
-        k_rx_node<<<grid, kRxThreads, 0, s>>>(dx0, dx1, deo, den, dL0, dto, dtt, dtl, dtri, dcap, dfix,
-                                               tau, nn);
-        ck(cudaGetLastError());
-        std::swap(dx0, dx1);
+        ck(launch_after(k_rx_tri, blocks(nt, kRxStepThreads), kRxStepThreads, s, a, (const double*)a.x0, nt));
+        ck(launch_after(k_rx_node, blocks(nn, kRxStepThreads), kRxStepThreads, s, a, (const double*)a.x0, a.x1, tau, nn));
+        std::swap(a.x0, a.x1);
         if (flip_every > 0 && (it + 1) % flip_every == 0 && e == cudaSuccess) {
-            ck(cudaMemcpyAsync(x.data(), dx0, 16 * nn, cudaMemcpyDeviceToHost, s));
+            const bool listed = ctl[1] == 0 && ctl[2] == 0;
+            ck(cudaMemcpyAsync(x.data(), a.x0, 16 * nn, cudaMemcpyDeviceToHost, s));
+            if (listed) {
+                k_rx_marks<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, a.x0, n_slots);
+                ck(cudaGetLastError());
+                nb.resize(n_slots);
+                marks.resize(n_slots);
+                ck(cudaMemcpyAsync(marks.data(), a.marks, n_slots, cudaMemcpyDeviceToHost, s));
+                if (!nb_fresh) ck(cudaMemcpyAsync(nb.data(), a.nb, 4 * n_slots, cudaMemcpyDeviceToHost, s));
+            }
             ck(cudaStreamSynchronize(s));
             if (e != cudaSuccess) break;
-            const int64_t k = lawson(x, t, keep);
+            if (!listed) host_neighbours(nn, t, nb, marks);
+            nb_fresh = true;
+            const int64_t k = lawson(x, t, nb, marks, keep);
             flips += k;
             if (k > 0) {
-                lists();
-                upload_lists();
+                relist();
+                nb_fresh = false;
             }
         }
     }
     if (e == cudaSuccess) {
-        ck(cudaMemcpyAsync(x.data(), dx0, 16 * nn, cudaMemcpyDeviceToHost, s));
+        ck(cudaMemcpyAsync(x.data(), a.x0, 16 * nn, cudaMemcpyDeviceToHost, s));
         ck(cudaStreamSynchronize(s));
     }
-    for (void* p : {(void*)dx0, (void*)dx1, (void*)dt, (void*)deo, (void*)den, (void*)dL0, (void*)dto,
-                    (void*)dtt, (void*)dtl, (void*)dH0, (void*)dcap, (void*)dfix, (void*)dtri})
-        if (p) cudaFree(p);
+    if (block) cudaFree(block);
     if (e != cudaSuccess) {
         err = std::string("mesh relaxation: ") + cudaGetErrorString(e);
         return UE_ERR_CUDA;

@@ -85,26 +85,18 @@ __device__ __forceinline__ double root(double n2, double* r) {
 __global__ void __launch_bounds__(kRxStepThreads) k_rx_tri(const __grid_constant__ RxDev a, const double* __restrict__ x,
                                                            int64_t n_tris) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int32_t n[3];
-    double h[3], h0 = 0.0;
-    uint8_t own[3];
-    if (t < n_tris) {
-        for (int q = 0; q < 3; ++q) {
-            n[q] = a.t[3 * t + q];
-            h[q] = a.h[n[q]];
-            own[q] = a.own[3 * t + q];
-        }
-        h0 = a.H0[t];
-    }
-    grid_dependency_wait();
-    grid_dependents_launch();
     if (t >= n_tris) return;
-    double px[3], py[3];
+    double px[3], py[3], h[3];
+    uint8_t own[3];
     for (int q = 0; q < 3; ++q) {
-        const double2 p = __ldcg(reinterpret_cast<const double2*>(x) + n[q]);
+        const int32_t n = a.t[3 * t + q];
+        const double2 p = reinterpret_cast<const double2*>(x)[n];
         px[q] = p.x;
         py[q] = p.y;
+        h[q] = a.h[n];
+        own[q] = a.own[3 * t + q];
     }
+    const double h0 = a.H0[t];
     const double a2 = fabs((px[1] - px[0]) * (py[2] - py[0]) - (py[1] - py[0]) * (px[2] - px[0]));
     double l2[3];
     double2* eo = reinterpret_cast<double2*>(a.edge_out) + 3 * t;
@@ -147,27 +139,24 @@ __global__ void __launch_bounds__(kRxStepThreads) k_rx_tri(const __grid_constant
 
 // Per node: its edge springs, its shares of its triangles' height springs, the smallest cap;
 // then the capped Euler step (fixed nodes copy through).  Bound by the latency of its gathers: the
-// first kRxHeld entries of both lists are read before the triangles' kernel has finished, and what
-// they name is then loaded at once.  20k nodes: 12 us (30 us with every edge's spring evaluated here,
+// first kRxHeld entries of both lists are read together, and what they name is then loaded at once.
+// (As a programmatic dependent of the triangles' kernel, the lists read before its end, a step took
+// 35 us instead of 29: waiting blocks held the registers of those to come.)  20k nodes: 12 us (30 us with every edge's spring evaluated here,
 // at both of its ends).
 constexpr int kRxHeld = 8;
 __global__ void __launch_bounds__(kRxStepThreads) k_rx_node(const __grid_constant__ RxDev a, const double* __restrict__ x,
                                                             double* __restrict__ xn, double tau, int64_t n_nodes) {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int32_t ne = 0, nt = 0;
-    double c = 0.0;
-    bool fixed = true;
-    const uint32_t* er = nullptr;
-    const int32_t* cd = nullptr;
-    if (v < n_nodes) {
-        const int32_t off = a.off[v];
-        ne = a.e_cnt[v];
-        nt = a.cnt[v];
-        c = a.cap[v];
-        fixed = a.fixed[v];
-        er = a.e_ref + 2 * (int64_t)off;
-        cd = a.code + off;
+    if (v >= n_nodes) return;
+    const double2 p = reinterpret_cast<const double2*>(x)[v];
+    if (a.fixed[v]) {
+        reinterpret_cast<double2*>(xn)[v] = p;
+        return;
     }
+    const int32_t off = a.off[v], ne = a.e_cnt[v], nt = a.cnt[v];
+    double c = a.cap[v];
+    const uint32_t* er = a.e_ref + 2 * (int64_t)off;
+    const int32_t* cd = a.code + off;
     uint32_t r[kRxHeld];
     int32_t s[kRxHeld];
 #pragma unroll
@@ -175,20 +164,12 @@ __global__ void __launch_bounds__(kRxStepThreads) k_rx_node(const __grid_constan
         r[i] = i < ne ? er[i] : 0u;
         s[i] = i < nt ? cd[i] : 0;
     }
-    grid_dependency_wait();
-    grid_dependents_launch();
-    if (v >= n_nodes) return;
-    const double2 p = __ldcg(reinterpret_cast<const double2*>(x) + v);
-    if (fixed) {
-        reinterpret_cast<double2*>(xn)[v] = p;
-        return;
-    }
-    auto edge = [&](uint32_t ref) { return __ldcg(reinterpret_cast<const double2*>(a.edge_out) + (ref >> 1)); };
+    auto edge = [&](uint32_t ref) { return reinterpret_cast<const double2*>(a.edge_out)[ref >> 1]; };
     auto share = [&](int32_t code, double* cap) {
         const int32_t t = code / 3;
         const double2* o = reinterpret_cast<const double2*>(a.tri_out) + 4 * (int64_t)t;
-        *cap = __ldcg(reinterpret_cast<const double*>(o + 3));
-        return __ldcg(o + (code - 3 * t));
+        *cap = reinterpret_cast<const double*>(o + 3)[0];
+        return o[code - 3 * t];
     };
     double2 ev[kRxHeld], tv[kRxHeld];
     double cv[kRxHeld];
@@ -377,20 +358,6 @@ __global__ void k_rx_marks(const __grid_constant__ RxDev m, const double* __rest
         if (!(det <= 0.999e-10 * l * l) || !(l * l > 1e-280) || !(l * l < 1e280)) mark |= kLook;
     }
     m.marks[s] = mark;
-}
-
-template <typename K, typename... A>
-cudaError_t launch_after(K kern, unsigned grid, int threads, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1] = {};
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 double orient2d(const std::vector<double>& x, int a, int b, int c) {
@@ -739,8 +706,9 @@ int mesh_relax(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, co
     std::vector<uint8_t> marks;
     bool nb_fresh = false;   // nb follows t
     for (int32_t it = 0; it < iters && e == cudaSuccess; ++it) {
-        ck(launch_after(k_rx_tri, blocks(nt, kRxStepThreads), kRxStepThreads, s, a, (const double*)a.x0, nt));
-        ck(launch_after(k_rx_node, blocks(nn, kRxStepThreads), kRxStepThreads, s, a, (const double*)a.x0, a.x1, tau, nn));
+        k_rx_tri<<<blocks(nt, kRxStepThreads), kRxStepThreads, 0, s>>>(a, a.x0, nt);
+        k_rx_node<<<blocks(nn, kRxStepThreads), kRxStepThreads, 0, s>>>(a, a.x0, a.x1, tau, nn);
+        ck(cudaGetLastError());
         std::swap(a.x0, a.x1);
         if (flip_every > 0 && (it + 1) % flip_every == 0 && e == cudaSuccess) {
             const bool listed = ctl[1] == 0 && ctl[2] == 0;

@@ -258,6 +258,10 @@ struct FlowDev {
     size_t sent_bytes = 0;
     int* hlist = nullptr;         // [grid * halo] remote neighbours
     int2* cnt = nullptr;          // [grid]
+    int edges = 0;                // FP64 without a frame: edge records per CTA, else 0
+    int2* erec = nullptr;         // [grid * edges]
+    int2* ecnt = nullptr;         // [grid]
+    int* eslot = nullptr;         // [interior edges] scratch of the plan
     int4* crec = nullptr;         // [frame cells]
     double* epart = nullptr;      // [kFlowChecks * grid] energy sums of a launch's checks, then
                                   // kFlowChecks counters (zero between launches)

@@ -110,6 +110,8 @@ struct FlowArgs {
     const int* hlist;       // halo per CTA: places (CTA * cap + slot, then the frame cells)
     const int2* cnt;        // per CTA: publishing triangles, remote neighbours
     const int4* crec;       // fper per CTA: offsets of a frame cell's neighbours, -1 none
+    const int2* erec;       // FP64 without a frame: edge records and {inner, all} edges per CTA
+    const int2* ecnt;
     const double* gtab;
     int one_grp;            // one source group: its g is staged in shared memory
     int n_t, n_ei, n_ei_pad;
@@ -146,6 +148,9 @@ struct PlanArgs {
     int* hlist;
     int2* cnt;
     int4* crec;
+    int2 *erec, *ecnt;
+    int* eslot;
+    int edges;              // edge records of a CTA
     unsigned* ctl;
     FrameDev f;
     int fper;
@@ -669,20 +674,13 @@ struct Flow {
         }
     }
 
-    // The energy of eq. 8 after a step (check c of the launch), without leaving the launch: each
-    // triangle adds its own term and those of the edges it is R of, and the last CTA to arrive sums
-    // the CTAs' shares in order and updates the watchdog.  Checks are handled in turn: the last
-    // arrival at one has arrived, and finished, at those before.  It is bound by the latency of its
-    // loads (three deep); ending the launch at every check instead and summing in two kernels cost
-    // 19 us more per check at 92k triangles (256 steps, a check every 32: 606 us, now 454 us).
-    __device__ __forceinline__ void energy(const FlowArgs<T>& a, int c) {
-        __shared__ double red[NT / 32];
-        __shared__ bool last;
-        const int tid = threadIdx.x;
+    // This thread's share of the energy of eq. 8: its triangles' own terms and those of the edges that
+    // they are R of.
+    __device__ __forceinline__ double energy(const FlowArgs<T>& a) const {
         double x = 0.0;
 #pragma unroll
         for (int i = 0; i < TS; ++i) {
-            const int l = tid + i * NT;
+            const int l = threadIdx.x + i * NT;
             if (l >= nloc) break;
             const int j = __ldg(&a.rec[(size_t)blockIdx.x * CAP + l].x);
             const int4 t = __ldg(a.tri + j);
@@ -694,27 +692,7 @@ struct Flow {
                 if (k < a.n_ei && !(code[q] & 1)) x += __ldg(a.chk.we + k) * (double)V[i][q] * (double)V[i][q];
             }
         }
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if ((tid & 31) == 0) red[tid >> 5] = x;
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < NT / 32; ++w) x += red[w];
-            a.epart[(size_t)c * gridDim.x + blockIdx.x] = x;
-            __threadfence();
-            last = SOLO || atomicAdd(a.ecount + c, 1u) == gridDim.x - 1;
-        }
-        __syncthreads();
-        if (last && tid < 32) {
-            __threadfence();
-            double w = 0.0;
-            for (int i = tid; i < (int)gridDim.x; i += 32) w += __ldcg(a.epart + (size_t)c * gridDim.x + i);
-            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-            if (tid == 0) {
-                watchdog_update(a.chk.wd, w);
-                __threadfence();
-            }
-        }
-        __syncthreads();
+        return x;
     }
 
     // Each edge by its R triangle, each interface edge by its triangle, each frame side by the
@@ -757,14 +735,47 @@ struct Flow {
     }
 };
 
-template <typename T, int SH, bool PLASMA, bool FRAME, bool SOLO>
-__global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constant__ FlowArgs<T> a) {
-    extern __shared__ __align__(16) unsigned char smraw[];
+// An energy check (check c of the launch) from the threads' shares, without leaving the launch: the
+// last CTA to arrive sums the CTAs' shares in order and updates the watchdog.  Checks are handled
+// in turn: the last arrival at one has arrived, and finished, at those before.  It is bound by the
+// latency of its loads (three deep); ending the launch at every check instead and summing in two
+// kernels cost 19 us more per check at 92k triangles (256 steps, a check every 32: 606 us, now 454 us).
+template <bool SOLO, typename T>
+__device__ __forceinline__ void energy_check(const FlowArgs<T>& a, int c, double x) {
+    __shared__ double red[32];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((tid & 31) == 0) red[tid >> 5] = x;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < (int)blockDim.x / 32; ++w) x += red[w];
+        a.epart[(size_t)c * gridDim.x + blockIdx.x] = x;
+        __threadfence();
+        last = SOLO || atomicAdd(a.ecount + c, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (last && tid < 32) {
+        __threadfence();
+        double w = 0.0;
+        for (int i = tid; i < (int)gridDim.x; i += 32) w += __ldcg(a.epart + (size_t)c * gridDim.x + i);
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        if (tid == 0) {
+            watchdog_update(a.chk.wd, w);
+            __threadfence();
+        }
+    }
+    __syncthreads();
+}
+
+// A launch of n_steps steps by F, with its checks.
+template <typename F, bool SOLO, typename T>
+__device__ __forceinline__ void flow_body(const FlowArgs<T>& a, unsigned char* sm) {
     const unsigned tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
     bool ok = true;
     if (SOLO || (int)blockIdx.x != a.skip) {
-        Flow<T, SH, PLASMA, FRAME, SOLO> f;
-        f.setup(a, smraw);
+        F f;
+        f.setup(a, sm);
         int c = 0, next = a.chk.first > 0 ? a.chk.first : a.n_steps + 1;
         bool go = true;
 #pragma unroll 1
@@ -778,7 +789,7 @@ __global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constan
                 if (!(go = f.template step<1>(a, s)) || ++s == end) break;
             }
             if (go && (s == next || (s == a.n_steps && a.chk.end))) {
-                f.energy(a, c++);
+                energy_check<SOLO>(a, c++, f.energy(a));
                 next += a.chk.period;
             }
         }
@@ -802,6 +813,385 @@ __global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constan
     }
 }
 
+template <typename T, int SH, bool PLASMA, bool FRAME, bool SOLO>
+__global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constant__ FlowArgs<T> a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    flow_body<Flow<T, SH, PLASMA, FRAME, SOLO>, SOLO>(a, smraw);
+}
+
+// --- FP64 without a frame -------------------------------------------------------------------
+// GB300's FP64 pipe takes two lanes per SM and clock, so what counts is FP64 instructions, and a
+// triangle's thread that computes its three edges computes every edge twice.  Here a thread holds
+// edges (J and their addresses in registers, U and the coefficients in shared memory) and triangles (B):
+// each step updates the edges once, U passing through shared memory, and sums the triangles:
+// 10.5 FP64 instructions per triangle with a current instead of 18, plus one side of the edges whose
+// other triangle is in another CTA.  Those come last in a CTA's edge list; the thread that holds one
+// polls the other triangle's word itself, after the inner edges have been computed.  On 241k
+// triangles with a current a step takes 6.7 us, in vacuum 3.9 (9.9 with a triangle's edges in its thread,
+// 11.9 as two launches).
+struct EdgeShape {
+    int ts, es, edges;   // triangle and edge slots per thread, edges of a CTA
+};
+constexpr EdgeShape kEdgeShapes[2] = {{1, 3, 3072}, {2, 5, 4608}};
+// a CTA with all its triangles and a full list of remote neighbours has this many edges at most
+static_assert(2 * kEdgeShapes[0].edges >= 3 * 1024 + kShapes[0].halo64 && 2 * kEdgeShapes[1].edges >= 3 * 2048 + kShapes[1].halo64);
+constexpr unsigned kEdgeMask = (1u << 28) - 1, kEdgeSrc = 1u << 28, kEdgeOwn = 1u << 29;
+
+// Accesses from packed words, each one volatile statement: hoisted out of the step loop, the
+// unpacked addresses and signs would not fit the registers.
+// the word of the place in an edge's w
+__device__ __forceinline__ void word_at(Word<double>& x, const unsigned long long* sl, unsigned w) {
+    asm volatile("{.reg .b32 i; .reg .b64 p; shr.u32 i, %3, 12; mad.wide.u32 p, i, 16, %2; ld.relaxed.gpu.global.v2.u64 {%0, %1}, [p];}"
+                 : "=l"(x.a), "=l"(x.b)
+                 : "l"(sl), "r"(w)
+                 : "memory");
+}
+// word_wait of it
+__device__ __forceinline__ bool word_wait_at(Word<double>& x, const unsigned long long* sl, unsigned w, unsigned tag) {
+    if (x.ready(tag)) return true;
+    const long long t0 = clock64();
+    for (unsigned n = 1;; ++n) {
+        word_at(x, sl, w);
+        if (x.ready(tag)) return true;
+        if ((n & 255u) == 0 && clock64() - t0 > (2LL << 30)) return false;
+    }
+}
+// B of the slot in an edge's w
+__device__ __forceinline__ double lds_slot(uint32_t bufs, unsigned w) {
+    double v;
+    asm volatile("{.reg .b32 t; and.b32 t, %1, 0xFFE; shl.b32 t, t, 2; add.u32 t, t, %2; ld.shared.f64 %0, [t];}"
+                 : "=d"(v)
+                 : "r"(w), "r"(bufs));
+    return v;
+}
+// U at the address in a half of w, negated when bit 16 + Q of signs is set
+template <bool HI, int Q>
+__device__ __forceinline__ double lds_signed(unsigned w, unsigned signs) {
+    double v;
+    if constexpr (HI)
+        asm volatile("{.reg .b32 t, s, l, h; shr.u32 t, %1, 16; shl.b32 s, %2, %3; and.b32 s, s, 0x80000000; ld.shared.v2.b32 {l, h}, [t]; xor.b32 h, h, s; mov.b64 %0, {l, h};}"
+                     : "=d"(v)
+                     : "r"(w), "r"(signs), "n"(15 - Q));
+    else
+        asm volatile("{.reg .b32 t, s, l, h; and.b32 t, %1, 65535; shl.b32 s, %2, %3; and.b32 s, s, 0x80000000; ld.shared.v2.b32 {l, h}, [t]; xor.b32 h, h, s; mov.b64 %0, {l, h};}"
+                     : "=d"(v)
+                     : "r"(w), "r"(signs), "n"(15 - Q));
+    return v;
+}
+
+struct __align__(16) EdgeSrc {
+    double c;
+    long long g;
+};
+template <int N>
+__device__ __forceinline__ EdgeSrc entry_at(const EdgeSrc* e) {
+    EdgeSrc v;
+    asm volatile("ld.global.nc.v2.b64 {%0,%1}, [%2+%3];" : "=d"(v.c), "=l"(v.g) : "l"(e), "n"((int)sizeof(v) * N));
+    return v;
+}
+
+template <int SH, bool PLASMA>
+struct EdgeFlow {
+    static constexpr int NT = 1024, TS = kEdgeShapes[SH].ts, ES = kEdgeShapes[SH].es, NE = kEdgeShapes[SH].edges;
+    static constexpr int CAP = NT * TS, VO = 8 * CAP, CO = VO + 8 * (NE + 2), PO = CO + 8 * NE, GO = PO + (PLASMA ? 8 * NE : 0);
+    static constexpr size_t SMEM = GO + 8 * (size_t)kFlowSteps;
+    static_assert(CO + 4096 < 65536, "16-bit shared addresses");
+};
+
+template <int SH, bool PLASMA, bool SOLO>
+struct Flow64 : EdgeFlow<SH, PLASMA> {
+    using L = EdgeFlow<SH, PLASMA>;
+    static constexpr int NT = L::NT, TS = L::TS, ES = L::ES, NE = L::NE, CAP = L::CAP, VO = L::VO, CO = L::CO, PO = L::PO;
+
+    double J[PLASMA ? ES : 1], b[TS], cB[TS];
+    unsigned w[ES];         // inner: shared addresses of B_R, B_L; cut: place << 12 | slot << 1 | here is R
+    unsigned n01[TS], n2s[TS];   // shared addresses of the three U, signs (1: negative) from bit 16
+    unsigned src;           // bit i: edge slot i has a source
+    int ni, ne, nloc, npub;
+    uint32_t bufs, own;
+    double* gs;
+    unsigned tag0;
+    bool ok;
+    unsigned long long* put[2];
+    const EdgeSrc* sent;
+
+    __device__ __forceinline__ void setup(const FlowArgs<double>& a, unsigned char* sm) {
+        const int tid = threadIdx.x;
+        bufs = smem_addr(sm);
+        own = bufs + 8u * (uint32_t)tid;
+        gs = reinterpret_cast<double*>(sm + L::GO);
+        nloc = max(0, min(a.per, a.n_t - (int)blockIdx.x * a.per));
+        npub = SOLO ? 0 : __ldg(&a.cnt[blockIdx.x].x);
+        const int2 en = __ldg(a.ecnt + blockIdx.x);
+        ni = en.x;
+        ne = en.y;
+        tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
+        ok = true;
+        const size_t first = (size_t)blockIdx.x * CAP + tid;
+        for (int p = 0; p < 2; ++p) put[p] = a.slots[p] + 2 * first;
+        const size_t e0 = (size_t)blockIdx.x * NE + tid;
+        sent = reinterpret_cast<const EdgeSrc*>(a.sent) + e0;
+        src = 0;
+#pragma unroll
+        for (int i = 0; i < ES; ++i) {
+            const int e = tid + i * NT;
+            w[i] = 0;
+            if constexpr (PLASMA) J[i] = 0.0;
+            if (e >= ne) continue;
+            const int2 r = __ldg(a.erec + e0 + i * NT);
+            const int k = r.x & kEdgeMask;
+            if (r.x & kEdgeSrc) src |= 1u << i;
+            w[i] = (unsigned)r.y + (e < ni ? bufs | (bufs << 16) : 0u);
+            *reinterpret_cast<double*>(sm + VO + 8 * e) = a.U[k];
+            *reinterpret_cast<double*>(sm + CO + 8 * e) = fabs(__ldg(a.cU + k));
+            if constexpr (PLASMA) {
+                J[i] = a.J[k];
+                *reinterpret_cast<double*>(sm + PO + 8 * e) = __ldg(a.pb + k);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = tid + i * NT;
+            n01[i] = n2s[i] = 0;
+            b[i] = cB[i] = 0.0;
+            if (l >= nloc) continue;
+            const int4 r = __ldg(a.rec + first + i * NT);
+            n01[i] = (unsigned)r.y + (bufs | (bufs << 16));
+            n2s[i] = (unsigned)r.z + bufs;
+            b[i] = a.B[r.x];
+            cB[i] = __ldg(a.cB64 + r.x);
+            reinterpret_cast<double*>(sm)[l] = b[i];
+        }
+        if (tid < 2) *reinterpret_cast<double*>(sm + VO + 8 * (NE + tid)) = 0.0;   // the walls' U
+        if (a.one_grp)
+            for (int e = tid; e < a.n_steps; e += NT) gs[e] = __ldg(a.gtab + e);
+        // published only after this CTA's reads of U and J are done: their owners write them back
+        // after later steps
+        if (!SOLO) __threadfence();
+        __syncthreads();
+        if constexpr (!SOLO) {
+            __threadfence();
+#pragma unroll
+            for (int i = 0; i < TS; ++i)
+                if (tid + i * NT < npub) slot_put(a.slots[0], (int)blockIdx.x * CAP + tid + i * NT, tag0, b[i]);
+        }
+    }
+
+    // Step s + 1 from the B of step s; remote B in the words of parity PB = s & 1.
+    template <int PB>
+    __device__ __forceinline__ bool step(const FlowArgs<double>& a, int s) {
+        const unsigned tag = tag0 + (unsigned)s;
+        inner<0>(a, s);
+        if constexpr (SOLO) {
+            __syncthreads();
+        } else {
+            cut<0>(a, a.slots[PB], tag, s);
+            ok = __syncthreads_and(ok ? 1 : 0) != 0;
+            if (!ok) return false;
+        }
+        sums<PB, 0>(tag);
+        __syncthreads();
+        return true;
+    }
+
+    template <int I>
+    __device__ __forceinline__ void update(const FlowArgs<double>& a, int s, double bR, double bL) {
+        const double uo = lds_at<VO + 8 * I * NT>(own, 0.0);
+        double un = rn_fma(lds_at<CO + 8 * I * NT>(own, 0.0), rn_sub(bR, bL), uo);
+        if constexpr (PLASMA) {
+            const double jn = rn_fma(a.pa, J[I], rn_mul(lds_at<PO + 8 * I * NT>(own, 0.0), uo));
+            un = rn_fma(a.mdt, jn, un);
+            J[I] = jn;
+        }
+        if ((src >> I) & 1u) {
+            const EdgeSrc se = entry_at<I * NT>(sent);
+            un = rn_fma(se.c, a.one_grp ? gs[s] : __ldg(a.gtab + se.g + s), un);
+        }
+        sts_at<VO + 8 * I * NT>(own, un);
+    }
+
+    template <int I>
+    __device__ __forceinline__ void inner(const FlowArgs<double>& a, int s) {
+        if constexpr (I < ES) {
+            if ((int)threadIdx.x + I * NT < ni) update<I>(a, s, lds_half<0, false>(w[I], 0.0), lds_half<0, true>(w[I], 0.0));
+            inner<I + 1>(a, s);
+        }
+    }
+
+    // Edges to other CTAs, two slots' polls in flight.
+    template <int I>
+    __device__ __forceinline__ bool is_cut() const {
+        const int e = (int)threadIdx.x + I * NT;
+        return e >= ni && e < ne;
+    }
+    template <int I>
+    __device__ __forceinline__ void arrive(const FlowArgs<double>& a, const unsigned long long* sl, unsigned tag, int s, Word<double>& x) {
+        if (!word_wait_at(x, sl, w[I], tag)) ok = false;
+        const double r = x.value(), h = lds_slot(bufs, w[I]);
+        update<I>(a, s, w[I] & 1u ? h : r, w[I] & 1u ? r : h);
+    }
+    template <int I>
+    __device__ __forceinline__ void cut(const FlowArgs<double>& a, const unsigned long long* sl, unsigned tag, int s) {
+        if constexpr (I < ES) {
+            Word<double> x, y;
+            if (is_cut<I>()) word_at(x, sl, w[I]);
+            if constexpr (I + 1 < ES) {
+                if (is_cut<I + 1>()) word_at(y, sl, w[I + 1]);
+            }
+            if (is_cut<I>()) arrive<I>(a, sl, tag, s, x);
+            if constexpr (I + 1 < ES) {
+                if (is_cut<I + 1>()) arrive<I + 1>(a, sl, tag, s, y);
+            }
+            cut<I + 2>(a, sl, tag, s);
+        }
+    }
+
+    template <int PB, int I>
+    __device__ __forceinline__ void sums(unsigned tag) {
+        if constexpr (I < TS) {
+            const int l = (int)threadIdx.x + I * NT;
+            if (l < nloc) {
+                const double v0 = lds_signed<false, 0>(n01[I], n2s[I]), v1 = lds_signed<true, 1>(n01[I], n2s[I]),
+                             v2 = lds_signed<false, 2>(n2s[I], n2s[I]);
+                b[I] = rn_fma(-cB[I], rn_add(rn_add(v0, v1), v2), b[I]);
+                sts_at<8 * I * NT>(own, b[I]);
+                if (!SOLO && l < npub) slot_put_at<I * NT>(put[PB ^ 1], tag + 1u, b[I]);
+            }
+            sums<PB, I + 1>(tag);
+        }
+    }
+
+    __device__ __forceinline__ double energy(const FlowArgs<double>& a) const {
+        double x = 0.0;
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = (int)threadIdx.x + i * NT;
+            if (l < nloc) x += __ldg(a.chk.S + __ldg(&a.rec[(size_t)blockIdx.x * CAP + l].x)) * b[i] * b[i];
+        }
+#pragma unroll
+        for (int i = 0; i < ES; ++i) {
+            const int e = (int)threadIdx.x + i * NT;
+            if (e >= ne) continue;
+            const unsigned k = (unsigned)__ldg(&a.erec[(size_t)blockIdx.x * NE + e].x);
+            const double u = lds_val<double>(own + VO + 8 * i * NT);
+            if (k & kEdgeOwn) x += __ldg(a.chk.we + (k & kEdgeMask)) * u * u;
+        }
+        return x;
+    }
+
+    __device__ __forceinline__ void write_back(const FlowArgs<double>& a) {
+        if (!SOLO) __threadfence();
+#pragma unroll
+        for (int i = 0; i < TS; ++i) {
+            const int l = (int)threadIdx.x + i * NT;
+            if (l < nloc) a.B[__ldg(&a.rec[(size_t)blockIdx.x * CAP + l].x)] = b[i];
+        }
+#pragma unroll
+        for (int i = 0; i < ES; ++i) {
+            const int e = (int)threadIdx.x + i * NT;
+            if (e >= ne) continue;
+            const unsigned k = (unsigned)__ldg(&a.erec[(size_t)blockIdx.x * NE + e].x);
+            if (!(k & kEdgeOwn)) continue;
+            a.U[k & kEdgeMask] = lds_val<double>(own + VO + 8 * i * NT);
+            if constexpr (PLASMA) a.J[k & kEdgeMask] = J[i];
+        }
+    }
+};
+
+template <int SH, bool PLASMA, bool SOLO>
+__global__ void __launch_bounds__(1024, 1) k_flow64(const __grid_constant__ FlowArgs<double> a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    flow_body<Flow64<SH, PLASMA, SOLO>, SOLO>(a, smraw);
+}
+
+// Its plan, after k_flow_order: a CTA's inner edges by their R triangle, then the cut ones, both in
+// stored order (fixed, so that energies repeat), and where each triangle finds its edges.
+__global__ void __launch_bounds__(1024) k_flow_edges(const __grid_constant__ PlanArgs a) {
+    __shared__ int wsum[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int j0 = blockIdx.x * a.per, nloc = max(0, min(a.per, a.n_t - j0)), p0 = (int)blockIdx.x * a.cap;
+    const double* cU = (const double*)a.cU;
+    int at[2], base = 0;   // edges before triangles tid and tid + 1024: inner | cut << 16
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int l = tid + 1024 * i;
+        int n = 0;
+        if (l < nloc) {
+            const int4 t = __ldg(a.tri + j0 + l);
+            const int code[3] = {t.x, t.y, t.z};
+            for (int q = 0; q < 3; ++q) {
+                const int k = code[q] >> 1;
+                if (k >= a.n_ei) continue;
+                const int2 r = __ldg(a.rl + k);
+                const int o = (code[q] & 1) ? r.x : r.y;
+                if (o < j0 || o >= j0 + nloc) n += 1 << 16;
+                else if (!(code[q] & 1)) ++n;
+            }
+        }
+        int inc = n;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        int before = base;
+        for (int k = 0; k < 32; ++k) {
+            before += k < warp ? wsum[k] : 0;
+            base += wsum[k];
+        }
+        at[i] = before + inc - n;
+        __syncthreads();
+    }
+    const int ni = base & 0xFFFF, nc = base >> 16;
+    if (tid == 0) a.ecnt[blockIdx.x] = make_int2(ni, ni + nc);
+    if (nc > a.halo || ni + nc > a.edges) {
+        if (tid == 0) atomicOr(a.ctl + 3, 1u);
+        return;
+    }
+    int2* erec = a.erec + (size_t)blockIdx.x * a.edges;
+    EdgeSrc* sent = (EdgeSrc*)a.sent + (size_t)blockIdx.x * a.edges;
+    for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int l = tid + 1024 * i;
+            if (l >= nloc) continue;
+            const int slot = a.place[j0 + l] - p0;
+            const int4 t = __ldg(a.tri + j0 + l);
+            const int code[3] = {t.x, t.y, t.z};
+            int in = at[i] & 0xFFFF, out = ni + (at[i] >> 16);
+            unsigned v[3], signs = 0;
+            for (int q = 0; q < 3; ++q) {
+                const int k = code[q] >> 1;
+                const bool neg = code[q] & 1;
+                int e = a.edges;   // a wall's: the slot that stays 0
+                if (k < a.n_ei) {
+                    const int2 r = __ldg(a.rl + k);
+                    const int o = neg ? r.x : r.y;
+                    const bool remote = o < j0 || o >= j0 + nloc;
+                    e = remote ? out++ : !neg ? in++ : pass == 1 ? a.eslot[k] : 0;
+                    if (neg) signs |= 1u << (16 + q);
+                    if (pass == 0 && (remote || !neg)) {
+                        int2 x = make_int2(k | (neg ? 0 : (int)kEdgeOwn), 0);
+                        if (remote) x.y = a.place[o] << 12 | slot << 1 | (neg ? 0 : 1);
+                        else x.y = 8 * slot | (8 * (a.place[o] - p0)) << 16;
+                        const int h = a.has_src && neg_bit(__ldg(cU + k)) ? src_index(a, k) : -1;
+                        if (h >= 0) {
+                            x.x |= (int)kEdgeSrc;
+                            sent[e] = EdgeSrc{__ldg((const double*)a.src_c + h), (long long)__ldg(a.src_grp + h) * a.gstride};
+                        }
+                        erec[e] = x;
+                        if (!remote) a.eslot[k] = e;
+                    }
+                }
+                v[q] = 8u * (unsigned)(a.cap + e);
+            }
+            if (pass == 1) a.rec[p0 + slot] = make_int4(j0 + l, (int)(v[0] | v[1] << 16), (int)(v[2] | signs), 0);
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void k_flow_init(unsigned* ctl) {
     if (threadIdx.x == 0) {
         ctl[0] = 1u;   // words start with tag 0
@@ -809,23 +1199,30 @@ __global__ void k_flow_init(unsigned* ctl) {
     }
 }
 
-template <typename T, bool PLASMA, bool FRAME, bool SOLO, int SH>
-cudaError_t launch_shape(const FlowArgs<T>& a, int grid, cudaStream_t s) {
-    auto kern = k_flow<T, SH, PLASMA, FRAME, SOLO>;
-    const size_t smem = flow_smem<T, PLASMA, SH>(FRAME ? a.fper : 0);
+template <typename T>
+cudaError_t launch_resident(void (*kern)(FlowArgs<T>), const FlowArgs<T>& a, int grid, int threads, size_t smem, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)kShapes[SH].nt);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = SOLO ? 0 : 1;
+    attr[0].val.cooperative = grid > 1 ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <typename T, bool PLASMA, bool FRAME, bool SOLO, int SH>
+cudaError_t launch_shape(const FlowArgs<T>& a, int grid, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8 && !FRAME)
+        return launch_resident<T>(k_flow64<SH, PLASMA, SOLO>, a, grid, 1024, EdgeFlow<SH, PLASMA>::SMEM, s);
+    else
+        return launch_resident<T>(k_flow<T, SH, PLASMA, FRAME, SOLO>, a, grid, kShapes[SH].nt,
+                                  flow_smem<T, PLASMA, SH>(FRAME ? a.fper : 0), s);
 }
 
 template <typename T, bool PLASMA, bool FRAME>
@@ -834,7 +1231,8 @@ cudaError_t launch_flow_pf(const FlowArgs<T>& a, const FlowDev& fl, cudaStream_t
         if constexpr (FRAME) return cudaErrorInvalidValue;
         else {
             if (fl.shape == 0) return launch_shape<T, PLASMA, false, true, 0>(a, 1, s);
-            return launch_shape<T, PLASMA, false, true, 1>(a, 1, s);
+            if constexpr (sizeof(T) == 4) return launch_shape<T, PLASMA, false, true, 1>(a, 1, s);
+            return cudaErrorInvalidValue;
         }
     }
     if (fl.shape == 0) return launch_shape<T, PLASMA, FRAME, false, 0>(a, fl.grid, s);
@@ -863,6 +1261,8 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
     a.hlist = fl.hlist;
     a.cnt = fl.cnt;
     a.crec = fl.crec;
+    a.erec = fl.erec;
+    a.ecnt = fl.ecnt;
     a.gtab = m.gtab;
     a.one_grp = m.n_src > 0 && m.n_grp == 1;
     a.n_t = (int)m.n_t;
@@ -887,6 +1287,7 @@ cudaError_t launch_flow_t(const FlowDev& fl, const DevMesh& m, void* Uif, int n_
 
 // Most shared memory of a CTA, a current's coefficients counted in (it may be set later).
 size_t smem_of(bool f64, int sh, int cells) {
+    if (f64 && cells == 0) return sh == 0 ? EdgeFlow<0, true>::SMEM : EdgeFlow<1, true>::SMEM;
     if (f64) return sh == 0 ? flow_smem<double, true, 0>(cells) : flow_smem<double, true, 1>(cells);
     return sh == 0   ? flow_smem<float, true, 0>(cells)
            : sh == 1 ? flow_smem<float, true, 1>(cells)
@@ -900,8 +1301,9 @@ bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
     fl = FlowDev();
     if (n_t < 1 || sms < 1 || n_t + n_fc >= INT32_MAX / 2) return false;
     // one CTA holds up to 2,048 triangles: without an exchange its step takes 0.3 to 0.6 us, less
-    // than the 0.9 us of one
-    if (n_fc == 0 && n_t <= 2048) {
+    // than the 0.9 us of one.  In FP64 one SM's pipe takes 2 to 3.3 us for 1,000 triangles, an exchange
+    // 1.2 to 1.4
+    if (n_fc == 0 && n_t <= (f64 ? 512 : 2048)) {
         fl.grid = 1;
         fl.shape = n_t <= 1024 ? 0 : 1;
         fl.per = (int)n_t;
@@ -922,6 +1324,11 @@ bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
     fl.halo = f64 ? kShapes[fl.shape].halo64 : kShapes[fl.shape].halo32;
     fl.slot_words = fl.grid > 1 ? ((int64_t)fl.grid * fl.cap + n_fc) * (f64 ? 2 : 1) : 0;
     fl.sent_bytes = (size_t)fl.grid * fl.cap * (f64 ? sizeof(SrcEntry<double>) : sizeof(SrcEntry<float>));
+    if (f64 && n_fc == 0) {
+        if ((int64_t)fl.grid * fl.cap > 1 << 20) return false;   // places in an edge record
+        fl.edges = kEdgeShapes[fl.shape].edges;
+        fl.sent_bytes = (size_t)fl.grid * fl.edges * sizeof(EdgeSrc);
+    }
     return true;
 }
 
@@ -958,9 +1365,14 @@ cudaError_t launch_flow_plan(const FlowDev& fl, const DevMesh& m, cudaStream_t s
     if (m.frame) a.f = *m.frame;
     a.fper = fl.fper;
     a.place = fl.place;
+    a.erec = fl.erec;
+    a.ecnt = fl.ecnt;
+    a.eslot = fl.eslot;
+    a.edges = fl.edges;
     if (m.precision == UE_PREC_FP64) {
         k_flow_order<double><<<fl.grid, 1024, 0, s>>>(a);
-        k_flow_plan<double><<<fl.grid, 1024, 0, s>>>(a);
+        if (fl.edges > 0) k_flow_edges<<<fl.grid, 1024, 0, s>>>(a);
+        else k_flow_plan<double><<<fl.grid, 1024, 0, s>>>(a);
     } else {
         k_flow_order<float><<<fl.grid, 1024, 0, s>>>(a);
         k_flow_plan<float><<<fl.grid, 1024, 0, s>>>(a);

@@ -1054,7 +1054,9 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
             ok = ok && alloc_into(m, fl.ctl, 4, 4, s) && alloc_into(m, fl.place, nt, 4, s) &&
                  alloc_into(m, fl.rec, slots, 16, s) &&
                  alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
-                 (fl.grid == 1 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
+                 (fl.grid == 1 || fl.edges > 0 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
+                 (fl.edges == 0 || (alloc_into(m, fl.erec, (size_t)fl.grid * fl.edges, 8, s) &&
+                                    alloc_into(m, fl.ecnt, fl.grid, 8, s) && alloc_into(m, fl.eslot, nei + 1, 4, s))) &&
                  (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
                  (m->watchdog_every <= 0 || alloc_into(m, fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8, s)) &&
                  (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));

@@ -102,6 +102,28 @@ def test_resident_fp64_with_two_slots(ue):
     _same(_run(ue, xy, tris, h, 33, 32, **kw), _run(ue, xy, tris, h, 33, -1, **kw))
 
 
+@pytest.mark.parametrize("n_t,shuffle", [(155_648, False), (155_649, False), (311_296, False), (7_000, True),
+                                         (60_000, True), (280_000, True)])
+@pytest.mark.parametrize("plasma", [False, True])
+def test_resident_fp64_edges_apart(ue, n_t, shuffle, plasma):
+    """FP64 at the edges of its shapes, and with nearly every edge between two CTAs (up to a full list of
+    remote neighbours, and past it, where the launches stay): fields bit for bit, a watchdog's energy."""
+    xy, tris, h = _lattice(n_t, 5, shuffle=shuffle)
+    kw = dict(plasma=plasma, precision=ue.UE_PREC_FP64, load=dict(reorder=ue.UE_REORDER_NONE) if shuffle else None)
+    a = _run(ue, xy, tris, h, 33, 32, watchdog_every=16, **kw)
+    b = _run(ue, xy, tris, h, 33, -1, **kw)
+    for x, y in zip(a[:-1], b[:-1]):
+        assert np.array_equal(x, y)
+    m = ue.Mesh(xy, tris, **(kw["load"] or {}))
+    m.geometry_build(dt_mode=ue.UE_DT_GIVEN, dt=0.1 * h, graph_chunk=32, watchdog_every=32, precision=ue.UE_PREC_FP64)
+    m.write_fields(B=np.cos(np.arange(m.n_tris)))
+    m.step_n(64)
+    W = m.check()[1]
+    # the same positive terms in another order
+    assert abs(W / m.energy() - 1) <= 4 * n_t * 1.2e-16
+    m.close()
+
+
 @pytest.mark.parametrize("n_t", [7_000, 400_000])
 def test_resident_with_scattered_neighbours(ue, n_t):
     """The caller's order kept and random: nearly every neighbour is in another CTA; the larger

@@ -334,13 +334,31 @@ cudaError_t launch_fields_in(const DevMesh& m, const double* E_caller, const dou
 cudaError_t launch_fields_out(const DevMesh& m, double* E_caller, double* B_caller,
                               double* J_caller, const int64_t* edge_caller,
                               const int64_t* perm_tri, const double* relen, cudaStream_t s);
+// The watchdog words (energy, reference, growth limit, flag) and the error words reset: values
+// travel as kernel arguments, so no host buffer outlives the call.
+struct Rearm {
+    double* wd;
+    double growth;
+    int* p_err;
+    unsigned *tb_err, *flow_err;
+};
+__device__ __forceinline__ void rearm_words(const Rearm& r) {
+    r.wd[0] = 0.0;
+    r.wd[1] = 0.0;
+    r.wd[2] = r.growth;
+    r.wd[3] = 0.0;
+    if (r.p_err) *r.p_err = 0;
+    if (r.tb_err) *r.tb_err = 0u;
+    if (r.flow_err) *r.flow_err = 0u;
+}
+cudaError_t launch_rearm(const Rearm& r, cudaStream_t s);
 // The same transfers in caller order, with the caller's arrays (double, or float when f32) in
 // pinned host memory at their mapped device addresses, or in device memory: k_of[n_e] = stored
 // interior edge of each caller edge or -1, inv[n_t] = stored triangle of each caller triangle.
-// E (and J) are written on every caller edge.
+// E (and J) are written on every caller edge.  A write re-arms the watchdog in the same launch.
 cudaError_t launch_fields_in_caller(const DevMesh& m, const void* E_caller, const void* B_caller,
                                     const void* J_caller, bool f32, const int32_t* k_of, const int32_t* inv,
-                                    const double* elen, int64_t n_e, cudaStream_t s);
+                                    const double* elen, int64_t n_e, const Rearm& r, cudaStream_t s);
 cudaError_t launch_fields_out_caller(const DevMesh& m, void* E_caller, void* B_caller, void* J_caller, bool f32,
                                      const int32_t* k_of, const int32_t* inv, const double* relen, int64_t n_e,
                                      cudaStream_t s);

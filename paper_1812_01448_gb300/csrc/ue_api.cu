@@ -1154,30 +1154,15 @@ bool direct_transfer(const ue_mesh* m, const void* E, const void* B, const void*
     return (!E || dE) && (!B || dB) && (!j || dj) && (E || B || j);
 }
 
-// The watchdog words (energy, reference, growth limit, flag) and the error words reset in one
-// launch: values travel as kernel arguments, so no host buffer outlives the call.
-__global__ void k_rearm(double* wd, double growth, int* p_err, unsigned* tb_err, unsigned* flow_err) {
-    if (threadIdx.x != 0) return;
-    wd[0] = 0.0;
-    wd[1] = 0.0;
-    wd[2] = growth;
-    wd[3] = 0.0;
-    if (p_err) *p_err = 0;
-    if (tb_err) *tb_err = 0u;
-    if (flow_err) *flow_err = 0u;
-}
-
 __global__ void k_put_step(long long* step, long long v) {
     if (threadIdx.x == 0) *step = v;
 }
 
-// Re-arm the watchdog and the error words after new fields are written.
-int rearm(ue_mesh* m, cudaStream_t s) {
+// What re-arms the watchdog and the error words after new fields are written.
+ue::Rearm rearm(ue_mesh* m) {
     m->since_check = 0;
     unsigned* tb_err = (m->variant == UE_VARIANT_BLOCKED && m->tb.done) ? m->tb.done + 1 : nullptr;
-    k_rearm<<<1, 32, 0, s>>>(m->wd, m->watchdog_growth, m->p_err, tb_err, m->flow.ctl ? m->flow.ctl + 2 : nullptr);
-    UE_CUDA(cudaGetLastError());
-    return UE_OK;
+    return {m->wd, m->watchdog_growth, m->p_err, tb_err, m->flow.ctl ? m->flow.ctl + 2 : nullptr};
 }
 
 // A step counter set by ue_set_step reaches the device in the stream of the next call that
@@ -1282,9 +1267,7 @@ int fields_f32(ue_mesh* m, float* E, float* B, float* j, bool write, cudaStream_
         m->direct_fields += (E ? 1 : 0) + (B ? 1 : 0) + (j ? 1 : 0);
     }
     if (write) {
-        UE_CUDA(ue::launch_fields_in_caller(m->dm, dE, dB, dj, true, m->d_kof, m->d_inv, m->d_elen, h.n_edges, s));
-        const int rc = rearm(m, s);
-        if (rc != UE_OK) return rc;
+        UE_CUDA(ue::launch_fields_in_caller(m->dm, dE, dB, dj, true, m->d_kof, m->d_inv, m->d_elen, h.n_edges, rearm(m), s));
     } else {
         UE_CUDA(ue::launch_fields_out_caller(m->dm, const_cast<void*>(dE), const_cast<void*>(dB),
                                              const_cast<void*>(dj), true, m->d_kof, m->d_inv, m->d_relen,
@@ -1915,7 +1898,7 @@ int ue_write_fields(ue_mesh* m, const double* E, const double* B, const double* 
         // pinned host arrays: the kernels read them in place
         const int rc = ensure_caller_maps(m, s);
         if (rc != UE_OK) return rc;
-        UE_CUDA(ue::launch_fields_in_caller(m->dm, dE, dB, dj, false, m->d_kof, m->d_inv, m->d_elen, h.n_edges, s));
+        UE_CUDA(ue::launch_fields_in_caller(m->dm, dE, dB, dj, false, m->d_kof, m->d_inv, m->d_elen, h.n_edges, rearm(m), s));
         m->direct_fields += (E ? 1 : 0) + (B ? 1 : 0) + (j ? 1 : 0);
     } else {
         if (E) UE_CUDA(cudaMemcpyAsync(m->d_Ec, E, 8 * h.n_edges, cudaMemcpyHostToDevice, s));
@@ -1923,6 +1906,7 @@ int ue_write_fields(ue_mesh* m, const double* E, const double* B, const double* 
         if (j) UE_CUDA(cudaMemcpyAsync(m->d_Jc, j, 8 * h.n_edges, cudaMemcpyHostToDevice, s));
         UE_CUDA(ue::launch_fields_in(m->dm, E ? m->d_Ec : nullptr, B ? m->d_Bc : nullptr,
                                      j ? m->d_Jc : nullptr, m->d_ecaller, m->d_perm, m->d_elen, s));
+        UE_CUDA(ue::launch_rearm(rearm(m), s));
     }
     if (m->dm.frame) {
         const ue::FrameDev& f = m->fd;
@@ -1935,10 +1919,6 @@ int ue_write_fields(ue_mesh* m, const double* E, const double* B, const double* 
         UE_CUDA(cudaMemsetAsync(f.V, 0, esz * (f.NX + 1) * f.NY, s));
         UE_CUDA(cudaMemsetAsync(f.Bx, 0, esz * f.n_fc, s));
         UE_CUDA(cudaMemsetAsync(f.By, 0, esz * f.n_fc, s));
-    }
-    {
-        const int rc = rearm(m, s);
-        if (rc != UE_OK) return rc;
     }
     UE_CUDA(cudaStreamSynchronize(s));
     return UE_OK;

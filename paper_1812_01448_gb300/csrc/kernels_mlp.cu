@@ -364,6 +364,245 @@ __global__ void __launch_bounds__(NT, 1) k_mlp_fwd_bf16(const float* __restrict_
     }
 }
 
+// The same forward with layer 2 on tcgen05 (kind::f16, FP32 accumulators in tensor memory), for large
+// sets of rows.  kTcGroups warp groups of 128 threads per SM each take 128 rows at a time:
+// - the rows arrive by bulk copies, kTcStages tiles ahead;
+// - layer 1 stays on mma.sync: its sums, which are rounded to BF16, keep their bits.  A C fragment,
+//   ReLU'd and rounded, has the layout of tcgen05.st.16x128b: it goes straight to tensor memory as
+//   layer 2's A operand;
+// - one thread issues b2 as a product of its own (three BF16 parts that add up to it, times ones) and the
+//   four K = 16 steps of 128 x 64 x 64 into the group's 64 accumulator columns;
+// - every thread reads its row's 64 sums back, relu and w3.
+// While one group waits for its products the others compute.  (With h1 through shared memory its
+// stores, the operand's reads and the other accesses kept the shared memory 55% busy: 132 us, 113 with
+// eight groups.)  5.07M rows: 107 us; the copy time of their 264 MB is 39.  k_mlp_fwd_bf16, whose 40
+// mma.sync per 16 rows bound it, 177 us.  Three or five groups, and layer 1 of the next tile computed
+// while the products run, change nothing (112, 113, 107): neither latency nor issue slots (44%) but
+// the pipes that the 16 mma.sync per 32 rows, ReLU and rounding share (ALU 50%, tensor 37%) are what is left.
+// Waits are bounded: when one runs out the group leaves its remaining scores NaN.
+constexpr int kTcGroups = 4, kTcStages = 3, kTcRows = 128;
+constexpr uint32_t kTcTile = kTcRows * kD * 4;   // bytes of a full input tile
+static_assert(kTcTile % 16 == 0);
+// D = FP32, A = B = BF16, B K-major, N = 64, M = 128
+constexpr uint32_t kTcInstr = (1u << 4) | (1u << 7) | (1u << 10) | ((64u / 8) << 17) | ((128u / 16) << 24);
+
+struct TcSmem {
+    unsigned char w2[kH * 128];              // [n][k], swizzled
+    unsigned char bias[kH * 128];            // [n][3 parts of b2, 0 ...], swizzled (16 columns are read)
+    float x[kTcGroups][kTcStages][kTcRows * kD];
+    float b1[kH], w3[kH];
+    uint64_t full[kTcGroups][kTcStages], done[kTcGroups];
+    uint32_t tmem;
+};
+
+// K-major operand, 128-byte swizzle, groups of 8 rows 1024 bytes apart
+__device__ __forceinline__ uint64_t tc_desc(const void* p) {
+    return (uint64_t)((smem_addr(p) & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t acc) {
+    asm volatile("{.reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;}" ::"r"(d),
+                 "r"(a), "l"(b), "r"(kTcInstr), "r"(acc)
+                 : "memory");
+}
+// 16 rows x 64 BF16 as pairs: c[2 j] = row lane / 4, columns 8 j + 2 (lane % 4) and the next, c[2 j + 1] the
+// same of row lane / 4 + 8
+__device__ __forceinline__ void tc_store_frag(uint32_t t, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(t),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+// 16 of a row's sums; the wait in the same statement, so that the registers are not read before it
+__device__ __forceinline__ void tc_load16(uint32_t t, float (&v)[16]) {
+    uint32_t* r = reinterpret_cast<uint32_t*>(v);
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(t)
+        : "memory");
+}
+// two products at once: acc += a * b on both halves
+__device__ __forceinline__ void fma2(unsigned long long& acc, float a0, float a1, unsigned long long b) {
+    asm("{.reg .b64 a; mov.b64 a, {%1, %2}; fma.rn.f32x2 %0, a, %3, %0;}" : "+l"(acc) : "f"(a0), "f"(a1), "l"(b));
+}
+// relu of two BF16 values (of a pair with a NaN, 0 for it, as fmaxf)
+__device__ __forceinline__ uint32_t relu2(uint32_t v) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0u));
+    return r;
+}
+// element (row, k) of a swizzled operand of 64 columns
+__device__ __forceinline__ __nv_bfloat16* tc_at(unsigned char* p, int row, int k) {
+    return reinterpret_cast<__nv_bfloat16*>(p + row * 128 + ((((k >> 3) ^ row) & 7) << 4) + 2 * (k & 7));
+}
+
+__global__ void __launch_bounds__(128 * kTcGroups, 1) k_mlp_fwd_tc(const float* __restrict__ P, const float* __restrict__ X,
+                                                                  int64_t n, float* __restrict__ z) {
+    constexpr int G = kTcGroups, ST = kTcStages, NT = 128 * G;
+    // tensor memory columns: the accumulators, h1 (two values per column) and the ones
+    constexpr uint32_t kAcc = 0, kH1 = 64 * G, kOnes = 96 * G, kCols = 512;
+    static_assert(kOnes + 8 <= kCols);
+    extern __shared__ unsigned char tc_raw[];
+    TcSmem& S = *reinterpret_cast<TcSmem*>(tc_raw + ((1024u - (smem_addr(tc_raw) & 1023u)) & 1023u));
+    const int tid = threadIdx.x, wg = tid >> 7, wt = tid & 127, warp = wt >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int64_t tiles = (n + kTcRows - 1) / kTcRows, stride = (int64_t)gridDim.x * G;
+    const int64_t tile0 = (int64_t)blockIdx.x * G + wg;
+    auto fetch = [&](int64_t tile, int st) {   // one thread
+        const uint32_t rows = (uint32_t)min((int64_t)kTcRows, n - tile * kTcRows);
+        bulk_g2s(S.x[wg][st], X + tile * kTcRows * kD, rows * kD * 4, &S.full[wg][st]);
+    };
+    if (wt == 0) {
+        for (int i = 0; i < ST; ++i) mbar_init(&S.full[wg][i], 1);
+        mbar_init(&S.done[wg], 1);
+        fence_mbar_init();
+        for (int i = 0; i < ST; ++i)
+            if (tile0 + i * stride < tiles) fetch(tile0 + i * stride, i);
+    }
+    __syncwarp();
+    if (tid < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&S.tmem)), "r"(kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    for (int i = tid; i < kH * kH; i += NT) *tc_at(S.w2, i >> 6, i & 63) = __float2bfloat16_rn(__ldg(P + kOffW2 + i));
+    for (int i = tid; i < kH * 16; i += NT) {
+        const int c = i >> 4, k = i & 15;
+        const float b = __ldg(P + kOffB2 + c);
+        const __nv_bfloat16 hi = __float2bfloat16_rz(b);
+        __nv_bfloat16 v = k == 0 ? hi : __float2bfloat16_rn(0.f);
+        if (k == 1 || k == 2) {
+            const float r = isfinite(b) ? b - __bfloat162float(hi) : 0.f;
+            const __nv_bfloat16 mid = __float2bfloat16_rz(r);
+            v = k == 1 ? mid : __float2bfloat16_rn(r - __bfloat162float(mid));
+        }
+        *tc_at(S.bias, c, k) = v;
+    }
+    if (tid < kH) {
+        S.b1[tid] = __ldg(P + kOffB1 + tid);
+        S.w3[tid] = __ldg(P + kOffW3 + tid);
+    }
+    const float b3 = __ldg(P + kOffB3);
+    // B fragments of layer 1, as in k_mlp_fwd_bf16
+    uint32_t w1[8][2];
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        const float* r1 = P + kOffW1 + (8 * nt + g) * kD;
+        w1[nt][0] = pack_bf16(__ldg(r1 + 2 * t), __ldg(r1 + 2 * t + 1));
+        w1[nt][1] = t < 2 ? pack_bf16(__ldg(r1 + 2 * t + 8), __ldg(r1 + 2 * t + 9)) : 0u;
+    }
+    fence_proxy_async();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm = *(volatile uint32_t*)&S.tmem, lanes = (uint32_t)(32 * warp) << 16;
+    if (wg == 0) {   // rows {1, 1, 1, 0 ...}
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %3, %3, %3, %3, %3};" ::"r"(tm + lanes + kOnes),
+                     "r"(0x3F803F80u), "r"(0x00003F80u), "r"(0u)
+                     : "memory");
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t acc_t = tm + kAcc + 64u * (uint32_t)wg, h1_t = tm + kH1 + 32u * (uint32_t)wg;
+    const uint64_t db = tc_desc(S.w2), dbias = tc_desc(S.bias);
+    bool ok = true;
+    uint32_t phase = 0, par = 0;
+    int st = 0;
+    int64_t tile = tile0;
+    for (; tile < tiles; tile += stride) {
+        uint32_t c[2][16];
+        if (!mbar_wait(&S.full[wg][st], par)) ok = false;
+        const float* xs = S.x[wg][st] + (32 * warp + g) * kD + 2 * t;
+        if (++st == ST) {
+            st = 0;
+            par ^= 1u;
+        }
+        uint32_t a[2][4];
+#pragma unroll
+        for (int sub = 0; sub < 2; ++sub) {
+            auto two = [&](int off) {
+                const float2 v = *reinterpret_cast<const float2*>(xs + 16 * sub * kD + off);
+                return pack_bf16(v.x, v.y);
+            };
+            a[sub][0] = two(0);
+            a[sub][1] = two(8 * kD);
+            a[sub][2] = t < 2 ? two(8) : 0u;
+            a[sub][3] = t < 2 ? two(8 * kD + 8) : 0u;
+        }
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            const float2 bb = *reinterpret_cast<const float2*>(S.b1 + nt * 8 + 2 * t);
+#pragma unroll
+            for (int sub = 0; sub < 2; ++sub) {
+                float v[4] = {bb.x, bb.y, bb.x, bb.y};
+                mma_bf16(v, a[sub][0], a[sub][1], a[sub][2], a[sub][3], w1[nt][0], w1[nt][1]);
+                c[sub][2 * nt] = relu2(pack_bf16(v[0], v[1]));
+                c[sub][2 * nt + 1] = relu2(pack_bf16(v[2], v[3]));
+            }
+        }
+        __syncwarp();
+        tc_store_frag(h1_t + lanes, c[0]);
+        tc_store_frag(h1_t + lanes + (16u << 16), c[1]);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        // the group's threads have read the inputs and the sums of the tile before, and written h1
+        uint32_t all;
+        asm volatile("{.reg .pred p, q; setp.ne.b32 p, %1, 0; bar.red.and.pred q, %2, 128, p; selp.u32 %0, 1, 0, q;}"
+                     : "=r"(all)
+                     : "r"(ok ? 1u : 0u), "r"(wg + 1)
+                     : "memory");
+        if (!all) {
+            ok = false;
+            break;
+        }
+        if (wt == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            tc_mma(acc_t, tm + kOnes, dbias, 0u);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tc_mma(acc_t, h1_t + 8u * k, db + 2u * k, 1u);   // 16 columns of B: 32 bytes
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(&S.done[wg])) : "memory");
+            if (tile + ST * stride < tiles) fetch(tile + ST * stride, st == 0 ? ST - 1 : st - 1);
+        }
+        __syncwarp();
+        if (!mbar_wait(&S.done[wg], phase)) ok = false;
+        phase ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        __syncwarp();
+        unsigned long long acc[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+        for (int quart = 0; quart < 4; ++quart) {
+            float v[16];
+            tc_load16(acc_t + lanes + 16u * quart, v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(S.w3 + 16 * quart + 4 * i);
+                fma2(acc[(2 * i) & 3], fmaxf(v[4 * i], 0.f), fmaxf(v[4 * i + 1], 0.f), w.x);
+                fma2(acc[(2 * i + 1) & 3], fmaxf(v[4 * i + 2], 0.f), fmaxf(v[4 * i + 3], 0.f), w.y);
+            }
+        }
+        auto sum = [](unsigned long long q) { return __uint_as_float((uint32_t)q) + __uint_as_float((uint32_t)(q >> 32)); };
+        const float s = (sum(acc[0]) + sum(acc[1])) + (sum(acc[2]) + sum(acc[3]));
+        const int64_t row = tile * kTcRows + wt;
+        if (row < n) z[row] = ok ? s + b3 : __int_as_float(0x7fffffff);
+    }
+    if (!ok) {   // a wait ran out: no scores, and the copies in flight end before their memory is given up
+        for (int64_t k = tile; k < tiles; k += stride)
+            if (k * kTcRows + wt < n) z[k * kTcRows + wt] = __int_as_float(0x7fffffff);
+        if (wt == 0)
+            for (int i = 0; i < ST; ++i) {
+                mbar_wait(&S.full[wg][i], 0);
+                mbar_wait(&S.full[wg][i], 1);
+            }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(kCols) : "memory");
+}
+
 // Fused inference for one mesh, one launch: features -> BF16 MLP -> score z_j + base_j, the
 // per-block maxima of the score (with its row), of K_jj and of the Gershgorin row bound; the
 // last block to finish (counter in the work space) reduces the block partials and computes the
@@ -938,6 +1177,16 @@ cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf
         // start is shorter, else 12
         const int64_t tiles = (n + 15) / 16;
         auto grid = [&](int nt) { return (unsigned)std::min<int64_t>((tiles + nt / 32 - 1) / (nt / 32), 152); };
+        // From 32,768 rows of 16-byte aligned inputs layer 2 goes to tcgen05: 20k rows 9.9 us either way,
+        // 40k 10.1 (10.9), 100k 10.5 (13.2), 1M 27 (45).
+        if (n >= 32768 && ((uintptr_t)X & 15u) == 0) {
+            const size_t smem = sizeof(TcSmem) + 1024;   // aligned to 1024 inside
+            const cudaError_t e = cudaFuncSetAttribute(k_mlp_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            const int64_t blocks = (n + kTcRows * kTcGroups - 1) / (kTcRows * kTcGroups);
+            k_mlp_fwd_tc<<<(unsigned)std::min<int64_t>(blocks, 152), 128 * kTcGroups, smem, s>>>(P, X, n, z);
+            return cudaGetLastError();
+        }
         if (tiles < 152 * 8 * 32) k_mlp_fwd_bf16<256><<<grid(256), 256, 0, s>>>(P, X, n, z);
         else k_mlp_fwd_bf16<384><<<grid(384), 384, 0, s>>>(P, X, n, z);
     } else {

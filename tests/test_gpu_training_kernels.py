@@ -49,6 +49,30 @@ def test_forward(lib, n, shift):
     assert z[n] == 7.0
 
 
+@pytest.mark.parametrize("n", [32_767, 32_768, 32_895, 152 * 512 - 1, 152 * 512 + 1, 4 * 152 * 512 + 129])
+def test_forward_of_many_rows(lib, n):
+    """Around the rows from which layer 2 runs on tcgen05, and around its tiles: against torch, and
+    against the same rows at an address that keeps the other kernel.  1e-5: both sum 64 products in FP32
+    (a few 2^-24 of terms below 1) from the same BF16 h1.  Rows with a NaN or an infinity agree too."""
+    torch, ue, p = lib
+    flat = torch.randn(n * 12, generator=torch.Generator().manual_seed(n))
+    X = flat.reshape(n, 12)
+    X[7, 3], X[130, 0], X[131, 5], X[n - 1, 11] = float("nan"), float("inf"), -float("inf"), float("nan")
+    off = torch.empty(n * 12 + 1, device="cuda")
+    off[1:] = flat.cuda()
+    z, y = torch.full((n + 1,), 7.0, device="cuda"), torch.full((n + 1,), 7.0, device="cuda")
+    ue.mlp_forward(p.cuda(), X.cuda(), z, bf16=True)
+    ue.mlp_forward(p.cuda(), off[1:].reshape(n, 12), y, bf16=True)
+    assert z[n] == 7.0 and y[n] == 7.0
+    assert torch.equal(z.isnan(), y.isnan()) and torch.equal(z.isinf(), y.isinf())
+    f = z.isfinite()
+    assert f.sum() >= n - 4
+    assert (z[f] - y[f]).abs().max() < 1e-5
+    ok = torch.isfinite(X).all(1)
+    err = (z[:n].cpu().double() - _layers(torch, p, X, True)[-1])[ok].abs()
+    assert err.max() < 4e-3 and err.median() < 2e-6
+
+
 @pytest.mark.parametrize("sizes", [[1], [0, 3, 0], [4095, 4096, 4097, 1], [512, 511, 513, 20_000]])
 def test_segment_argmax(lib, sizes):
     torch, ue, _ = lib

@@ -14,7 +14,7 @@
 // shared memory, values between CTAs through tagged words (exchange.cuh); larger ones launch once per
 // product.  Measured for 200 products (was: two launches per product through edge values, each
 // normalised by a reduction in the last block):
-//   10k triangles 2.70 ms -> 0.38, 234k 5.38 ms -> 0.68 (3.4 us per product), 1.9M 23.5 ms -> 9.6.
+//   10k triangles 2.70 ms -> 0.27, 234k 5.38 ms -> 0.62 (3.1 us per product), 1.9M 23.5 ms -> 9.6.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -179,7 +179,11 @@ __global__ void __launch_bounds__(kThreads) k_pw_step(const int4* __restrict__ n
 
 // kSeg products (or the rest) in one cooperative launch.  CTA c keeps triangles [c per, (c+1) per);
 // a thread holds slots tid + i * NT; the iterate and, with several slots, the records' weights sit
-// in shared memory.  Layout and exchange as in kernels_flow.cu.
+// in shared memory.  Exchange as in kernels_flow.cu: with several slots the CTA polls its remote
+// neighbours into shared memory and a barrier follows; with one, whose product is all latency, each
+// thread polls those of its triangle itself, a store, a poll and four FMAs (10k triangles: 1.94 us
+// per product with the list and its barrier, now 1.33; with two slots a thread's polls hold up its other
+// slot: 234k triangles 3.1 us, 3.5 that way, and the same with the triangles that publish in front).
 struct PowerArgs {
     const int4* nb;
     const double2* w;
@@ -194,18 +198,23 @@ struct PowerArgs {
 };
 
 constexpr unsigned kPwPublish = 1u << 16;
-constexpr unsigned kPwFar = 1u << 17;   // 3 bits: neighbour polled by this thread (the list is full)
+constexpr unsigned kPwFar = 1u << 17;   // 3 bits: a remote neighbour that the list had no room for
+__device__ __forceinline__ int far_of(const int4* nb, int j, int q) {
+    const int4 r = __ldg(nb + j);
+    return q == 0 ? r.x : q == 1 ? r.y : r.z;
+}
 
 template <int TS>
 __host__ __device__ constexpr size_t power_smem(int cap, int hcap) {
-    return (TS > 1 ? 32 * (size_t)cap : 0) + 16 * ((size_t)cap + hcap) + 4 * (size_t)hcap;
+    return (TS > 1 ? 32 * (size_t)cap : 0) + 16 * ((size_t)cap + (TS > 1 ? hcap : 0)) + 4 * (size_t)hcap;
 }
 
 template <int NT, int TS, bool SOLO>
 __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
+    constexpr bool OWN = TS == 1;   // threads poll for themselves
     __shared__ int s_hcnt;
-    const int tid = threadIdx.x, nth = TS > 1 ? NT : (int)blockDim.x, cap = TS * nth, bcap = cap + a.hcap;
+    const int tid = threadIdx.x, nth = TS > 1 ? NT : (int)blockDim.x, cap = TS * nth, bcap = cap + (OWN ? 0 : a.hcap);
     double2* W = reinterpret_cast<double2*>(smraw);
     double* Vb = reinterpret_cast<double*>(W + (TS > 1 ? 2 * cap : 0));
     int* hlist = reinterpret_cast<int*>(Vb + 2 * bcap);
@@ -223,7 +232,8 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
         v[i] = old[i] = 0.0;
         n01[i] = n2f[i] = 0;
         if (l >= nloc) continue;
-        const int4 r = __ldg(a.nb + j0 + l);
+        const int j = j0 + l;
+        const int4 r = __ldg(a.nb + j);
         const int o[3] = {r.x, r.y, r.z};
         unsigned off[3], f = 0;
 #pragma unroll
@@ -235,7 +245,7 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
                 f |= kPwPublish;
                 if (pos < a.hcap) {
                     hlist[pos] = o[q];
-                    n = cap + pos;
+                    n = cap + pos;   // beyond the slots: the list's entry
                 } else {
                     f |= kPwFar << q;
                 }
@@ -244,7 +254,7 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
         }
         n01[i] = off[0] | (off[1] << 16);
         n2f[i] = off[2] | f;
-        const double2 x = __ldg(a.w + 2 * (int64_t)(j0 + l)), y = __ldg(a.w + 2 * (int64_t)(j0 + l) + 1);
+        const double2 x = __ldg(a.w + 2 * (int64_t)j), y = __ldg(a.w + 2 * (int64_t)j + 1);
         const double2 xs = make_double2(sc * x.x, sc * x.y), ys = make_double2(sc * y.x, sc * y.y);
         if constexpr (TS > 1) {
             W[2 * l] = xs;
@@ -253,9 +263,9 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
             wa[0] = xs;
             wb[0] = ys;
         }
-        v[i] = up * a.v[j0 + l];
+        v[i] = up * a.v[j];
         Vb[l] = v[i];
-        if (!SOLO && (f & kPwPublish)) slot_put(a.slots[0], j0 + l, a.tag0, v[i]);
+        if (!SOLO && (f & kPwPublish)) slot_put(a.slots[0], j, a.tag0, v[i]);
     }
     __syncthreads();
     const int hn = SOLO ? 0 : min(s_hcnt, a.hcap);
@@ -263,22 +273,22 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
     for (int s = 0; s < a.n_it; ++s) {
         const int p = s & 1;
         const unsigned tag = a.tag0 + (unsigned)s;
+        const unsigned long long* sl = p ? a.slots[1] : a.slots[0];
         double* Vp = Vb + (p ? bcap : 0);
         double* Vn = Vb + (p ? 0 : bcap);
-        if constexpr (SOLO) {
-            if (s > 0) __syncthreads();
-        } else {
+        const uint32_t va = smem_addr(Vp);
+        if constexpr (!SOLO && !OWN) {
             constexpr int kPoll = 2;
             for (int e0 = tid; e0 < hn; e0 += kPoll * nth) {
                 Word<double> x[kPoll];
 #pragma unroll
                 for (int u = 0; u < kPoll; ++u)
-                    if (e0 + u * nth < hn) x[u].load(p ? a.slots[1] : a.slots[0], hlist[e0 + u * nth]);
+                    if (e0 + u * nth < hn) x[u].load(sl, hlist[e0 + u * nth]);
 #pragma unroll
                 for (int u = 0; u < kPoll; ++u) {
                     const int e = e0 + u * nth;
                     if (e < hn) {
-                        if (!word_wait(x[u], p ? a.slots[1] : a.slots[0], hlist[e], tag)) ok = false;
+                        if (!word_wait(x[u], sl, hlist[e], tag)) ok = false;
                         Vp[cap + e] = x[u].value();
                     }
                 }
@@ -286,7 +296,6 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
             ok = __syncthreads_and(ok ? 1 : 0) != 0;
             if (!ok) break;
         }
-        const uint32_t va = smem_addr(Vp);
 #pragma unroll
         for (int i = 0; i < TS; ++i) {
             const int l = tid + i * nth;
@@ -299,36 +308,64 @@ __global__ void __launch_bounds__(NT, 1) k_pw_res(const __grid_constant__ PowerA
                 x = wa[0];
                 y = wb[0];
             }
-            double n[3] = {lds_val<double>(va + (n01[i] & 0xFFFFu)), lds_val<double>(va + (n01[i] >> 16)),
-                           lds_val<double>(va + (n2f[i] & 0xFFFFu))};
-            if (!SOLO && (n2f[i] & (7u * kPwFar))) {
-                const int4 r = __ldg(a.nb + j0 + l);
-                const int o[3] = {r.x, r.y, r.z};
+            double n[3];
+            if (OWN && !SOLO && (n2f[i] & kPwPublish)) {
+                const unsigned off[3] = {n01[i] & 0xFFFFu, n01[i] >> 16, n2f[i] & 0xFFFFu};
+                Word<double> t[3];
+                int at[3];
+#pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    if (!(n2f[i] & (kPwFar << q))) continue;
-                    Word<double> t;
-                    t.load(p ? a.slots[1] : a.slots[0], o[q]);
-                    if (!word_wait(t, p ? a.slots[1] : a.slots[0], o[q], tag)) ok = false;
-                    n[q] = t.value();
+                    at[q] = -1;
+                    if (off[q] >= 8u * (unsigned)cap) at[q] = hlist[(off[q] >> 3) - cap];
+                    else if (n2f[i] & (kPwFar << q)) at[q] = far_of(a.nb, j0 + l, q);
+                    if (at[q] >= 0) t[q].load(sl, at[q]);
+                    else n[q] = lds_val<double>(va + off[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if (at[q] >= 0) {
+                        if (!word_wait(t[q], sl, at[q], tag)) ok = false;
+                        n[q] = t[q].value();
+                    }
+            } else {
+                n[0] = lds_val<double>(va + (n01[i] & 0xFFFFu));
+                n[1] = lds_val<double>(va + (n01[i] >> 16));
+                n[2] = lds_val<double>(va + (n2f[i] & 0xFFFFu));
+                if (!OWN && !SOLO && (n2f[i] & (7u * kPwFar))) {
+                    for (int q = 0; q < 3; ++q) {
+                        if (!(n2f[i] & (kPwFar << q))) continue;
+                        const int o = far_of(a.nb, j0 + l, q);
+                        Word<double> t;
+                        t.load(sl, o);
+                        if (!word_wait(t, sl, o, tag)) ok = false;
+                        n[q] = t.value();
+                    }
                 }
             }
             old[i] = v[i];
             v[i] = fma(-y.x, n[2], fma(-x.y, n[1], fma(-x.x, n[0], y.y * v[i])));
-            Vn[l] = v[i];
             if (!SOLO && (n2f[i] & kPwPublish) && s + 1 < a.n_it) slot_put(p ? a.slots[0] : a.slots[1], j0 + l, tag + 1u, v[i]);
+            Vn[l] = v[i];
+        }
+        if constexpr (SOLO) {
+            __syncthreads();
+        } else if constexpr (OWN) {
+            ok = __syncthreads_and(ok ? 1 : 0) != 0;
+            if (!ok) break;
         }
     }
-    if (!SOLO) ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    if constexpr (!SOLO && !OWN) ok = __syncthreads_and(ok ? 1 : 0) != 0;
     if (!ok && tid == 0) atomicOr(&a.ctl->err, 1u);
     double num = 0.0, den = 0.0;
 #pragma unroll
     for (int i = 0; i < TS; ++i) {
         const int l = tid + i * nth;
         if (l >= nloc) break;
-        const double t = a.S[j0 + l] * old[i];
+        const int j = j0 + l;
+        const double t = a.S[j] * old[i];
         num += t * v[i];
         den += t * old[i];
-        if (!a.last) a.v[j0 + l] = v[i];
+        if (!a.last) a.v[j] = v[i];
     }
     __syncthreads();
     power_sums<NT>(num, den, a.part, a.ctl);
@@ -363,7 +400,7 @@ PowerPlan power_plan(int64_t n_t, int sms) {
     const int cap = ts * pl.threads;
     if (pl.grid > 1) {
         const size_t fixed = ts > 1 ? power_smem<2>(cap, 0) : power_smem<1>(cap, 0);
-        pl.hcap = (int)std::min(std::min<size_t>(3 * (size_t)cap, (kSmem - fixed) / 20), (size_t)(8192 - cap)) & ~3;
+        pl.hcap = (int)std::min(std::min<size_t>(3 * (size_t)cap, (kSmem - fixed) / (ts > 1 ? 20 : 4)), (size_t)(8192 - cap)) & ~3;
     }
     return pl;
 }

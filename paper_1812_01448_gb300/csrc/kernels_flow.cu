@@ -19,7 +19,9 @@
 // it carries the step they need.  Two words per triangle, alternating: a triangle writes step
 // s + 1 only after its neighbours' step s has arrived, hence after they have read its step s - 1,
 // which the word held.  Per step a CTA polls its remote neighbours once into shared memory, one
-// barrier, then every triangle reads its neighbours there.  All CTAs are resident (cooperative
+// barrier, then every triangle reads its neighbours there; with one triangle per thread, where a step
+// is all latency, each thread polls its own (90k triangles: 0.97 us per step with the list, now 0.84;
+// with several slots a thread's polls hold up its others).  All CTAs are resident (cooperative
 // launch) and every wait is bounded: one that runs out sets the error word and ends the launch.
 //
 // A plan made once (k_flow_plan, after the source is set) orders each CTA's triangles into slots:
@@ -27,10 +29,10 @@
 // with a source or a conductor's edge, so that few warps take that branch, then the others in
 // stored order; and it turns each triangle's neighbours into shared-memory addresses.
 //
-// What bounds it: one exchange through L2 (store, poll, barrier: about 0.9 us) up to some 1,000
+// What bounds it: one exchange through L2 (store, poll, barrier: about 0.8 us) up to some 1,000
 // triangles per SM, then the SM's issue slots (about 25 instructions per triangle; everything a slot
 // needs is at a compile-time offset from one register).  Measured per step on GB300, with a line
-// source, against graph replays of the two plain kernels: 90k triangles 0.97 us (6.2), 305k 1.20,
+// source, against graph replays of the two plain kernels: 90k triangles 0.84 us (6.2), 305k 1.20,
 // 1.2M 3.06 (9.3); one CTA alone 0.41 us on 1,040 triangles, 0.30 without a source (2.9).  Against
 // k_tbp (8 steps per launch, ring-ordered tiles) on 500k triangles 1.38 us (5.0), with a plasma
 // current 1.70 (k_tb 4.7), with a 16-cell PML frame 1.75 (10.0: the frame's tiles step by plain
@@ -412,12 +414,14 @@ struct Flow {
     static constexpr int NT = kShapes[SH].nt, TS = kShapes[SH].ts, CAP = NT * TS;
     static constexpr int STRIDE = kBuffer<T, SH> * (int)sizeof(T);   // bytes between the two buffers
     static constexpr bool CR = kCoefRegs<T, TS>;
+    static constexpr bool OWN = TS == 1 && !FRAME && !SOLO;   // threads poll for themselves
     static_assert(STRIDE + 2048 < 65536, "16-bit shared addresses");
 
     T V[TS][3], J[PLASMA ? TS : 1][3], b[TS];
     Vec4<T> Cr[CR ? TS : 1];
     T Pr[CR && PLASMA ? TS : 1][3];
     unsigned n01[TS], n2f[TS];
+    int at[OWN ? 3 : 1];    // places of the remote neighbours, -1: the neighbour is in this CTA
     // frame cell: sides X in bottom, top, left, right order, each with the cell's own
     // counter-clockwise sign, so that every one advances by (own B - neighbour's B)
     T X[FRAME ? 4 : 1], Bx, By;
@@ -448,7 +452,7 @@ struct Flow {
         nloc = max(0, min(a.per, a.n_t - j0));
         const int2 cn2 = __ldg(a.cnt + blockIdx.x);
         npub = SOLO ? 0 : cn2.x;
-        hn = SOLO ? 0 : cn2.y;
+        hn = SOLO || OWN ? 0 : cn2.y;
         tag0 = SOLO ? 0u : *(volatile unsigned*)a.ctl;
         ok = true;
         const size_t first = (size_t)blockIdx.x * CAP + tid;
@@ -464,6 +468,14 @@ struct Flow {
             const int4 r = __ldg(rec + l);
             n01[i] = (unsigned)r.y + (bufs | (bufs << 16));
             n2f[i] = (unsigned)r.z + bufs;
+            if constexpr (OWN) {
+                const unsigned off[3] = {(unsigned)r.y & 0xFFFFu, (unsigned)r.y >> 16, (unsigned)r.z & 0xFFFFu};
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int h = (int)(off[q] / (unsigned)sizeof(T)) - CAP;
+                    at[q] = h < 0 ? -1 : __ldg(a.hlist + (size_t)blockIdx.x * kHalo<T, SH> + h);
+                }
+            }
             const int4 t = __ldg(a.tri + r.x);
             const int code[3] = {t.x, t.y, t.z};
             T c[3], pb[3];
@@ -576,7 +588,7 @@ struct Flow {
         const unsigned tag = tag0 + (unsigned)s;
         if constexpr (SOLO) {
             if (s > 0) __syncthreads();
-        } else {
+        } else if constexpr (!OWN) {
             // the remote neighbours' B, a few polls in flight per thread
             constexpr int kPoll = 4;
             const unsigned long long* sl = a.slots[PB];
@@ -614,7 +626,8 @@ struct Flow {
             }
         }
         slots_from<PB, 0>(a, s, tag);
-        return true;
+        if constexpr (OWN) ok = __syncthreads_and(ok ? 1 : 0) != 0;
+        return ok;
     }
 
     template <int PB, int I>
@@ -629,8 +642,26 @@ struct Flow {
                 if constexpr (CR) c = Cr[I];
                 else c = lds4_at<2 * STRIDE + I * NT * (int)sizeof(Vec4<T>)>(bufs + threadIdx.x * (uint32_t)sizeof(Vec4<T>), T(0));
                 const T cq[3] = {c.x, c.y, c.z};
-                const T nv[3] = {lds_half<RD, false>(n01[I], T(0)), lds_half<RD, true>(n01[I], T(0)),
-                                 lds_half<RD, false>(n2f[I], T(0))};
+                T nv[3];
+                if (OWN && l < npub) {
+                    Word<T> w[3];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        if (at[q] >= 0) w[q].load(a.slots[PB], at[q]);
+                    if (at[0] < 0) nv[0] = lds_half<RD, false>(n01[I], T(0));
+                    if (at[1] < 0) nv[1] = lds_half<RD, true>(n01[I], T(0));
+                    if (at[2] < 0) nv[2] = lds_half<RD, false>(n2f[I], T(0));
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        if (at[q] >= 0) {
+                            if (!word_wait(w[q], a.slots[PB], at[q], tag)) ok = false;
+                            nv[q] = w[q].value();
+                        }
+                } else {
+                    nv[0] = lds_half<RD, false>(n01[I], T(0));
+                    nv[1] = lds_half<RD, true>(n01[I], T(0));
+                    nv[2] = lds_half<RD, false>(n2f[I], T(0));
+                }
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     const T uo = V[I][q];

@@ -1014,7 +1014,25 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
     const HostMesh& h = m->hm;
     const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;
     const int64_t nt = h.n_tris, nei = h.n_ei, nn = h.n_nodes, ne = h.n_edges;
+    m->flow = ue::FlowDev();
+    const int64_t W = m->fr.W, NX = m->fr.nx + 2 * W;
+    const int64_t n_fc = 2 * W * NX + 2 * W * m->fr.ny;
+    if (m->variant != UE_VARIANT_PERSISTENT && m->graph_chunk > 0 && m->tb_test_cta < 0) {
+        int dev = 0, sms = 0, coop = 0;
+        UE_CUDA(cudaGetDevice(&dev));
+        UE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        if (!coop || !ue::flow_shape(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) m->flow = ue::FlowDev();
+    }
+    const size_t flow_slots = (size_t)m->flow.grid * m->flow.cap;
     m->reserve = (size_t)(16 * nn + nt * (150 + 3 * (int64_t)esz) + nei * (64 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
+    // the resident step's arrays with them: on small meshes, whose slots are mostly spare, they are
+    // the larger part and took further chunks, 60 us each
+    if (m->flow.grid > 0)
+        m->reserve += 16 * flow_slots + m->flow.sent_bytes + 4 * (size_t)nt + 16 * (size_t)m->flow.slot_words +
+                      (size_t)m->flow.grid * (4 * (size_t)m->flow.halo + 16 + 8 * (size_t)m->flow.edges) +
+                      (m->flow.edges > 0 ? 4 * (size_t)nei : 0) + 16 * (size_t)n_fc +
+                      (m->watchdog_every > 0 ? 8 * (size_t)ue::kFlowChecks * (m->flow.grid + 1) : 0) + 12 * kAlign;
     bool ok = alloc_into(m, m->d_xy, 2 * nn, 8, s) && alloc_into(m, m->d_tri_nodes, 3 * nt, 4, s) &&
               alloc_into(m, m->d_edge_nodes, 2 * nei + 2, 4, s) &&
               alloc_into(m, m->d_edge_opp, 2 * nei + 2, 4, s) &&
@@ -1039,28 +1057,18 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
          alloc_into(m, dm.U, dm.n_ei_pad + (n_if + 3) / 4 * 4, esz, s) &&
          alloc_into(m, dm.B, dm.n_t_pad, esz, s) && alloc_into(m, dm.step, 1, 8, s);
     if (ok && m->precision == UE_PREC_FP64) ok = alloc_into(m, dm.cB, dm.n_t_pad, 8, s);
-    m->flow = ue::FlowDev();
-    if (m->variant != UE_VARIANT_PERSISTENT && m->graph_chunk > 0 && m->tb_test_cta < 0) {
-        int dev = 0, sms = 0, coop = 0;
-        UE_CUDA(cudaGetDevice(&dev));
-        UE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        const int64_t W = m->fr.W, NX = m->fr.nx + 2 * W;
-        const int64_t n_fc = 2 * W * NX + 2 * W * m->fr.ny;
-        if (coop && ue::flow_shape(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) {
-            ue::FlowDev& fl = m->flow;
-            fl.skip = m->flow_skip;
-            const size_t slots = (size_t)fl.grid * fl.cap;
-            ok = ok && alloc_into(m, fl.ctl, 4, 4, s) && alloc_into(m, fl.place, nt, 4, s) &&
-                 alloc_into(m, fl.rec, slots, 16, s) &&
-                 alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
-                 (fl.grid == 1 || fl.edges > 0 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
-                 (fl.edges == 0 || (alloc_into(m, fl.erec, (size_t)fl.grid * fl.edges, 8, s) &&
-                                    alloc_into(m, fl.ecnt, fl.grid, 8, s) && alloc_into(m, fl.eslot, nei + 1, 4, s))) &&
-                 (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
-                 (m->watchdog_every <= 0 || alloc_into(m, fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8, s)) &&
-                 (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));
-        }
+    if (m->flow.grid > 0) {
+        ue::FlowDev& fl = m->flow;
+        fl.skip = m->flow_skip;
+        ok = ok && alloc_into(m, fl.ctl, 4, 4, s) && alloc_into(m, fl.place, nt, 4, s) &&
+             alloc_into(m, fl.rec, flow_slots, 16, s) &&
+             alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
+             (fl.grid == 1 || fl.edges > 0 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
+             (fl.edges == 0 || (alloc_into(m, fl.erec, (size_t)fl.grid * fl.edges, 8, s) &&
+                                alloc_into(m, fl.ecnt, fl.grid, 8, s) && alloc_into(m, fl.eslot, nei + 1, 4, s))) &&
+             (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
+             (m->watchdog_every <= 0 || alloc_into(m, fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8, s)) &&
+             (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));
     }
     {
         int g = m->flow.grid > 0 ? ue::kFlowSteps : 64;

@@ -615,10 +615,8 @@ int bake_source(ue_mesh* m, cudaStream_t s) {
     int rc = bake_source_mesh(m, s);
     if (rc != UE_OK) return rc;
     if (m->flow.grid > 0) {
-        DevMesh v = m->dm;
-        v.frame = m->fr.W > 0 ? &m->fd : nullptr;
         unsigned over = 0;
-        UE_CUDA(ue::launch_flow_plan(m->flow, v, s));
+        UE_CUDA(ue::launch_flow_plan(m->flow, m->dm, s));
         UE_CUDA(cudaMemcpyAsync(&over, m->flow.ctl + 3, 4, cudaMemcpyDeviceToHost, s));
         UE_CUDA(cudaStreamSynchronize(s));
         if (over) m->flow.grid = 0;   // neighbours too scattered: this mesh keeps its launches
@@ -1199,10 +1197,9 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
         return UE_OK;
     }
     void* Uif = nullptr;
+    // the frame that was built: one attached or taken off since waits for the next build
     if (m->has_reg) Uif = (float*)m->reg.dm.U + m->reg.f.u_off;
-    else if (m->fr.W > 0) Uif = (char*)dm.U + (m->precision == UE_PREC_FP64 ? 8 : 4) * dm.n_ei_pad;
-    DevMesh v = dm;
-    v.frame = m->fr.W > 0 ? &m->fd : nullptr;
+    else if (dm.frame) Uif = (char*)dm.U + (m->precision == UE_PREC_FP64 ? 8 : 4) * dm.n_ei_pad;
     int64_t launched = 0;
     *used = true;
     for (int64_t left = n; left > 0;) {
@@ -1228,7 +1225,7 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
             }
         }
         UE_CUDA(ue::launch_gtab(dm, batch, s));
-        const cudaError_t e = ue::launch_flow(m->flow, v, Uif, batch, chk, s);
+        const cudaError_t e = ue::launch_flow(m->flow, dm, Uif, batch, chk, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && left == n) {
             cudaGetLastError();
             m->flow.grid = 0;

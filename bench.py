@@ -407,6 +407,7 @@ def run_native(args):
         torch.cuda.synchronize()
         barrier()
     launches = m.stats()["kernel_launches"] - launches0
+    resident = m.stats()["resident_launches"] > 0    # a mesh that fits the chip: not the variant's kernels
     ms_total = max_over_ranks(ev0.elapsed_time(ev1), dist)
     value = world * n_t * args.steps / (ms_total * 1e-3)
 
@@ -511,7 +512,8 @@ def run_native(args):
                        "n_edges": m.n_edges, "dt": dt, "rho": rho,
                        "variant": (f"blocked k={args.block_depth} {args.tiler} tiles<={args.tile_tris} "
                                 f"threads={args.tb_threads or 512} {args.tb_kernel} kernel" if blocked
-                                else args.variant) + f", CUDA graph chunk {graph_steps} steps",
+                                else args.variant) +
+                               (", resident launches" if resident else f", CUDA graph chunk {graph_steps} steps"),
                        "l2": (f"working set {step_bytes / 1e6:.0f} MB per step > {L2_BYTES / 1e6:.0f} MB L2; no flush"
                               if step_bytes > L2_BYTES else
                               f"working set {step_bytes / 1e6:.0f} MB per step < {L2_BYTES / 1e6:.0f} MB L2: "
@@ -566,7 +568,7 @@ def run_cavity(args):
     res = {}
     for name, load, opts in (("one CTA", dict(reorder=ue.UE_REORDER_GREEDY, tile_tris=4096),
                               dict(variant=ue.UE_VARIANT_BLOCKED, block_depth=8)),
-                             ("plain", dict(), dict(graph_chunk=32))):
+                             ("plain", dict(), dict(variant=ue.UE_VARIANT_PLAIN | ue.UE_VARIANT_NO_RESIDENT, graph_chunk=32))):
         m = ue.Mesh(ms.xy, ms.tris, **load)
         m.geometry_build(stream=stream, dt_mode=ue.UE_DT_GIVEN, dt=dt, **opts)
         m.write_fields(E=np.zeros(m.n_edges), B=B0, stream=stream)

@@ -71,6 +71,9 @@ extern "C" {
                                  /* tiles (UE_REORDER_KD, _GREEDY or _GREEDY_RINGS)           */
 #define UE_VARIANT_PERSISTENT 3  /* one cooperative launch per chunk of steps, timed grid     */
                                  /* barriers between half-steps; FP32                         */
+/* Added to PLAIN or BLOCKED: calls long enough to run resident (ue_step_n) replay the variant's */
+/* CUDA graphs instead, as larger meshes do.  The results are the same bit for bit.          */
+#define UE_VARIANT_NO_RESIDENT 256
 
 #define UE_RHO_GIVEN 0
 #define UE_RHO_POWER 1
@@ -103,7 +106,7 @@ typedef struct ue_options {
     int32_t dt_mode;       /* UE_DT_*                                                        */
     int32_t power_iters;   /* power-iteration steps (default 200)                            */
     uint32_t power_seed;   /* start vector: SplitMix64(seed * 2^32 + caller triangle id)     */
-    int32_t variant;       /* UE_VARIANT_* (0 = default: plain)                              */
+    int32_t variant;       /* UE_VARIANT_* (0 = default: plain), + UE_VARIANT_NO_RESIDENT    */
     int32_t graph_chunk;   /* steps per captured CUDA graph launch; 0 = default, <0 = none   */
     int32_t tile_tris;     /* UE_REORDER_KD / _GREEDY / _GREEDY_RINGS: maximum triangles per tile (ue_mesh_load) */
     int32_t block_depth;   /* UE_VARIANT_BLOCKED: steps per launch, 1..15                    */
@@ -141,7 +144,7 @@ typedef struct ue_stats_t {
                                  /* in place in pinned host memory (no staging copy)          */
     int32_t tb_kernel_used;      /* UE_VARIANT_BLOCKED: the kernel its launches run (UE_TBK_*) */
                                  /* (long calls on small meshes run resident: ue_step_n)      */
-    int32_t reserved2;
+    int32_t resident_launches;   /* resident launches of ue_step_n so far (among the above)   */
 } ue_stats_t;
 
 /* Kernels of the blocked variant (ue_stats_t.tb_kernel_used). */
@@ -228,7 +231,8 @@ int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
 /* Advance n_steps leap-frog steps, asynchronously on `stream`.  A call of a graph chunk of steps
  * or more on a mesh small enough for the chip's registers and shared memory (about 1.2M
  * triangles in FP32, 600k with a current or a frame, 300k in FP64, provided neighbouring triangles
- * are mostly stored close together; plain and blocked variants, graph_chunk >= 0) runs resident: one
+ * are mostly stored close together; plain and blocked variants without UE_VARIANT_NO_RESIDENT,
+ * graph_chunk >= 0) runs resident: one
  * cooperative launch for up to 1024 steps, with the same results bit for bit.  Its waits are
  * bounded; one that runs out is reported by ue_check (UE_ERR_TIMEOUT).  Errors of the launches are
  * reported here; device-side conditions surface at the next synchronous call. */

@@ -17,6 +17,7 @@ UE_DT_GIVEN, UE_DT_POWER, UE_DT_LEARNED = 0, 1, 2
 UE_RHO_GIVEN, UE_RHO_POWER, UE_RHO_LEARNED, UE_RHO_POWER_FALLBACK = 0, 1, 2, 3
 UE_MLP_PARAMS = 5057
 UE_VARIANT_PLAIN, UE_VARIANT_BLOCKED, UE_VARIANT_PERSISTENT = 1, 2, 3
+UE_VARIANT_NO_RESIDENT = 256   # added to PLAIN or BLOCKED
 UE_TB_SPLIT, UE_TB_FUSED = 0, 1
 UE_STATIC_MAX_TRIS, UE_STATIC_MAX_EDGES = 1 << 18, 1 << 19
 
@@ -42,7 +43,7 @@ class Stats(C.Structure):
                 ("bytes_per_step", C.c_double), ("kernel_launches", C.c_int64),
                 ("dt_setup_ms", C.c_double), ("rho_lo", C.c_double), ("rho_hi", C.c_double),
                 ("rho_hat", C.c_double), ("direct_fields", C.c_int64), ("tb_kernel_used", C.c_int32),
-                ("reserved2", C.c_int32)]
+                ("resident_launches", C.c_int32)]
 
 
 P = C.c_void_p

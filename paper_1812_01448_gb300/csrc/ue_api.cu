@@ -79,6 +79,7 @@ struct ue_mesh {
     int64_t steps_done = 0;
     int64_t step_pending = -1;   // ue_set_step's value, put on the device by the next call that steps
     int64_t launches = 0;
+    int32_t resident_launches = 0;
 
     // device tables and geometry (stored numbering)
     double* d_xy = nullptr;
@@ -127,6 +128,7 @@ struct ue_mesh {
     int tb_kernel = UE_TB_SPLIT;
     int tb_test_cta = -1;
     int flow_skip = -1;
+    bool no_resident = false;        // UE_VARIANT_NO_RESIDENT
     int cur = 0;                     // buffer holding the current fields
 
     // dt selection
@@ -1015,7 +1017,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
     m->flow = ue::FlowDev();
     const int64_t W = m->fr.W, NX = m->fr.nx + 2 * W;
     const int64_t n_fc = 2 * W * NX + 2 * W * m->fr.ny;
-    if (m->variant != UE_VARIANT_PERSISTENT && m->graph_chunk > 0 && m->tb_test_cta < 0) {
+    if (m->variant != UE_VARIANT_PERSISTENT && !m->no_resident && m->graph_chunk > 0 && m->tb_test_cta < 0) {
         int dev = 0, sms = 0, coop = 0;
         UE_CUDA(cudaGetDevice(&dev));
         UE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1234,6 +1236,7 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
         }
         UE_CUDA(e);
         launched += 1 + (dm.n_src > 0 ? 1 : 0);
+        ++m->resident_launches;
         left -= batch;
         m->since_check = since;
     }
@@ -1429,6 +1432,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     ue_options d;
     ue_options_default(&d);
     const ue_options& o = opt ? *opt : d;
+    const int32_t variant = o.variant & ~UE_VARIANT_NO_RESIDENT;
     if (o.precision != UE_PREC_FP32 && o.precision != UE_PREC_FP64)
         return fail(UE_ERR_ARG, "unknown precision");
     if (o.dt_mode == UE_DT_GIVEN && !(o.dt > 0)) return fail(UE_ERR_ARG, "dt must be > 0");
@@ -1438,12 +1442,12 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
         return fail(UE_ERR_ARG, "power iteration needs iters >= 1 and safety > 0");
     if (o.dt_mode == UE_DT_LEARNED && (!o.mlp_params || !(o.learned_margin >= 1.0)))
         return fail(UE_ERR_ARG, "learned dt needs mlp_params and learned_margin >= 1");
-    if (o.variant != 0 && o.variant != UE_VARIANT_PLAIN && o.variant != UE_VARIANT_BLOCKED &&
+    if (variant != 0 && variant != UE_VARIANT_PLAIN && variant != UE_VARIANT_BLOCKED &&
         o.variant != UE_VARIANT_PERSISTENT)
         return fail(UE_ERR_ARG, "unknown variant");
-    if (o.variant == UE_VARIANT_PERSISTENT && (o.precision != UE_PREC_FP32 || o.timeout_ms < 1))
+    if (variant == UE_VARIANT_PERSISTENT && (o.precision != UE_PREC_FP32 || o.timeout_ms < 1))
         return fail(UE_ERR_ARG, "the persistent variant is FP32 only and needs timeout_ms >= 1");
-    if (o.variant == UE_VARIANT_BLOCKED) {
+    if (variant == UE_VARIANT_BLOCKED) {
         if (o.precision != UE_PREC_FP32) return fail(UE_ERR_ARG, "the blocked variant is FP32 only");
         if (m->hm.tile_tri_off.size() < 2) return fail(UE_ERR_ARG, "the blocked variant needs tiles (UE_REORDER_KD, UE_REORDER_GREEDY or UE_REORDER_GREEDY_RINGS)");
         if (o.block_depth < 1 || o.block_depth > 15) return fail(UE_ERR_ARG, "block_depth must be in 1..15");
@@ -1452,7 +1456,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     }
     const bool framed = m->fr.W > 0;
     if (framed) {
-        if (o.variant == UE_VARIANT_PERSISTENT)
+        if (variant == UE_VARIANT_PERSISTENT)
             return fail(UE_ERR_ARG, "a framed mesh steps with the plain or the blocked variant");
         if (o.dt_mode == UE_DT_LEARNED)
             return fail(UE_ERR_ARG, "a framed mesh takes its dt from UE_DT_GIVEN or UE_DT_POWER");
@@ -1476,7 +1480,8 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     m->reg = ue::RegionDev();
     m->reg_host = ue::Region();
     m->cur = 0;
-    m->variant = o.variant == 0 ? UE_VARIANT_PLAIN : o.variant;
+    m->variant = variant == 0 ? UE_VARIANT_PLAIN : variant;
+    m->no_resident = (o.variant & UE_VARIANT_NO_RESIDENT) != 0;
     m->block_depth = o.block_depth;
     m->tb_threads = o.tb_threads == 1024 ? 1024 : 512;
     if (o.tb_kernel != UE_TB_SPLIT && o.tb_kernel != UE_TB_FUSED) return fail(UE_ERR_ARG, "tb_kernel must be UE_TB_SPLIT or UE_TB_FUSED");
@@ -1653,6 +1658,7 @@ int ue_batch_create(ue_mesh* const* meshes, int32_t n, void* stream, ue_mesh** o
     B->block_depth = m0->block_depth;
     B->tb_threads = m0->tb_threads;
     B->graph_chunk = m0->graph_chunk;
+    for (int32_t i = 0; i < n; ++i) B->no_resident = B->no_resident || meshes[i]->no_resident;
     B->watchdog_every = m0->watchdog_every;
     B->watchdog_growth = m0->watchdog_growth;
     B->dt = m0->dt;
@@ -2725,6 +2731,7 @@ int ue_stats(const ue_mesh* m, ue_stats_t* out) {
     out->rho_hi = m->rho_hi;
     out->rho_hat = m->rho_hat;
     out->direct_fields = m->direct_fields;
+    out->resident_launches = m->resident_launches;
     if (m->variant == UE_VARIANT_BLOCKED && m->built) {
         const bool whole = !m->dm.plasma && !m->has_reg && !m->ts.hdr.empty() && ue::tbf1_fits(m->tb, m->ts.hdr.data());
         out->tb_kernel_used = whole ? UE_TBK_WHOLE_MESH : ue::tb_kernel_used(m->tb, m->dm);

@@ -286,6 +286,9 @@ struct FlowChecks {
     double* wd = nullptr;
 };
 cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_steps, const FlowChecks& chk, cudaStream_t s);
+// Loads the kernel of m's next launch; cudaErrorCooperativeLaunchTooLarge when the device cannot hold
+// its CTAs at once.
+cudaError_t flow_ready(const FlowDev& fl, const DevMesh& m);
 
 // Launchers (kernels_step.cu).
 // g(t) table for the next `count` steps (no-op without a source).

@@ -1230,10 +1230,18 @@ __global__ void k_flow_init(unsigned* ctl) {
     }
 }
 
+// no steps: looks only whether the launch fits (flow_ready)
 template <typename T>
 cudaError_t launch_resident(void (*kern)(FlowArgs<T>), const FlowArgs<T>& a, int grid, int threads, size_t smem, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    if (a.n_steps == 0) {
+        int dev = 0, sms = 0, per = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem)) != cudaSuccess) return e;
+        return per * sms >= grid ? cudaSuccess : cudaErrorCooperativeLaunchTooLarge;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
@@ -1416,6 +1424,11 @@ cudaError_t launch_flow(const FlowDev& fl, const DevMesh& m, void* Uif, int n_st
     if ((chk.first > 0 || chk.end) && (!fl.epart || !chk.we || !chk.S || !chk.wd)) return cudaErrorInvalidValue;
     return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, Uif, n_steps, chk, s)
                                        : launch_flow_t<float>(fl, m, Uif, n_steps, chk, s);
+}
+
+cudaError_t flow_ready(const FlowDev& fl, const DevMesh& m) {
+    return m.precision == UE_PREC_FP64 ? launch_flow_t<double>(fl, m, nullptr, 0, FlowChecks(), nullptr)
+                                       : launch_flow_t<float>(fl, m, nullptr, 0, FlowChecks(), nullptr);
 }
 
 }  // namespace ue

@@ -1183,9 +1183,17 @@ int flush_step(ue_mesh* m, cudaStream_t s) {
     return UE_OK;
 }
 
-// n steps by the resident kernel, in place in the current field buffer.  `unit`: the steps between
-// watchdog checks of the launches this replaces.  *used is false, and nothing stepped, when the
-// device cannot hold the launch's CTAs at once (the caller then makes its launches).
+// Whether calls of *unit steps (a graph chunk, the steps between the watchdog checks of the launches)
+// or more run resident; shorter ones launch step by step.
+bool runs_resident(const ue_mesh* m, int64_t* unit) {
+    *unit = m->variant == UE_VARIANT_BLOCKED ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
+    // with the watchdog on a launch takes whole units
+    return ue::flow_takes(m->flow, m->dm) && (m->watchdog_every <= 0 || *unit <= ue::kFlowSteps);
+}
+
+// n steps by the resident kernel, in place in the current field buffer, for a mesh that runs_resident
+// with `unit`.  *used is false, and nothing stepped, when the device cannot hold the launch's CTAs at
+// once (the caller then makes its launches).
 int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) {
     DevMesh& dm = m->dm;
     const int64_t every = m->watchdog_every;
@@ -1193,11 +1201,7 @@ int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) 
     // the steps since the last check reach `every`, then every `period`
     const int64_t period = every > 0 ? (every + unit - 1) / unit * unit : 0;
     int64_t most = ue::kFlowSteps;
-    if (every > 0) most = unit > most ? unit : std::max(unit, std::min(most / unit * unit, ue::kFlowChecks / 2 * period));
-    if (most > ue::kFlowSteps) {   // a unit beyond one launch (a very long graph chunk)
-        *used = false;
-        return UE_OK;
-    }
+    if (every > 0) most = std::max(unit, std::min(most / unit * unit, ue::kFlowChecks / 2 * period));
     void* Uif = nullptr;
     // the frame that was built: one attached or taken off since waits for the next build
     if (m->has_reg) Uif = (float*)m->reg.dm.U + m->reg.f.u_off;
@@ -2005,14 +2009,11 @@ int ue_step_n(ue_mesh* m, int64_t n, void* stream) {
         m->launches += launched;
         return UE_OK;
     }
-    if (ue::flow_takes(m->flow, m->dm)) {
-        const int64_t unit = m->variant == UE_VARIANT_BLOCKED ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
-        // calls of a graph chunk or more, which would replay graphs; shorter ones launch step by step
-        if (n >= unit) {
-            bool used = false;
-            const int rc = flow_steps(m, n, unit, s, &used);
-            if (rc != UE_OK || used) return rc;
-        }
+    int64_t unit = 0;
+    if (runs_resident(m, &unit) && n >= unit) {
+        bool used = false;
+        const int rc = flow_steps(m, n, unit, s, &used);
+        if (rc != UE_OK || used) return rc;
     }
     if (m->variant == UE_VARIANT_BLOCKED) {
         const int64_t k = m->block_depth;
@@ -2081,9 +2082,17 @@ int ue_step_prepare(ue_mesh* m, void* stream) {
     if (!m || !m->built) return fail(UE_ERR_ARG, "geometry not built");
     cudaStream_t s = (cudaStream_t)stream;
     if (m->graph_chunk <= 0 || m->variant == UE_VARIANT_PERSISTENT) return UE_OK;
+    if (m->variant == UE_VARIANT_BLOCKED && !m->dm.plasma && !m->has_reg && !m->ts.hdr.empty() &&
+        ue::tbf1_fits(m->tb, m->ts.hdr.data()))
+        return UE_OK;   // one launch per call, no graph
+    int64_t unit = 0;
+    if (runs_resident(m, &unit)) {   // no graph either; the kernel is loaded, and its CTAs' room looked at, here
+        const cudaError_t e = ue::flow_ready(m->flow, m->dm);
+        if (e == cudaSuccess) return UE_OK;
+        if (e != cudaErrorCooperativeLaunchTooLarge) UE_CUDA(e);
+        m->flow.grid = 0;
+    }
     if (m->variant == UE_VARIANT_BLOCKED) {
-        if (!m->dm.plasma && !m->has_reg && !m->ts.hdr.empty() && ue::tbf1_fits(m->tb, m->ts.hdr.data()))
-            return UE_OK;   // one launch per call, no graph
         for (int p = 0; p < 2; ++p) {
             const int rc = ensure_graph_tb(m, p);
             if (rc != UE_OK) return rc;
@@ -2091,7 +2100,6 @@ int ue_step_prepare(ue_mesh* m, void* stream) {
         }
         return UE_OK;
     }
-    if (ue::flow_takes(m->flow, m->dm)) return UE_OK;   // the calls long enough for a graph run resident
     const int rc = ensure_graph(m);
     if (rc != UE_OK) return rc;
     UE_CUDA(cudaGraphUpload(m->gexec, s));

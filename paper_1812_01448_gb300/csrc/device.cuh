@@ -319,12 +319,13 @@ cudaError_t launch_coeff(const DevMesh& m, const double* elen, const double* d, 
                          const int32_t* tri_code, double dt, cudaStream_t s);
 // FP64 power iteration on K = -L_E L_B in the S metric; returns rho in *rho (synchronous).
 // With a frame, the iterate covers the triangles and the frame cells (start vector keyed by
-// n_t + frame cell), and K is the operator of the coupled system.
+// n_t + frame cell), and K is the operator of the coupled system.  small: by edges and triangles as with
+// a frame, on half the work space.
 cudaError_t power_iteration(const int2* rl, const int4* tri, const double* elen, const double* d,
                             const double* S, const int64_t* perm_tri, int64_t n_t, int64_t n_ei,
                             int iters, uint32_t seed, double* work, double* rho, cudaStream_t s,
-                            const FrameDev* frame = nullptr);
-size_t power_iteration_work_doubles(int64_t n_t, int64_t n_ei, const FrameDev* frame = nullptr);
+                            const FrameDev* frame, bool small);
+size_t power_iteration_work_doubles(int64_t n_t, int64_t n_ei, const FrameDev* frame, bool small);
 // The same without a frame (kernels_power.cu); work holds power_work_doubles doubles.
 size_t power_work_doubles(int64_t n_t);
 cudaError_t power_iteration_mesh(const int2* rl, const int4* tri, const double* elen, const double* d,

@@ -770,27 +770,28 @@ cudaError_t launch_source_flags(const DevMesh& m, const int32_t* k, int64_t n, b
     return cudaGetLastError();
 }
 
-size_t power_iteration_work_doubles(int64_t n_t, int64_t n_ei, const FrameDev* f) {
-    if (!f) return power_work_doubles(n_t);
+size_t power_iteration_work_doubles(int64_t n_t, int64_t n_ei, const FrameDev* f, bool small) {
+    if (!f && !small) return power_work_doubles(n_t);
     const int64_t nb = (n_t + kThreads - 1) / kThreads;
+    if (!f) return (size_t)(3 * n_t + 2 * n_ei + 1 + 2 * nb + 8 + 2);
     const int64_t nc = n_t + f->n_fc, nbf = (f->n_fc + kThreads - 1) / kThreads;
     const int64_t ng = f->u_off + f->n_if;
     const int64_t nh = (int64_t)f->NX * (f->NY + 1), nv = (int64_t)(f->NX + 1) * f->NY;
     return (size_t)(2 * nc + n_t + ng + n_ei + nh + nv + 2 * (nb + nbf) + 8 + 2);
 }
 
-// Without a frame: kernels_power.cu.  With one, an edge and a triangle launch per iteration (the
-// reductions in the triangles' last block), the iterate normalised on the fly by the scale its
-// previous reduction left, and the frame's side and cell launches between them, its cells'
-// partials summed by the triangles' last block after their own.
+// Without a frame: kernels_power.cu.  With one, or on the small work space, an edge and a triangle
+// launch per iteration (the reductions in the triangles' last block), the iterate normalised on the fly
+// by the scale its previous reduction left, and a frame's side and cell launches between them, its
+// cells' partials summed by the triangles' last block after their own.
 cudaError_t power_iteration(const int2* rl, const int4* tri, const double* elen, const double* d,
                             const double* S, const int64_t* perm_tri, int64_t n_t, int64_t n_ei,
                             int iters, uint32_t seed, double* work, double* rho, cudaStream_t s,
-                            const FrameDev* f) {
-    if (!f) return power_iteration_mesh(rl, tri, elen, d, S, perm_tri, n_t, n_ei, iters, seed, work, rho, s);
-    const int64_t nb = (n_t + kThreads - 1) / kThreads, nbf = (f->n_fc + kThreads - 1) / kThreads;
-    const int64_t nc = n_t + f->n_fc, ng = f->u_off + f->n_if;
-    const int64_t nh = (int64_t)f->NX * (f->NY + 1), nv = (int64_t)(f->NX + 1) * f->NY;
+                            const FrameDev* f, bool small) {
+    if (!f && !small) return power_iteration_mesh(rl, tri, elen, d, S, perm_tri, n_t, n_ei, iters, seed, work, rho, s);
+    const int64_t nb = (n_t + kThreads - 1) / kThreads, nbf = f ? (f->n_fc + kThreads - 1) / kThreads : 0;
+    const int64_t nc = n_t + (f ? f->n_fc : 0), ng = f ? f->u_off + f->n_if : n_ei + 1;
+    const int64_t nh = f ? (int64_t)f->NX * (f->NY + 1) : 0, nv = f ? (int64_t)(f->NX + 1) * f->NY : 0;
     double* w[2] = {work, work + nc};
     double* invS = work + 2 * nc;
     double* g = invS + n_t;
@@ -802,17 +803,19 @@ cudaError_t power_iteration(const int2* rl, const int4* tri, const double* elen,
     unsigned int* counter = reinterpret_cast<unsigned int*>(part + 2 * (nb + nbf) + 8);
     cudaError_t e;
     if ((e = cudaMemsetAsync(g, 0, sizeof(double) * ng, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(gH, 0, sizeof(double) * (nh + nv), s)) != cudaSuccess) return e;
+    if (f && (e = cudaMemsetAsync(gH, 0, sizeof(double) * (nh + nv), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(counter, 0, sizeof(double), s)) != cudaSuccess) return e;
     k_pi_prep<<<blocks_for(n_ei > n_t ? n_ei : n_t), kThreads, 0, s>>>(elen, d, S, c, invS, n_ei, n_t);
-    k_fpi_start<<<(unsigned)nbf, kThreads, 0, s>>>(*f, w[0], seed, n_t, part + 2 * nb);
+    if (f) k_fpi_start<<<(unsigned)nbf, kThreads, 0, s>>>(*f, w[0], seed, n_t, part + 2 * nb);
     k_pi_start<<<(unsigned)nb, kThreads, 0, s>>>(w[0], perm_tri, S, seed, n_t, part, sc[0], counter, nbf);
     for (int it = 0; it < iters; ++it) {
         const int cur = it & 1;
         if (n_ei > 0) k_pi_edge<<<blocks_for(n_ei), kThreads, 0, s>>>(rl, c, w[cur], sc[cur], g, n_ei);
-        k_fpi_edge<<<blocks_for(f->n_fc + f->n_if), kThreads, 0, s>>>(*f, w[cur], sc[cur], n_t, g, gH, gV);
-        k_fpi_cell<<<(unsigned)nbf, kThreads, 0, s>>>(*f, g, gH, gV, w[cur], sc[cur], w[cur ^ 1], n_t,
-                                                     part + 2 * nb);
+        if (f) {
+            k_fpi_edge<<<blocks_for(f->n_fc + f->n_if), kThreads, 0, s>>>(*f, w[cur], sc[cur], n_t, g, gH, gV);
+            k_fpi_cell<<<(unsigned)nbf, kThreads, 0, s>>>(*f, g, gH, gV, w[cur], sc[cur], w[cur ^ 1], n_t,
+                                                         part + 2 * nb);
+        }
         k_pi_tri<<<(unsigned)nb, kThreads, 0, s>>>(tri, invS, g, w[cur], sc[cur], w[cur ^ 1], part,
                                                   sc[cur ^ 1], counter, n_t, nbf);
     }

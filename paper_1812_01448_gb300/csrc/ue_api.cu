@@ -11,6 +11,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -273,9 +274,13 @@ void dev_free_all(ue_mesh* m, cudaStream_t s, bool keep_arena = false) {
     arena_reset(m, keep_arena);
 }
 
+// The resident step's arrays are given up where memory is short: the mesh then keeps its launches.
+bool drop_flow(ue_mesh* m, cudaStream_t s);
+
 template <typename P>
 bool alloc_into(ue_mesh* m, P*& out, size_t count, size_t elem, cudaStream_t s) {
     out = (P*)dev_alloc(m, count * elem, s);
+    if (!out && drop_flow(m, s)) out = (P*)dev_alloc(m, count * elem, s);
     return out != nullptr;
 }
 
@@ -290,6 +295,19 @@ void dev_release(ue_mesh* m, void* p, cudaStream_t s) {
             m->allocs.pop_back();
             return;
         }
+}
+
+bool drop_flow(ue_mesh* m, cudaStream_t s) {
+    ue::FlowDev& fl = m->flow;
+    if (fl.grid == 0 && !fl.rec) return false;
+    cudaDeviceSynchronize();   // no launch still uses them
+    for (void* p : {(void*)fl.slots, (void*)fl.place, (void*)fl.rec, fl.sent, (void*)fl.hlist, (void*)fl.cnt,
+                    (void*)fl.erec, (void*)fl.ecnt, (void*)fl.eslot, (void*)fl.crec, (void*)fl.epart})
+        dev_release(m, p, s);
+    unsigned* ctl = fl.ctl;    // its error word may not have been read yet
+    fl = ue::FlowDev();
+    fl.ctl = ctl;
+    return true;
 }
 
 #define UE_CUDA(call)                                                                   \
@@ -1057,18 +1075,22 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
          alloc_into(m, dm.U, dm.n_ei_pad + (n_if + 3) / 4 * 4, esz, s) &&
          alloc_into(m, dm.B, dm.n_t_pad, esz, s) && alloc_into(m, dm.step, 1, 8, s);
     if (ok && m->precision == UE_PREC_FP64) ok = alloc_into(m, dm.cB, dm.n_t_pad, 8, s);
-    if (m->flow.grid > 0) {
+    if (ok && m->flow.grid > 0) {
         ue::FlowDev& fl = m->flow;
         fl.skip = m->flow_skip;
-        ok = ok && alloc_into(m, fl.ctl, 4, 4, s) && alloc_into(m, fl.place, nt, 4, s) &&
-             alloc_into(m, fl.rec, flow_slots, 16, s) &&
-             alloc_into(m, fl.sent, fl.sent_bytes, 1, s) && alloc_into(m, fl.cnt, fl.grid, 8, s) &&
-             (fl.grid == 1 || fl.edges > 0 || alloc_into(m, fl.hlist, (size_t)fl.grid * fl.halo, 4, s)) &&
-             (fl.edges == 0 || (alloc_into(m, fl.erec, (size_t)fl.grid * fl.edges, 8, s) &&
-                                alloc_into(m, fl.ecnt, fl.grid, 8, s) && alloc_into(m, fl.eslot, nei + 1, 4, s))) &&
-             (n_fc == 0 || alloc_into(m, fl.crec, n_fc, 16, s)) &&
-             (m->watchdog_every <= 0 || alloc_into(m, fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8, s)) &&
-             (fl.slot_words == 0 || alloc_into(m, fl.slots, 2 * fl.slot_words, 8, s));
+        auto get = [&](auto*& p, size_t count, size_t elem) {
+            p = static_cast<std::remove_reference_t<decltype(p)>>(dev_alloc(m, count * elem, s));
+            return p != nullptr;
+        };
+        const bool all = get(fl.ctl, 4, 4) && get(fl.place, nt, 4) && get(fl.rec, flow_slots, 16) &&
+                         get(fl.sent, fl.sent_bytes, 1) && get(fl.cnt, fl.grid, 8) &&
+                         (fl.grid == 1 || fl.edges > 0 || get(fl.hlist, (size_t)fl.grid * fl.halo, 4)) &&
+                         (fl.edges == 0 || (get(fl.erec, (size_t)fl.grid * fl.edges, 8) && get(fl.ecnt, fl.grid, 8) &&
+                                            get(fl.eslot, nei + 1, 4))) &&
+                         (n_fc == 0 || get(fl.crec, n_fc, 16)) &&
+                         (m->watchdog_every <= 0 || get(fl.epart, (size_t)ue::kFlowChecks * (fl.grid + 1), 8)) &&
+                         (fl.slot_words == 0 || get(fl.slots, 2 * fl.slot_words, 8));
+        if (!all) drop_flow(m, s);
     }
     {
         int g = m->flow.grid > 0 ? ue::kFlowSteps : 64;
@@ -1087,8 +1109,8 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         return fail(UE_ERR_ALLOC, "device allocation failed");
     }
     {
+        if (m->flow.ctl) UE_CUDA(ue::launch_flow_init(m->flow, s));
         if (m->flow.grid > 0) {
-            UE_CUDA(ue::launch_flow_init(m->flow, s));
             if (m->flow.slot_words > 0) UE_CUDA(cudaMemsetAsync(m->flow.slots, 0, 16 * m->flow.slot_words, s));
             if (m->flow.epart)   // its counters
                 UE_CUDA(cudaMemsetAsync(m->flow.epart + (size_t)ue::kFlowChecks * m->flow.grid, 0, 8 * ue::kFlowChecks, s));
@@ -1547,10 +1569,15 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
         if (nrc != UE_OK) return nrc;
         llock.lock();
         if (!(lres = learned_res())) return fail(UE_ERR_ALLOC, "learned dt result buffer");
-    } else if (o.dt_mode == UE_DT_POWER) {
-        if (!alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, framed ? &m->fd : nullptr), 8, s))
-            return fail(UE_ERR_ALLOC, "power iteration work space");
     }
+    const ue::FrameDev* frame = framed ? &m->fd : nullptr;
+    bool small = false;   // half the work space, where memory is short
+    auto power_work = [&]() {
+        if (alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, false), 8, s)) return true;
+        small = true;
+        return alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, true), 8, s);
+    };
+    if (o.dt_mode == UE_DT_POWER && !power_work()) return fail(UE_ERR_ALLOC, "power iteration work space");
     UE_CUDA(cudaStreamSynchronize(s));
     Range nvtx_dt("ue_geometry_build: dt, coefficients, tiles");
     const auto t_dt0 = std::chrono::steady_clock::now();
@@ -1574,12 +1601,10 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
         }
     }
     if (need_power) {
-        if (!pwork && !alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, framed ? &m->fd : nullptr), 8, s))
-            return fail(UE_ERR_ALLOC, "power iteration work space");
+        if (!pwork && !power_work()) return fail(UE_ERR_ALLOC, "power iteration work space");
         double rho = 0;
         UE_CUDA(ue::power_iteration(m->d_rl, dm.tri, m->d_elen, m->d_d, m->d_S, m->d_perm, nt, nei,
-                                    o.power_iters, o.power_seed, pwork, &rho, s,
-                                    framed ? &m->fd : nullptr));
+                                    o.power_iters, o.power_seed, pwork, &rho, s, frame, small));
         if (!(rho > 0) || !std::isfinite(rho)) return fail(UE_ERR_DUAL, "power iteration gave rho <= 0");
         m->rho = rho;
         m->rho_source = o.dt_mode == UE_DT_LEARNED ? UE_RHO_POWER_FALLBACK : UE_RHO_POWER;

@@ -85,7 +85,11 @@ extern "C" {
 typedef struct ue_mesh ue_mesh;  /* opaque, owned by the library until ue_mesh_free        */
 
 /* Device allocator hooks: alloc(bytes, stream, ctx) returns a device pointer or NULL;
- * free(ptr, stream, ctx) releases it.  Both NULL = cudaMalloc / cudaFree.  Pointers must be
+ * free(ptr, stream, ctx) releases it.  Both NULL = cudaMalloc / cudaFree; blocks
+ * of up to 64 MB are then cut from a few larger ones, which stay with the mesh for its next build, and
+ * up to 64 MB of what calls have returned for its next calls; ue_mesh_free gives all back.  Where memory
+ * is short the faster paths do without theirs (no resident step, half the power iteration's work
+ * space) before a call fails.  Pointers must be
  * 16-byte aligned (the blocked kernels move records and fields with TMA bulk copies): one that
  * is not is handed back to free and the call fails with UE_ERR_ALLOC. */
 typedef void* (*ue_alloc_fn)(size_t bytes, void* stream, void* ctx);
@@ -399,7 +403,7 @@ int ue_mesh_flip(const double* xy, int64_t n_nodes, const int32_t* tris, int64_t
  * column).  omega: n_modes doubles, descending.  B: NULL or n_modes * n_tris doubles, mode i
  * at B + i*n_tris in caller triangle order, normalised to sum_j S_j B_j^2 = 1 (sign
  * arbitrary).  Synchronous; the work space, about 3 n_tris * 2 n_modes
- * doubles, comes from the mesh's allocator and is returned.
+ * doubles, comes from the mesh's allocator and is returned to it.
  * Errors: UE_ERR_ARG (also on a mesh with a PML frame); UE_ERR_ALLOC; UE_ERR_DUAL if the block
  * loses rank; UE_ERR_CUDA. */
 int ue_modes(ue_mesh* m, int32_t n_modes, int32_t iters, uint32_t seed, double* omega, double* B,

@@ -16,6 +16,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "arena.h"
 #include "device.cuh"
 #include "ue_internal.h"
 
@@ -55,6 +56,22 @@ struct FrameHost {
     std::vector<double> iface;    // 6 per edge: x_a, y_a, x_b, y_b, inward normal
 };
 
+// The device under a mesh's arena.
+const ue::Arena::Ops kDeviceOps = {
+    [](size_t bytes) -> void* {
+        void* p = nullptr;
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    },
+    [](void* p) { cudaFree(p); },
+    [] { cudaDeviceSynchronize(); },
+    [] {
+        int dev = -1;
+        cudaGetDevice(&dev);
+        return dev;
+    }};
+
 }  // namespace
 
 struct ue_mesh {
@@ -63,13 +80,7 @@ struct ue_mesh {
     ue_free_fn free_fn = nullptr;
     void* alloc_ctx = nullptr;
     std::vector<void*> allocs;
-    // without callbacks: small blocks are cut from a few large ones (Arena below)
-    struct Piece {
-        char* p;
-        size_t bytes;
-    };
-    std::vector<Piece> chunks, spare, pieces;   // from cudaMalloc; free parts of them; parts in use
-    size_t reserve = 0;                         // least size of the next chunk
+    ue::Arena arena{kDeviceOps};     // without callbacks
 
     bool built = false;
     int precision = UE_PREC_FP32;
@@ -169,84 +180,11 @@ struct ue_mesh {
 
 namespace {
 
-// Device memory without allocator callbacks.  A cudaMalloc and its cudaFree cost about 60 us and a
-// setup makes some 27 of them: blocks up to kDirect are cut, first fit, from chunks (the first as
-// large as a setup's arrays), larger ones come from cudaMalloc as before.  A released block is reused
-// only after the device has gone idle, as cudaFree waits too, so work on another stream that
-// still reads it is safe.  A rebuild starts from one chunk of the size that the last build took.
-constexpr size_t kDirect = (size_t)64 << 20, kChunk = (size_t)2 << 20, kAlign = 256;
+// Without callbacks, blocks beyond this are cudaMalloc's own.
+constexpr size_t kDirect = (size_t)64 << 20;
 
-void* arena_alloc(ue_mesh* m, size_t bytes) {
-    bytes = (bytes + kAlign - 1) / kAlign * kAlign;
-    for (int pass = 0; pass < 2; ++pass) {
-        for (size_t i = 0; i < m->spare.size(); ++i) {
-            ue_mesh::Piece& f = m->spare[i];
-            if (f.bytes < bytes) continue;
-            char* p = f.p;
-            f.p += bytes;
-            f.bytes -= bytes;
-            if (f.bytes == 0) m->spare.erase(m->spare.begin() + i);
-            m->pieces.push_back({p, bytes});
-            return p;
-        }
-        if (pass == 1) break;
-        size_t held = 0;
-        for (const ue_mesh::Piece& c : m->chunks) held += c.bytes;
-        const size_t want = std::max(bytes, std::max(kChunk, std::min(std::max(held / 4, m->reserve), 4 * kDirect)));
-        m->reserve = 0;
-        void* c = nullptr;
-        size_t got = want;
-        if (cudaMalloc(&c, want) != cudaSuccess) {   // little memory left: no more than asked for
-            cudaGetLastError();
-            got = bytes;
-            if (want == bytes || cudaMalloc(&c, bytes) != cudaSuccess) {
-                cudaGetLastError();
-                return nullptr;
-            }
-        }
-        m->chunks.push_back({(char*)c, got});
-        m->spare.push_back({(char*)c, got});
-    }
-    return nullptr;
-}
-
-bool arena_release(ue_mesh* m, void* p) {
-    for (size_t i = 0; i < m->pieces.size(); ++i)
-        if (m->pieces[i].p == p) {
-            cudaDeviceSynchronize();
-            m->spare.push_back(m->pieces[i]);
-            m->pieces[i] = m->pieces.back();
-            m->pieces.pop_back();
-            return true;
-        }
-    return false;
-}
-
-// All blocks of the arena free again.  keep: as one chunk for the next build.
-void arena_reset(ue_mesh* m, bool keep) {
-    m->pieces.clear();
-    m->spare.clear();
-    size_t held = 0;
-    for (const ue_mesh::Piece& c : m->chunks) held += c.bytes;
-    if (keep && m->chunks.size() == 1) {
-        cudaDeviceSynchronize();
-        m->spare = m->chunks;
-        return;
-    }
-    for (const ue_mesh::Piece& c : m->chunks) cudaFree(c.p);
-    m->chunks.clear();
-    void* c = nullptr;
-    if (keep && held > 0) {
-        if (cudaMalloc(&c, held) == cudaSuccess) {
-            m->chunks.push_back({(char*)c, held});
-            m->spare = m->chunks;
-        } else {
-            cudaGetLastError();
-        }
-    }
-}
-
-void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s) {
+// temp: released before the call returns (Scratch)
+void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s, bool temp = false) {
     if (bytes == 0) bytes = 16;
     void* p = nullptr;
     if (m->alloc) {
@@ -256,10 +194,10 @@ void* dev_alloc(ue_mesh* m, size_t bytes, cudaStream_t s) {
             p = nullptr;
         }
     } else if (bytes <= kDirect) {
-        return arena_alloc(m, bytes);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        p = nullptr;
+        return m->arena.alloc(bytes, temp);
+    } else if (!(p = kDeviceOps.get(bytes))) {
+        m->arena.give_back();
+        p = kDeviceOps.get(bytes);
     }
     if (p) m->allocs.push_back(p);
     return p;
@@ -271,22 +209,22 @@ void dev_free_all(ue_mesh* m, cudaStream_t s, bool keep_arena = false) {
         else cudaFree(p);
     }
     m->allocs.clear();
-    arena_reset(m, keep_arena);
+    m->arena.reset(keep_arena);
 }
 
 // The resident step's arrays are given up where memory is short: the mesh then keeps its launches.
 bool drop_flow(ue_mesh* m, cudaStream_t s);
 
 template <typename P>
-bool alloc_into(ue_mesh* m, P*& out, size_t count, size_t elem, cudaStream_t s) {
-    out = (P*)dev_alloc(m, count * elem, s);
-    if (!out && drop_flow(m, s)) out = (P*)dev_alloc(m, count * elem, s);
+bool alloc_into(ue_mesh* m, P*& out, size_t count, size_t elem, cudaStream_t s, bool temp = false) {
+    out = (P*)dev_alloc(m, count * elem, s, temp);
+    if (!out && drop_flow(m, s)) out = (P*)dev_alloc(m, count * elem, s, temp);
     return out != nullptr;
 }
 
 // Release one allocation made by dev_alloc (no-op for NULL).
 void dev_release(ue_mesh* m, void* p, cudaStream_t s) {
-    if (!p || arena_release(m, p)) return;
+    if (!p || m->arena.release(p)) return;
     for (size_t i = 0; i < m->allocs.size(); ++i)
         if (m->allocs[i] == p) {
             if (m->free_fn) m->free_fn(p, (void*)s, m->alloc_ctx);
@@ -309,6 +247,25 @@ bool drop_flow(ue_mesh* m, cudaStream_t s) {
     fl.ctl = ctl;
     return true;
 }
+
+// What one call allocates and gives back as it returns.
+struct Scratch {
+    ue_mesh* m;
+    cudaStream_t s;
+    std::vector<void*> blocks;
+    Scratch(ue_mesh* m_, cudaStream_t s_) : m(m_), s(s_) {}
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    ~Scratch() {
+        for (void* p : blocks) dev_release(m, p, s);
+    }
+    template <typename P>
+    bool get(P*& out, size_t count, size_t elem) {
+        if (!alloc_into(m, out, count, elem, s, true)) return false;
+        blocks.push_back(out);
+        return true;
+    }
+};
 
 #define UE_CUDA(call)                                                                   \
     do {                                                                                \
@@ -545,7 +502,8 @@ int bake_plasma(ue_mesh* m, cudaStream_t s) {
     if (!dm.pb && !alloc_into(m, dm.pb, dm.n_ei_pad, esz, s)) return fail(UE_ERR_ALLOC, "plasma coefficient");
     UE_CUDA(cudaMemsetAsync(dm.pb, 0, esz * dm.n_ei_pad, s));
     double* d_n = nullptr;
-    if (!alloc_into(m, d_n, m->hm.n_nodes, 8, s)) return fail(UE_ERR_ALLOC, "plasma density");
+    Scratch tmp(m, s);
+    if (!tmp.get(d_n, m->hm.n_nodes, 8)) return fail(UE_ERR_ALLOC, "plasma density");
     UE_CUDA(cudaMemcpyAsync(d_n, m->plasma_n.data(), 8 * m->hm.n_nodes, cudaMemcpyHostToDevice, s));
     UE_CUDA(cudaMemsetAsync(dm.J, 0, esz * dm.n_ei_pad, s));
     UE_CUDA(ue::launch_plasma_coeff(dm, d_n, m->d_edge_nodes, m->plasma_nu, m->dt, s));
@@ -1042,15 +1000,16 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         if (!coop || !ue::flow_shape(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) m->flow = ue::FlowDev();
     }
-    const size_t flow_slots = (size_t)m->flow.grid * m->flow.cap;
-    m->reserve = (size_t)(16 * nn + nt * (150 + 3 * (int64_t)esz) + nei * (64 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
+    const size_t flow_slots = (size_t)m->flow.grid * m->flow.cap, kAlign = ue::Arena::kAlign;
+    size_t reserve = (size_t)(16 * nn + nt * (150 + 3 * (int64_t)esz) + nei * (64 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
     // the resident step's arrays with them: on small meshes, whose slots are mostly spare, they are
     // the larger part and took further chunks, 60 us each
     if (m->flow.grid > 0)
-        m->reserve += 16 * flow_slots + m->flow.sent_bytes + 4 * (size_t)nt + 16 * (size_t)m->flow.slot_words +
+        reserve += 16 * flow_slots + m->flow.sent_bytes + 4 * (size_t)nt + 16 * (size_t)m->flow.slot_words +
                       (size_t)m->flow.grid * (4 * (size_t)m->flow.halo + 16 + 8 * (size_t)m->flow.edges) +
                       (m->flow.edges > 0 ? 4 * (size_t)nei : 0) + 16 * (size_t)n_fc +
                       (m->watchdog_every > 0 ? 8 * (size_t)ue::kFlowChecks * (m->flow.grid + 1) : 0) + 12 * kAlign;
+    m->arena.reserve(reserve);
     bool ok = alloc_into(m, m->d_xy, 2 * nn, 8, s) && alloc_into(m, m->d_tri_nodes, 3 * nt, 4, s) &&
               alloc_into(m, m->d_edge_nodes, 2 * nei + 2, 4, s) &&
               alloc_into(m, m->d_edge_opp, 2 * nei + 2, 4, s) &&
@@ -2423,8 +2382,8 @@ int ue_frame_state(ue_mesh* m, double* Bx, double* By, double* Ex, double* Ey, i
     const ue::FrameDev& f = m->fd;
     const int64_t nh = (int64_t)f.NX * (f.NY + 1), nv = (int64_t)(f.NX + 1) * f.NY;
     double *tx = nullptr, *ty = nullptr, *th = nullptr, *tv = nullptr;
-    if (!alloc_into(m, tx, f.n_fc, 8, s) || !alloc_into(m, ty, f.n_fc, 8, s) || !alloc_into(m, th, nh, 8, s) ||
-        !alloc_into(m, tv, nv, 8, s))
+    Scratch tmp(m, s);
+    if (!tmp.get(tx, f.n_fc, 8) || !tmp.get(ty, f.n_fc, 8) || !tmp.get(th, nh, 8) || !tmp.get(tv, nv, 8))
         return fail(UE_ERR_ALLOC, "frame state buffers");
     const bool f64 = m->precision == UE_PREC_FP64;
     if (write) {
@@ -2441,7 +2400,6 @@ int ue_frame_state(ue_mesh* m, double* Bx, double* By, double* Ex, double* Ey, i
         UE_CUDA(cudaMemcpyAsync(Ey, tv, 8 * nv, cudaMemcpyDeviceToHost, s));
     }
     UE_CUDA(cudaStreamSynchronize(s));
-    for (double* p : {tx, ty, th, tv}) dev_release(m, p, s);
     return UE_OK;
 }
 
@@ -2451,17 +2409,14 @@ int ue_frame_fields(ue_mesh* m, double* B, double* Ex, double* Ey, void* stream)
     const ue::FrameDev& f = m->fd;
     const int64_t nh = (int64_t)f.NX * (f.NY + 1), nv = (int64_t)(f.NX + 1) * f.NY;
     double *tB = nullptr, *tx = nullptr, *ty = nullptr;
-    if ((B && !alloc_into(m, tB, f.n_fc, 8, s)) || (Ex && !alloc_into(m, tx, nh, 8, s)) ||
-        (Ey && !alloc_into(m, ty, nv, 8, s)))
+    Scratch tmp(m, s);
+    if ((B && !tmp.get(tB, f.n_fc, 8)) || (Ex && !tmp.get(tx, nh, 8)) || (Ey && !tmp.get(ty, nv, 8)))
         return fail(UE_ERR_ALLOC, "frame export buffers");
     UE_CUDA(ue::launch_frame_out(f, m->precision == UE_PREC_FP64, tB, tx, ty, s));
     if (B) UE_CUDA(cudaMemcpyAsync(B, tB, 8 * f.n_fc, cudaMemcpyDeviceToHost, s));
     if (Ex) UE_CUDA(cudaMemcpyAsync(Ex, tx, 8 * nh, cudaMemcpyDeviceToHost, s));
     if (Ey) UE_CUDA(cudaMemcpyAsync(Ey, ty, 8 * nv, cudaMemcpyDeviceToHost, s));
     UE_CUDA(cudaStreamSynchronize(s));
-    dev_release(m, tB, s);
-    dev_release(m, tx, s);
-    dev_release(m, ty, s);
     return UE_OK;
 }
 
@@ -2470,8 +2425,9 @@ int ue_get_geometry(ue_mesh* m, double* O, double* S, double* elen, double* d) {
     const HostMesh& h = m->hm;
     cudaStream_t s = nullptr;
     double *tO = nullptr, *tS = nullptr, *tl = nullptr, *td = nullptr;
-    if ((O && !alloc_into(m, tO, 2 * h.n_tris, 8, s)) || (S && !alloc_into(m, tS, h.n_tris, 8, s)) ||
-        (elen && !alloc_into(m, tl, h.n_edges, 8, s)) || (d && !alloc_into(m, td, h.n_edges, 8, s)))
+    Scratch tmp(m, s);
+    if ((O && !tmp.get(tO, 2 * h.n_tris, 8)) || (S && !tmp.get(tS, h.n_tris, 8)) || (elen && !tmp.get(tl, h.n_edges, 8)) ||
+        (d && !tmp.get(td, h.n_edges, 8)))
         return fail(UE_ERR_ALLOC, "geometry export buffers");
     UE_CUDA(ue::launch_scatter_geometry(m->d_O, m->d_S, m->d_elen, m->d_d, m->d_perm, m->d_ecaller,
                                         h.n_tris, h.n_ei, h.n_edges, tO, tS, tl, td, s));
@@ -2679,20 +2635,14 @@ int ue_modes_low(ue_mesh* m, int32_t n_modes, int32_t iters, int32_t degree, uin
     if (nt < bw) return fail(UE_ERR_ARG, "ue_modes_low: the mesh has fewer triangles than the block of vectors");
     double* work = nullptr;
     double* Bd = nullptr;
-    if (!alloc_into(m, work, ue::modes_low_work_doubles(nt, bw), 8, s) ||
-        (B && !alloc_into(m, Bd, (size_t)n_modes * nt, 8, s)))
+    Scratch tmp(m, s);
+    if (!tmp.get(work, ue::modes_low_work_doubles(nt, bw), 8) || (B && !tmp.get(Bd, (size_t)n_modes * nt, 8)))
         return fail(UE_ERR_ALLOC, "ue_modes_low work space");
     bool lost = false;
     UE_CUDA(ue::modes_low_run(m->d_rl, m->dm.tri, m->d_elen, m->d_d, m->d_S, m->d_perm, nt, nei, n_modes,
                               iters, degree, seed, work, omega, Bd, &lost, s));
-    if (lost) {
-        dev_release(m, work, s);
-        if (Bd) dev_release(m, Bd, s);
-        return fail(UE_ERR_DUAL, "ue_modes_low: the block of vectors lost rank");
-    }
+    if (lost) return fail(UE_ERR_DUAL, "ue_modes_low: the block of vectors lost rank");
     if (B) UE_CUDA(cudaMemcpy(B, Bd, sizeof(double) * n_modes * nt, cudaMemcpyDeviceToHost));
-    dev_release(m, work, s);
-    if (Bd) dev_release(m, Bd, s);
     return UE_OK;
 }
 
@@ -2711,20 +2661,15 @@ int ue_modes(ue_mesh* m, int32_t n_modes, int32_t iters, uint32_t seed, double* 
         return fail(UE_ERR_ARG, "ue_modes: the mesh has fewer triangles than the block of vectors");
     double* work = nullptr;
     double* Bd = nullptr;
-    if (!alloc_into(m, work, ue::modes_work_doubles(nt, ue::modes_block_size(n_modes)), 8, s) ||
-        (B && !alloc_into(m, Bd, (size_t)n_modes * nt, 8, s)))
+    Scratch tmp(m, s);
+    if (!tmp.get(work, ue::modes_work_doubles(nt, ue::modes_block_size(n_modes)), 8) ||
+        (B && !tmp.get(Bd, (size_t)n_modes * nt, 8)))
         return fail(UE_ERR_ALLOC, "ue_modes work space");
     bool lost = false;
     UE_CUDA(ue::modes_run(m->d_rl, m->dm.tri, m->d_elen, m->d_d, m->d_S, m->d_perm, nt, nei, n_modes,
                           iters, seed, work, omega, Bd, &lost, s));
-    if (lost) {
-        dev_release(m, work, s);
-        if (Bd) dev_release(m, Bd, s);
-        return fail(UE_ERR_DUAL, "ue_modes: the block of vectors lost rank (fewer independent modes than asked)");
-    }
+    if (lost) return fail(UE_ERR_DUAL, "ue_modes: the block of vectors lost rank (fewer independent modes than asked)");
     if (B) UE_CUDA(cudaMemcpy(B, Bd, sizeof(double) * n_modes * nt, cudaMemcpyDeviceToHost));
-    dev_release(m, work, s);
-    if (Bd) dev_release(m, Bd, s);
     return UE_OK;
 }
 

@@ -242,6 +242,10 @@ int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
  * reported here; device-side conditions surface at the next synchronous call. */
 int ue_step_n(ue_mesh* m, int64_t n_steps, void* stream);
 
+/* The largest mesh or batch, in triangles of a vacuum medium without a frame, whose long calls run
+ * resident on the current device (0: none, or no device; one whose neighbours lie far apart may not at any size). */
+int ue_resident_capacity(int32_t precision, int64_t* n_tris);
+
 /* Capture and instantiate now the CUDA graphs that ue_step_n replays (a blocked mesh: one per
  * field buffer parity; the plain variant: one), and upload them on `stream`, so that the first
  * ue_step_n call long enough to use them pays no capture.  On a mesh whose long calls run resident

@@ -13,4 +13,4 @@ from ._native import (UE_DT_GIVEN, UE_DT_LEARNED, UE_DT_POWER, UE_PREC_FP32,  # 
                       UE_REORDER_RCM, UE_VARIANT_BLOCKED,
                       UE_TB_FUSED, UE_TB_SPLIT, UE_VARIANT_NO_RESIDENT, UE_VARIANT_PERSISTENT, UE_VARIANT_PLAIN, UEError)
 from .api import (Mesh, adam, batch_create, mesh_flip, mesh_relax, mlp_backward, mlp_forward, options,  # noqa: F401
-                  power_iteration_static, rho_loss, seg_argmax, triangulate)
+                  power_iteration_static, resident_capacity, rho_loss, seg_argmax, triangulate)

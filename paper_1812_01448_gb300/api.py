@@ -446,6 +446,13 @@ def triangulate(xy, segs=None, holes=None, drop_exterior: bool = False):
     return out[:nt.value].copy(), nf.value
 
 
+def resident_capacity(precision: int = N.UE_PREC_FP32) -> int:
+    """The most triangles of a mesh or batch whose long calls run resident (ue_resident_capacity)."""
+    n = C.c_int64()
+    N.check(N.lib().ue_resident_capacity(int(precision), C.byref(n)), "ue_resident_capacity")
+    return n.value
+
+
 def batch_create(meshes, stream=None) -> Mesh:
     """ue_batch_create: one Mesh object advancing all the given built meshes together.
 

@@ -269,6 +269,8 @@ struct FlowDev {
 };
 // n_fc: cells of a PML frame stepped with the mesh.  False when the mesh does not fit.
 bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl);
+// The most triangles that fit, without a frame.
+int64_t flow_capacity(bool f64, int sms);
 // Whether m, as it stands, steps by it (the largest shape takes vacuum media only).
 bool flow_takes(const FlowDev& fl, const DevMesh& m);
 cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s);

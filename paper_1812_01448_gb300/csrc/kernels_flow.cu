@@ -1371,6 +1371,16 @@ bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl) {
     return true;
 }
 
+int64_t flow_capacity(bool f64, int sms) {
+    FlowDev fl;
+    int64_t lo = 0, hi = (int64_t)sms * 512 * 16 + 1;   // fits (none does), does not
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) / 2;
+        (flow_shape(mid, 0, f64, sms, fl) ? lo : hi) = mid;
+    }
+    return lo;
+}
+
 bool flow_takes(const FlowDev& fl, const DevMesh& m) { return fl.grid > 0 && (fl.shape != kVacuumShape || !m.plasma); }
 
 cudaError_t launch_flow_init(const FlowDev& fl, cudaStream_t s) {

@@ -2061,6 +2061,17 @@ int ue_step_n(ue_mesh* m, int64_t n, void* stream) {
     return UE_OK;
 }
 
+int ue_resident_capacity(int32_t precision, int64_t* n_tris) {
+    if (!n_tris || (precision != UE_PREC_FP32 && precision != UE_PREC_FP64)) return fail(UE_ERR_ARG, "bad arguments");
+    int dev = 0, sms = 0, coop = 0;
+    *n_tris = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return UE_OK;   // no device
+    UE_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    *n_tris = coop ? ue::flow_capacity(precision == UE_PREC_FP64, sms) : 0;
+    return UE_OK;
+}
+
 int ue_step_prepare(ue_mesh* m, void* stream) {
     Range nvtx_range("ue_step_prepare");
     if (!m || !m->built) return fail(UE_ERR_ARG, "geometry not built");

@@ -8,7 +8,9 @@ or 1024 threads).
 The tuner times each candidate on a sample of the meshes, spread over their size
 distribution, as a real batch: built by the library, stepped inside its CUDA graphs, timed
 with CUDA events on the launching stream.  Each mesh keeps its own source; a fixed small dt
-is used because speed does not depend on it.
+is used because speed does not depend on it.  A sample may fit the chip, and step resident whatever
+its plain or blocked form, where the whole batch does not: it is then kept from the resident step,
+so that what is timed is what the batch will launch.
 
 Only the library's calls are sequenced here; all stepping work runs in libue.so.
 """
@@ -18,7 +20,7 @@ import time
 
 import numpy as np
 
-from .api import Mesh, batch_create
+from .api import Mesh, batch_create, resident_capacity
 from . import _native as N
 
 # (variant, tiler, tile_tris, block_depth, tb_threads); plain and persistent use the tiled
@@ -57,16 +59,21 @@ def _steps_for(steps: int, depth: int) -> int:
 
 
 def time_batch(items, variant: str, tile_tris: int, block_depth: int, tb_threads: int,
-               steps: int = 192, warmup: int = 48, stream=None, meshes=None, tiler: str = "kd") -> float:
+               steps: int = 192, warmup: int = 48, stream=None, meshes=None, tiler: str = "kd",
+               resident: bool = True) -> float:
     """Triangle-steps/s of one configuration on a batch of ``items`` = (MeshArrays, source
     edge ids, amplitudes, omega0).  ``meshes`` may hold already loaded Mesh objects of the same
-    items, tiler and tile size (they are rebuilt for this variant)."""
+    items, tiler and tile size (they are rebuilt for this variant).  resident=False keeps a batch
+    that fits the chip from the resident step."""
     import torch
     own = meshes is None
     if own:
         meshes = [Mesh(ms.xy, ms.tris, reorder=TILERS[tiler], tile_tris=tile_tris) for ms, *_ in items]
+    code = _VARIANT[variant]
+    if not resident and variant != "persistent":
+        code |= N.UE_VARIANT_NO_RESIDENT
     for m, (ms, ids, amp, w0) in zip(meshes, items):
-        m.geometry_build(stream=stream, dt_mode=N.UE_DT_GIVEN, dt=1e-7, variant=_VARIANT[variant],
+        m.geometry_build(stream=stream, dt_mode=N.UE_DT_GIVEN, dt=1e-7, variant=code,
                          block_depth=block_depth, tb_threads=tb_threads, graph_chunk=32)
         m.set_source(ids, amp, w0, 0.1, 0.05)
     b = batch_create(meshes, stream)
@@ -95,8 +102,10 @@ def autotune_batch(items, candidates=DEFAULT_CANDIDATES, sample: int = 32, steps
     """Time every candidate on a spread sample of ``items``; return (best, table).  ``best``
     and each row of ``table`` are dicts with variant, tile_tris, block_depth, tb_threads and
     rate (triangle-steps/s on the sample), plus the tiler; the table also records the tuning
-    time."""
-    idx = spread([ms.n_tris for ms, *_ in items], sample)
+    time and whether the whole batch fits the chip (its plain and blocked forms then step alike)."""
+    sizes = [ms.n_tris for ms, *_ in items]
+    resident = sum(sizes) <= resident_capacity()
+    idx = spread(sizes, sample)
     sub = [items[i] for i in idx]
     t0 = time.perf_counter()
     table = []
@@ -110,7 +119,7 @@ def autotune_batch(items, candidates=DEFAULT_CANDIDATES, sample: int = 32, steps
                 row = dict(variant=variant, tiler=tiler, tile_tris=tile, block_depth=depth, tb_threads=threads)
                 try:
                     row["rate"] = time_batch(sub, variant, tile, depth, threads, steps=steps, stream=stream,
-                                             meshes=meshes, tiler=tiler)
+                                             meshes=meshes, tiler=tiler, resident=resident)
                 except N.UEError as e:
                     # a configuration the library refuses for these meshes (a tile with its halo
                     # beyond the blocked kernel's capacity): recorded, not chosen
@@ -126,5 +135,5 @@ def autotune_batch(items, candidates=DEFAULT_CANDIDATES, sample: int = 32, steps
         raise ValueError("autotune_batch: the library refused every candidate for these meshes")
     best = max(usable, key=lambda r: r["rate"])
     return dict(best), {"rows": table, "sample_meshes": len(sub),
-                        "sample_tris": int(sum(ms.n_tris for ms, *_ in sub)),
+                        "sample_tris": int(sum(ms.n_tris for ms, *_ in sub)), "resident": resident,
                         "seconds": time.perf_counter() - t0}

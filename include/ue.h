@@ -309,13 +309,17 @@ int ue_get_geometry(ue_mesh* m, double* O, double* S, double* elen, double* d);
  *   K = -L_E L_B, of a built mesh without a PML frame (UE_ERR_ARG otherwise);
  *   log rho_hat = max_j (z_j + base_j).
  * ue_mlp_forward: z[n] for rows X[12*n]; bf16 = 1 tensor cores (BF16 in, FP32 accumulate),
- *   0 = FP32 debug path.  params: UE_MLP_PARAMS floats on the device.
+ *   0 = FP32 debug path.  params: UE_MLP_PARAMS floats on the device.  The tensor-core kernel's waits
+ *   are bounded (about a second): where one runs out the rows it still had to score hold NaN, and
+ *   the first of these calls but ue_rho_features to begin after that, on this device, returns
+ *   UE_ERR_TIMEOUT and does nothing else.  The first call to run it pins 64 bytes of host memory.
  * ue_mlp_backward: grad[UE_MLP_PARAMS] = sum over m rows of dz[i] * dz_i/dparams for rows[i]
  *   (same rounding as the forward); work holds m * UE_MLP_PARAMS floats.
  * ue_adam: one Adam step (t >= 1) on n floats.
  * ue_seg_argmax: per segment s of rows [off[s], off[s+1]): best = max (z + base), arg.
  * ue_rho_loss: dz[s] = 2 (best[s] - target[s]), loss[s] = (best[s] - target[s])^2.
  * All asynchronous on `stream`. */
+#define UE_MLP_TEST_TIMEOUT (-0x7FFFFFFF)   /* tests only, as bf16: 1 with a wait that runs out */
 int ue_rho_features(ue_mesh* m, float* X, float* base, void* stream);
 int ue_mlp_forward(const float* params, const float* X, int64_t n, int32_t bf16, float* z,
                    void* stream);

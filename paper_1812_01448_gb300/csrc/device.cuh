@@ -385,8 +385,11 @@ int mlp_n_params();
 cudaError_t launch_features(const double* xy, const int32_t* tri_nodes, const int32_t* tri_code,
                             const int32_t* tri_nb, const double* elen, const double* d, const double* S,
                             int64_t n_t, int64_t n_ei, float* X, float* base, cudaStream_t s);
-cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf16, float* z,
-                               cudaStream_t s);
+// err (device-visible host memory, or NULL): set when a bounded wait of the kernel runs out, which only
+// the kernel of mlp_forward_waits has; test: one of its waits does.
+bool mlp_forward_waits(const float* X, int64_t n, int bf16);
+cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf16, float* z, unsigned* err,
+                               bool test, cudaStream_t s);
 cudaError_t launch_mlp_backward(const float* P, const float* X, const int64_t* rows, const float* dz,
                                 int64_t m, int bf16, float* work, float* grad, cudaStream_t s);
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1,

@@ -379,7 +379,8 @@ __global__ void __launch_bounds__(NT, 1) k_mlp_fwd_bf16(const float* __restrict_
 // mma.sync per 16 rows bound it, 177 us.  Three or five groups, and layer 1 of the next tile computed
 // while the products run, change nothing (112, 113, 107): neither latency nor issue slots (44%) but
 // the pipes that the 16 mma.sync per 32 rows, ReLU and rounding share (ALU 50%, tensor 37%) are what is left.
-// Waits are bounded: when one runs out the group leaves its remaining scores NaN.
+// Waits are bounded: when one runs out the group leaves its remaining scores NaN and sets *err (host
+// memory; NULL: none).
 constexpr int kTcGroups = 4, kTcStages = 3, kTcRows = 128;
 constexpr uint32_t kTcTile = kTcRows * kD * 4;   // bytes of a full input tile
 static_assert(kTcTile % 16 == 0);
@@ -440,7 +441,8 @@ __device__ __forceinline__ __nv_bfloat16* tc_at(unsigned char* p, int row, int k
 }
 
 __global__ void __launch_bounds__(128 * kTcGroups, 1) k_mlp_fwd_tc(const float* __restrict__ P, const float* __restrict__ X,
-                                                                  int64_t n, float* __restrict__ z) {
+                                                                  int64_t n, float* __restrict__ z,
+                                                                  volatile unsigned* err, int test) {
     constexpr int G = kTcGroups, ST = kTcStages, NT = 128 * G;
     // tensor memory columns: the accumulators, h1 (two values per column) and the ones
     constexpr uint32_t kAcc = 0, kH1 = 64 * G, kOnes = 96 * G, kCols = 512;
@@ -458,6 +460,8 @@ __global__ void __launch_bounds__(128 * kTcGroups, 1) k_mlp_fwd_tc(const float* 
         for (int i = 0; i < ST; ++i) mbar_init(&S.full[wg][i], 1);
         mbar_init(&S.done[wg], 1);
         fence_mbar_init();
+        // tests only: one group also waits for bytes that no copy brings
+        if (test && tid == 0 && blockIdx.x == 0) asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], 16;" ::"r"(smem_addr(&S.full[0][0])) : "memory");
         for (int i = 0; i < ST; ++i)
             if (tile0 + i * stride < tiles) fetch(tile0 + i * stride, i);
     }
@@ -591,11 +595,16 @@ __global__ void __launch_bounds__(128 * kTcGroups, 1) k_mlp_fwd_tc(const float* 
     if (!ok) {   // a wait ran out: no scores, and the copies in flight end before their memory is given up
         for (int64_t k = tile; k < tiles; k += stride)
             if (k * kTcRows + wt < n) z[k * kTcRows + wt] = __int_as_float(0x7fffffff);
-        if (wt == 0)
+        if (wt == 0) {
             for (int i = 0; i < ST; ++i) {
                 mbar_wait(&S.full[wg][i], 0);
                 mbar_wait(&S.full[wg][i], 1);
             }
+            if (err) {
+                *err = 1u;
+                __threadfence_system();
+            }
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -1169,8 +1178,11 @@ cudaError_t launch_features(const double* xy, const int32_t* tri_nodes, const in
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf16, float* z,
-                               cudaStream_t s) {
+// Whether the forward on n rows takes the kernel with bounded waits.
+bool mlp_forward_waits(const float* X, int64_t n, int bf16) { return bf16 && n >= 32768 && ((uintptr_t)X & 15u) == 0; }
+
+cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf16, float* z, unsigned* err,
+                               bool test, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     if (bf16) {
         // one block per SM (a warp's registers hold the network); few tiles per warp: 8 warps, whose
@@ -1179,12 +1191,12 @@ cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf
         auto grid = [&](int nt) { return (unsigned)std::min<int64_t>((tiles + nt / 32 - 1) / (nt / 32), 152); };
         // From 32,768 rows of 16-byte aligned inputs layer 2 goes to tcgen05: 20k rows 9.9 us either way,
         // 40k 10.1 (10.9), 100k 10.5 (13.2), 1M 27 (45).
-        if (n >= 32768 && ((uintptr_t)X & 15u) == 0) {
+        if (mlp_forward_waits(X, n, bf16)) {
             const size_t smem = sizeof(TcSmem) + 1024;   // aligned to 1024 inside
             const cudaError_t e = cudaFuncSetAttribute(k_mlp_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             const int64_t blocks = (n + kTcRows * kTcGroups - 1) / (kTcRows * kTcGroups);
-            k_mlp_fwd_tc<<<(unsigned)std::min<int64_t>(blocks, 152), 128 * kTcGroups, smem, s>>>(P, X, n, z);
+            k_mlp_fwd_tc<<<(unsigned)std::min<int64_t>(blocks, 152), 128 * kTcGroups, smem, s>>>(P, X, n, z, err, test ? 1 : 0);
             return cudaGetLastError();
         }
         if (tiles < 152 * 8 * 32) k_mlp_fwd_bf16<256><<<grid(256), 256, 0, s>>>(P, X, n, z);

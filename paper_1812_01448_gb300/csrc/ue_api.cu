@@ -948,6 +948,61 @@ LearnedRes* learned_res() {
     return &r;
 }
 
+// The word in host memory that the network's forward pass sets when a bounded wait runs out; one per
+// device, made on its first use.  NULL when there is none to be had: the failure then shows as NaN only.
+struct MlpError {
+    std::atomic<unsigned*> host{nullptr};
+    unsigned* dev = nullptr;
+};
+std::mutex g_mlp_mu;
+MlpError g_mlp[kMaxDevices];
+
+MlpError* mlp_error() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    return &g_mlp[dev];
+}
+
+unsigned* mlp_error_word() {
+    MlpError* e = mlp_error();
+    if (!e || e->host.load(std::memory_order_acquire)) return e ? e->dev : nullptr;
+    std::lock_guard<std::mutex> lock(g_mlp_mu);
+    if (e->host.load(std::memory_order_relaxed)) return e->dev;
+    void *h = nullptr, *d = nullptr;
+    // a capture, here or on another thread, goes on
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (cudaHostAlloc(&h, 64, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) h = nullptr;
+    if (h && cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+        cudaFreeHost(h);
+        h = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!h) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    std::memset(h, 0, 64);
+    e->dev = (unsigned*)d;
+    e->host.store((unsigned*)h, std::memory_order_release);
+    return e->dev;
+}
+
+// A forward pass on this device has run out of time since this was last asked.
+bool mlp_timed_out() {
+    MlpError* e = mlp_error();
+    volatile unsigned* h = e ? e->host.load(std::memory_order_acquire) : nullptr;
+    if (!h || *h == 0u) return false;
+    *h = 0u;
+    return true;
+}
+
+#define UE_MLP_CHECK()                                                                                   \
+    do {                                                                                                 \
+        if (mlp_timed_out())                                                                             \
+            return fail(UE_ERR_TIMEOUT, "a wait of the network's forward pass ran out of time: rows of z are NaN"); \
+    } while (0)
+
 // Learned rho: one fused launch (features -> BF16 MLP -> max of z + base, max K_jj, max
 // Gershgorin bound, then the local Rayleigh quotient near the argmax triangle), synchronous.
 // Sets m->rho_hat, m->rho_lo, m->rho_hi.  Caller holds g_learned_mu.
@@ -2464,13 +2519,16 @@ int ue_rho_features(ue_mesh* m, float* X, float* base, void* stream) {
 
 int ue_mlp_forward(const float* params, const float* X, int64_t n, int32_t bf16, float* z, void* stream) {
     if (!params || !X || !z || n < 0) return fail(UE_ERR_ARG, "bad arguments");
-    UE_CUDA(ue::launch_mlp_forward(params, X, n, bf16 ? 1 : 0, z, (cudaStream_t)stream));
+    UE_MLP_CHECK();
+    unsigned* err = ue::mlp_forward_waits(X, n, bf16 ? 1 : 0) ? mlp_error_word() : nullptr;
+    UE_CUDA(ue::launch_mlp_forward(params, X, n, bf16 ? 1 : 0, z, err, bf16 == UE_MLP_TEST_TIMEOUT, (cudaStream_t)stream));
     return UE_OK;
 }
 
 int ue_mlp_backward(const float* params, const float* X, const int64_t* rows, const float* dz,
                     int64_t m, int32_t bf16, float* work, float* grad, void* stream) {
     if (!params || !X || !grad || m < 0 || (m > 0 && (!rows || !dz || !work))) return fail(UE_ERR_ARG, "bad arguments");
+    UE_MLP_CHECK();
     UE_CUDA(ue::launch_mlp_backward(params, X, rows, dz, m, bf16 ? 1 : 0, work, grad, (cudaStream_t)stream));
     return UE_OK;
 }
@@ -2478,6 +2536,7 @@ int ue_mlp_backward(const float* params, const float* X, const int64_t* rows, co
 int ue_adam(float* params, const float* grad, float* m1, float* m2, int32_t n, float lr, float beta1,
             float beta2, float eps, int32_t t, void* stream) {
     if (!params || !grad || !m1 || !m2 || n < 1 || t < 1) return fail(UE_ERR_ARG, "bad arguments");
+    UE_MLP_CHECK();
     UE_CUDA(ue::launch_adam(params, grad, m1, m2, n, lr, beta1, beta2, eps, t, (cudaStream_t)stream));
     return UE_OK;
 }
@@ -2485,12 +2544,14 @@ int ue_adam(float* params, const float* grad, float* m1, float* m2, int32_t n, f
 int ue_seg_argmax(const float* z, const float* base, const int64_t* off, int32_t n_seg, float* best,
                   int64_t* arg, void* stream) {
     if (!z || !base || !off || !best || !arg || n_seg < 0) return fail(UE_ERR_ARG, "bad arguments");
+    UE_MLP_CHECK();
     UE_CUDA(ue::launch_seg_argmax(z, base, off, n_seg, best, arg, (cudaStream_t)stream));
     return UE_OK;
 }
 
 int ue_rho_loss(const float* best, const float* target, int32_t n_seg, float* dz, float* loss, void* stream) {
     if (!best || !target || !dz || !loss || n_seg < 0) return fail(UE_ERR_ARG, "bad arguments");
+    UE_MLP_CHECK();
     UE_CUDA(ue::launch_rho_loss(best, target, n_seg, dz, loss, (cudaStream_t)stream));
     return UE_OK;
 }

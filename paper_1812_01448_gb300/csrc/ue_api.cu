@@ -624,7 +624,17 @@ int bake_source_mesh(ue_mesh* m, cudaStream_t s) {
     dm.grp_par = dm.gtab = nullptr;
     dm.n_src = (int64_t)m->src_k.size();
     dm.n_grp = 0;
-    if (dm.n_src == 0) return UE_OK;
+    if (dm.n_src == 0) {
+        // the tiles' counts of source edges: the pipelined kernel goes by them
+        ue::TileSet& ts = m->ts;
+        if (m->variant == UE_VARIANT_BLOCKED && m->tb.hdr && ts.max_src > 0) {
+            for (int64_t t = 0; t < ts.n_tiles; ++t) ts.hdr[t * ue::TileSet::kHdr + 8] = ts.hdr[t * ue::TileSet::kHdr + 9] = 0;
+            ts.max_src = 0;
+            UE_CUDA(cudaMemcpyAsync(m->tb.hdr, ts.hdr.data(), 4 * ts.hdr.size(), cudaMemcpyHostToDevice, s));
+            UE_CUDA(cudaStreamSynchronize(s));
+        }
+        return UE_OK;
+    }
     if (!m->is_batch) m->grp_par[0] = m->dt;   // a rebuild may have changed dt
     dm.n_grp = (int)(m->grp_par.size() / 4);
     const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;

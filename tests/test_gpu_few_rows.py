@@ -1,0 +1,36 @@
+"""The training kernels' forms for many segments, at the lines between the forms."""
+import numpy as np
+import pytest
+
+from test_gpu_training_kernels import _layers, lib  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_seg", [304, 305, 608, 609, 2432, 2433, 2440, 20_001])
+def test_argmax_of_many_segments(lib, n_seg):  # noqa: F811
+    """512 and 256 threads a segment, 128 (two segments a block) and a warp each (eight), with empty segments,
+    segments of one row and of several passes, ties, NaN and infinities."""
+    torch, ue, _ = lib
+    rng = np.random.default_rng(n_seg)
+    sizes = rng.choice([0, 1, 7, 31, 32, 33, 255, 256, 257, 300, 1025], n_seg)
+    sizes[n_seg // 2] = 9001
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    z = rng.integers(0, 40, off[-1]).astype(np.float32)
+    base = rng.integers(0, 3, off[-1]).astype(np.float32)
+    z[rng.integers(0, off[-1], 50)] = np.nan
+    base[rng.integers(0, off[-1], 50)] = -np.inf
+    z[rng.integers(0, off[-1], 5)] = np.inf
+    best = torch.full((n_seg + 1,), 7.0, device="cuda")
+    arg = torch.full((n_seg + 1,), 7, dtype=torch.int64, device="cuda")
+    ue.seg_argmax(torch.from_numpy(z).cuda(), torch.from_numpy(base).cuda(), torch.from_numpy(off).cuda(), best[:n_seg], arg[:n_seg])
+    with np.errstate(invalid="ignore"):
+        t = z + base
+    t[np.isnan(t)] = -np.inf
+    want_b, want_a = np.full(n_seg, -np.inf, np.float32), np.full(n_seg, -1, np.int64)
+    for s in range(n_seg):
+        seg = t[off[s]:off[s + 1]]
+        if seg.size and seg.max() > -np.inf:
+            want_b[s], want_a[s] = seg.max(), off[s] + int(np.argmax(seg))
+    assert np.array_equal(best.cpu().numpy()[:n_seg], want_b) and np.array_equal(arg.cpu().numpy()[:n_seg], want_a)
+    assert float(best[n_seg]) == 7.0 and int(arg[n_seg]) == 7

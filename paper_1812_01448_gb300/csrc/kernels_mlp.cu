@@ -254,6 +254,33 @@ __device__ __forceinline__ void mlp16(const PackedNet& N, uint32_t a0, uint32_t 
     s1 = x1;
 }
 
+// Forward on few rows: one warp per 16, the network packed in the block's shared memory.  A warp takes
+// a tile or two, and filling the registers of k_mlp_fwd_bf16 with the whole network took longer than
+// reading what a tile needs.
+__global__ void __launch_bounds__(128) k_mlp_fwd_few(const float* __restrict__ P, const float* __restrict__ X, int64_t n,
+                                                     float* __restrict__ z) {
+    __shared__ __align__(16) PackedNet net;
+    pack_net(net, P, threadIdx.x, blockDim.x);
+    __syncthreads();
+    const float b3 = net.b3[0];
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); tile * 16 < n; tile += warps) {
+        const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
+        auto xv = [&](int64_t r, int c) { return (r < n && c < kD) ? __ldg(X + r * kD + c) : 0.f; };
+        const uint32_t a0 = pack_bf16(xv(r0, 2 * t), xv(r0, 2 * t + 1));
+        const uint32_t a1 = pack_bf16(xv(r1, 2 * t), xv(r1, 2 * t + 1));
+        const uint32_t a2 = pack_bf16(xv(r0, 2 * t + 8), xv(r0, 2 * t + 9));
+        const uint32_t a3 = pack_bf16(xv(r1, 2 * t + 8), xv(r1, 2 * t + 9));
+        float s0, s1;
+        mlp16(net, a0, a1, a2, a3, s0, s1);
+        if (t == 0) {
+            if (r0 < n) z[r0] = s0 + b3;
+            if (r1 < n) z[r1] = s1 + b3;
+        }
+    }
+}
+
 // Forward on BF16 tensor cores (mma.sync m16n8k16, FP32 accumulation): one warp per 16 rows.  The
 // whole network sits in a warp's registers as B fragments (16 for layer 1, 64 for layer 2), so a
 // tile is its loads, its products and its ReLUs; the next tile's inputs are loaded a tile ahead.
@@ -1194,18 +1221,24 @@ cudaError_t launch_mlp_forward(const float* P, const float* X, int64_t n, int bf
                                bool test, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     if (bf16) {
-        // one block per SM (a warp's registers hold the network); few tiles per warp: 8 warps, whose
-        // start is shorter, else 12
         const int64_t tiles = (n + 15) / 16;
         auto grid = [&](int nt) { return (unsigned)std::min<int64_t>((tiles + nt / 32 - 1) / (nt / 32), 152); };
         // From 32,768 rows of 16-byte aligned inputs layer 2 goes to tcgen05: 20k rows 9.9 us either way,
-        // 40k 10.1 (10.9), 100k 10.5 (13.2), 1M 27 (45).
+        // 40k 10.1 (10.9), 100k 10.5 (13.2), 1M 27 (45).  Inputs off that alignment keep the network in
+        // registers from 50,000 rows, one block per SM: 8 warps, whose start is shorter, while a warp has
+        // few tiles, else 12.  Rows in a train of calls, in shared memory against registers: 16 rows
+        // 6.4 us (8.2), 20k 8.2 (10.2), 32k 8.3 (10.3), 50k 10.3 (10.3), 100k 16.4 (12.3).
         if (mlp_forward_waits(X, n, bf16)) {
             const size_t smem = sizeof(TcSmem) + 1024;   // aligned to 1024 inside
             const cudaError_t e = cudaFuncSetAttribute(k_mlp_fwd_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             const int64_t blocks = (n + kTcRows * kTcGroups - 1) / (kTcRows * kTcGroups);
             k_mlp_fwd_tc<<<(unsigned)std::min<int64_t>(blocks, 152), 128 * kTcGroups, smem, s>>>(P, X, n, z, err, test ? 1 : 0);
+            return cudaGetLastError();
+        }
+        if (n < 50000) {
+            const unsigned blocks = (unsigned)((tiles + 3) / 4);
+            k_mlp_fwd_few<<<blocks, 128, 0, s>>>(P, X, n, z);
             return cudaGetLastError();
         }
         if (tiles < 152 * 8 * 32) k_mlp_fwd_bf16<256><<<grid(256), 256, 0, s>>>(P, X, n, z);

@@ -1,4 +1,4 @@
-"""The training kernels' forms for many segments, at the lines between the forms."""
+"""The training kernels' forms for few rows and many segments, at the lines between the forms."""
 import numpy as np
 import pytest
 
@@ -34,3 +34,19 @@ def test_argmax_of_many_segments(lib, n_seg):  # noqa: F811
             want_b[s], want_a[s] = seg.max(), off[s] + int(np.argmax(seg))
     assert np.array_equal(best.cpu().numpy()[:n_seg], want_b) and np.array_equal(arg.cpu().numpy()[:n_seg], want_a)
     assert float(best[n_seg]) == 7.0 and int(arg[n_seg]) == 7
+
+
+@pytest.mark.parametrize("n", [1, 15, 17, 64, 65, 32_767, 49_999, 50_000, 50_001])
+@pytest.mark.parametrize("shift", [1, 2])
+def test_forward_off_the_alignment(lib, n, shift):  # noqa: F811
+    """Around the line between the network in shared memory and in registers; bounds as for the other
+    forms: an h1 that lies within an accumulation error of a BF16 midpoint may round the other way."""
+    torch, ue, p = lib
+    flat = torch.randn(n * 12 + 2, generator=torch.Generator().manual_seed(n))
+    X = flat[shift:shift + n * 12].reshape(n, 12)
+    z = torch.full((n + 1,), 7.0, device="cuda")
+    ue.mlp_forward(p.cuda(), flat.cuda()[shift:shift + n * 12].reshape(n, 12), z[:n], bf16=True)
+    ref = _layers(torch, p, X, True)[-1]
+    err = (z[:n].cpu().double() - ref).abs()
+    assert err.max() < 1e-3 * ref.abs().max() + 1e-3 and err.median() < 2e-6
+    assert z[n] == 7.0

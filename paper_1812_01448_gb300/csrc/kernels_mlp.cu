@@ -1027,8 +1027,10 @@ __device__ __forceinline__ float rb(float x, int bf16) {
 // weights per thread and its unit's biases) over its rows, four rows at a time: 64 threads, one per
 // hidden unit, take a row forward and back, then all 256 add the four outer products.  One sum per
 // block is written; with one gradient row per mesh row (20 KB) the sum over them read it all
-// again, one thread per parameter in a row: 19 + 16 us on 400 rows, milliseconds on 20,000, against
-// 16 + 4 us here on 400 rows (bound by the latency of a row's chain of sums).
+// again, one thread per parameter in a row: 37 us together on 400 rows, milliseconds on 20,000, against
+// 13 here on 400 rows (bound by the latency of the weights and of a row's chain of sums).  Up to four rows
+// are one block, which writes the gradient itself: 8.2 us for a row, 14.4 with the sum over blocks and the
+// weights loaded as they were stored.
 constexpr int kBwdRows = 4, kBwdThreads = kH * kBwdRows, kW2P = kH + 1;   // padded row: no bank conflicts
 __global__ void __launch_bounds__(kBwdThreads) k_mlp_bwd(const float* __restrict__ P, const float* __restrict__ X,
                                                          const int64_t* __restrict__ rows, const float* __restrict__ dz,
@@ -1036,8 +1038,22 @@ __global__ void __launch_bounds__(kBwdThreads) k_mlp_bwd(const float* __restrict
     __shared__ float w1[kH * (kD + 1)], w2[kH * kW2P], b1[kH], b2[kH], w3[kH];
     __shared__ float x[kBwdRows][kD], h1[kBwdRows][kH], h2[kBwdRows][kH], d1[kBwdRows][kH], d2[kBwdRows][kH], dzr[kBwdRows];
     const int tid = threadIdx.x, o = tid & (kH - 1), p = tid / kH;   // hidden unit, row of the group
-    for (int i = tid; i < kH * kD; i += kBwdThreads) w1[(i / kD) * (kD + 1) + i % kD] = rb(P[kOffW1 + i], bf16);
-    for (int i = tid; i < kH * kH; i += kBwdThreads) w2[(i / kH) * kW2P + i % kH] = rb(P[kOffW2 + i], bf16);
+    // all of a thread's weights in flight at once: a call on few rows is this latency and a row's
+    float v1[kH * kD / kBwdThreads], v2[kH * kH / kBwdThreads];
+#pragma unroll
+    for (int u = 0; u < kH * kD / kBwdThreads; ++u) v1[u] = __ldg(P + kOffW1 + tid + u * kBwdThreads);
+#pragma unroll
+    for (int u = 0; u < kH * kH / kBwdThreads; ++u) v2[u] = __ldg(P + kOffW2 + tid + u * kBwdThreads);
+#pragma unroll
+    for (int u = 0; u < kH * kD / kBwdThreads; ++u) {
+        const int i = tid + u * kBwdThreads;
+        w1[(i / kD) * (kD + 1) + i % kD] = rb(v1[u], bf16);
+    }
+#pragma unroll
+    for (int u = 0; u < kH * kH / kBwdThreads; ++u) {
+        const int i = tid + u * kBwdThreads;
+        w2[(i / kH) * kW2P + i % kH] = rb(v2[u], bf16);
+    }
     if (tid < kH) {
         b1[tid] = P[kOffB1 + tid];
         b2[tid] = P[kOffB2 + tid];
@@ -1255,8 +1271,8 @@ cudaError_t launch_mlp_backward(const float* P, const float* X, const int64_t* r
     // at most two blocks per SM; no more shares than the m gradient rows `work` holds
     const int64_t groups = (m + kBwdRows - 1) / kBwdRows;
     const int blocks = (int)(groups < 304 ? groups : 304);
-    k_mlp_bwd<<<blocks, kBwdThreads, 0, s>>>(P, X, rows, dz, m, bf16, work);
-    k_colsum<<<(kNParams + kSumParams - 1) / kSumParams, kSumParams * kSumSlices, 0, s>>>(work, blocks, grad);
+    k_mlp_bwd<<<blocks, kBwdThreads, 0, s>>>(P, X, rows, dz, m, bf16, blocks > 1 ? work : grad);
+    if (blocks > 1) k_colsum<<<(kNParams + kSumParams - 1) / kSumParams, kSumParams * kSumSlices, 0, s>>>(work, blocks, grad);
     return cudaGetLastError();
 }
 

@@ -50,3 +50,22 @@ def test_forward_off_the_alignment(lib, n, shift):  # noqa: F811
     err = (z[:n].cpu().double() - ref).abs()
     assert err.max() < 1e-3 * ref.abs().max() + 1e-3 and err.median() < 2e-6
     assert z[n] == 7.0
+
+
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 8])
+def test_backward_of_one_block_and_two(lib, m):  # noqa: F811
+    """One block writes the gradient itself; the sum over several blocks' shares adds the same rows."""
+    torch, ue, p = lib
+    g = torch.Generator().manual_seed(m)
+    X, rows = torch.randn(50, 12, generator=g).cuda(), torch.randint(0, 50, (m,), generator=g).cuda()
+    dz, k = torch.randn(m, generator=g).cuda(), p.shape[0]
+    grad, part, work = torch.full((k,), 7.0, device="cuda"), torch.zeros(k, device="cuda"), torch.full((m * k,), 3.0, device="cuda")
+    ue.mlp_backward(p.cuda(), X, rows, dz, grad, work)
+    total = torch.zeros(k, dtype=torch.float64)
+    size = torch.zeros(k, dtype=torch.float64)
+    for i in range(m):
+        ue.mlp_backward(p.cuda(), X, rows[i:i + 1], dz[i:i + 1], part, work)
+        total += part.cpu().double()
+        size += part.cpu().double().abs()
+    # the same products, at most m + 1 FP32 additions each
+    assert ((grad.cpu().double() - total).abs() <= (m + 1) * 2.0 ** -24 * size).all()

@@ -475,7 +475,7 @@ cudaError_t modes_run(const int2* rl, const int4* tri, const double* elen, const
     // start: the random block made S-orthonormal
     if ((e = k.orthonormalize(V, W)) != cudaSuccess || (*lost_rank = k.lost)) return e;
     std::swap(V, W);
-    int p = 1;
+    int p = 1, last = 1;
     for (int it = 0; it < iters;) {
         p = std::min(p, iters - it);
         const double* X = V;   // V stays: a block that lost rank over p products is taken again one by one
@@ -495,12 +495,16 @@ cudaError_t modes_run(const int2* rl, const int4* tri, const double* elen, const
             continue;
         }
         it += p;
+        last = p;
         std::swap(V, Y == W ? W : W2);
         p = products_until_qr(k.R, m, p);
     }
-    // once more, now near identity: columns S-orthonormal to rounding for Rayleigh-Ritz
-    if ((e = k.orthonormalize(V, W)) != cudaSuccess || (*lost_rank = k.lost)) return e;
-    std::swap(V, W);
+    // After several products once more, now near identity: columns S-orthonormal to rounding for
+    // Rayleigh-Ritz, as they are after one (on 2k triangles this is 20 of the 150 us of a single iteration)
+    if (last > 1) {
+        if ((e = k.orthonormalize(V, W)) != cudaSuccess || (*lost_rank = k.lost)) return e;
+        std::swap(V, W);
+    }
     // Rayleigh-Ritz: H = V^T S K V, its eigenvectors rotate V into the modes
     k.product(V, W);
     if ((e = k.gram(V, W)) != cudaSuccess) return e;

@@ -65,6 +65,7 @@ struct RxDev {
 // node of more is listed on the host.
 constexpr int kRxValence = 32;
 constexpr uint8_t kSeed = 1, kLook = 2;
+constexpr int64_t kRxMarked = 384;
 
 // 1/|w| and |w| of w^2 = n2: one Heron step on n2 rsqrt(n2) gives the root to about half an ulp, so
 // springs and caps keep the precision of a square root and a division at the cost of one rsqrt.
@@ -667,6 +668,9 @@ int mesh_relax(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, co
         if (e == cudaSuccess && r != cudaSuccess) e = r;
     };
     const int64_t n_slots = 3 * nt;
+    // Marks and neighbours of few triangles are sooner found on the host (about 0.1 us a triangle) than
+    // launched, copied and waited for (25 us)
+    const bool marked = flip_every > 0 && nt >= kRxMarked;
     auto blocks = [](int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); };
     int32_t ctl[4] = {};
     // after a change of t: the lists of every node and, where flips follow, the neighbours
@@ -678,7 +682,7 @@ int mesh_relax(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, co
         k_rx_offsets<<<blocks(nn, kRxThreads), kRxThreads, 0, s>>>(a, nn);
         k_rx_fill<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, n_slots);
         k_rx_lists<<<blocks(nn, kRxStepThreads), kRxStepThreads, 0, s>>>(a, nn);
-        if (flip_every > 0) k_rx_nb<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, n_slots);
+        if (marked) k_rx_nb<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, n_slots);
         ck(cudaGetLastError());
         ck(cudaMemcpyAsync(ctl, a.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, s));
         ck(cudaStreamSynchronize(s));   // t may change after this
@@ -711,7 +715,7 @@ int mesh_relax(const double* xy, int64_t nn, const int32_t* tris, int64_t nt, co
         ck(cudaGetLastError());
         std::swap(a.x0, a.x1);
         if (flip_every > 0 && (it + 1) % flip_every == 0 && e == cudaSuccess) {
-            const bool listed = ctl[1] == 0 && ctl[2] == 0;
+            const bool listed = marked && ctl[1] == 0 && ctl[2] == 0;
             ck(cudaMemcpyAsync(x.data(), a.x0, 16 * nn, cudaMemcpyDeviceToHost, s));
             if (listed) {
                 k_rx_marks<<<blocks(n_slots, kRxThreads), kRxThreads, 0, s>>>(a, a.x0, n_slots);

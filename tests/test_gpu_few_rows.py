@@ -1,8 +1,11 @@
-"""The training kernels' forms for few rows and many segments, at the lines between the forms."""
+"""The training kernels' forms for few rows, few triangles and many segments, at the lines between the forms."""
 import numpy as np
 import pytest
 
+import meshgen
+from oracle import relax
 from test_gpu_training_kernels import _layers, lib  # noqa: F401
+from test_oracle_relax import _scramble
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +72,19 @@ def test_backward_of_one_block_and_two(lib, m):  # noqa: F811
         size += part.cpu().double().abs()
     # the same products, at most m + 1 FP32 additions each
     assert ((grad.cpu().double() - total).abs() <= (m + 1) * 2.0 ** -24 * size).all()
+
+
+@pytest.mark.parametrize("points", [60, 180, 195, 205, 230])
+def test_relaxation_around_the_line_for_host_marks(lib, points):  # noqa: F811
+    """384 triangles: below, the flips' neighbours and marks are made on the host."""
+    _, ue, _ = lib
+    ms = meshgen.random_delaunay(points, seed=points)
+    tris = _scramble(ms.xy, relax.orient_ccw(ms.xy, ms.tris), points // 3, seed=3).astype(np.int32)
+    h = np.full(len(ms.xy), 1.2 / points ** 0.5)
+    x, t, k = ue.mesh_relax(ms.xy, tris, 6, flip_every=2, h_nodes=h)
+    y, u, f = ms.xy, tris, 0
+    for _ in range(3):
+        y, u, _ = ue.mesh_relax(y, u, 2, flip_every=0, h_nodes=h)
+        u, n = ue.mesh_flip(y, u)
+        f += n
+    assert k == f > 0 and np.array_equal(t, u) and np.array_equal(x, y)

@@ -266,6 +266,7 @@ struct FlowDev {
     double* epart = nullptr;      // [kFlowChecks * grid] energy sums of a launch's checks, then
                                   // kFlowChecks counters (zero between launches)
     int skip = -1;                // tests only: this CTA returns at once
+    bool planned = false;         // the plan has been made, and fits
 };
 // n_fc: cells of a PML frame stepped with the mesh.  False when the mesh does not fit.
 bool flow_shape(int64_t n_t, int64_t n_fc, bool f64, int sms, FlowDev& fl);

@@ -118,6 +118,8 @@ struct ue_mesh {
     // plasma and source, kept on the host so that a rebuild can re-bake them
     std::vector<double> plasma_n;
     double plasma_nu = 0;
+    void* src_block = nullptr;        // the source's device arrays
+    bool src_baked = false;           // they, and what follows from them, are made
     std::vector<int32_t> src_k;       // stored edge ids
     std::vector<double> src_amp;
     std::vector<int32_t> src_grp;     // source group of each entry (0 for a single mesh)
@@ -537,7 +539,11 @@ int bake_plasma(ue_mesh* m, cudaStream_t s) {
     return UE_OK;
 }
 
-int bake_source_mesh(ue_mesh* m, cudaStream_t s);
+struct SourceUpload {
+    std::vector<char> block;
+    std::vector<int32_t> rec;
+};
+int bake_source_mesh(ue_mesh* m, cudaStream_t s, SourceUpload& up);
 
 // The region of a framed blocked mesh: coefficients again (the mesh's cU carries the source
 // flags) and its own table {local edge, source index}; the rest of the source state is the
@@ -562,7 +568,7 @@ int region_sources(ue_mesh* m, cudaStream_t s) {
     for (size_t i = 0; i < m->src_k.size(); ++i) src_of[m->src_k[i]] = (int32_t)i;
     std::vector<int32_t> lk, li;
     const std::vector<int64_t>& eg = m->reg_host.egid;
-    for (size_t l = 0; l < eg.size(); ++l)
+    for (size_t l = 0; l < eg.size() && g.n_src > 0; ++l)
         if (src_of[eg[l]] >= 0) {
             lk.push_back((int32_t)l);
             li.push_back(src_of[eg[l]]);
@@ -589,15 +595,20 @@ int region_sources(ue_mesh* m, cudaStream_t s) {
     return UE_OK;
 }
 
+// The source on the device, and what follows from it: the resident step's plan, the tiles' records, the
+// region's table.  One wait for all but the last.  Without memory the mesh is left with no source.
 int bake_source(ue_mesh* m, cudaStream_t s) {
-    int rc = bake_source_mesh(m, s);
-    if (rc != UE_OK) return rc;
+    if (m->src_baked && m->dm.n_src == 0 && m->src_k.empty()) return UE_OK;   // none before, none now
+    SourceUpload up;   // until the copies are done
+    const int rc = bake_source_mesh(m, s, up);
+    if (rc != UE_OK && rc != UE_ERR_ALLOC) return rc;
+    const std::string why = g_err;
+    m->src_baked = true;
+    unsigned over = 0;
     if (m->flow.grid > 0) {
-        unsigned over = 0;
         UE_CUDA(ue::launch_flow_plan(m->flow, m->dm, s));
-        UE_CUDA(cudaMemcpyAsync(&over, m->flow.ctl + 3, 4, cudaMemcpyDeviceToHost, s));
-        UE_CUDA(cudaStreamSynchronize(s));
-        if (over) m->flow.grid = 0;   // neighbours too scattered: this mesh keeps its launches
+        // which neighbours are remote does not depend on the source: looked at once
+        if (!m->flow.planned) UE_CUDA(cudaMemcpyAsync(&over, m->flow.ctl + 3, 4, cudaMemcpyDeviceToHost, s));
     }
     if (m->variant == UE_VARIANT_BLOCKED && m->tb.erec) {
         // the tile records carry the source flags of the coefficients (the pipelined kernel
@@ -605,105 +616,113 @@ int bake_source(ue_mesh* m, cudaStream_t s) {
         UE_CUDA(ue::launch_tb_fill(m->tb, m->dm, s));
         if (m->tb.frec) UE_CUDA(ue::launch_tbf_fill(m->tb, m->dm, s));
         m->tb.max_src = m->ts.max_src;
-        UE_CUDA(cudaStreamSynchronize(s));
     }
-    if (!m->has_reg) return rc;
-    return region_sources(m, s);
+    UE_CUDA(cudaStreamSynchronize(s));
+    m->flow.planned = m->flow.grid > 0;
+    if (over) m->flow.grid = 0;   // neighbours too scattered: this mesh keeps its launches
+    const int rrc = m->has_reg ? region_sources(m, s) : UE_OK;
+    return rc != UE_OK ? fail(rc, why) : rrc;
 }
 
-int bake_source_mesh(ue_mesh* m, cudaStream_t s) {
+// Everything of the source in one block with one upload (an array each took up to 30 us of a call's 75).
+int bake_source_mesh(ue_mesh* m, cudaStream_t s, SourceUpload& up) {
     DevMesh& dm = m->dm;
-    if (dm.n_src > 0 && dm.src_k) UE_CUDA(ue::launch_source_flags(dm, dm.src_k, dm.n_src, false, s));
+    if (dm.n_src > 0) UE_CUDA(ue::launch_source_flags(dm, dm.src_k, dm.n_src, false, s));
     UE_CUDA(cudaStreamSynchronize(s));
-    for (void* p : {(void*)dm.src_k, (void*)dm.src_grp, dm.src_c, (void*)dm.src_hash,
-                    (void*)dm.grp_par, (void*)dm.gtab})
-        dev_release(m, p, s);
+    dev_release(m, m->src_block, s);
+    m->src_block = nullptr;
     dm.src_k = dm.src_grp = nullptr;
     dm.src_c = nullptr;
     dm.src_hash = nullptr;
     dm.grp_par = dm.gtab = nullptr;
-    dm.n_src = (int64_t)m->src_k.size();
-    dm.n_grp = 0;
-    if (dm.n_src == 0) {
-        // the tiles' counts of source edges: the pipelined kernel goes by them
-        ue::TileSet& ts = m->ts;
-        if (m->variant == UE_VARIANT_BLOCKED && m->tb.hdr && ts.max_src > 0) {
-            for (int64_t t = 0; t < ts.n_tiles; ++t) ts.hdr[t * ue::TileSet::kHdr + 8] = ts.hdr[t * ue::TileSet::kHdr + 9] = 0;
-            ts.max_src = 0;
-            UE_CUDA(cudaMemcpyAsync(m->tb.hdr, ts.hdr.data(), 4 * ts.hdr.size(), cudaMemcpyHostToDevice, s));
-            UE_CUDA(cudaStreamSynchronize(s));
-        }
-        return UE_OK;
-    }
-    if (!m->is_batch) m->grp_par[0] = m->dt;   // a rebuild may have changed dt
-    dm.n_grp = (int)(m->grp_par.size() / 4);
-    const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;
-    int32_t *k = nullptr, *grp = nullptr;
-    double *amp = nullptr, *par = nullptr, *gt = nullptr;
-    void* c = nullptr;
-    if (!alloc_into(m, k, dm.n_src, 4, s) || !alloc_into(m, amp, dm.n_src, 8, s) ||
-        !alloc_into(m, c, dm.n_src, esz, s) || !alloc_into(m, grp, dm.n_src, 4, s) ||
-        !alloc_into(m, par, m->grp_par.size(), 8, s) ||
-        !alloc_into(m, gt, (size_t)dm.gtab_size * dm.n_grp, 8, s))
-        return fail(UE_ERR_ALLOC, "source arrays");
-    UE_CUDA(cudaMemcpyAsync(k, m->src_k.data(), 4 * dm.n_src, cudaMemcpyHostToDevice, s));
-    UE_CUDA(cudaMemcpyAsync(amp, m->src_amp.data(), 8 * dm.n_src, cudaMemcpyHostToDevice, s));
-    UE_CUDA(cudaMemcpyAsync(grp, m->src_grp.data(), 4 * dm.n_src, cudaMemcpyHostToDevice, s));
-    UE_CUDA(cudaMemcpyAsync(par, m->grp_par.data(), 8 * m->grp_par.size(), cudaMemcpyHostToDevice, s));
-    dm.src_k = k;
-    dm.src_c = c;
-    dm.src_grp = grp;
-    dm.grp_par = par;
-    dm.gtab = gt;
-    UE_CUDA(ue::launch_source_coeff(dm, amp, m->d_elen, s));
-    UE_CUDA(ue::launch_source_flags(dm, k, dm.n_src, true, s));
+    dm.n_src = dm.n_grp = 0;
+    int64_t n = (int64_t)m->src_k.size();
+    if (n > 0 && !m->is_batch) m->grp_par[0] = m->dt;   // a rebuild may have changed dt
+    const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4, n_grp = m->grp_par.size() / 4;
     // open-addressing table {stored edge id, source index}, load factor <= 1/2
     int bits = 4;
-    while ((int64_t(1) << bits) < 2 * dm.n_src) ++bits;
+    while ((int64_t(1) << bits) < 2 * n) ++bits;
     const uint32_t size = 1u << bits;
-    std::vector<int32_t> tab(2 * (size_t)size, -1);
-    for (int64_t i = 0; i < dm.n_src; ++i) {
-        uint32_t h = ((uint32_t)m->src_k[i] * 2654435761u) >> (32 - bits);
-        while (tab[2 * h] != -1) h = (h + 1) & (size - 1);
-        tab[2 * h] = m->src_k[i];
-        tab[2 * h + 1] = (int32_t)i;
+    size_t bytes = 0;
+    auto part = [&](size_t b) {
+        const size_t at = bytes;
+        bytes += (b + 255) / 256 * 256;
+        return at;
+    };
+    const size_t amp = part(8 * n), par = part(32 * n_grp), hash = part(8 * (size_t)size), k = part(4 * n), grp = part(4 * n);
+    const size_t sent = bytes, c = part(esz * n), gtab = part(8 * n_grp * (size_t)dm.gtab_size);
+    int rc = UE_OK;
+    char* b = nullptr;
+    if (n > 0 && !alloc_into(m, b, bytes, 1, s)) {
+        rc = fail(UE_ERR_ALLOC, "source arrays");
+        n = 0;
     }
-    int2* dh = nullptr;
-    if (!alloc_into(m, dh, size, 8, s)) return fail(UE_ERR_ALLOC, "source table");
-    UE_CUDA(cudaMemcpyAsync(dh, tab.data(), 8 * (size_t)size, cudaMemcpyHostToDevice, s));
-    dm.src_hash = dh;
-    dm.src_bits = bits;
-    UE_CUDA(cudaStreamSynchronize(s));
-    dev_release(m, amp, s);
-    if (m->variant == UE_VARIANT_BLOCKED) {
-        // per-tile source records: (local edge, source index) for every local copy of a source edge
-        std::vector<int32_t> src_of(m->hm.n_ei, -1);
-        for (size_t i = 0; i < m->src_k.size(); ++i) src_of[m->src_k[i]] = (int32_t)i;
-        std::vector<int32_t> rec;
+    if (m->variant == UE_VARIANT_BLOCKED && (n > 0 || m->tb.tsrc)) {
+        // per-tile source records: (local edge, source index) for every local copy of a source edge; none,
+        // and their counts zero, without a source (the pipelined kernel goes by the counts)
+        dev_release(m, m->tb.tsrc, s);
+        m->tb.tsrc = nullptr;
         ue::TileSet& ts = m->ts;
-        int maxn = 0;
-        for (int64_t t = 0; t < ts.n_tiles; ++t) {
-            int32_t* h = &ts.hdr[t * ue::TileSet::kHdr];
-            h[8] = (int32_t)(rec.size() / 2);
-            const int64_t off = h[7], nel = h[5];
-            for (int64_t l = 0; l < nel; ++l) {
-                const int32_t src = src_of[ts.erec[4 * (off + l)]];
-                if (src >= 0) {
-                    rec.push_back((int32_t)l);
-                    rec.push_back(src);
+        auto records = [&]() {
+            std::vector<int32_t> src_of(n > 0 ? m->hm.n_ei : 0, -1);
+            for (int64_t i = 0; i < n; ++i) src_of[m->src_k[i]] = (int32_t)i;
+            std::vector<int32_t>& rec = up.rec;
+            rec.clear();
+            int maxn = 0;
+            for (int64_t t = 0; t < ts.n_tiles; ++t) {
+                int32_t* h = &ts.hdr[t * ue::TileSet::kHdr];
+                h[8] = (int32_t)(rec.size() / 2);
+                const int64_t off = h[7], nel = n > 0 ? h[5] : 0;
+                for (int64_t l = 0; l < nel; ++l) {
+                    const int32_t src = src_of[ts.erec[4 * (off + l)]];
+                    if (src >= 0) {
+                        rec.push_back((int32_t)l);
+                        rec.push_back(src);
+                    }
                 }
+                h[9] = (int32_t)(rec.size() / 2) - h[8];
+                if (h[9] > maxn) maxn = h[9];
             }
-            h[9] = (int32_t)(rec.size() / 2) - h[8];
-            if (h[9] > maxn) maxn = h[9];
+            ts.max_src = maxn;
+        };
+        records();
+        if (n > 0 && !alloc_into(m, m->tb.tsrc, up.rec.size() / 2 + 1, 8, s)) {
+            rc = fail(UE_ERR_ALLOC, "tile source records");
+            dev_release(m, b, s);
+            n = 0;
+            records();
         }
-        ts.max_src = maxn;
-        int2* d = nullptr;
-        if (!alloc_into(m, d, rec.size() / 2 + 1, 8, s)) return fail(UE_ERR_ALLOC, "tile source records");
-        if (!rec.empty()) UE_CUDA(cudaMemcpyAsync(d, rec.data(), 4 * rec.size(), cudaMemcpyHostToDevice, s));
-        m->tb.tsrc = d;
+        if (!up.rec.empty()) UE_CUDA(cudaMemcpyAsync(m->tb.tsrc, up.rec.data(), 4 * up.rec.size(), cudaMemcpyHostToDevice, s));
         UE_CUDA(cudaMemcpyAsync(m->tb.hdr, ts.hdr.data(), 4 * ts.hdr.size(), cudaMemcpyHostToDevice, s));
     }
-    UE_CUDA(cudaStreamSynchronize(s));
+    if (n == 0) return rc;
+    up.block.assign(sent, 0);
+    char* h = up.block.data();
+    std::memcpy(h + amp, m->src_amp.data(), 8 * n);
+    std::memcpy(h + par, m->grp_par.data(), 32 * n_grp);
+    std::memcpy(h + k, m->src_k.data(), 4 * n);
+    std::memcpy(h + grp, m->src_grp.data(), 4 * n);
+    int32_t* tab = reinterpret_cast<int32_t*>(h + hash);
+    std::fill(tab, tab + 2 * (size_t)size, -1);
+    for (int64_t i = 0; i < n; ++i) {
+        uint32_t e = ((uint32_t)m->src_k[i] * 2654435761u) >> (32 - bits);
+        while (tab[2 * e] != -1) e = (e + 1) & (size - 1);
+        tab[2 * e] = m->src_k[i];
+        tab[2 * e + 1] = (int32_t)i;
+    }
+    UE_CUDA(cudaMemcpyAsync(b, h, sent, cudaMemcpyHostToDevice, s));
+    m->src_block = b;
+    dm.n_src = n;
+    dm.n_grp = (int)n_grp;
+    dm.src_k = reinterpret_cast<int32_t*>(b + k);
+    dm.src_grp = reinterpret_cast<int32_t*>(b + grp);
+    dm.src_c = b + c;
+    dm.src_hash = reinterpret_cast<int2*>(b + hash);
+    dm.src_bits = bits;
+    dm.grp_par = reinterpret_cast<double*>(b + par);
+    dm.gtab = reinterpret_cast<double*>(b + gtab);
+    UE_CUDA(ue::launch_source_coeff(dm, reinterpret_cast<const double*>(b + amp), m->d_elen, s));
+    UE_CUDA(ue::launch_source_flags(dm, dm.src_k, n, true, s));
     return UE_OK;
 }
 
@@ -1523,6 +1542,8 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     m->d_xbad = nullptr;
     m->built = false;
     m->dm = DevMesh();
+    m->src_block = nullptr;
+    m->src_baked = false;
     m->tb = ue::TBDev();
     m->flow = ue::FlowDev();
     m->fd = ue::FrameDev();

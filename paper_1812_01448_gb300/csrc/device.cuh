@@ -232,6 +232,8 @@ cudaError_t launch_tbf1(const TBDev& t, const DevMesh& m, long long n_steps, int
 int tb_kernel_used(const TBDev& t, const DevMesh& m);
 // whether launch_tb runs the pipelined persistent form k_tbp for these tiles
 bool tb_pipelined(int max_tri_loc, int max_edge_loc, int threads, bool plasma);
+// triangle slots per thread of the 512-thread kernels (4, 6 or 8) when every tile runs at once, else 0
+int tb_one_wave(const TBDev& t);
 cudaError_t launch_tb_fill(const TBDev& t, const DevMesh& m, cudaStream_t s);
 // k steps of the blocked kernel reading buffer `cur`, writing buffer cur ^ 1; the source uses
 // g-table entries gbase .. gbase + k - 1.

@@ -776,6 +776,12 @@ bool tb_pipelined(int max_tri_loc, int max_edge_loc, int threads, bool plasma) {
     return threads != 1024 && ts > 0;
 }
 
+int tb_one_wave(const TBDev& t) {
+    if (t.threads == 1024 || t.n_tiles == 0 || t.n_tiles > t.sms) return 0;
+    if (t.max_tri_loc <= 4 * kNT && t.max_edge_loc <= 6 * kNT) return 4;
+    return t.max_tri_loc <= 6 * kNT && t.max_edge_loc <= 9 * kNT ? 6 : 8;
+}
+
 cudaError_t launch_tb_fill(const TBDev& t, const DevMesh& m, cudaStream_t s) {
     const int64_t n = t.n_trec > t.n_erec ? t.n_trec : t.n_erec;
     if (n == 0) return cudaSuccess;

@@ -1248,16 +1248,28 @@ int flush_step(ue_mesh* m, cudaStream_t s) {
     return UE_OK;
 }
 
-// Whether calls of *unit steps (a graph chunk, the steps between the watchdog checks of the launches)
-// or more run resident; shorter ones launch step by step.
-bool runs_resident(const ue_mesh* m, int64_t* unit) {
-    *unit = m->variant == UE_VARIANT_BLOCKED ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
+// The fewest steps of a call that runs resident, at least *unit (a graph chunk, the steps between the
+// watchdog checks of the launches); 0: none does.  A resident call takes 20 to 25 us and, on a mesh of
+// up to 100k triangles, 1.0 to 1.2 us per step.  That is less than the plain launches at any length, and
+// than blocked ones too but where all the tiles run at once: then a launch of k steps on small ones takes
+// about 2.7 + 0.7 k us (with a source 1.5 times that) and a call 10.  Measured, launches against resident:
+// 9.8k triangles in tiles of 1,000, k = 8: 32 steps 45 us (57), 256 steps 289 (313); 90k: 32 steps 47 (57),
+// 256 steps 290 (316); k = 4 on 5k: 32 steps 53 (58), 64 steps 98 (95); with a source, k = 8, 22k in tiles
+// of 256: 32 steps 61 (64), 64 steps 111 (99).  In tiles of 1,400 to 2,000, k = 8: 45k 32 steps 54 (59),
+// 64 steps 98 (96), 256 steps 356 (313); 2.6k, where a CTA has 32 triangles, 256 steps 342 (362).
+int64_t resident_from(const ue_mesh* m, int64_t* unit) {
+    const bool blocked = m->variant == UE_VARIANT_BLOCKED;
+    *unit = blocked ? (int64_t)tb_chunk_launches(m) * m->block_depth : m->graph_chunk;
     // with the watchdog on a launch takes whole units
-    return ue::flow_takes(m->flow, m->dm) && (m->watchdog_every <= 0 || *unit <= ue::kFlowSteps);
+    if (!ue::flow_takes(m->flow, m->dm) || (m->watchdog_every > 0 && *unit > ue::kFlowSteps)) return 0;
+    if (!blocked || m->has_reg || m->block_depth < 4) return *unit;
+    const int slots = ue::tb_one_wave(m->tb);
+    const bool deep = m->block_depth >= 6 && m->dm.n_src == 0;
+    if (deep && (slots == 4 || (slots == 6 && m->hm.n_tris <= 4096))) return 0;
+    return slots == 4 || (deep && slots == 6) ? std::max<int64_t>(*unit, 64) : *unit;
 }
 
-// n steps by the resident kernel, in place in the current field buffer, for a mesh that runs_resident
-// with `unit`.  *used is false, and nothing stepped, when the device cannot hold the launch's CTAs at
+// n steps by the resident kernel, in place in the current field buffer (resident_from).  *used is false, and nothing stepped, when the device cannot hold the launch's CTAs at
 // once (the caller then makes its launches).
 int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) {
     DevMesh& dm = m->dm;
@@ -2080,7 +2092,8 @@ int ue_step_n(ue_mesh* m, int64_t n, void* stream) {
         return UE_OK;
     }
     int64_t unit = 0;
-    if (runs_resident(m, &unit) && n >= unit) {
+    const int64_t from = resident_from(m, &unit);
+    if (from > 0 && n >= from) {
         bool used = false;
         const int rc = flow_steps(m, n, unit, s, &used);
         if (rc != UE_OK || used) return rc;
@@ -2167,11 +2180,12 @@ int ue_step_prepare(ue_mesh* m, void* stream) {
         ue::tbf1_fits(m->tb, m->ts.hdr.data()))
         return UE_OK;   // one launch per call, no graph
     int64_t unit = 0;
-    if (runs_resident(m, &unit)) {   // no graph either; the kernel is loaded, and its CTAs' room looked at, here
+    const int64_t from = resident_from(m, &unit);
+    if (from > 0) {   // the kernel is loaded, and its CTAs' room looked at, here
         const cudaError_t e = ue::flow_ready(m->flow, m->dm);
-        if (e == cudaSuccess) return UE_OK;
-        if (e != cudaErrorCooperativeLaunchTooLarge) UE_CUDA(e);
-        m->flow.grid = 0;
+        if (e == cudaErrorCooperativeLaunchTooLarge) m->flow.grid = 0;
+        else if (e != cudaSuccess) UE_CUDA(e);
+        else if (from <= unit) return UE_OK;   // no call replays a graph
     }
     if (m->variant == UE_VARIANT_BLOCKED) {
         for (int p = 0; p < 2; ++p) {

@@ -233,12 +233,13 @@ int ue_write_fields_f32(ue_mesh* m, const float* E, const float* B, const float*
 int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
 
 /* Advance n_steps leap-frog steps, asynchronously on `stream`.  A call of a graph chunk of steps
- * or more on a mesh small enough for the chip's registers and shared memory (about 1.2M
+ * or more (blocked meshes of few, small tiles: 64 or more, or none) on a mesh small enough for the chip's registers and shared memory (about 1.2M
  * triangles in FP32, 600k with a current or a frame, 300k in FP64, provided neighbouring triangles
  * are mostly stored close together; plain and blocked variants without UE_VARIANT_NO_RESIDENT,
  * graph_chunk >= 0) runs resident: one
  * cooperative launch for up to 1024 steps, with the same results bit for bit.  Its waits are
- * bounded; one that runs out is reported by ue_check (UE_ERR_TIMEOUT).  Errors of the launches are
+ * bounded (about a second); one that runs out is reported by ue_check (UE_ERR_TIMEOUT), and the fields are
+ * then of no use: some CTAs have written theirs back, others not.  Errors of the launches are
  * reported here; device-side conditions surface at the next synchronous call. */
 int ue_step_n(ue_mesh* m, int64_t n_steps, void* stream);
 
@@ -268,8 +269,8 @@ int ue_energy(ue_mesh* m, double* W, void* stream);
 
 /* Watchdog state (synchronous): *W = energy at the last check, *flag = 0 ok, 1 non-finite
  * energy, 2 energy grew by more than watchdog_growth between two checks.  Returns
- * UE_ERR_UNSTABLE when the flag is set, UE_ERR_TIMEOUT (flag 3) when a grid barrier of the
- * persistent variant ran out of time.  ue_write_fields re-arms both. */
+ * UE_ERR_UNSTABLE when the flag is set, UE_ERR_TIMEOUT (flag 3) when a wait of a resident, pipelined
+ * blocked or persistent launch ran out of time.  ue_write_fields re-arms both. */
 int ue_check(ue_mesh* m, double* W, int32_t* flag);
 
 /* Step counter used by the source time t = (n + 1/2) dt (checkpoint / resume).  ue_set_step

@@ -1068,6 +1068,10 @@ int learned_rho(ue_mesh* m, const ue_options& o, LearnedRes* r, cudaStream_t s) 
     return UE_OK;
 }
 
+// The watchdog's four words, then the resident step's control words: one copy reads both (ue_check took
+// 14 us, 23 with a copy of the error word after that of the watchdog's).
+constexpr int kWatchWords = 6;
+
 // Allocate the device arrays of a mesh (variant, precision, graph_chunk and block_depth set)
 // and upload its connectivity tables.  Coefficients are zeroed.
 int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
@@ -1125,7 +1129,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
             p = static_cast<std::remove_reference_t<decltype(p)>>(dev_alloc(m, count * elem, s));
             return p != nullptr;
         };
-        const bool all = get(fl.ctl, 4, 4) && get(fl.place, nt, 4) && get(fl.rec, flow_slots, 16) &&
+        const bool all = get(fl.place, nt, 4) && get(fl.rec, flow_slots, 16) &&
                          get(fl.sent, fl.sent_bytes, 1) && get(fl.cnt, fl.grid, 8) &&
                          (fl.grid == 1 || fl.edges > 0 || get(fl.hlist, (size_t)fl.grid * fl.halo, 4)) &&
                          (fl.edges == 0 || (get(fl.erec, (size_t)fl.grid * fl.edges, 8) && get(fl.ecnt, fl.grid, 8) &&
@@ -1142,7 +1146,7 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
             g = tb_chunk_launches(m) * m->block_depth;
         dm.gtab_size = g;
     }
-    ok = ok && alloc_into(m, m->wd, 4, 8, s) &&
+    ok = ok && alloc_into(m, m->wd, kWatchWords, 8, s) &&
          alloc_into(m, m->wd_part, ue::energy_parts(nei, nt), 8, s);
     if (!ok) {
         dev_free_all(m, s);
@@ -1152,8 +1156,9 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         return fail(UE_ERR_ALLOC, "device allocation failed");
     }
     {
-        if (m->flow.ctl) UE_CUDA(ue::launch_flow_init(m->flow, s));
         if (m->flow.grid > 0) {
+            m->flow.ctl = reinterpret_cast<unsigned*>(m->wd + 4);
+            UE_CUDA(ue::launch_flow_init(m->flow, s));
             if (m->flow.slot_words > 0) UE_CUDA(cudaMemsetAsync(m->flow.slots, 0, 16 * m->flow.slot_words, s));
             if (m->flow.epart)   // its counters
                 UE_CUDA(cudaMemsetAsync(m->flow.epart + (size_t)ue::kFlowChecks * m->flow.grid, 0, 8 * ue::kFlowChecks, s));
@@ -2257,7 +2262,7 @@ int ue_energy(ue_mesh* m, double* W, void* stream) {
 
 int ue_check(ue_mesh* m, double* W, int32_t* flag) {
     if (!m || !m->built) return fail(UE_ERR_ARG, "geometry not built");
-    double wd[4];
+    double wd[kWatchWords];
     UE_CUDA(cudaMemcpy(wd, m->wd, sizeof(wd), cudaMemcpyDeviceToHost));
     if (W) *W = wd[1];
     if (flag) *flag = (int32_t)wd[3];
@@ -2278,9 +2283,9 @@ int ue_check(ue_mesh* m, double* W, int32_t* flag) {
         }
     }
     if (m->flow.ctl) {
-        unsigned e = 0;
-        UE_CUDA(cudaMemcpy(&e, m->flow.ctl + 2, 4, cudaMemcpyDeviceToHost));
-        if (e) {
+        unsigned ctl[4];
+        std::memcpy(ctl, wd + 4, sizeof(ctl));
+        if (ctl[2]) {
             if (flag) *flag = 3;
             return fail(UE_ERR_TIMEOUT, "a wait of the resident step kernel ran out of time");
         }

@@ -85,13 +85,12 @@ extern "C" {
 typedef struct ue_mesh ue_mesh;  /* opaque, owned by the library until ue_mesh_free        */
 
 /* Device allocator hooks: alloc(bytes, stream, ctx) returns a device pointer or NULL;
- * free(ptr, stream, ctx) releases it.  Both NULL = cudaMalloc / cudaFree; blocks
- * of up to 64 MB are then cut from a few larger ones, which stay with the mesh for its next build, and
- * up to 64 MB of what calls have returned for its next calls; ue_mesh_free gives all back.  Where memory
- * is short the faster paths do without theirs (no resident step, half the power iteration's work
- * space) before a call fails.  Pointers must be
- * 16-byte aligned (the blocked kernels move records and fields with TMA bulk copies): one that
- * is not is handed back to free and the call fails with UE_ERR_ALLOC. */
+ * free(ptr, stream, ctx) releases it.  Both NULL = cudaMalloc / cudaFree; blocks of up to 64 MB are
+ * then cut from a few larger ones, which stay with the mesh for its next build, and up to 64 MB of what
+ * calls have returned for its next calls; ue_mesh_free gives all back.  Where memory is short the
+ * faster paths do without theirs (no resident step, half the power iteration's work space) before a
+ * call fails.  Pointers must be 16-byte aligned (the blocked kernels move records and fields with TMA
+ * bulk copies): one that is not is handed back to free and the call fails with UE_ERR_ALLOC. */
 typedef void* (*ue_alloc_fn)(size_t bytes, void* stream, void* ctx);
 typedef void (*ue_free_fn)(void* ptr, void* stream, void* ctx);
 
@@ -233,18 +232,20 @@ int ue_write_fields_f32(ue_mesh* m, const float* E, const float* B, const float*
 int ue_read_fields_f32(ue_mesh* m, float* E, float* B, float* j, void* stream);
 
 /* Advance n_steps leap-frog steps, asynchronously on `stream`.  A call of a graph chunk of steps
- * or more (blocked meshes of few, small tiles: 64 or more, or none) on a mesh small enough for the chip's registers and shared memory (about 1.2M
- * triangles in FP32, 600k with a current or a frame, 300k in FP64, provided neighbouring triangles
- * are mostly stored close together; plain and blocked variants without UE_VARIANT_NO_RESIDENT,
- * graph_chunk >= 0) runs resident: one
- * cooperative launch for up to 1024 steps, with the same results bit for bit.  Its waits are
- * bounded (about a second); one that runs out is reported by ue_check (UE_ERR_TIMEOUT), and the fields are
- * then of no use: some CTAs have written theirs back, others not.  Errors of the launches are
- * reported here; device-side conditions surface at the next synchronous call. */
+ * or more (blocked meshes whose tiles, at most as many as the device has SMs, are small: 64 steps or
+ * more, or at no length, where their launches are faster) on a mesh small enough for the chip's
+ * registers and shared memory (about 1.2M triangles in FP32, 600k with a current or a frame, 300k in
+ * FP64, provided neighbouring triangles are mostly stored close together; plain and blocked variants
+ * without UE_VARIANT_NO_RESIDENT, graph_chunk >= 0) runs resident: one cooperative launch for up to
+ * 1024 steps, with the same results bit for bit.  Its waits are bounded (about a second); one that runs
+ * out is reported by ue_check (UE_ERR_TIMEOUT), and the fields are then of no use: some CTAs have
+ * written theirs back, others not.  Errors of the launches are reported here; device-side conditions
+ * surface at the next synchronous call. */
 int ue_step_n(ue_mesh* m, int64_t n_steps, void* stream);
 
 /* The largest mesh or batch, in triangles of a vacuum medium without a frame, whose long calls run
- * resident on the current device (0: none, or no device; one whose neighbours lie far apart may not at any size). */
+ * resident on the current device (0: none, or no device; one whose neighbours lie far apart may not
+ * at any size). */
 int ue_resident_capacity(int32_t precision, int64_t* n_tris);
 
 /* Capture and instantiate now the CUDA graphs that ue_step_n replays (a blocked mesh: one per

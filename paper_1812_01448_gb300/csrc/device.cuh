@@ -156,7 +156,7 @@ __host__ __device__ __forceinline__ void frame_ij(const FrameDev& f, int64_t c, 
     }
 }
 
-// Everything the step kernels need, in the stored numbering.// Everything the step kernels need, in the stored numbering.
+// Everything the step kernels need, in the stored numbering.
 struct DevMesh {
     int precision = 0;            // UE_PREC_*
     int64_t n_t = 0, n_ei = 0, n_nodes = 0;

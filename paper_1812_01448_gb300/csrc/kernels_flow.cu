@@ -30,14 +30,21 @@
 // stored order; and it turns each triangle's neighbours into shared-memory addresses.
 //
 // What bounds it: one exchange through L2 (store, poll, barrier: about 0.8 us) up to some 1,000
-// triangles per SM, then the SM's issue slots (about 25 instructions per triangle; everything a slot
-// needs is at a compile-time offset from one register).  Measured per step on GB300, with a line
+// triangles per SM, then that exchange and the latency of a slot's chain of shared gathers and arithmetic
+// at 16 warps per SM (500k triangles: issue slots 32% busy, the shared-memory path 42%; an instruction
+// waits 11.5 cycles, 3.7 of them for the words of other CTAs and 1.4 at the barrier; about 25 instructions
+// per triangle, everything a slot needs at a compile-time offset from one register).  Measured per step on GB300, with a line
 // source, against graph replays of the two plain kernels: 90k triangles 0.84 us (6.2), 305k 1.20,
 // 1.2M 3.06 (9.3); one CTA alone 0.41 us on 1,040 triangles, 0.30 without a source (2.9).  Against
 // k_tbp (8 steps per launch, ring-ordered tiles) on 500k triangles 1.38 us (5.0), with a plasma
 // current 1.70 (k_tb 4.7), with a 16-cell PML frame 1.75 (10.0: the frame's tiles step by plain
 // launches).  With slots in stored order, neighbours found at each launch and unpacked addresses
 // hoisted into (then spilled) registers the same steps took 1.23, 1.89, -, 0.52, 2.44, 4.4 and 4.3.
+// 1,024 threads leave 64 registers each.  What still spills, in bytes of stores and loads per thread: two
+// slots with a current 44 and 56, with a frame 76 and 96, with both 196 and 216; the 16-slot shape, on
+// 512 threads, 152 and 172; FP64 with a frame, where a thread
+// computes its triangle's three edges, 380 to 1,032 and 464 to 1,168 (146k triangles with a 16-cell
+// frame: 8.1 us per step with a current, the launches 12.1).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -857,7 +864,8 @@ __global__ void __launch_bounds__(kShapes[SH].nt, 1) k_flow(const __grid_constan
 // each step updates the edges once, U passing through shared memory, and sums the triangles:
 // 10.5 FP64 instructions per triangle with a current instead of 18, plus one side of the edges whose
 // other triangle is in another CTA.  Those come last in a CTA's edge list; the thread that holds one
-// polls the other triangle's word itself, after the inner edges have been computed.  On 241k
+// polls the other triangle's word itself, after the inner edges have been computed.  The larger shape
+// spills: 84 bytes of stores and 212 of loads per thread, with a current 220 and 452.  On 241k
 // triangles with a current a step takes 6.7 us, in vacuum 3.9 (9.9 with a triangle's edges in its thread,
 // 11.9 as two launches).
 struct EdgeShape {

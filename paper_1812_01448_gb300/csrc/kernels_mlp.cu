@@ -287,7 +287,8 @@ __global__ void __launch_bounds__(128) k_mlp_fwd_few(const float* __restrict__ P
 // Bound by the warp-level tensor pipe: 40 products per 16 rows, about 15 cycles each on every SM
 // quarter, which is why the gain over fragments read from shared memory at every tile (460
 // instructions per tile, scalar input loads) is small.  5.07M rows: 192 -> 177 us at 384 threads per
-// SM (197 at 256, 195 at 512, where registers spill); 100k rows: 17 -> 13 us at 256 (15 at 384).
+// SM (197 at 256, 195 at 512, where registers spill); 100k rows: 17 -> 13 us at 256 (15 at 384).  Only
+// inputs off 16-byte alignment, of 50,000 rows or more, come here.
 template <int NT>
 __global__ void __launch_bounds__(NT, 1) k_mlp_fwd_bf16(const float* __restrict__ P,
                                                         const float* __restrict__ X, int64_t n,

@@ -27,7 +27,6 @@ namespace {
 
 thread_local std::string g_err;
 
-
 int fail(int code, const std::string& msg) {
     g_err = msg;
     return code;

@@ -1072,8 +1072,9 @@ int learned_rho(ue_mesh* m, const ue_options& o, LearnedRes* r, cudaStream_t s) 
 constexpr int kWatchWords = 6;
 
 // Allocate the device arrays of a mesh (variant, precision, graph_chunk and block_depth set)
-// and upload its connectivity tables.  Coefficients are zeroed.
-int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
+// and upload its connectivity tables.  Coefficients are zeroed.  work: bytes that the build takes for a
+// while after this.
+int alloc_and_upload(ue_mesh* m, size_t work, cudaStream_t s) {
     const HostMesh& h = m->hm;
     const size_t esz = m->precision == UE_PREC_FP64 ? 8 : 4;
     const int64_t nt = h.n_tris, nei = h.n_ei, nn = h.n_nodes, ne = h.n_edges;
@@ -1087,15 +1088,38 @@ int alloc_and_upload(ue_mesh* m, cudaStream_t s) {
         UE_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
         if (!coop || !ue::flow_shape(nt, n_fc, m->precision == UE_PREC_FP64, sms, m->flow)) m->flow = ue::FlowDev();
     }
-    const size_t flow_slots = (size_t)m->flow.grid * m->flow.cap, kAlign = ue::Arena::kAlign;
-    size_t reserve = (size_t)(16 * nn + nt * (150 + 3 * (int64_t)esz) + nei * (64 + 2 * (int64_t)esz) + 20 * ne) + 32 * kAlign;
-    // the resident step's arrays with them: on small meshes, whose slots are mostly spare, they are
-    // the larger part and took further chunks, 60 us each
-    if (m->flow.grid > 0)
-        reserve += 16 * flow_slots + m->flow.sent_bytes + 4 * (size_t)nt + 16 * (size_t)m->flow.slot_words +
-                      (size_t)m->flow.grid * (4 * (size_t)m->flow.halo + 16 + 8 * (size_t)m->flow.edges) +
-                      (m->flow.edges > 0 ? 4 * (size_t)nei : 0) + 16 * (size_t)n_fc +
-                      (m->watchdog_every > 0 ? 8 * (size_t)ue::kFlowChecks * (m->flow.grid + 1) : 0) + 12 * kAlign;
+    const size_t flow_slots = (size_t)m->flow.grid * m->flow.cap;
+    // the first chunks: these arrays, the resident step's (on small meshes, whose slots are mostly spare,
+    // the larger part), and the work space, whose room the caller maps and a source then take
+    size_t reserve = 0;
+    auto count = [&](int n, size_t bytes) {   // n arrays
+        if (bytes < ue::Arena::kOwn) reserve += n * ((bytes + ue::Arena::kAlign - 1) / ue::Arena::kAlign * ue::Arena::kAlign);
+    };
+    count(1, 16 * (size_t)nn);                   // xy
+    count(2, 12 * (size_t)nt);                   // nodes and codes of triangles
+    count(2, 16 * (size_t)nt + 64);              // O, records
+    count(3, 8 * (size_t)nt);                    // order, S, B for transfers
+    count(8, 8 * (size_t)nei + 64);              // nodes, opposite nodes, triangles, order, |e|, d, 1/|e|, d/|e|
+    count(2, 8 * (size_t)ne);                    // E, j for transfers
+    count(m->precision == UE_PREC_FP64 ? 2 : 1, esz * (size_t)nt + 64);   // B, dt/S
+    count(2, esz * (size_t)nei + 64);            // coefficients, U
+    if (m->flow.grid > 0) {
+        const ue::FlowDev& fl = m->flow;
+        count(1, 16 * flow_slots);
+        count(1, fl.sent_bytes);
+        count(1, 4 * (size_t)nt);
+        count(1, 16 * (size_t)fl.slot_words);
+        count(2, 8 * (size_t)fl.grid);
+        if (fl.grid > 1 && fl.edges == 0) count(1, 4 * (size_t)fl.grid * fl.halo);
+        if (fl.edges > 0) {
+            count(1, 8 * (size_t)fl.grid * fl.edges);
+            count(1, 4 * (size_t)nei + 4);
+        }
+        if (n_fc > 0) count(1, 16 * (size_t)n_fc);
+        if (m->watchdog_every > 0) count(1, 8 * (size_t)ue::kFlowChecks * (fl.grid + 1));
+    }
+    count(1, 8 * ue::energy_parts(nei, nt));
+    reserve += std::max(work < ue::Arena::kOwn ? work : 0, 4 * (size_t)(ne + nt)) + 32 * ue::Arena::kAlign;
     m->arena.reserve(reserve);
     bool ok = alloc_into(m, m->d_xy, 2 * nn, 8, s) && alloc_into(m, m->d_tri_nodes, 3 * nt, 4, s) &&
               alloc_into(m, m->d_edge_nodes, 2 * nei + 2, 4, s) &&
@@ -1581,7 +1605,7 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
         return fail(UE_ERR_ARG, "watchdog_every must be >= 0 and watchdog_growth > 1");
     m->watchdog_every = o.watchdog_every;
     m->watchdog_growth = o.watchdog_growth;
-    int arc = alloc_and_upload(m, s);
+    int arc = alloc_and_upload(m, o.dt_mode == UE_DT_POWER && !framed ? 8 * ue::power_iteration_work_doubles(h.n_tris, h.n_ei, nullptr, false) : 0, s);
     if (arc != UE_OK) return arc;
     if (framed && (arc = setup_frame(m, s)) != UE_OK) return arc;
     DevMesh& dm = m->dm;
@@ -1634,9 +1658,9 @@ int ue_geometry_build(ue_mesh* m, const ue_options* opt, void* stream) {
     const ue::FrameDev* frame = framed ? &m->fd : nullptr;
     bool small = false;   // half the work space, where memory is short
     auto power_work = [&]() {
-        if (alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, false), 8, s)) return true;
+        if (alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, false), 8, s, true)) return true;
         small = true;
-        return alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, true), 8, s);
+        return alloc_into(m, pwork, ue::power_iteration_work_doubles(nt, nei, frame, true), 8, s, true);
     };
     if (o.dt_mode == UE_DT_POWER && !power_work()) return fail(UE_ERR_ALLOC, "power iteration work space");
     UE_CUDA(cudaStreamSynchronize(s));
@@ -1790,7 +1814,7 @@ int ue_batch_create(ue_mesh* const* meshes, int32_t n, void* stream, ue_mesh** o
                 H.tile_tri_off.push_back(h.tile_tri_off[t] + t_off[i]);
         }
     }
-    int rc = alloc_and_upload(B, s);
+    int rc = alloc_and_upload(B, 0, s);
     if (rc != UE_OK) {
         ue_mesh_free(B);
         return rc;

@@ -119,6 +119,24 @@ int calls() {   // eigenmode calls of varying width between a build's arrays: 60
     return 0;
 }
 
+int large() {   // large blocks apart, chunks of several bounded
+    Arena a(ops);
+    a.reserve(300 << 20);
+    std::vector<char*> p;
+    for (int i = 0; i < 60; ++i) p.push_back((char*)a.alloc(i % 6 == 0 ? 20 << 20 : 3 << 20, false));
+    size_t own = 0;
+    for (auto& c : dev) {
+        CHECK(c.second <= Arena::kGrow);
+        own += c.second == (size_t)20 << 20;
+    }
+    CHECK(own == 10);
+    const int g = gets;
+    a.reset(true);
+    for (int i = 0; i < 60; ++i) CHECK(a.alloc(i % 6 == 0 ? 20 << 20 : 3 << 20, false));
+    CHECK(gets == g);
+    return 0;
+}
+
 int refused() {
     Arena a(ops);
     limit = 40 << 20;
@@ -150,14 +168,17 @@ int rebuilds() {
     a.reset(true);
     CHECK(build(8, 8 << 20) && gets == g);       // the same chunk
     CHECK(build(20, 0) && dev.size() > 1);       // grown past it
-    a.reset(true);
-    CHECK(total == 0);
     g = gets;
-    CHECK(build(28, 8 << 20) && gets == g + 1);  // one chunk of what that took
     a.reset(true);
-    CHECK(build(3, 3 << 20) && gets == g + 1);
+    CHECK(build(28, 28 << 20) && gets == g);     // the same chunks
+    void* t = a.alloc(20 << 20, true);
+    CHECK(t && a.release(t));
+    g = gets;
+    a.reset(true);
+    CHECK((t = a.alloc(20 << 20, true)) && gets == g && a.release(t));   // and what a call returned
+    CHECK(build(3, 3 << 20) && gets == g);
     a.reset(true);                               // far larger than the last build: not kept
-    CHECK(total == 0 && build(3, 3 << 20) && total == (size_t)3 << 20);
+    CHECK(total == 0 && build(3, 3 << 20) && total == (size_t)4 << 20);
     g = gets;
     cur = 1;                                     // another device
     a.reset(true);
@@ -169,7 +190,7 @@ int rebuilds() {
 
 int main(int, char** v) {
     const std::string s = v[1];
-    const int rc = s == "blocks" ? blocks() : s == "joining" ? joining() : s == "calls" ? calls() : s == "refused" ? refused() : rebuilds();
+    const int rc = s == "blocks" ? blocks() : s == "joining" ? joining() : s == "calls" ? calls() : s == "refused" ? refused() : s == "large" ? large() : rebuilds();
     if (rc == 0 && total != 0) { puts("chunks left"); return 1; }
     return rc;
 }
@@ -186,7 +207,7 @@ def driver(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("case", ["blocks", "joining", "calls", "refused", "rebuilds"])
+@pytest.mark.parametrize("case", ["blocks", "joining", "calls", "large", "refused", "rebuilds"])
 def test_arena(driver, case):
     r = subprocess.run([driver, case], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout

@@ -361,6 +361,7 @@ __device__ __forceinline__ void rearm_words(const Rearm& r) {
     if (r.flow_err) *r.flow_err = 0u;
 }
 cudaError_t launch_rearm(const Rearm& r, cudaStream_t s);
+cudaError_t launch_put_step(long long* step, long long v, cudaStream_t s);
 // The same transfers in caller order, with the caller's arrays (double, or float when f32) in
 // pinned host memory at their mapped device addresses, or in device memory: k_of[n_e] = stored
 // interior edge of each caller edge or -1, inv[n_t] = stored triangle of each caller triangle.

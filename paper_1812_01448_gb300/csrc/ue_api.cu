@@ -1255,10 +1255,6 @@ bool direct_transfer(const ue_mesh* m, const void* E, const void* B, const void*
     return (!E || dE) && (!B || dB) && (!j || dj) && (E || B || j);
 }
 
-__global__ void k_put_step(long long* step, long long v) {
-    if (threadIdx.x == 0) *step = v;
-}
-
 // What re-arms the watchdog and the error words after new fields are written.
 ue::Rearm rearm(ue_mesh* m) {
     m->since_check = 0;
@@ -1270,8 +1266,7 @@ ue::Rearm rearm(ue_mesh* m) {
 // steps, ordered before its kernels.
 int flush_step(ue_mesh* m, cudaStream_t s) {
     if (m->step_pending < 0) return UE_OK;
-    k_put_step<<<1, 32, 0, s>>>(m->dm.step, (long long)m->step_pending);
-    UE_CUDA(cudaGetLastError());
+    UE_CUDA(ue::launch_put_step(m->dm.step, (long long)m->step_pending, s));
     m->step_pending = -1;
     return UE_OK;
 }
@@ -1297,8 +1292,9 @@ int64_t resident_from(const ue_mesh* m, int64_t* unit) {
     return slots == 4 || (deep && slots == 6) ? std::max<int64_t>(*unit, 64) : *unit;
 }
 
-// n steps by the resident kernel, in place in the current field buffer (resident_from).  *used is false, and nothing stepped, when the device cannot hold the launch's CTAs at
-// once (the caller then makes its launches).
+// n steps by the resident kernel, in place in the current field buffer (resident_from).  *used is false,
+// and nothing stepped, when the device cannot hold the launch's CTAs at once (the caller then makes its
+// launches).
 int flow_steps(ue_mesh* m, int64_t n, int64_t unit, cudaStream_t s, bool* used) {
     DevMesh& dm = m->dm;
     const int64_t every = m->watchdog_every;

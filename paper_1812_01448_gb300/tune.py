@@ -102,7 +102,7 @@ def autotune_batch(items, candidates=DEFAULT_CANDIDATES, sample: int = 32, steps
     """Time every candidate on a spread sample of ``items``; return (best, table).  ``best``
     and each row of ``table`` are dicts with variant, tile_tris, block_depth, tb_threads and
     rate (triangle-steps/s on the sample), plus the tiler; the table also records the tuning
-    time and whether the whole batch fits the chip (its plain and blocked forms then step alike)."""
+    time and whether the whole batch fits the chip (its plain and blocked forms then mostly step alike)."""
     sizes = [ms.n_tris for ms, *_ in items]
     resident = sum(sizes) <= resident_capacity()
     idx = spread(sizes, sample)
